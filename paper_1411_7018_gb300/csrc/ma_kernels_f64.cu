@@ -23,6 +23,7 @@
 #include "ma_point.cuh"
 #include "ma_transfer.cuh"
 #include "ma_residual.cuh"
+#include "ma_smooth_f2.cuh"
 
 namespace ma {
 
@@ -81,6 +82,57 @@ cudaError_t launch_colour(double* u, const double* rhs, int n, double h6, unsign
     k_smooth_colour<PI, PJ, PK><<<grid, dim3(BX, BY), 0, s>>>(u, rhs, n, h6, ev);
     return cudaGetLastError();
 }
+
+// ---------------------------------------------------------------------------
+// The same sweep with the point update of ma_smooth_f2.cuh, on grids of
+// kF2MinN points a side and more.  Below, the colours of a level fill few
+// warps and the fused tail (which shares those sizes) runs the FP64 form.
+// Colours 3 and 4 follow each other in the order and differ in all three
+// parities, a corner offset the stencil lacks, so they are independent and one
+// launch sweeps both: blocks with z below nk0 take colour C, the rest colour
+// D.  NN > 0 fixes the grid size at compile time for the sizes that stream
+// from HBM: the 18 neighbour offsets become immediates of the loads.
+// ---------------------------------------------------------------------------
+template <int C, int NN>
+__device__ __forceinline__ void smooth_f2_block(double* u, const double* __restrict__ rhs, int n_rt,
+                                                const smoothf2::Params& P, unsigned long long* events, int bz)
+{
+    const int n = NN > 0 ? NN : n_rt;
+    const int i = ((C & 1) ? 1 : 2) + 2 * (int)(blockIdx.x * BX + threadIdx.x);
+    const int j = ((C & 2) ? 1 : 2) + 2 * (int)(blockIdx.y * BY + threadIdx.y);
+    const int k = ((C & 4) ? 1 : 2) + 2 * bz;
+    if (i > n - 2 || j > n - 2 || k > n - 2) return;
+    smoothf2::point<long long>(u, rhs, lin(i, j, k, n), n, (long long)n * n, P, events);
+}
+
+template <int C, int D, int NN>
+__global__ void __launch_bounds__(BX * BY) k_smooth_f2(double* u, const double* __restrict__ rhs, int n,
+                                                        smoothf2::Params P, unsigned long long* events, int nk0)
+{
+    const int bz = blockIdx.z;
+    if (C == D || bz < nk0) smooth_f2_block<C, NN>(u, rhs, n, P, events, bz);
+    else smooth_f2_block<D, NN>(u, rhs, n, P, events, bz - nk0);
+}
+
+template <int C, int D>
+cudaError_t launch_smooth_f2(double* u, const double* rhs, int n, const smoothf2::Params& P, unsigned long long* ev,
+                             cudaStream_t s)
+{
+    // colour 3 holds the larger i and j ranges of the pair (3, 4)
+    const int ni = colour_count(n, C & 1), nj = colour_count(n, (C >> 1) & 1), nk0 = colour_count(n, (C >> 2) & 1);
+    const int nk = nk0 + (C == D ? 0 : colour_count(n, (D >> 2) & 1));
+    const dim3 grid((ni + BX - 1) / BX, (nj + BY - 1) / BY, nk), blk(BX, BY);
+    count_launches(1);
+    switch (n) {
+    case 129: k_smooth_f2<C, D, 129><<<grid, blk, 0, s>>>(u, rhs, n, P, ev, nk0); break;
+    case 257: k_smooth_f2<C, D, 257><<<grid, blk, 0, s>>>(u, rhs, n, P, ev, nk0); break;
+    case 513: k_smooth_f2<C, D, 513><<<grid, blk, 0, s>>>(u, rhs, n, P, ev, nk0); break;
+    default: k_smooth_f2<C, D, 0><<<grid, blk, 0, s>>>(u, rhs, n, P, ev, nk0); break;
+    }
+    return cudaGetLastError();
+}
+
+constexpr int kF2MinN = 33;
 
 // ---------------------------------------------------------------------------
 // Block reduction of (max |x|, sum x^2) in a fixed order (deterministic).
@@ -976,6 +1028,20 @@ static inline double pow6(double h) { const double h2 = h * h; return 64.0 * h2 
 cudaError_t launch_smooth(double* u, const double* rhs, int n, double h, int nsweeps,
                           unsigned long long* events, cudaStream_t s)
 {
+    smoothf2::Params P;
+    if (n >= kF2MinN && smoothf2::make_params(h, &P)) {
+        for (int sw = 0; sw < nsweeps; ++sw) {
+            cudaError_t e;
+            if ((e = launch_smooth_f2<0, 0>(u, rhs, n, P, events, s)) != cudaSuccess) return e;
+            if ((e = launch_smooth_f2<1, 1>(u, rhs, n, P, events, s)) != cudaSuccess) return e;
+            if ((e = launch_smooth_f2<2, 2>(u, rhs, n, P, events, s)) != cudaSuccess) return e;
+            if ((e = launch_smooth_f2<3, 4>(u, rhs, n, P, events, s)) != cudaSuccess) return e;
+            if ((e = launch_smooth_f2<5, 5>(u, rhs, n, P, events, s)) != cudaSuccess) return e;
+            if ((e = launch_smooth_f2<6, 6>(u, rhs, n, P, events, s)) != cudaSuccess) return e;
+            if ((e = launch_smooth_f2<7, 7>(u, rhs, n, P, events, s)) != cudaSuccess) return e;
+        }
+        return cudaSuccess;
+    }
     const double h6 = pow6(h);
     for (int sw = 0; sw < nsweeps; ++sw) {
         cudaError_t e;

@@ -1345,6 +1345,7 @@ __global__ void k_f32_to_f64(const float* __restrict__ e, double* __restrict__ u
 // of the correction operator, rounded to FP32 from the FP64 Hessian the
 // residual already formed; the shell is not stored.
 struct CmF32Out {
+    static constexpr bool kUnorm = false;
     float* r;
     float* b;        // colour-major B store of the level
     float inv_4h2;   // 1 / (4 h^2)
@@ -1830,7 +1831,7 @@ cudaError_t launch_residual_f2(const double* u, const double* rhs, double* r, in
     count_launches(1);
     const int kz = n < 16 ? n : 16;
     const int kchunk = (n + kz - 1) / kz;
-    resid::launch_k_residual_f2(resid::grid_for(n, kz), s, u, rhs, resid::NaturalF2Out{r}, n,
+    resid::launch_k_residual_f2(resid::grid_for(n, kz), s, u, rhs, resid::NaturalF2Out<false>{r}, n,
                                 1.0 / (64.0 * h2 * h2 * h2), nullptr, kchunk);
     return cudaGetLastError();
 }

@@ -172,10 +172,9 @@ inline dim3 grid_for(int n, int kz) { return dim3((n + RX - 1) / RX, (n + RY - 1
 //    significant bits), with Knuth's two-sum and the FMA form of Dekker's
 //    exact product: |error| of a few 2^-46 relative to the sum of the
 //    magnitudes of the determinant's terms.
-// A stencil that spans up to three binades is handled the same way with each
-// significand shifted to the smallest exponent; one whose values change sign
-// across several binades, or are zero, huge or tiny, takes the FP64
-// evaluation instead.
+// A stencil that changes binade or sign is handled the same way, each value
+// as a fixed-point number of the largest one's scale with 7 bits to spare; one
+// whose largest value is zero, huge or tiny takes the FP64 evaluation.
 // ---------------------------------------------------------------------------
 namespace f2 {
 
@@ -221,6 +220,15 @@ __device__ __forceinline__ F2 add(F2 x, F2 y)
     return fast_two_sum(s.hi, s.lo + (x.lo + y.lo));
 }
 
+// The sum left unnormalised (|lo| may reach a few half ulps of hi): saves the
+// three dependent operations of the last step where the result only enters a
+// product, whose cross terms then drop |lo|^2, or an add.
+__device__ __forceinline__ F2 add_u(F2 x, F2 y)
+{
+    const F2 s = two_sum(x.hi, y.hi);
+    return {s.hi, s.lo + (x.lo + y.lo)};
+}
+
 __device__ __forceinline__ F2 neg(F2 x) { return {-x.hi, -x.lo}; }
 
 // Exact FP32 value of an integer y in [0, 2^23) or, for the signed form, in
@@ -230,12 +238,15 @@ __device__ __forceinline__ F2 neg(F2 x) { return {-x.hi, -x.lo}; }
 __device__ __forceinline__ float u23_to_f(unsigned y) { return __int_as_float(0x4B000000 | (int)y) - 8388608.0f; }
 __device__ __forceinline__ float s22_to_f(int y) { return __int_as_float(0x4B400000 + y) - 12582912.0f; }
 
-// x * scale as hi + lo, exact, for |x| < 2^45: x = a 2^23 + c with c in
-// [0, 2^23) and |a| < 2^22; scale a power of two.
-__device__ __forceinline__ F2 from_i45(long long x, float scale)
+// x * U as hi + lo, exact, for |x| < 2^45 and U a power of two: x = a 2^23 + c
+// with c in [0, 2^23) and |a| < 2^22.  Each piece is placed in the significand
+// of 1.5 2^23 (or 2^23) and one FMA scales it and takes the constant off, all
+// of it exact.  U23 = 2^23 U.
+__device__ __forceinline__ F2 from_i45(long long x, float U, float U23)
 {
-    const F2 r = fast_two_sum(s22_to_f((int)(x >> 23)) * 8388608.0f, u23_to_f((unsigned)x & 0x7fffffu));
-    return {r.hi * scale, r.lo * scale};
+    const float a = fmaf(__int_as_float(0x4B400000 + (int)(x >> 23)), U23, -12582912.0f * U23);
+    const float c = fmaf(__int_as_float(0x4B000000 | ((int)x & 0x7fffff)), U, -8388608.0f * U);
+    return fast_two_sum(a, c);
 }
 
 // x * scale as hi + lo, |x| < 2^68 (exact to ~2^-48 relative), scale a
@@ -266,13 +277,18 @@ __device__ __forceinline__ F2 from_f64(double x)
 }
 
 // det(H) for the symmetric 3x3 H = [[A, R, S], [R, B, T], [S, T, C]]: the
-// cofactor expansion along the first row.
+// cofactor expansion along the first row.  UNORM leaves the sums inside
+// unnormalised: about 15 of 91 operations fewer, and up to twice the error
+// (1.7e-15 against 1.4e-15 of max f on the rational-arithmetic test's 129^3
+// points, where FP64's rounded neighbour sums leave 4e-12).
+template <bool UNORM = false>
 __device__ __forceinline__ F2 det3(const F2& A, const F2& B, const F2& C, const F2& R, const F2& S, const F2& T)
 {
-    const F2 c1 = add(mul_u(B, C), neg(mul_u(T, T)));
-    const F2 c2 = add(mul_u(R, C), neg(mul_u(S, T)));
-    const F2 c3 = add(mul_u(R, T), neg(mul_u(B, S)));
-    return add(add(mul_u(A, c1), neg(mul_u(R, c2))), mul_u(S, c3));
+    auto sum = [](F2 x, F2 y) { return UNORM ? add_u(x, y) : add(x, y); };
+    const F2 c1 = sum(mul_u(B, C), neg(mul_u(T, T)));
+    const F2 c2 = sum(mul_u(R, C), neg(mul_u(S, T)));
+    const F2 c3 = sum(mul_u(R, T), neg(mul_u(B, S)));
+    return sum(sum(mul_u(A, c1), neg(mul_u(R, c2))), mul_u(S, c3));
 }
 
 // The exact paths accept binades E with 2^(E-1075) and the cube of the
@@ -289,18 +305,26 @@ struct ResF2 {
     f2::F2 H[6];   // 4 h^2 D^2_h u: xx, yy, zz, xy, xz, yz
 };
 
-__device__ __forceinline__ ResF2 residual_point_f2(const double* __restrict__ u, long long p, long long sy,
-                                                   long long sz, double rhs, f2::F2 inv_h6, double inv_h6_d)
+// H = 2^kexp 4 h^2 D^2_h u at interior point p, formed exactly in int64 and
+// held as two-float values; false (H unset) where the stencil's largest value
+// is zero, huge or tiny.  -20 <= kexp <= 40 keeps every scaled unit inside
+// FP32's range.
+template <typename Idx>
+__device__ __forceinline__ bool gather_f2(const double* __restrict__ u, Idx p, Idx sy, Idx sz, int kexp, f2::F2* H,
+                                          long long* centre)
 {
     const long long* q = reinterpret_cast<const long long*>(u) + p;
     const long long b0 = __ldg(q);
     const long long bxp = __ldg(q + 1), bxm = __ldg(q - 1);
     const long long byp = __ldg(q + sy), bym = __ldg(q - sy);
     const long long bzp = __ldg(q + sz), bzm = __ldg(q - sz);
-    const long long rpp = __ldg(q + sy + 1), rmm = __ldg(q - sy - 1), rpm = __ldg(q + sy - 1), rmp = __ldg(q - sy + 1);
-    const long long spp = __ldg(q + sz + 1), smm = __ldg(q - sz - 1), spm = __ldg(q + sz - 1), smp = __ldg(q - sz + 1);
-    const long long tpp = __ldg(q + sz + sy), tmm = __ldg(q - sz - sy), tpm = __ldg(q + sz - sy),
-                    tmp = __ldg(q - sz + sy);
+    const long long rpp = __ldg(q + (sy + 1)), rmm = __ldg(q - (sy + 1)), rpm = __ldg(q + (sy - 1)),
+                    rmp = __ldg(q - (sy - 1));
+    const long long spp = __ldg(q + (sz + 1)), smm = __ldg(q - (sz + 1)), spm = __ldg(q + (sz - 1)),
+                    smp = __ldg(q - (sz - 1));
+    const long long tpp = __ldg(q + (sz + sy)), tmm = __ldg(q - (sz + sy)), tpm = __ldg(q + (sz - sy)),
+                    tmp = __ldg(q - (sz - sy));
+    *centre = b0;
     // one sign and one exponent: the top 12 bits of every pattern equal b0's
     const unsigned h0 = (unsigned)(b0 >> 32);
     unsigned diff = 0;
@@ -310,65 +334,87 @@ __device__ __forceinline__ ResF2 residual_point_f2(const double* __restrict__ u,
     MA_F2_CK(spp); MA_F2_CK(smm); MA_F2_CK(spm); MA_F2_CK(smp);
     MA_F2_CK(tpp); MA_F2_CK(tmm); MA_F2_CK(tpm); MA_F2_CK(tmp);
 #undef MA_F2_CK
-    const int E = (int)((h0 >> 20) & 0x7ff);
-    ResF2 out;
-    auto finish = [&](long long A, long long B, long long C, long long R, long long S, long long T, float unit) {
-        // |x| < 2^45 for all six (the common case on fine grids): the two-piece
-        // conversion; otherwise the three-piece one
-        const unsigned long long big = 1ull << 45;
-        if ((unsigned long long)(A + big) < 2 * big && (unsigned long long)(B + big) < 2 * big &&
-            (unsigned long long)(C + big) < 2 * big && (unsigned long long)(R + big) < 2 * big &&
-            (unsigned long long)(S + big) < 2 * big && (unsigned long long)(T + big) < 2 * big) {
-            out.H[0] = f2::from_i45(A, unit);
-            out.H[1] = f2::from_i45(B, unit);
-            out.H[2] = f2::from_i45(C, unit);
-            out.H[3] = f2::from_i45(R, unit);
-            out.H[4] = f2::from_i45(S, unit);
-            out.H[5] = f2::from_i45(T, unit);
-        } else {
-            out.H[0] = f2::from_i64(A, unit);
-            out.H[1] = f2::from_i64(B, unit);
-            out.H[2] = f2::from_i64(C, unit);
-            out.H[3] = f2::from_i64(R, unit);
-            out.H[4] = f2::from_i64(S, unit);
-            out.H[5] = f2::from_i64(T, unit);
-        }
-        const f2::F2 d = f2::det3(out.H[0], out.H[1], out.H[2], out.H[3], out.H[4], out.H[5]);
-        out.val = f2::add(f2::from_f64(rhs), f2::neg(f2::mul(d, inv_h6)));
-    };
-    if ((diff >> 20) == 0 && E >= f2::kMinE && E <= f2::kMaxE) {
-        // ulp of the binade, negated for negative values
-        const float unit = __int_as_float(((E - 1075 + 127) << 23) | (int)(h0 & 0x80000000u));
-        finish(4 * ((bxp - b0) + (bxm - b0)), 4 * ((byp - b0) + (bym - b0)), 4 * ((bzp - b0) + (bzm - b0)),
-               (rpp - rmp) - (rpm - rmm), (spp - smp) - (spm - smm), (tpp - tmp) - (tpm - tmm), unit);
-        return out;
-    }
-    // The stencil spans a few binades: each value as its signed significand
-    // shifted to the smallest exponent among them, still exact in int64
-    // (53 bits + a shift of at most 3), in units of that exponent's ulp.
-    {
+    int E = (int)((h0 >> 20) & 0x7ff);
+    int sign = (int)(h0 & 0x80000000u);   // the ulp of the binade, negated for negative values
+    // a quarter of the diagonal entries, and the off-diagonal ones, in ulps
+    long long A, B, C, R, S, T;
+    if ((diff >> 20) == 0) {
+        if (E < f2::kMinE || E > f2::kMaxE) return false;
+        A = (bxp - b0) + (bxm - b0);
+        B = (byp - b0) + (bym - b0);
+        C = (bzp - b0) + (bzm - b0);
+        R = (rpp - rmp) - (rpm - rmm);
+        S = (spp - smp) - (spm - smm);
+        T = (tpp - tmp) - (tpm - tmm);
+    } else {
+        // The stencil changes binade or sign: each value as its signed
+        // significand in units of 2^-7 of the largest one's ulp.  Exact down
+        // to 2^-7 of the largest value, truncated by less than 2^-7 of its
+        // ulp below (a sum in FP64 rounds by half of one); four of them fit
+        // int64.
         auto ex = [](long long b) { return (int)((b >> 52) & 0x7ff); };
-        int emin = ex(b0), emax = emin;
-#define MA_F2_MM(v) emin = min(emin, ex(v)), emax = max(emax, ex(v))
+#define MA_F2_MM(v) E = max(E, ex(v))
         MA_F2_MM(bxp); MA_F2_MM(bxm); MA_F2_MM(byp); MA_F2_MM(bym); MA_F2_MM(bzp); MA_F2_MM(bzm);
         MA_F2_MM(rpp); MA_F2_MM(rmm); MA_F2_MM(rpm); MA_F2_MM(rmp);
         MA_F2_MM(spp); MA_F2_MM(smm); MA_F2_MM(spm); MA_F2_MM(smp);
         MA_F2_MM(tpp); MA_F2_MM(tmm); MA_F2_MM(tpm); MA_F2_MM(tmp);
 #undef MA_F2_MM
-        if (emax - emin <= 3 && emin >= f2::kMinE - 3 && emax <= f2::kMaxE) {
-            auto sg = [emin](long long b) -> long long {
-                const long long m = ((b & 0x000FFFFFFFFFFFFFll) | 0x0010000000000000ll) << (((b >> 52) & 0x7ff) - emin);
-                return b < 0 ? -m : m;
-            };
-            const long long m0 = sg(b0);
-            const float unit = __int_as_float((emin - 1075 + 127) << 23);
-            finish(4 * ((sg(bxp) - m0) + (sg(bxm) - m0)), 4 * ((sg(byp) - m0) + (sg(bym) - m0)),
-                   4 * ((sg(bzp) - m0) + (sg(bzm) - m0)), (sg(rpp) - sg(rmp)) - (sg(rpm) - sg(rmm)),
-                   (sg(spp) - sg(smp)) - (sg(spm) - sg(smm)), (sg(tpp) - sg(tmp)) - (sg(tpm) - sg(tmm)), unit);
-            return out;
-        }
+        if (E < f2::kMinE || E > f2::kMaxE) return false;
+        auto sg = [E, ex](long long b) -> long long {
+            const int e = ex(b);
+            const long long m = (b & 0x000FFFFFFFFFFFFFll) | (e > 0 ? 0x0010000000000000ll : 0ll);
+            const long long v = (m << 7) >> min(E - e, 63);
+            return b < 0 ? -v : v;
+        };
+        const long long m0 = sg(b0);
+        A = (sg(bxp) - m0) + (sg(bxm) - m0);
+        B = (sg(byp) - m0) + (sg(bym) - m0);
+        C = (sg(bzp) - m0) + (sg(bzm) - m0);
+        R = (sg(rpp) - sg(rmp)) - (sg(rpm) - sg(rmm));
+        S = (sg(spp) - sg(smp)) - (sg(spm) - sg(smm));
+        T = (sg(tpp) - sg(tmp)) - (sg(tpm) - sg(tmm));
+        E -= 7;
+        sign = 0;
     }
-    // FP64 evaluation (the stencil crosses a binade)
+    const float unit = __int_as_float(((E - 1075 + 127 + kexp) << 23) | sign);
+    const float unit4 = 4.0f * unit;
+    // |x| < 2^45 for all six (the common case on fine grids): the two-piece
+    // conversion; otherwise the three-piece one
+    int big = 0;
+#define MA_F2_HW(x) big |= (int)((x) >> 32) ^ (int)((x) >> 63)
+    MA_F2_HW(A); MA_F2_HW(B); MA_F2_HW(C); MA_F2_HW(R); MA_F2_HW(S); MA_F2_HW(T);
+#undef MA_F2_HW
+    if (big < (1 << 13)) {
+        const float u23 = 8388608.0f * unit, u423 = 8388608.0f * unit4;
+        H[0] = f2::from_i45(A, unit4, u423);
+        H[1] = f2::from_i45(B, unit4, u423);
+        H[2] = f2::from_i45(C, unit4, u423);
+        H[3] = f2::from_i45(R, unit, u23);
+        H[4] = f2::from_i45(S, unit, u23);
+        H[5] = f2::from_i45(T, unit, u23);
+    } else {
+        H[0] = f2::from_i64(A, unit4);
+        H[1] = f2::from_i64(B, unit4);
+        H[2] = f2::from_i64(C, unit4);
+        H[3] = f2::from_i64(R, unit);
+        H[4] = f2::from_i64(S, unit);
+        H[5] = f2::from_i64(T, unit);
+    }
+    return true;
+}
+
+template <bool UNORM = false>
+__device__ __forceinline__ ResF2 residual_point_f2(const double* __restrict__ u, long long p, long long sy,
+                                                   long long sz, double rhs, f2::F2 inv_h6, double inv_h6_d)
+{
+    ResF2 out;
+    long long b0;
+    if (gather_f2<long long>(u, p, sy, sz, 0, out.H, &b0)) {
+        const f2::F2 d = f2::det3<UNORM>(out.H[0], out.H[1], out.H[2], out.H[3], out.H[4], out.H[5]);
+        out.val = f2::add(f2::from_f64(rhs), f2::neg(f2::mul(d, inv_h6)));
+        return out;
+    }
+    // FP64 evaluation
     HessS H = gather_hess(u, p, sy, sz, __longlong_as_double(b0));
     const double v = fma(-det0(H), inv_h6_d, rhs);
     const double hs[6] = {H.A, H.B, H.C, H.R, H.S, H.T};
@@ -409,7 +455,7 @@ __device__ __forceinline__ void residual_f2_block(const double* __restrict__ u, 
                 out.zero(p);
                 continue;
             }
-            const ResF2 r = residual_point_f2(u, p, sy, sz, rhs[p], inv_h6, inv_h6_d);
+            const ResF2 r = residual_point_f2<Out::kUnorm>(u, p, sy, sz, rhs[p], inv_h6, inv_h6_d);
             const float v32 = r.val.hi;
             mx = fmaxf(mx, fabsf(v32));
             ss = fmaf(v32, v32, ss);
@@ -458,7 +504,10 @@ void launch_k_residual_f2(dim3 grid, cudaStream_t s, const double* u, const doub
 }
 
 // FP64 output of the two-float residual (hi + lo rounded once to double).
+// UNORM: the determinant with unnormalised sums (f2::det3).
+template <bool UNORM>
 struct NaturalF2Out {
+    static constexpr bool kUnorm = UNORM;
     double* r;
     __device__ __forceinline__ void put2(long long p, int, int, int, int, const ResF2& v) const
     {

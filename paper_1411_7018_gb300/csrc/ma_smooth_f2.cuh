@@ -1,0 +1,118 @@
+// ma_smooth_f2.cuh -- the FP64 smoother's point update (Section 2) with its
+// arithmetic off the FP64 pipe.  GB300 issues FP64 at 1/64 of its FP32 rate,
+// and the FP64 form of this update (35 FP64 operations a point) held that pipe
+// at 85 % of its peak: 137 us per colour at 257^3, against 20 us for the
+// bytes.  Here the six second differences are exact integers
+// (resid::gather_f2), the determinant at the shifted Hessian is taken in
+// two-float arithmetic, and two FP64 operations are left, the addition of the
+// change to the centre value.
+//
+// Measured per sweep under graph replay (Example 4 / random cosine, us), FP64
+// form -> this one: 257^3 1075 / 1076 -> 343 / 406, 129^3 152 / 152 -> 68 / 80,
+// 65^3 34 / 34 -> 25 / 26, 33^3 26 / 26 -> 20 / 20.  Bound at 257^3 by issue
+// (about 450 integer and FP32 instructions a point); at 33^3 by the length of
+// one point's dependent chain, 7 launches a sweep.  The random cosine's values
+// cross more binades, so more warps take gather_f2's fixed-point branch.
+//
+// Scaling: H = 2^k 4 h^2 D^2_h u with 2^k next to 1 / (4 h^2), so that the
+// entries have the size of D^2 u and their products stay inside FP32's range
+// whatever the step; the local equation det(H - z I) = (2^k 4 h^2)^3 rhs has the
+// root of Eq. (realroots) at v = v0 + z / (8 2^k).
+//
+// The root is found as smallest_root finds it: Newton in FP32 on the rounded
+// entries, then one Newton correction whose residual is evaluated to about 2^-45
+// of the entries' cube (in FP64 there), with the FP32 derivative.  The second
+// differences it starts from are exact, where the FP64 gather rounds the
+// neighbour sums to 2^-53 |u|, so from 17^3 up the result lies closer to the
+// exact update.  A point that smallest_root would not solve by that path
+// (rhs <= 0, degenerate, no convergence), or whose stencil gather_f2 refuses,
+// takes the FP64 form.
+#pragma once
+
+#include "ma_point.cuh"
+#include "ma_residual.cuh"
+
+namespace ma {
+namespace smoothf2 {
+
+struct Params {
+    double h6;      // 64 h^6, the right-hand side's factor of the FP64 form
+    double kz;      // 2^-k / 8: z to the change of u
+    float chi, clo; // (2^k 4 h^2)^3 as two floats
+    int kexp;       // k
+};
+
+// false: k would leave gather_f2's range, the grid keeps the FP64 form.
+inline bool make_params(double h, Params* P)
+{
+    const double h2 = h * h;
+    int e = 0;
+    const double m = frexp(4.0 * h2, &e);   // 4 h^2 = m 2^e, m in [1/2, 1)
+    P->kexp = m < 0.70710678118654752 ? 1 - e : -e;
+    if (P->kexp < -20 || P->kexp > 40) return false;
+    const double q = ldexp(4.0 * h2, P->kexp), c = q * q * q;
+    P->h6 = 64.0 * h2 * h2 * h2;
+    P->kz = ldexp(0.125, -P->kexp);
+    P->chi = (float)c;
+    P->clo = (float)(c - (double)P->chi);
+    return true;
+}
+
+// The FP64 form, for the points the fast path leaves.
+static __device__ __noinline__ void point_f64(double* u, const double* __restrict__ rhs, long long p, long long sy,
+                                              long long sz, double h6, unsigned long long* events)
+{
+    const double v0 = u[p];
+    const HessS H = gather_hess(u, p, sy, sz, v0);
+    bool nonconvex = false;
+    const double z = smallest_root(H, __dmul_rn(h6, rhs[p]), &nonconvex);
+    u[p] = fma(0.125, z, v0);
+    if (nonconvex && events) atomicAdd(events, 1ull);
+}
+
+// a - z as two floats, z one float
+__device__ __forceinline__ resid::f2::F2 shift(resid::f2::F2 a, float z)
+{
+    const resid::f2::F2 s = resid::f2::two_sum(a.hi, -z);
+    return resid::f2::fast_two_sum(s.hi, s.lo + a.lo);
+}
+
+template <typename Idx>
+__device__ __forceinline__ void point(double* u, const double* __restrict__ rhs, Idx p, Idx sy, Idx sz,
+                                      const Params& P, unsigned long long* events)
+{
+    using namespace resid;
+    f2::F2 H[6];
+    long long b0;
+    const double b = __ldg(rhs + p);
+    // rhs > 0 by its bits (NaN passes and fails to converge below)
+    if (gather_f2<Idx>(u, p, sy, sz, P.kexp, H, &b0) && __double_as_longlong(b) > 0) {
+        const f2::F2 r6 = f2::mul(f2::from_f64(b), f2::F2{P.chi, P.clo});
+        HessSf F;
+        F.A = H[0].hi; F.B = H[1].hi; F.C = H[2].hi;
+        F.R = H[3].hi; F.S = H[4].hi; F.T = H[5].hi;
+        const float scale = fabsf(F.A) + fabsf(F.B) + fabsf(F.C) + fabsf(F.R) + fabsf(F.S) + fabsf(F.T);
+        const float d0 = det_shift_f(F, 0.0f);
+        float z = is_pd<HessSf, float>(F, d0) ? 0.0f : gershgorin_low<HessSf, float>(F) - cbrtf(r6.hi);
+        bool conv = false;
+        for (int it = 0; it < 60; ++it) {
+            const float dz = __fdividef(det_shift_f(F, z) - r6.hi, minors_shift_f(F, z));
+            z += dz;
+            if (!isfinite(z)) break;
+            if (fabsf(dz) <= 2e-6f * scale) { conv = true; break; }
+        }
+        const float m = minors_shift_f(F, z);
+        // the scale's window keeps the cube's low parts inside FP32's range
+        if (conv && m > 0.05f * scale * scale && r6.hi > 0.0f && scale > 9.5e-7f && scale < 1.0e9f) {
+            const f2::F2 d = f2::det3<true>(shift(H[0], z), shift(H[1], z), shift(H[2], z), H[3], H[4], H[5]);
+            const f2::F2 g = f2::add_u(d, f2::neg(r6));
+            const float dz = __fdividef(g.hi + g.lo, m);
+            u[p] = fma(P.kz, f2d(z) + f2d(dz), __longlong_as_double(b0));
+            return;
+        }
+    }
+    point_f64(u, rhs, p, sy, sz, P.h6, events);
+}
+
+}  // namespace smoothf2
+}  // namespace ma

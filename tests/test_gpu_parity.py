@@ -456,3 +456,53 @@ def test_single_level_hierarchy_solves(n, precision):
     O.solve(ref, pr.f, pr.h, tol=1e-13, max_cycles=60, params=O.Params(coarsest_n=n))
     bound = 1e-10 if precision != M.MA_FP32 else 1e-6
     assert np.max(np.abs(got - ref)) <= bound * np.max(np.abs(ref))
+
+
+# ---------------------------------------------------------------------------
+# the two-float forms of the FP64 kernels (grids from 33^3 up)
+# ---------------------------------------------------------------------------
+
+@pytest.mark.parametrize("n", [33, 37, 67])   # the smallest grid that takes them, and ragged ones
+@pytest.mark.parametrize("length,shift", [(1.0, 0.0), (1e-3, 0.0), (1e3, 0.0), (1e-7, 0.0), (1.0, -1.5), (1.0, -40.0),
+                                          (1.0, 1e7)])
+def test_smooth_in_two_floats_over_scales_signs_and_binades(n, length, shift):
+    """Two sweeps against the oracle with the step and the values' binades
+    moved: u(x) = L^2 u0(x / L) + c has the Hessian of u0 on a cube of side L.
+    c = -1.5 puts a sign change through the grid, 1e7 and L = 1e-7 leave the
+    exact integer path (FP64 form).  A sweep rounds each stencil sum at
+    2^-53 |u|, which moves a point by a few |u| 2^-53: 1e-12 max|u| holds 4500
+    of them.  Where c dominates, the oracle's own rounding is the larger part."""
+    pr, u0 = perturbed("exp", n, 1e-4)
+    u0 = length ** 2 * u0 + shift
+    h = length / (n - 1)
+    f = pr.f.copy()
+    if abs(shift) < 1e6:
+        f[np.random.default_rng(1).random(f.shape) < 0.01] *= -1.0   # rhs <= 0: counted, FP64 form
+    else:
+        # the oracle's Hessian is rounding noise of |u| / h^2 here: solve for a rhs far above it
+        f *= 1e6
+    ref = u0.copy()
+    ev_ref = O.gs_sweep(ref, f, h) + O.gs_sweep(ref, f, h)
+    u = dev(u0)
+    ev = torch.zeros(1, dtype=torch.int64, device="cuda")
+    M.ma_smooth(u, dev(f), n, h, 2, events=ev)
+    got = host(u)
+    assert int(ev.item()) == ev_ref
+    assert np.max(np.abs(got - ref)) <= 1e-12 * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("n", [33, 35])
+def test_smooth_in_two_floats_from_a_zero_interior(n):
+    """Values that span every binade down to 0 (zero interior inside the
+    Dirichlet shell), Hessians far from positive definite there, a right-hand
+    side with negative entries: the bound of the test above."""
+    pr = P.make("exp", n)
+    u0, f = pr.initial(), pr.f.copy()
+    f[np.random.default_rng(3).random(f.shape) < 0.1] *= -1.0
+    ref = u0.copy()
+    ev_ref = O.gs_sweep(ref, f, pr.h)
+    u = dev(u0)
+    ev = torch.zeros(1, dtype=torch.int64, device="cuda")
+    M.ma_smooth(u, dev(f), n, pr.h, 1, events=ev)
+    assert int(ev.item()) == ev_ref
+    assert np.max(np.abs(host(u) - ref)) <= 1e-12 * np.max(np.abs(ref))
