@@ -195,7 +195,7 @@ cudaError_t mixed_fmg_step(ma_hierarchy* H, int l)
     cudaError_t e;
     if ((e = refresh_base(H, 0, l)) != cudaSuccess) return e;
     ma::Level& F = H->lev[l];
-    if ((e = ma::launch_residual64_to32(F.u, F.rhs, F.rhs32, F.bstore, F.n, F.h, H->partials, H->s)) != cudaSuccess)
+    if ((e = ma::launch_residual64_to32(F.u, F.rhs, F.rhs32, F.bstore, F.n, F.h, nullptr, H->s)) != cudaSuccess)
         return e;
     for (int c = 0; c < ma::kFmgCorrCycles; ++c)
         if ((e = corr_vcycle_from(H, l)) != cudaSuccess) return e;

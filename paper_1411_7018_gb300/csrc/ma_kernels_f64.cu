@@ -212,6 +212,60 @@ __global__ void __launch_bounds__(BX * BY) k_coarse_rhs(const double* __restrict
     coarse_rhs_block(wc, rc, bc, nc, inv_H6, blockIdx);
 }
 
+// out = r + det(D^2_h u) (SIGN = 1, the coarse right-hand side) or r - det
+// (SIGN = -1, the residual without norms) inside and 0 on the shell, with exact
+// integer second differences and a two-float determinant (resid::gather_f2): one
+// point a thread, the grid size at compile time for the sizes of a hierarchy's
+// larger levels.  The FP64 forms of the two were bound by the FP64 pipe
+// (257^3: 754 us residual, 800 us right-hand side); this one by issue, 254 us
+// at 257^3, 36 against 98 at 129^3, 8.4 against 22 at 65^3, 3.8 against 7.2 at
+// 33^3 (Example 4, graph replay).  Runs of planes a thread, as the residual
+// with norms walks them, keep more values live (76 registers for 64): 297 us.
+template <int NN, int SIGN>
+__global__ void __launch_bounds__(BX * BY) k_operator_f2(const double* __restrict__ u, const double* __restrict__ r,
+                                                         double* __restrict__ out, int n_rt, double inv_h6)
+{
+    using namespace resid;
+    const int n = NN > 0 ? NN : n_rt;
+    const int i = blockIdx.x * BX + threadIdx.x;
+    const int j = blockIdx.y * BY + threadIdx.y;
+    const int k = blockIdx.z;
+    if (i >= n || j >= n) return;
+    const long long p = lin(i, j, k, n), sz = (long long)n * n;
+    if (i == 0 || j == 0 || k == 0 || i == n - 1 || j == n - 1 || k == n - 1) {
+        out[p] = 0.0;
+        return;
+    }
+    f2::F2 H[6];
+    long long b0;
+    const double rv = __ldg(r + p);
+    if (gather_f2<long long>(u, p, n, sz, 0, H, &b0)) {
+        const float ih = (float)(SIGN * inv_h6);
+        const f2::F2 d = f2::mul(f2::det3<true>(H[0], H[1], H[2], H[3], H[4], H[5]),
+                                 f2::F2{ih, (float)(SIGN * inv_h6 - (double)ih)});
+        const f2::F2 v = f2::add(f2::from_f64(rv), d);
+        out[p] = f2d(v.hi) + f2d(v.lo);
+        return;
+    }
+    const HessS G = gather_hess(u, p, n, sz, __longlong_as_double(b0));
+    out[p] = fma(SIGN * det0(G), inv_h6, rv);
+}
+
+template <int SIGN>
+cudaError_t launch_operator_f2(const double* u, const double* r, double* out, int n, double inv_h6, cudaStream_t s)
+{
+    const dim3 g = xfer::grid_of(n), b(BX, BY);
+    switch (n) {
+    case 33: k_operator_f2<33, SIGN><<<g, b, 0, s>>>(u, r, out, n, inv_h6); break;
+    case 65: k_operator_f2<65, SIGN><<<g, b, 0, s>>>(u, r, out, n, inv_h6); break;
+    case 129: k_operator_f2<129, SIGN><<<g, b, 0, s>>>(u, r, out, n, inv_h6); break;
+    case 257: k_operator_f2<257, SIGN><<<g, b, 0, s>>>(u, r, out, n, inv_h6); break;
+    case 513: k_operator_f2<513, SIGN><<<g, b, 0, s>>>(u, r, out, n, inv_h6); break;
+    default: k_operator_f2<0, SIGN><<<g, b, 0, s>>>(u, r, out, n, inv_h6); break;
+    }
+    return cudaGetLastError();
+}
+
 // rhs := f, u := g (whole grids); counts interior points with f not finite
 // or f <= 0 and shell points with g not finite.
 __global__ void k_copy_rhs_bc(const double* __restrict__ f, const double* __restrict__ g, double* __restrict__ rhs,
@@ -1071,6 +1125,12 @@ cudaError_t launch_residual(const double* u, const double* rhs, double* r, int n
     count_launches(1);
     const dim3 g = reduce_grid(n);
     const int kchunk = (n + (int)g.z - 1) / (int)g.z;
+    if (n >= kF2MinN) {
+        if (!partials) return launch_operator_f2<-1>(u, rhs, r, n, 1.0 / pow6(h), s);
+        resid::launch_k_residual_f2(resid::grid_for(n, g.z), s, u, rhs, resid::NaturalF2Out<true>{r}, n, 1.0 / pow6(h),
+                                    partials, kchunk);
+        return cudaGetLastError();
+    }
     resid::k_residual_col<resid::NaturalF64Out><<<resid::grid_for(n, g.z), dim3(resid::RX, resid::RY), 0, s>>>(
         u, rhs, resid::NaturalF64Out{r}, n, 1.0 / pow6(h), partials, kchunk);
     return cudaGetLastError();
@@ -1127,7 +1187,9 @@ cudaError_t launch_restrict_level(const double* uf, const double* rf, int nf, do
 cudaError_t launch_coarse_rhs(const double* wc, const double* rc, double* bc, int nc, double H, cudaStream_t s)
 {
     count_launches(1);
-    k_coarse_rhs<<<grid_of(nc), dim3(BX, BY), 0, s>>>(wc, rc, bc, nc, 1.0 / pow6(H));
+    const double inv_H6 = 1.0 / pow6(H);
+    if (nc >= kF2MinN) return launch_operator_f2<1>(wc, rc, bc, nc, inv_H6, s);
+    k_coarse_rhs<<<grid_of(nc), dim3(BX, BY), 0, s>>>(wc, rc, bc, nc, inv_H6);
     return cudaGetLastError();
 }
 

@@ -1841,7 +1841,8 @@ cudaError_t launch_residual64_to32(const double* u, const double* rhs, float* r_
 {
     const double h2 = h * h;
     count_launches(1);
-    const int kz = n < 16 ? n : 16;
+    // without norms one plane a block (the partials' count fixes the grid with them)
+    const int kz = n < 16 || !partials ? n : 16;
     const int kchunk = (n + kz - 1) / kz;
     resid::launch_k_residual_f2(resid::grid_for(n, kz), s, u, rhs, CmF32Out{r_cm, (float*)bstore, (float)(0.25 / h2)},
                                 n, 1.0 / (64.0 * h2 * h2 * h2), partials, kchunk);

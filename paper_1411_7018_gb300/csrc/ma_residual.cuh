@@ -488,14 +488,17 @@ __global__ void __launch_bounds__(RX * RY) k_residual_f2(const double* __restric
     residual_f2_block<Out, NN>(u, rhs, out, n, inv_h6, partials, kchunk, blockIdx, gridDim);
 }
 
-// Launch with the grid size fixed at compile time for the sizes that stream
-// from HBM.
+// Launch with the grid size fixed at compile time for the sizes of a
+// hierarchy's larger levels (the runtime form takes up to 115 registers for
+// its 64-bit offsets).
 template <typename Out>
 void launch_k_residual_f2(dim3 grid, cudaStream_t s, const double* u, const double* rhs, Out out, int n,
                           double inv_h6, double* partials, int kchunk)
 {
     const dim3 blk(RX, RY);
     switch (n) {
+    case 33: k_residual_f2<Out, 33><<<grid, blk, 0, s>>>(u, rhs, out, n, inv_h6, partials, kchunk); break;
+    case 65: k_residual_f2<Out, 65><<<grid, blk, 0, s>>>(u, rhs, out, n, inv_h6, partials, kchunk); break;
     case 129: k_residual_f2<Out, 129><<<grid, blk, 0, s>>>(u, rhs, out, n, inv_h6, partials, kchunk); break;
     case 257: k_residual_f2<Out, 257><<<grid, blk, 0, s>>>(u, rhs, out, n, inv_h6, partials, kchunk); break;
     case 513: k_residual_f2<Out, 513><<<grid, blk, 0, s>>>(u, rhs, out, n, inv_h6, partials, kchunk); break;

@@ -506,3 +506,24 @@ def test_smooth_in_two_floats_from_a_zero_interior(n):
     M.ma_smooth(u, dev(f), n, pr.h, 1, events=ev)
     assert int(ev.item()) == ev_ref
     assert np.max(np.abs(host(u) - ref)) <= 1e-12 * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("name,n", [("exp", 33), ("sine", 35), ("cosine", 63), ("sine", 65), ("exp", 129)])
+def test_two_float_residual_and_coarse_rhs_match_oracle(name, n):
+    """The residual and the coarse right-hand side on the sizes that take the
+    two-float forms (each compile-time size and ragged ones; sine changes sign
+    inside the grid), with the FP64 kernels' bound (the oracle's own rounding
+    is the larger part of it), and 0 on the shell."""
+    pr, u0 = perturbed(name, n, 1e-6)
+    r = torch.full_like(dev(u0), 7.0)
+    M.ma_residual(dev(u0), dev(pr.f), r, n, pr.h)
+    got, ref = host(r), O.residual(u0, pr.f, pr.h)
+    assert np.max(np.abs(got - ref)) <= _residual_bound(u0, pr.h, name)
+    r0 = 1e-3 * np.random.default_rng(n).standard_normal((n, n, n))
+    b = torch.full_like(dev(u0), 7.0)
+    M.ma_coarse_rhs(dev(u0), dev(r0), b, n, pr.h)
+    gb = host(b)
+    assert np.max(np.abs(gb - O.coarse_rhs(u0, r0, pr.h))) <= _residual_bound(u0, pr.h, name)
+    shell = np.ones_like(gb, bool)
+    shell[1:-1, 1:-1, 1:-1] = False
+    assert np.all(got[shell] == 0.0) and np.all(gb[shell] == 0.0)
