@@ -958,16 +958,213 @@ __global__ void __launch_bounds__(BX * BY) k_coarse_rhs_corr(const float* __rest
     coarse_rhs_corr_block(w, bstore, resc, rhs_cm, n, inv_h2, blockIdx);
 }
 
-// Coarsest correction grid: one block, shared memory, FP32 sweeps until
-// max|de| <= 2e-6 max|e| (FP32 resolution of the correction; at most 40
-// sweeps), or a fixed count.
-constexpr int CT = 256;
+// ---- correction grids in one block's shared memory ---------------------------
+// A sweep of a small grid is a chain of colour phases, each as long as one
+// point's dependent chain (loads, Hessian, the Newton steps of the root) and a
+// barrier; the points of a phase fill few warps.  So a phase runs on no more
+// warps than it has points for (a whole block's barrier, and idle warps at
+// it, cost more than the phase), a point's position comes from multiplications
+// by reciprocals in place of integer divisions, and its B and rhs, which no
+// phase writes, are loaded one phase ahead.
 
 __device__ __forceinline__ S3f corr_hess_sm(const float* e, int p, int sy, int sz, float e0, float inv_h2)
 {
     return hess_from_diff([&](int di, int dj, int dk) -> float { return e[p + di + dj * sy + dk * sz] - e0; },
                           inv_h2);
 }
+
+// Index arithmetic of a grid of n <= 17 points a side.  t / d as
+// t (65536 / d + 1) >> 16: exact for t d <= 65536.
+struct SmallGrid {
+    int n, a, b, ma, mb, mi, mn;   // a, b: interior indices of parity 0, 1; m*: reciprocals of a, b, n - 2, n
+    __device__ __forceinline__ explicit SmallGrid(int n_) : n(n_), a((n_ - 3) / 2), b((n_ - 1) / 2)
+    {
+        ma = a > 0 ? 65536 / a + 1 : 0;
+        mb = 65536 / b + 1;
+        mi = 65536 / (n - 2) + 1;
+        mn = 65536 / n + 1;
+    }
+    __device__ __forceinline__ int count(int c) const
+    {
+        return ((c & 1) ? b : a) * ((c & 2) ? b : a) * ((c & 4) ? b : a);
+    }
+    __device__ __forceinline__ int offset(int c) const   // cm_offset
+    {
+        const int sj = (c & 2) ? b : a, sk = (c & 4) ? b : a;
+        return ((c & 4) ? (a + b) * (a + b) * a : 0) + ((c & 2) ? (a + b) * a * sk : 0) + ((c & 1) ? a * sj * sk : 0);
+    }
+    // linear index of point t of colour c
+    __device__ __forceinline__ int point(int c, int t) const
+    {
+        const bool pi = c & 1, pj = c & 2, pk = c & 4;
+        const int y0 = (t * (pi ? mb : ma)) >> 16, x = t - y0 * (pi ? b : a);
+        const int z = (y0 * (pj ? mb : ma)) >> 16, y = y0 - z * (pj ? b : a);
+        return (((pk ? 1 : 2) + 2 * z) * n + (pj ? 1 : 2) + 2 * y) * n + (pi ? 1 : 2) + 2 * x;
+    }
+    // interior point q in natural order: (i, j, k), its linear index returned
+    __device__ __forceinline__ int interior(int q, int* i, int* j, int* k) const
+    {
+        const int y0 = (q * mi) >> 16, z = (y0 * mi) >> 16;
+        *i = 1 + q - y0 * (n - 2);
+        *j = 1 + y0 - z * (n - 2);
+        *k = 1 + z;
+        return (*k * n + *j) * n + *i;
+    }
+    // colour-major slot and colour count of interior point (i, j, k)
+    __device__ __forceinline__ int slot(int i, int j, int k, int* cnt, int* off) const
+    {
+        const int c = (i & 1) | ((j & 1) << 1) | ((k & 1) << 2);
+        const int ni = (i & 1) ? b : a, nj = (j & 1) ? b : a;
+        *cnt = count(c);
+        *off = offset(c);
+        return (((k - 1) >> 1) * nj + ((j - 1) >> 1)) * ni + ((i - 1) >> 1);
+    }
+};
+
+__device__ __forceinline__ S3f load_b_sm(const float* b, int cnt)
+{
+    S3f B;
+    B.xx = b[0]; B.yy = b[cnt]; B.zz = b[2 * cnt]; B.xy = b[3 * cnt]; B.xz = b[4 * cnt]; B.yz = b[5 * cnt];
+    return B;
+}
+
+// Warps that run a grid's colour phases, and their barrier: one warp up to
+// 5^3 (at most 9 points a phase), four up to 9^3 (at most 91), the block above.
+__device__ __forceinline__ int phase_threads(int n, int block) { return n <= 5 ? 32 : (n <= 9 ? 128 : block); }
+
+__device__ __forceinline__ void phase_barrier(int n)
+{
+    if (n <= 5) __syncwarp();
+    else if (n <= 9) asm volatile("bar.sync 1, 128;" ::: "memory");
+    else __syncthreads();
+}
+
+// Visits the points of a phase sequence: phase q (0 .. nq - 1) holds colour
+// first(q) and, where it is not negative, colour second(q).  body(p, B, r,
+// slot_colour...) updates one point.  NT threads of the block enter.
+template <typename First, typename Second, typename Body>
+__device__ __forceinline__ void run_phases(const SmallGrid& G, const float* sb, const float* sr, int nq, int nt,
+                                           First first, Second second, Body body)
+{
+    struct Pt {
+        int p, cnt;
+        const float *b, *r;
+    };
+    const int tid = threadIdx.x;
+    auto locate = [&](int q, int t, Pt* P) -> bool {
+        int c = first(q);
+        const int d = second(q), nc = G.count(c);
+        if (t >= nc) {
+            if (d < 0) return false;
+            t -= nc;
+            c = d;
+            if (t >= G.count(d)) return false;
+        }
+        const int off = G.offset(c);
+        P->cnt = G.count(c);
+        P->p = G.point(c, t);
+        P->b = sb + 6 * off + t;
+        P->r = sr + off + t;
+        return true;
+    };
+    if (G.n <= 9) {   // at most one point a thread: its B and rhs one phase ahead
+        Pt cur, nxt;
+        S3f B = {0, 0, 0, 0, 0, 0}, Bn = B;
+        float r = 0.0f, rn = 0.0f;
+        bool on = locate(0, tid, &cur);
+        if (on) {
+            B = load_b_sm(cur.b, cur.cnt);
+            r = *cur.r;
+        }
+        for (int q = 0; q < nq; ++q) {
+            const bool onn = q + 1 < nq && locate(q + 1, tid, &nxt);
+            if (onn) {
+                Bn = load_b_sm(nxt.b, nxt.cnt);
+                rn = *nxt.r;
+            }
+            if (on) body(cur.p, B, r);
+            phase_barrier(G.n);
+            on = onn;
+            cur = nxt;
+            B = Bn;
+            r = rn;
+        }
+        return;
+    }
+    for (int q = 0; q < nq; ++q) {
+        const int tot = G.count(first(q)) + (second(q) >= 0 ? G.count(second(q)) : 0);
+        for (int t = tid; t < tot; t += nt) {
+            Pt P;
+            if (locate(q, t, &P)) body(P.p, load_b_sm(P.b, P.cnt), *P.r);
+        }
+        phase_barrier(G.n);
+    }
+}
+
+// Ascending colour order in 7 phases: colours 3 and 4 differ in all three
+// parities, so they are independent and share one.
+__device__ __forceinline__ int asc_first(int q) { return q <= 3 ? q : q + 1; }
+__device__ __forceinline__ int asc_second(int q) { return q == 3 ? 4 : -1; }
+
+// Coarsest correction grid in shared memory: FP32 sweeps in ascending order
+// until max|de| <= 2e-6 max|e| (FP32 resolution of the correction; at most 40
+// sweeps), or a fixed count.  Every thread of the block enters; ends with a
+// block barrier.
+__device__ __forceinline__ void coarsest_corr_sm(float* se, const float* sb, const float* sr, int n, float inv_h2,
+                                                 float h2half, int sweeps, unsigned long long* ev)
+{
+    const int max_sweeps = sweeps > 0 ? sweeps : 40;
+    const int nt = phase_threads(n, (int)blockDim.x);
+    __shared__ float red[32][2];
+    if (n == 3) {   // one unknown
+        if (threadIdx.x == 0) {
+            const S3f B = load_b_sm(sb, 1);
+            const float r = sr[0];
+            float v = se[13];
+            for (int s = 0; s < max_sweeps; ++s) {
+                const float e0 = v;
+                const S3f K = corr_hess_sm(se, 13, 3, 9, e0, inv_h2);
+                bool nonconvex = false;
+                v = fmaf(h2half, corr_root(B, K, r, &nonconvex), e0);
+                *ev += nonconvex ? 1ull : 0ull;
+                if (sweeps == 0 && fabsf(v - e0) <= 2e-6f * fabsf(v)) break;
+            }
+            se[13] = v;
+        }
+    } else if ((int)threadIdx.x < nt) {
+        const SmallGrid G(n);
+        for (int s = 0; s < max_sweeps; ++s) {
+            float du = 0.0f, um = 0.0f;
+            run_phases(G, sb, sr, 7, nt, asc_first, asc_second, [&](int p, const S3f& B, float r) {
+                const float e0 = se[p];
+                const S3f K = corr_hess_sm(se, p, n, n * n, e0, inv_h2);
+                bool nonconvex = false;
+                const float v = fmaf(h2half, corr_root(B, K, r, &nonconvex), e0);
+                se[p] = v;
+                du = fmaxf(du, fabsf(v - e0));
+                um = fmaxf(um, fabsf(v));
+                *ev += nonconvex ? 1ull : 0ull;
+            });
+            if (sweeps > 0) continue;
+            for (int o = 16; o > 0; o >>= 1) {
+                du = fmaxf(du, __shfl_xor_sync(0xffffffffu, du, o));
+                um = fmaxf(um, __shfl_xor_sync(0xffffffffu, um, o));
+            }
+            if (nt > 32) {
+                if ((threadIdx.x & 31) == 0) { red[threadIdx.x >> 5][0] = du; red[threadIdx.x >> 5][1] = um; }
+                phase_barrier(n);
+                du = um = 0.0f;
+                for (int w = 0; w < nt / 32; ++w) { du = fmaxf(du, red[w][0]); um = fmaxf(um, red[w][1]); }
+                phase_barrier(n);   // red is free again
+            }
+            if (du <= 2e-6f * um) break;
+        }
+    }
+    __syncthreads();
+}
+
+// Coarsest correction grid: one block.
+constexpr int CT = 256;
 
 // smem: e (n^3, natural), B (6 floats per interior point, colour-major),
 // rhs (colour-major).
@@ -981,57 +1178,12 @@ __device__ __forceinline__ void coarsest_corr_body(float* e, const float* __rest
     float* se = smf;
     float* sb = smf + m;
     float* sr = smf + m + 6 * mi;
-    __shared__ float red[CT / 32][2];
-    __shared__ int stop;
     for (int q = threadIdx.x; q < m; q += CT) se[q] = e[q];
     for (int q = threadIdx.x; q < 6 * mi; q += CT) sb[q] = bstore[q];
     for (int q = threadIdx.x; q < mi; q += CT) sr[q] = rhs_cm[q];
     __syncthreads();
-    const int max_sweeps = sweeps > 0 ? sweeps : 40;
     unsigned long long ev = 0;
-    for (int s = 0; s < max_sweeps; ++s) {
-        float du = 0.0f, um = 0.0f;
-        long long off = 0;
-        for (int c = 0; c < 8; ++c) {
-            const int pi = c & 1, pj = (c >> 1) & 1, pk = (c >> 2) & 1;
-            const int ni = colour_count(n, pi), nj = colour_count(n, pj), nk = colour_count(n, pk);
-            const int cnt = (ni > 0 && nj > 0 && nk > 0) ? ni * nj * nk : 0;
-            for (int t = threadIdx.x; t < cnt; t += CT) {
-                const int i = (pi ? 1 : 2) + 2 * (t % ni);
-                const int j = (pj ? 1 : 2) + 2 * ((t / ni) % nj);
-                const int k = (pk ? 1 : 2) + 2 * (t / (ni * nj));
-                const int p = (k * n + j) * n + i;
-                const float e0 = se[p];
-                const float* b = sb + 6 * off + t;
-                S3f B;
-                B.xx = b[0]; B.yy = b[cnt]; B.zz = b[2 * cnt]; B.xy = b[3 * cnt]; B.xz = b[4 * cnt]; B.yz = b[5 * cnt];
-                const S3f K = corr_hess_sm(se, p, n, n * n, e0, inv_h2);
-                bool nonconvex = false;
-                const float z = corr_root(B, K, sr[off + t], &nonconvex);
-                const float v = fmaf(h2half, z, e0);
-                se[p] = v;
-                du = fmaxf(du, fabsf(v - e0));
-                um = fmaxf(um, fabsf(v));
-                ev += nonconvex ? 1ull : 0ull;
-            }
-            off += cnt;
-            __syncthreads();
-        }
-        if (sweeps > 0) continue;
-        for (int o = 16; o > 0; o >>= 1) {
-            du = fmaxf(du, __shfl_down_sync(0xffffffffu, du, o));
-            um = fmaxf(um, __shfl_down_sync(0xffffffffu, um, o));
-        }
-        if ((threadIdx.x & 31) == 0) { red[threadIdx.x >> 5][0] = du; red[threadIdx.x >> 5][1] = um; }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            float a = 0.0f, b = 0.0f;
-            for (int w = 0; w < CT / 32; ++w) { a = fmaxf(a, red[w][0]); b = fmaxf(b, red[w][1]); }
-            stop = (a <= 2e-6f * b) ? 1 : 0;
-        }
-        __syncthreads();
-        if (stop) break;
-    }
+    coarsest_corr_sm(se, sb, sr, n, inv_h2, h2half, sweeps, &ev);
     for (int q = threadIdx.x; q < m; q += CT) e[q] = se[q];
     if (events && ev) atomicAdd(events, ev);
 }
@@ -1056,7 +1208,7 @@ __global__ void __launch_bounds__(CT) k_coarsest_corr(float* e, const float* __r
 // bound levels by one.
 // ---------------------------------------------------------------------------
 constexpr int kTailMaxN = 17;
-constexpr int TT = 1024;
+constexpr int TT = 512;
 
 struct TailLevel {
     int n;
@@ -1065,6 +1217,7 @@ struct TailLevel {
     float* e;            // global iterate (read on the top level, written back there)
     const float* b;      // global colour-major B store
     const float* rhs;    // global colour-major rhs (read on the top level)
+    int oe, ow, orr, ob, orhs;   // places of the level's fields in shared memory, in floats (set_tail_offsets)
 };
 
 struct TailArgs {
@@ -1080,6 +1233,22 @@ __host__ __device__ inline int tail_level_floats(int n, bool top)
     return m /* e */ + (top ? 0 : m) /* w */ + m /* res */ + 6 * mi /* B */ + mi /* rhs */;
 }
 
+// Lays the levels out in shared memory; the host fills the offsets in, so that
+// every access is an offset from the block's base.
+inline void set_tail_offsets(TailArgs* A)
+{
+    int q = 0;
+    for (int l = 0; l < A->nlev; ++l) {
+        TailLevel& V = A->lev[l];
+        const int m = V.n * V.n * V.n, mi = (V.n - 2) * (V.n - 2) * (V.n - 2);
+        V.oe = q; q += m;
+        V.ow = q; q += l > 0 ? m : 0;
+        V.orr = q; q += m;
+        V.ob = q; q += 6 * mi;
+        V.orhs = q; q += mi;
+    }
+}
+
 struct TailSmem {
     float *e, *w, *r, *b, *rhs;
 };
@@ -1089,79 +1258,28 @@ struct TailSmem {
 // that the tail and the level-by-level cycle give the same bits under any
 // tuning.  Pairs: colours c and c^7 in one phase (independent: the stencil
 // of a colour-c point holds every colour but c^7), phases (0, 7), (1, 6),
-// (2, 5), (3, 4), the colour-pair kernel's sweep; otherwise one colour a
-// phase in ascending order.  Each point runs the separate kernels'
-// arithmetic; a colour with no points takes no barrier.
-__device__ __forceinline__ void tail_smooth(const TailSmem& S, int n, float inv_h2, float h2half, int nsw, bool pairs,
-                                            unsigned long long* ev)
+// (2, 5), (3, 4), the colour-pair kernel's sweep; otherwise ascending.  Each
+// point runs the separate kernels' arithmetic.  Every thread of the block
+// enters; ends with a block barrier.
+__device__ __forceinline__ void tail_smooth(const TailSmem& S, const SmallGrid& G, float inv_h2, float h2half, int nsw,
+                                            bool pairs, unsigned long long* ev)
 {
-    int cnts[8], offs[8];
-    {
-        int off = 0;
-        for (int c = 0; c < 8; ++c) {
-            const int ni = colour_count(n, c & 1), nj = colour_count(n, (c >> 1) & 1),
-                      nk = colour_count(n, (c >> 2) & 1);
-            cnts[c] = (ni > 0 && nj > 0 && nk > 0) ? ni * nj * nk : 0;
-            offs[c] = off;
-            off += cnts[c];
-        }
+    const int n = G.n, nt = phase_threads(n, (int)blockDim.x);
+    if ((int)threadIdx.x < nt && nsw > 0) {
+        const int per = pairs ? 4 : 7;
+        run_phases(
+            G, S.b, S.rhs, nsw * per, nt, [&](int q) { return pairs ? q & 3 : asc_first(q % 7); },
+            [&](int q) { return pairs ? (q & 3) ^ 7 : asc_second(q % 7); },
+            [&](int p, const S3f& B, float r) {
+                const float e0 = S.e[p];
+                const S3f K = corr_hess_sm(S.e, p, n, n * n, e0, inv_h2);
+                bool nonconvex = false;
+                const float z = corr_root(B, K, r, &nonconvex);
+                S.e[p] = fmaf(h2half, z, e0);
+                *ev += nonconvex ? 1ull : 0ull;
+            });
     }
-    auto point = [&](int c, int t) {
-        const int pi = c & 1, pj = (c >> 1) & 1, pk = (c >> 2) & 1;
-        const int ni = colour_count(n, pi), nj = colour_count(n, pj);
-        const int cnt = cnts[c], off = offs[c];
-        const int i = (pi ? 1 : 2) + 2 * (t % ni);
-        const int j = (pj ? 1 : 2) + 2 * ((t / ni) % nj);
-        const int k = (pk ? 1 : 2) + 2 * (t / (ni * nj));
-        const int p = (k * n + j) * n + i;
-        const float* bp = S.b + 6 * off + t;
-        S3f B;
-        B.xx = bp[0]; B.yy = bp[cnt]; B.zz = bp[2 * cnt]; B.xy = bp[3 * cnt]; B.xz = bp[4 * cnt];
-        B.yz = bp[5 * cnt];
-        const float e0 = S.e[p];
-        const S3f K = corr_hess_sm(S.e, p, n, n * n, e0, inv_h2);
-        bool nonconvex = false;
-        const float z = corr_root(B, K, S.rhs[off + t], &nonconvex);
-        S.e[p] = fmaf(h2half, z, e0);
-        *ev += nonconvex ? 1ull : 0ull;
-    };
-    for (int sw = 0; sw < nsw; ++sw) {
-        if (pairs) {
-            for (int c = 0; c < 4; ++c) {
-                const int d = c ^ 7, nc_ = cnts[c], tot = cnts[c] + cnts[d];
-                if (tot == 0) continue;
-                for (int t = threadIdx.x; t < tot; t += TT) {
-                    if (t < nc_) point(c, t);
-                    else point(d, t - nc_);
-                }
-                __syncthreads();
-            }
-        } else {
-            for (int c = 0; c < 8; ++c) {
-                if (cnts[c] == 0) continue;
-                for (int t = threadIdx.x; t < cnts[c]; t += TT) point(c, t);
-                __syncthreads();
-            }
-        }
-    }
-}
-
-// B and rhs of interior point (i, j, k) in the colour-major shared copies.
-__device__ __forceinline__ int tail_cm(int i, int j, int k, int n, int* cnt)
-{
-    const CmPos c = cm_pos(i, j, k, n);
-    *cnt = (int)c.cnt;
-    return (int)(c.off + c.idx);
-}
-
-__device__ __forceinline__ S3f tail_b(const float* b, int i, int j, int k, int n)
-{
-    const CmPos c = cm_pos(i, j, k, n);
-    const float* bp = b + 6 * c.off + c.idx;
-    const int cnt = (int)c.cnt;
-    S3f B;
-    B.xx = bp[0]; B.yy = bp[cnt]; B.zz = bp[2 * cnt]; B.xy = bp[3 * cnt]; B.xz = bp[4 * cnt]; B.yz = bp[5 * cnt];
-    return B;
+    __syncthreads();
 }
 
 __device__ __forceinline__ float tail_line(const float* uc, const float* wc, int nc, int Ic, int J0, int K0, int oj,
@@ -1179,51 +1297,43 @@ __device__ __forceinline__ float tail_line(const float* uc, const float* wc, int
 __device__ __forceinline__ void corr_tail_body(const TailArgs& A)
 {
     extern __shared__ float tsm[];
-    TailSmem S[4];
-    {
-        float* q = tsm;
-        for (int l = 0; l < A.nlev; ++l) {
-            const int n = A.lev[l].n, m = n * n * n, mi = (n - 2) * (n - 2) * (n - 2);
-            S[l].e = q; q += m;
-            S[l].w = l > 0 ? q : nullptr; q += l > 0 ? m : 0;
-            S[l].r = q; q += m;
-            S[l].b = q; q += 6 * mi;
-            S[l].rhs = q; q += mi;
-        }
-    }
+    auto fields = [&](int l) {
+        const TailLevel& V = A.lev[l];
+        return TailSmem{tsm + V.oe, tsm + V.ow, tsm + V.orr, tsm + V.ob, tsm + V.orhs};
+    };
     // inputs: the top level's iterate and rhs, every level's B; residual
     // shells 0 (restrictions only read the interior, as in the separate path)
     for (int l = 0; l < A.nlev; ++l) {
         const int n = A.lev[l].n, m = n * n * n, mi = (n - 2) * (n - 2) * (n - 2);
-        for (int q = threadIdx.x; q < 6 * mi; q += TT) S[l].b[q] = A.lev[l].b[q];
-        for (int q = threadIdx.x; q < m; q += TT) S[l].r[q] = 0.0f;
+        const TailSmem S = fields(l);
+        for (int q = threadIdx.x; q < 6 * mi; q += TT) S.b[q] = A.lev[l].b[q];
+        for (int q = threadIdx.x; q < m; q += TT) S.r[q] = 0.0f;
         if (l == 0) {
-            for (int q = threadIdx.x; q < m; q += TT) S[0].e[q] = A.lev[0].e[q];
-            for (int q = threadIdx.x; q < mi; q += TT) S[0].rhs[q] = A.lev[0].rhs[q];
+            for (int q = threadIdx.x; q < m; q += TT) S.e[q] = A.lev[0].e[q];
+            for (int q = threadIdx.x; q < mi; q += TT) S.rhs[q] = A.lev[0].rhs[q];
         }
     }
     __syncthreads();
     unsigned long long ev = 0;
     const int L = A.nlev;
     for (int l = 0; l < L - 1; ++l) {
-        const TailSmem& F = S[l];
-        const TailSmem& C = S[l + 1];
+        const TailSmem F = fields(l);
+        const TailSmem C = fields(l + 1);
         const int nf = A.lev[l].n, nc = A.lev[l + 1].n;
-        tail_smooth(F, nf, A.lev[l].inv_h2, A.lev[l].h2half, A.nu1, A.lev[l].pairs != 0, &ev);
+        const SmallGrid GF(nf), GC(nc);
+        tail_smooth(F, GF, A.lev[l].inv_h2, A.lev[l].h2half, A.nu1, A.lev[l].pairs != 0, &ev);
         // residual on the fine interior
         for (int q = threadIdx.x; q < (nf - 2) * (nf - 2) * (nf - 2); q += TT) {
-            const int i = 1 + q % (nf - 2), j = 1 + (q / (nf - 2)) % (nf - 2), k = 1 + q / ((nf - 2) * (nf - 2));
-            const int p = (k * nf + j) * nf + i;
-            int cnt;
-            const int cm = tail_cm(i, j, k, nf, &cnt);
-            const S3f B = tail_b(F.b, i, j, k, nf);
+            int i, j, k, cnt, off;
+            const int p = GF.interior(q, &i, &j, &k), sl = GF.slot(i, j, k, &cnt, &off);
+            const S3f B = load_b_sm(F.b + 6 * off + sl, cnt);
             const S3f K = corr_hess_sm(F.e, p, nf, nf * nf, F.e[p], A.lev[l].inv_h2);
-            F.r[p] = F.rhs[cm] - delta_det(B, K);
+            F.r[p] = F.rhs[off + sl] - delta_det(B, K);
         }
         __syncthreads();
         // restriction: coarse residual, approximation restriction of e
         for (int pc = threadIdx.x; pc < nc * nc * nc; pc += TT) {
-            const int I = pc % nc, J = (pc / nc) % nc, K = pc / (nc * nc);
+            const int J0 = (pc * GC.mn) >> 16, K = (J0 * GC.mn) >> 16, I = pc - J0 * nc, J = J0 - K * nc;
             const int pf = ((2 * K) * nf + 2 * J) * nf + 2 * I;
             const bool inside = I > 0 && J > 0 && K > 0 && I < nc - 1 && J < nc - 1 && K < nc - 1;
             C.r[pc] = inside ? xfer::weighted_restrict(F.r, pf, nf, (long long)nf * nf, A.kind) : 0.0f;
@@ -1235,76 +1345,30 @@ __device__ __forceinline__ void corr_tail_body(const TailArgs& A)
         __syncthreads();
         // coarse right-hand side N_H(w_H) + res_H, colour-major
         for (int q = threadIdx.x; q < (nc - 2) * (nc - 2) * (nc - 2); q += TT) {
-            const int i = 1 + q % (nc - 2), j = 1 + (q / (nc - 2)) % (nc - 2), k = 1 + q / ((nc - 2) * (nc - 2));
-            const int p = (k * nc + j) * nc + i;
-            int cnt;
-            const int cm = tail_cm(i, j, k, nc, &cnt);
-            const S3f B = tail_b(C.b, i, j, k, nc);
+            int i, j, k, cnt, off;
+            const int p = GC.interior(q, &i, &j, &k), sl = GC.slot(i, j, k, &cnt, &off);
+            const S3f B = load_b_sm(C.b + 6 * off + sl, cnt);
             const S3f K = corr_hess_sm(C.w, p, nc, nc * nc, C.w[p], A.lev[l + 1].inv_h2);
-            C.rhs[cm] = delta_det(B, K) + C.r[p];
+            C.rhs[off + sl] = delta_det(B, K) + C.r[p];
         }
         __syncthreads();
     }
-    {   // coarsest grid: sweeps until max|de| <= 2e-6 max|e| (at most 40), or a fixed count
-        const TailSmem& Bt = S[L - 1];
-        const int n = A.lev[L - 1].n;
-        __shared__ float red[TT / 32][2];
-        __shared__ int stop;
-        const int max_sweeps = A.coarse_sweeps > 0 ? A.coarse_sweeps : 40;
-        for (int s = 0; s < max_sweeps; ++s) {
-            float du = 0.0f, um = 0.0f;
-            int off = 0;
-            for (int c = 0; c < 8; ++c) {
-                const int pi = c & 1, pj = (c >> 1) & 1, pk = (c >> 2) & 1;
-                const int ni = colour_count(n, pi), nj = colour_count(n, pj), nk = colour_count(n, pk);
-                const int cnt = (ni > 0 && nj > 0 && nk > 0) ? ni * nj * nk : 0;
-                for (int t = threadIdx.x; t < cnt; t += TT) {
-                    const int i = (pi ? 1 : 2) + 2 * (t % ni);
-                    const int j = (pj ? 1 : 2) + 2 * ((t / ni) % nj);
-                    const int k = (pk ? 1 : 2) + 2 * (t / (ni * nj));
-                    const int p = (k * n + j) * n + i;
-                    const float e0 = Bt.e[p];
-                    const float* b = Bt.b + 6 * off + t;
-                    S3f Bm;
-                    Bm.xx = b[0]; Bm.yy = b[cnt]; Bm.zz = b[2 * cnt]; Bm.xy = b[3 * cnt]; Bm.xz = b[4 * cnt];
-                    Bm.yz = b[5 * cnt];
-                    const S3f K = corr_hess_sm(Bt.e, p, n, n * n, e0, A.lev[L - 1].inv_h2);
-                    bool nonconvex = false;
-                    const float z = corr_root(Bm, K, Bt.rhs[off + t], &nonconvex);
-                    const float v = fmaf(A.lev[L - 1].h2half, z, e0);
-                    Bt.e[p] = v;
-                    du = fmaxf(du, fabsf(v - e0));
-                    um = fmaxf(um, fabsf(v));
-                    ev += nonconvex ? 1ull : 0ull;
-                }
-                off += cnt;
-                __syncthreads();
-            }
-            if (A.coarse_sweeps > 0) continue;
-            for (int o = 16; o > 0; o >>= 1) {
-                du = fmaxf(du, __shfl_down_sync(0xffffffffu, du, o));
-                um = fmaxf(um, __shfl_down_sync(0xffffffffu, um, o));
-            }
-            if ((threadIdx.x & 31) == 0) { red[threadIdx.x >> 5][0] = du; red[threadIdx.x >> 5][1] = um; }
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                float a = 0.0f, b = 0.0f;
-                for (int w = 0; w < TT / 32; ++w) { a = fmaxf(a, red[w][0]); b = fmaxf(b, red[w][1]); }
-                stop = (a <= 2e-6f * b) ? 1 : 0;
-            }
-            __syncthreads();
-            if (stop) break;
-        }
+    {
+        const TailSmem S = fields(L - 1);
+        coarsest_corr_sm(S.e, S.b, S.rhs, A.lev[L - 1].n, A.lev[L - 1].inv_h2, A.lev[L - 1].h2half, A.coarse_sweeps,
+                         &ev);
     }
     for (int l = L - 2; l >= 0; --l) {
-        const TailSmem& F = S[l];
-        const TailSmem& C = S[l + 1];
+        const TailSmem F = fields(l);
+        const TailSmem C = fields(l + 1);
         const int nf = A.lev[l].n, nc = A.lev[l + 1].n;
+        const SmallGrid GF(nf);
         // prolongation e_h += I(e_H - w_H) on the fine interior, each value formed as xfer::k_prolong forms it
         for (int q = threadIdx.x; q < (nf - 2) * (nf - 2) * (nf - 2); q += TT) {
-            const int i = 1 + q % (nf - 2), j = 1 + (q / (nf - 2)) % (nf - 2), k = 1 + q / ((nf - 2) * (nf - 2));
+            int i, j, k;
+            const int p = GF.interior(q, &i, &j, &k);
             const int J0 = j >> 1, K0 = k >> 1, oj = j & 1, ok = k & 1;
-            const float w = 1.0f / (float)(1 << (oj + ok));
+            const float w = oj + ok == 2 ? 0.25f : (oj + ok == 1 ? 0.5f : 1.0f);
             float v;
             if (i & 1) {
                 const int I = i >> 1;
@@ -1314,14 +1378,13 @@ __device__ __forceinline__ void corr_tail_body(const TailArgs& A)
             } else {
                 v = tail_line(C.e, C.w, nc, i >> 1, J0, K0, oj, ok, w);
             }
-            const int p = (k * nf + j) * nf + i;
             F.e[p] = F.e[p] + v;
         }
         __syncthreads();
-        tail_smooth(F, nf, A.lev[l].inv_h2, A.lev[l].h2half, A.nu2, A.lev[l].pairs != 0, &ev);
+        tail_smooth(F, GF, A.lev[l].inv_h2, A.lev[l].h2half, A.nu2, A.lev[l].pairs != 0, &ev);
     }
     const int m0 = A.lev[0].n * A.lev[0].n * A.lev[0].n;
-    for (int q = threadIdx.x; q < m0; q += TT) A.lev[0].e[q] = S[0].e[q];
+    for (int q = threadIdx.x; q < m0; q += TT) A.lev[0].e[q] = tsm[A.lev[0].oe + q];
     if (A.events && ev) atomicAdd(A.events, ev);
 }
 
@@ -1748,6 +1811,7 @@ cudaError_t launch_corr_vcycle_tail(const TailSpec* lv, int nlev, int nu1, int n
     A.approx = approx;
     A.coarse_sweeps = coarse_sweeps;
     A.events = events;
+    set_tail_offsets(&A);
     count_launches(1);
     k_corr_vcycle_tail<<<1, TT, tail_smem_bytes(ns, nlev), s>>>(A);
     return cudaGetLastError();
@@ -2015,7 +2079,14 @@ struct OpTail {
         int inst;
         TailArgs A;
     };
-    static __device__ __forceinline__ void run(const Job& J, int) { corr_tail_body(J.A); }
+    static __device__ __forceinline__ void run(const Job& J, int)
+    {
+        __shared__ TailArgs A;   // one copy from the job table in place of loads through it
+        const int* src = reinterpret_cast<const int*>(&J.A);
+        for (int q = threadIdx.x; q < (int)(sizeof(TailArgs) / sizeof(int)); q += NT) reinterpret_cast<int*>(&A)[q] = src[q];
+        __syncthreads();
+        corr_tail_body(A);
+    }
 };
 
 struct OpCoarsest {
@@ -2362,6 +2433,7 @@ void build_sequence(TableBuilder& T, const BatchInstance* in, int count, const B
                     A.approx = p.approx;
                     A.coarse_sweeps = p.coarse_sweeps;
                     A.events = I.events;
+                    set_tail_offsets(&A);
                     const int sm = tail_smem_bytes(ns, A.nlev);
                     tsmem = sm > tsmem ? sm : tsmem;
                     tj.push_back(J);
