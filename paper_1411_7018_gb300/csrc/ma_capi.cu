@@ -183,7 +183,7 @@ cudaError_t vcycle_from(ma_hierarchy* H, int l0)
 // With finest_vcycle false the finest level only receives the interpolated
 // iterate (the mixed-precision solve continues from there).
 cudaError_t refresh_base(ma_hierarchy* H, int apply, int l0 = 0);
-cudaError_t corr_vcycle_from(ma_hierarchy* H, int l0);
+cudaError_t corr_vcycles_from(ma_hierarchy* H, int l0, int cycles);
 
 // An FMG level of the mixed solve below the finest: one outer iteration with
 // kFmgCorrCycles FP32 correction V-cycles from level l, in place of
@@ -197,8 +197,7 @@ cudaError_t mixed_fmg_step(ma_hierarchy* H, int l)
     ma::Level& F = H->lev[l];
     if ((e = ma::launch_residual64_to32(F.u, F.rhs, F.rhs32, F.bstore, F.n, F.h, nullptr, H->s)) != cudaSuccess)
         return e;
-    for (int c = 0; c < ma::kFmgCorrCycles; ++c)
-        if ((e = corr_vcycle_from(H, l)) != cudaSuccess) return e;
+    if ((e = corr_vcycles_from(H, l, ma::kFmgCorrCycles)) != cudaSuccess) return e;
     return ma::launch_update(F.u, F.e, F.n, 1, H->s);
 }
 
@@ -249,11 +248,19 @@ cudaError_t refresh_base(ma_hierarchy* H, int apply, int l0)
     return cudaSuccess;
 }
 
-// One FAS V-cycle (Algorithm 1 structure) for N(e) = rhs32 from level l0
-// down and back, starting from the current e on level l0.  The levels with
-// n <= 17 (the tail, down to the coarsest grid) run as one single-block
-// launch with the same arithmetic.
-cudaError_t corr_vcycle_from(ma_hierarchy* H, int l0)
+// First level of the cycles from l0 that the cluster launch takes (33^3 or
+// 17^3, down to the coarsest grid, which is 9^3 or smaller), or -1.
+int cluster_level(const ma_hierarchy* H, int l0)
+{
+    if (!H->corr_cluster || H->lev[H->L - 1].n > 9) return -1;
+    for (int l = l0; l < H->L; ++l)
+        if (H->lev[l].n <= ma::corr_cluster_max_n()) return H->lev[l].n >= 17 ? l : -1;
+    return -1;
+}
+
+// One cycle from level l0; lc >= 0: `cluster` runs the levels from lc down.
+template <typename Launch>
+cudaError_t corr_vcycle_levels(ma_hierarchy* H, int l0, int lc, Launch cluster)
 {
     cudaStream_t s = H->s;
     const ma_hier_desc& d = H->d;
@@ -262,6 +269,7 @@ cudaError_t corr_vcycle_from(ma_hierarchy* H, int l0)
     while (lt > l0 && H->lev[lt - 1].n <= ma::corr_tail_max_n()) --lt;
     const bool fused = H->lev[lt].n <= ma::corr_tail_max_n();
     if (!fused) lt = H->L - 1;
+    if (lc >= 0) lt = lc;
     for (int l = l0; l < lt; ++l) {
         ma::Level& F = H->lev[l];
         ma::Level& C = H->lev[l + 1];
@@ -275,7 +283,9 @@ cudaError_t corr_vcycle_from(ma_hierarchy* H, int l0)
         if ((e = ma::launch_coarse_rhs_corr(C.w32, C.bstore, C.res32, C.rhs32, C.n, C.h, s)) != cudaSuccess)
             return e;
     }
-    if (fused) {
+    if (lc >= 0) {
+        if ((e = cluster(1)) != cudaSuccess) return e;
+    } else if (fused) {
         ma::TailSpec spec[4];
         const int nlev = H->L - lt;
         for (int q = 0; q < nlev; ++q) {
@@ -302,7 +312,33 @@ cudaError_t corr_vcycle_from(ma_hierarchy* H, int l0)
     return cudaSuccess;
 }
 
-cudaError_t corr_vcycle(ma_hierarchy* H) { return corr_vcycle_from(H, 0); }
+// `cycles` FAS V-cycles (Algorithm 1 structure) for N(e) = rhs32 from level l0
+// down and back, starting from the current e on level l0.  The levels up to
+// 33^3 run as one launch of a thread-block cluster, or, where that is not to
+// be had, those up to 9^3 (the tail, down to the coarsest grid) as one
+// single-block launch, with the same arithmetic.
+cudaError_t corr_vcycles_from(ma_hierarchy* H, int l0, int cycles)
+{
+    const int lc = cluster_level(H, l0);
+    ma::TailSpec spec[5];
+    const int nspec = lc >= 0 ? H->L - lc : 0;
+    for (int q = 0; q < nspec; ++q) {
+        ma::Level& A = H->lev[lc + q];
+        spec[q] = ma::TailSpec{A.n, A.h, A.e, A.bstore, A.rhs32};
+    }
+    auto cluster = [&](int count) {
+        return ma::launch_corr_vcycle_cluster(spec, nspec, count, H->d.nu1, H->d.nu2, H->d.restrict_kind,
+                                              H->d.approx_restrict, H->d.coarse_sweeps, H->events, H->s);
+    };
+    if (cycles > 0 && lc == l0) return cluster(cycles);
+    for (int c = 0; c < cycles; ++c) {
+        const cudaError_t e = corr_vcycle_levels(H, l0, lc, cluster);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+cudaError_t corr_vcycles(ma_hierarchy* H, int cycles) { return corr_vcycles_from(H, 0, cycles); }
 
 // ---- FP32 mode: the correction machinery with B = 0 -------------------------
 // With B = 0 the correction operator N(e) = det(B + K(e)) - det(B) is
@@ -359,7 +395,7 @@ cudaError_t fp32_fmg(ma_hierarchy* H)
         } else if ((e = ma::launch_interpolate_f32(C.e, C.n, F.e, s)) != cudaSuccess) {
             return e;
         }
-        if ((e = corr_vcycle_from(H, l)) != cudaSuccess) return e;
+        if ((e = corr_vcycles_from(H, l, 1)) != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
@@ -440,8 +476,7 @@ cudaError_t mixed_iteration(ma_hierarchy* H)
     if ((e = refresh_base(H, 0)) != cudaSuccess) return e;
     if ((e = mixed_residual(H)) != cudaSuccess) return e;
     const int inner = H->d.inner_cycles > 0 ? H->d.inner_cycles : 3;
-    for (int c = 0; c < inner; ++c)
-        if ((e = corr_vcycle(H)) != cudaSuccess) return e;
+    if ((e = corr_vcycles(H, inner)) != cudaSuccess) return e;
     return refresh_base(H, 1);
 }
 
@@ -534,6 +569,7 @@ ma_status ma_create_hierarchy(const ma_hier_desc* desc, void* dev_workspace, siz
     H->s = (cudaStream_t)stream;
     cudaError_t e = cudaGetDevice(&H->device);
     if (e == cudaSuccess) e = ma::prepare_kernels();
+    if (e == cudaSuccess && desc->precision != MA_FP64) H->corr_cluster = ma::prepare_corr_cluster();
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&H->cap, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaMallocHost((void**)&H->host, 8 * sizeof(double));
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&H->sv.ev, cudaEventDisableTiming);
@@ -627,7 +663,7 @@ ma_status ma_vcycle(ma_hierarchy* H, int ncycles)
     DeviceGuard g(H->device);
     if (H->d.precision == MA_FP32) {
         MA_CK(fp32_prepare(H));
-        for (int c = 0; c < ncycles; ++c) MA_CK(corr_vcycle(H));
+        MA_CK(corr_vcycles(H, ncycles));
         MA_CK(ma::launch_f32_to_f64(H->lev[0].e, H->lev[0].u, H->lev[0].n, H->s));
         return MA_OK;
     }
@@ -739,8 +775,7 @@ ma_status ma_solve_begin(ma_hierarchy* H, const ma_solve_opts* opts)
             // Algorithm 2 step 5 on the finest level: one outer iteration
             // (the FP32 correction cycles) completes the FMG pass
             const int inner = H->d.inner_cycles > 0 ? H->d.inner_cycles : 3;
-            for (int c = 0; c < inner; ++c)
-                if ((e = corr_vcycle(H)) != cudaSuccess) return e;
+            if ((e = corr_vcycles(H, inner)) != cudaSuccess) return e;
             if ((e = refresh_base(H, 1)) != cudaSuccess) return e;
             return mixed_residual(H);
         }
@@ -761,13 +796,12 @@ static cudaError_t launch_cycle(ma_hierarchy* H)
     return run_graph(H, H->g_cycle, [&]() -> cudaError_t {
         cudaError_t e;
         if (H->d.precision == MA_FP32) {
-            if ((e = corr_vcycle(H)) != cudaSuccess) return e;
+            if ((e = corr_vcycles(H, 1)) != cudaSuccess) return e;
             return fp32_residual(H);
         }
         if (mixed) {
             const int inner = H->d.inner_cycles > 0 ? H->d.inner_cycles : 3;
-            for (int c = 0; c < inner; ++c)
-                if ((e = corr_vcycle(H)) != cudaSuccess) return e;
+            if ((e = corr_vcycles(H, inner)) != cudaSuccess) return e;
             if ((e = refresh_base(H, 1)) != cudaSuccess) return e;
             return mixed_residual(H);
         }

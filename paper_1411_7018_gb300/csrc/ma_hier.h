@@ -47,6 +47,7 @@ struct ma_hierarchy {
     ma::Level lev[ma::kMaxLevels];
     cudaStream_t s = nullptr;
     int device = 0;
+    bool corr_cluster = false;           // the device runs the 16-block cluster of the small correction levels
     char* ws = nullptr;
     size_t bytes = 0;
     double* partials = nullptr;          // norm partials (2 per block)

@@ -114,6 +114,14 @@ int corr_tail_max_n();            // 0 when the fused tail is switched off
 bool set_corr_tail(int max_n);     // 0 off, 1 default, or 3 / 5 / 9 / 17; false otherwise
 cudaError_t launch_corr_vcycle_tail(const TailSpec* lv, int nlev, int nu1, int nu2, int kind, int approx,
                                     int coarse_sweeps, unsigned long long* events, cudaStream_t s);
+// cycles V-cycles over levels 33^3 or 17^3 (the first entry) down to the
+// coarsest grid, 9^3 among them, in one launch of a 16-block cluster.
+// prepare_corr_cluster: sets the kernel's limits on the current device and
+// tells whether it can run such a cluster; call outside stream capture.
+int corr_cluster_max_n();         // 33, or 0 when a tail bound is set by hand
+bool prepare_corr_cluster();
+cudaError_t launch_corr_vcycle_cluster(const TailSpec* lv, int nlev, int cycles, int nu1, int nu2, int kind,
+                                       int approx, int coarse_sweeps, unsigned long long* events, cudaStream_t s);
 cudaError_t launch_residual_corr_choice(int choice, const float* e, const void* bstore, const float* rhs_cm,
                                         float* res, int n, double h, cudaStream_t s);
 cudaError_t launch_residual_corr(const float* e, const void* bstore, const float* rhs_cm, float* res, int n,

@@ -1234,15 +1234,16 @@ __host__ __device__ inline int tail_level_floats(int n, bool top)
 }
 
 // Lays the levels out in shared memory; the host fills the offsets in, so that
-// every access is an offset from the block's base.
-inline void set_tail_offsets(TailArgs* A)
+// every access is an offset from the block's base.  top: the first level is
+// the one the cycle enters (it has no restricted approximation w).
+inline void set_tail_offsets(TailArgs* A, bool top = true)
 {
     int q = 0;
     for (int l = 0; l < A->nlev; ++l) {
         TailLevel& V = A->lev[l];
         const int m = V.n * V.n * V.n, mi = (V.n - 2) * (V.n - 2) * (V.n - 2);
         V.oe = q; q += m;
-        V.ow = q; q += l > 0 ? m : 0;
+        V.ow = q; q += l > 0 || !top ? m : 0;
         V.orr = q; q += m;
         V.ob = q; q += 6 * mi;
         V.orhs = q; q += mi;
@@ -1294,34 +1295,50 @@ __device__ __forceinline__ float tail_line(const float* uc, const float* wc, int
     return s * w;
 }
 
-__device__ __forceinline__ void corr_tail_body(const TailArgs& A)
+__device__ __forceinline__ TailSmem tail_fields(const TailArgs& A, float* tsm, int l)
 {
-    extern __shared__ float tsm[];
-    auto fields = [&](int l) {
-        const TailLevel& V = A.lev[l];
-        return TailSmem{tsm + V.oe, tsm + V.ow, tsm + V.orr, tsm + V.ob, tsm + V.orhs};
-    };
-    // inputs: the top level's iterate and rhs, every level's B; residual
-    // shells 0 (restrictions only read the interior, as in the separate path)
+    const TailLevel& V = A.lev[l];
+    return TailSmem{tsm + V.oe, tsm + V.ow, tsm + V.orr, tsm + V.ob, tsm + V.orhs};
+}
+
+// Every level's B; residual shells 0 (restrictions only read the interior, as
+// in the separate path).
+__device__ __forceinline__ void tail_load_base(const TailArgs& A, float* tsm)
+{
     for (int l = 0; l < A.nlev; ++l) {
         const int n = A.lev[l].n, m = n * n * n, mi = (n - 2) * (n - 2) * (n - 2);
-        const TailSmem S = fields(l);
+        const TailSmem S = tail_fields(A, tsm, l);
         for (int q = threadIdx.x; q < 6 * mi; q += TT) S.b[q] = A.lev[l].b[q];
         for (int q = threadIdx.x; q < m; q += TT) S.r[q] = 0.0f;
-        if (l == 0) {
-            for (int q = threadIdx.x; q < m; q += TT) S.e[q] = A.lev[0].e[q];
-            for (int q = threadIdx.x; q < mi; q += TT) S.rhs[q] = A.lev[0].rhs[q];
-        }
+    }
+}
+
+// rhs_H = N_H(w_H) + res_H of level l, colour-major.
+__device__ __forceinline__ void tail_coarse_rhs(const TailArgs& A, float* tsm, int l)
+{
+    const TailSmem C = tail_fields(A, tsm, l);
+    const int nc = A.lev[l].n;
+    const SmallGrid GC(nc);
+    for (int q = threadIdx.x; q < (nc - 2) * (nc - 2) * (nc - 2); q += TT) {
+        int i, j, k, cnt, off;
+        const int p = GC.interior(q, &i, &j, &k), sl = GC.slot(i, j, k, &cnt, &off);
+        const S3f B = load_b_sm(C.b + 6 * off + sl, cnt);
+        const S3f K = corr_hess_sm(C.w, p, nc, nc * nc, C.w[p], A.lev[l].inv_h2);
+        C.rhs[off + sl] = delta_det(B, K) + C.r[p];
     }
     __syncthreads();
-    unsigned long long ev = 0;
+}
+
+// The cycle from level 0 of the tail, whose e and rhs are in place, down and back.
+__device__ __forceinline__ void tail_cycle(const TailArgs& A, float* tsm, unsigned long long* ev)
+{
     const int L = A.nlev;
     for (int l = 0; l < L - 1; ++l) {
-        const TailSmem F = fields(l);
-        const TailSmem C = fields(l + 1);
+        const TailSmem F = tail_fields(A, tsm, l);
+        const TailSmem C = tail_fields(A, tsm, l + 1);
         const int nf = A.lev[l].n, nc = A.lev[l + 1].n;
         const SmallGrid GF(nf), GC(nc);
-        tail_smooth(F, GF, A.lev[l].inv_h2, A.lev[l].h2half, A.nu1, A.lev[l].pairs != 0, &ev);
+        tail_smooth(F, GF, A.lev[l].inv_h2, A.lev[l].h2half, A.nu1, A.lev[l].pairs != 0, ev);
         // residual on the fine interior
         for (int q = threadIdx.x; q < (nf - 2) * (nf - 2) * (nf - 2); q += TT) {
             int i, j, k, cnt, off;
@@ -1343,24 +1360,16 @@ __device__ __forceinline__ void corr_tail_body(const TailArgs& A)
             C.e[pc] = w;
         }
         __syncthreads();
-        // coarse right-hand side N_H(w_H) + res_H, colour-major
-        for (int q = threadIdx.x; q < (nc - 2) * (nc - 2) * (nc - 2); q += TT) {
-            int i, j, k, cnt, off;
-            const int p = GC.interior(q, &i, &j, &k), sl = GC.slot(i, j, k, &cnt, &off);
-            const S3f B = load_b_sm(C.b + 6 * off + sl, cnt);
-            const S3f K = corr_hess_sm(C.w, p, nc, nc * nc, C.w[p], A.lev[l + 1].inv_h2);
-            C.rhs[off + sl] = delta_det(B, K) + C.r[p];
-        }
-        __syncthreads();
+        tail_coarse_rhs(A, tsm, l + 1);
     }
     {
-        const TailSmem S = fields(L - 1);
+        const TailSmem S = tail_fields(A, tsm, L - 1);
         coarsest_corr_sm(S.e, S.b, S.rhs, A.lev[L - 1].n, A.lev[L - 1].inv_h2, A.lev[L - 1].h2half, A.coarse_sweeps,
-                         &ev);
+                         ev);
     }
     for (int l = L - 2; l >= 0; --l) {
-        const TailSmem F = fields(l);
-        const TailSmem C = fields(l + 1);
+        const TailSmem F = tail_fields(A, tsm, l);
+        const TailSmem C = tail_fields(A, tsm, l + 1);
         const int nf = A.lev[l].n, nc = A.lev[l + 1].n;
         const SmallGrid GF(nf);
         // prolongation e_h += I(e_H - w_H) on the fine interior, each value formed as xfer::k_prolong forms it
@@ -1381,14 +1390,407 @@ __device__ __forceinline__ void corr_tail_body(const TailArgs& A)
             F.e[p] = F.e[p] + v;
         }
         __syncthreads();
-        tail_smooth(F, GF, A.lev[l].inv_h2, A.lev[l].h2half, A.nu2, A.lev[l].pairs != 0, &ev);
+        tail_smooth(F, GF, A.lev[l].inv_h2, A.lev[l].h2half, A.nu2, A.lev[l].pairs != 0, ev);
     }
+}
+
+__device__ __forceinline__ void corr_tail_body(const TailArgs& A)
+{
+    extern __shared__ float tsm[];
+    tail_load_base(A, tsm);
+    {   // the top level's iterate and rhs
+        const int n = A.lev[0].n, m = n * n * n, mi = (n - 2) * (n - 2) * (n - 2);
+        const TailSmem S = tail_fields(A, tsm, 0);
+        for (int q = threadIdx.x; q < m; q += TT) S.e[q] = A.lev[0].e[q];
+        for (int q = threadIdx.x; q < mi; q += TT) S.rhs[q] = A.lev[0].rhs[q];
+    }
+    __syncthreads();
+    unsigned long long ev = 0;
+    tail_cycle(A, tsm, &ev);
     const int m0 = A.lev[0].n * A.lev[0].n * A.lev[0].n;
     for (int q = threadIdx.x; q < m0; q += TT) A.lev[0].e[q] = tsm[A.lev[0].oe + q];
     if (A.events && ev) atomicAdd(A.events, ev);
 }
 
 __global__ void __launch_bounds__(TT, 1) k_corr_vcycle_tail(TailArgs A) { corr_tail_body(A); }
+
+// ---------------------------------------------------------------------------
+// Correction V-cycles from a level of 33^3 or 17^3 down to the coarsest grid
+// and back in one cluster of 16 thread blocks.  Level by level those two grids
+// take 16 colour-pair launches and 4 transfers each a cycle, 1.8 us and more
+// apiece whatever their work; here a phase is a cluster barrier.
+//
+// A block owns planes of k: at 33^3 the odd plane 2m + 1 and the even plane
+// 2m + 2 (m its rank), at 17^3 the plane m + 1, in shared memory with one
+// plane of its neighbours on either side.  A phase updates the even planes'
+// colour and the odd planes' colour of a pair (at most 481 points a block,
+// one a thread), and each new value also goes to the neighbour block that
+// holds its plane as a halo.  Points of the pair's other colour, which a
+// neighbour may be writing into the halo meanwhile, are not in the stencil.
+// Coarse plane K = m + 1 of the 17^3 grid sits on the block's own fine plane
+// 2m + 2, so restriction and prolongation stay inside the block but for the
+// halo of r.  The levels up to 9^3 run as the single-block tail does, in the
+// first block.  Every point runs the arithmetic of the separate kernels: the
+// same bits.  B, which nothing here writes, is read from global memory one
+// phase ahead.
+// ---------------------------------------------------------------------------
+constexpr int KC = 16;      // blocks of the cluster
+constexpr int TC = 512;     // threads of a block
+
+struct ClusterLevel {
+    float inv_h2, h2half;
+    int pairs;
+    float* e;             // global, natural layout (top level: read and written back)
+    const float* b;       // global colour-major B
+    const float* rhs;     // global colour-major rhs (top level: read)
+};
+
+struct ClusterArgs {
+    int top33;            // enter at 33^3 (else at 17^3)
+    ClusterLevel l33, l17;
+    TailArgs tail;        // the levels from 9^3 down
+    int cycles;
+};
+
+__device__ __forceinline__ unsigned cluster_rank()
+{
+    unsigned r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+
+// All threads of the cluster: writes before it, also those into other blocks'
+// shared memory, are visible after it.
+__device__ __forceinline__ void cluster_barrier()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+__device__ __forceinline__ void store_remote(float* smem, unsigned rank, float v)
+{
+    unsigned a = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("mapa.shared::cluster.u32 %0, %0, %1;\n" : "+r"(a) : "r"(rank));
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+
+__device__ __forceinline__ float load_remote(const float* smem, unsigned rank)
+{
+    unsigned a = (unsigned)__cvta_generic_to_shared(smem);
+    float v;
+    asm volatile("mapa.shared::cluster.u32 %0, %0, %1;\n" : "+r"(a) : "r"(rank));
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+    return v;
+}
+
+// One level of the cluster: N points a side, P planes a block (local planes
+// 1 .. P; 0 and P + 1 are the neighbours').  Local plane q is plane m P + q.
+template <int N, int P>
+struct Slab {
+    static constexpr int PL = N * N, A = (N - 3) / 2, B = (N - 1) / 2, M2 = (N - 2) * (N - 2);
+    float *e, *r, *rh;          // [P + 2][N][N], the same, [P][M2]
+    const float* b;             // global colour-major B
+    unsigned m;                 // block rank
+    float inv_h2, h2half;
+
+    __device__ __forceinline__ int planes() const { return max(0, min(P, N - 2 - (int)m * P)); }
+    static __device__ __forceinline__ int ni(int c) { return (c & 1) ? B : A; }
+    static __device__ __forceinline__ int nj(int c) { return (c & 2) ? B : A; }
+    // points of in-plane colours before c & 3
+    static __device__ __forceinline__ int in_plane(int c)
+    {
+        return ((c & 1) ? A * ((c & 2) ? B : A) : 0) + ((c & 2) ? (A + B) * A : 0);
+    }
+    static __device__ __forceinline__ int offset(int c) { return (int)cm_offset(N, c); }
+
+    // A new value of local plane q at in-plane place s, and its copies in the
+    // neighbours' halos.
+    __device__ __forceinline__ void put(float* f, int q, int s, float v) const
+    {
+        f[q * PL + s] = v;
+        if (q == 1 && m > 0) store_remote(f + (P + 1) * PL + s, m - 1, v);
+        if (q == P && m + 1 < KC) store_remote(f + s, m + 1, v);
+    }
+
+    struct Pt {
+        int q, s, cnt;      // local plane, in-plane place, points of the colour
+        const float *b, *r;
+    };
+
+    // Point t of a phase that sweeps colour ce of even planes and colour co of
+    // odd ones (-1: none).
+    __device__ __forceinline__ bool locate(int ce, int co, int t, Pt* X) const
+    {
+        int q, c;
+        const int np = planes();
+        if (P == 1) {
+            q = 1;
+            c = ((m + 1) & 1) ? co : ce;
+            if (np < 1 || c < 0) return false;
+        } else {            // local plane 1 is odd, 2 even
+            const int no = co >= 0 && np >= 1 ? ni(co) * nj(co) : 0;
+            q = 1;
+            c = co;
+            if (t >= no) {
+                t -= no;
+                q = 2;
+                c = ce;
+                if (c < 0 || np < 2) return false;
+            }
+        }
+        if (t >= ni(c) * nj(c)) return false;
+        const int d = ni(c), y = (c & 1) ? t / B : t / A, x = t - y * d;
+        const int k = (int)m * P + q, kk = (k - ((k & 1) ? 1 : 2)) >> 1;
+        X->q = q;
+        X->s = (((c & 2) ? 1 : 2) + 2 * y) * N + ((c & 1) ? 1 : 2) + 2 * x;
+        X->cnt = d * nj(c) * ((c & 4) ? B : A);
+        X->b = b + 6 * offset(c) + kk * (d * nj(c)) + t;
+        X->r = rh + (q - 1) * M2 + in_plane(c) + t;
+        return true;
+    }
+
+    // Interior point t of the block's planes in natural order.
+    __device__ __forceinline__ bool interior(int t, int* q, int* i, int* j) const
+    {
+        const int p = t / M2, u = t - p * M2, y = u / (N - 2);
+        *q = 1 + p;
+        *j = 1 + y;
+        *i = 1 + u - y * (N - 2);
+        return p < planes();
+    }
+    // B and the rhs slot of the interior point (i, j) of local plane q
+    __device__ __forceinline__ S3f base(int q, int i, int j, int* slot) const
+    {
+        const int k = (int)m * P + q;
+        const int c = (i & 1) | ((j & 1) << 1) | ((k & 1) << 2);
+        const int u = ((j - 1) >> 1) * ni(c) + ((i - 1) >> 1), pl = ni(c) * nj(c);
+        *slot = (q - 1) * M2 + in_plane(c) + u;
+        return load_b(b + 6 * offset(c) + ((k - 1) >> 1) * pl + u, pl * ((c & 4) ? B : A));
+    }
+
+    __device__ __forceinline__ S3f hess(const float* f, int q, int s) const
+    {
+        return corr_hess_sm(f, q * PL + s, N, PL, f[q * PL + s], inv_h2);
+    }
+
+    // nsw sweeps; every phase ends with the cluster's barrier.
+    __device__ __forceinline__ void smooth(int nsw, int pairs, unsigned long long* ev) const
+    {
+        const int per = pairs ? 4 : 7, nq = nsw * per;
+        // ascending: 0, 1, 2, (3, 4), 5, 6, 7
+        auto even = [&](int w) { return pairs ? w : (w <= 3 ? w : -1); };
+        auto odd = [&](int w) { return pairs ? w ^ 7 : (w >= 3 ? w + 1 : -1); };
+        Pt cur, nxt;
+        S3f Bc = {0, 0, 0, 0, 0, 0}, Bn = Bc;
+        float rc = 0.0f, rn = 0.0f;
+        bool on = nq > 0 && locate(even(0), odd(0), threadIdx.x, &cur);
+        if (on) {
+            Bc = load_b(cur.b, cur.cnt);
+            rc = *cur.r;
+        }
+        int w = 0;
+        for (int t = 0; t < nq; ++t) {
+            w = w + 1 == per ? 0 : w + 1;
+            const bool onn = t + 1 < nq && locate(even(w), odd(w), threadIdx.x, &nxt);
+            if (onn) {
+                Bn = load_b(nxt.b, nxt.cnt);
+                rn = *nxt.r;
+            }
+            if (on) {
+                const float e0 = e[cur.q * PL + cur.s];
+                const S3f K = hess(e, cur.q, cur.s);
+                bool nonconvex = false;
+                put(e, cur.q, cur.s, fmaf(h2half, corr_root(Bc, K, rc, &nonconvex), e0));
+                *ev += nonconvex ? 1ull : 0ull;
+            }
+            cluster_barrier();
+            on = onn;
+            cur = nxt;
+            Bc = Bn;
+            rc = rn;
+        }
+    }
+
+    // r = rhs - N(e) on the block's planes, with halos.
+    __device__ __forceinline__ void residual() const
+    {
+        for (int t = threadIdx.x; t < P * M2; t += TC) {
+            int q, i, j, slot;
+            if (!interior(t, &q, &i, &j)) continue;
+            const S3f Bm = base(q, i, j, &slot);
+            put(r, q, j * N + i, rh[slot] - delta_det(Bm, hess(e, q, j * N + i)));
+        }
+        cluster_barrier();
+    }
+
+    // rhs = N(w) + r on the block's planes (Algorithm 1 step 5).
+    __device__ __forceinline__ void coarse_rhs(const float* w) const
+    {
+        for (int t = threadIdx.x; t < P * M2; t += TC) {
+            int q, i, j, slot;
+            if (!interior(t, &q, &i, &j)) continue;
+            const S3f Bm = base(q, i, j, &slot);
+            rh[slot] = delta_det(Bm, hess(w, q, j * N + i)) + r[q * PL + j * N + i];
+        }
+        __syncthreads();
+    }
+
+    // The top level's iterate and right-hand side from global memory.
+    __device__ __forceinline__ void load(const float* ge, const float* grhs) const
+    {
+        for (int t = threadIdx.x; t < (P + 2) * PL; t += TC) {
+            const int k = (int)m * P + t / PL;
+            e[t] = k < N ? ge[k * PL + t % PL] : 0.0f;
+        }
+        for (int t = threadIdx.x; t < P * M2; t += TC) {
+            int q, i, j;
+            if (!interior(t, &q, &i, &j)) continue;
+            const int k = (int)m * P + q, c = (i & 1) | ((j & 1) << 1) | ((k & 1) << 2);
+            const int u = ((j - 1) >> 1) * ni(c) + ((i - 1) >> 1);
+            rh[(q - 1) * M2 + in_plane(c) + u] = grhs[offset(c) + ((k - 1) >> 1) * (ni(c) * nj(c)) + u];
+        }
+    }
+
+    __device__ __forceinline__ void store(float* ge) const
+    {
+        for (int t = threadIdx.x; t < P * M2; t += TC) {
+            int q, i, j;
+            if (!interior(t, &q, &i, &j)) continue;
+            ge[((int)m * P + q) * PL + j * N + i] = e[q * PL + j * N + i];
+        }
+    }
+};
+
+// Trilinear correction of one fine point from the coarse planes dlo (K0) and
+// dhi (K0 + 1) of e_H - w_H, formed as xfer::k_prolong forms it.
+template <int NC>
+__device__ __forceinline__ float cluster_prolong(const float* dlo, const float* dhi, int i, int j, int ok)
+{
+    const int J0 = j >> 1, oj = j & 1, I = i >> 1;
+    const float w = oj + ok == 2 ? 0.25f : (oj + ok == 1 ? 0.5f : 1.0f);
+    auto line = [&](int Ic) {
+        float s = 0.0f;
+        s += dlo[J0 * NC + Ic];
+        if (oj) s += dlo[(J0 + 1) * NC + Ic];
+        if (ok) {
+            s += dhi[J0 * NC + Ic];
+            if (oj) s += dhi[(J0 + 1) * NC + Ic];
+        }
+        return s * w;
+    };
+    return (i & 1) ? (line(I) + line(I + 1)) * 0.5f : line(I);
+}
+
+constexpr int kClusterFloats33 = 2 * 4 * 33 * 33 + 2 * 31 * 31;
+constexpr int kClusterFloats17 = 3 * 3 * 17 * 17 + 15 * 15 + 2 * 17 * 17;
+
+__global__ void __launch_bounds__(TC, 1) k_corr_vcycle_cluster(const __grid_constant__ ClusterArgs A)
+{
+    extern __shared__ float csm[];
+    const unsigned m = cluster_rank();
+    float* q = csm;
+    auto take = [&](int f) {
+        float* p = q;
+        q += f;
+        return p;
+    };
+    Slab<33, 2> F;
+    F.e = take(4 * 33 * 33); F.r = take(4 * 33 * 33); F.rh = take(2 * 31 * 31);
+    F.b = A.l33.b; F.m = m; F.inv_h2 = A.l33.inv_h2; F.h2half = A.l33.h2half;
+    Slab<17, 1> C;
+    C.e = take(3 * 17 * 17);
+    float* w17 = take(3 * 17 * 17);
+    C.r = take(3 * 17 * 17); C.rh = take(15 * 15);
+    C.b = A.l17.b; C.m = m; C.inv_h2 = A.l17.inv_h2; C.h2half = A.l17.h2half;
+    float* d = take(2 * 17 * 17);   // planes of e_H - w_H
+    float* tsm = q;                 // first block: the levels from 9^3 down
+    const TailArgs& T = A.tail;
+    const TailLevel& V9 = T.lev[0];
+    unsigned long long ev = 0;
+    if (A.top33) F.load(A.l33.e, A.l33.rhs);
+    else C.load(A.l17.e, A.l17.rhs);
+    if (m == 0) tail_load_base(T, tsm);
+    cluster_barrier();   // every block is running before its memory is written from another
+    for (int cyc = 0; cyc < A.cycles; ++cyc) {
+        if (A.top33) {
+            F.smooth(T.nu1, A.l33.pairs, &ev);
+            F.residual();
+            // coarse plane K = m + 1 on the block's fine plane 2m + 2, and plane 0 in the first block
+            for (int t = threadIdx.x; t < (m == 0 ? 2 : 1) * C.PL; t += TC) {
+                const int own = t < C.PL, s = own ? t : t - C.PL, J = s / 17, I = s - J * 17;
+                const int K = own ? (int)m + 1 : 0, pf = (own ? 2 : 0) * F.PL + 2 * J * 33 + 2 * I;
+                const bool in = I > 0 && J > 0 && K > 0 && I < 16 && J < 16 && K < 16;
+                const float rv = in ? xfer::weighted_restrict(F.r, pf, 33, F.PL, T.kind) : 0.0f;
+                const float wv = in && T.approx == 1 ? xfer::weighted_restrict(F.e, pf, 33, F.PL, T.kind) : F.e[pf];
+                if (own) {
+                    C.r[C.PL + s] = rv;
+                    C.put(w17, 1, s, wv);
+                    C.put(C.e, 1, s, wv);
+                } else {
+                    w17[s] = wv;
+                    C.e[s] = wv;
+                }
+            }
+            cluster_barrier();
+            C.coarse_rhs(w17);
+        }
+        C.smooth(T.nu1, A.l17.pairs, &ev);
+        C.residual();
+        // plane K of the 9^3 grid sits on fine plane 2K: local plane 1 of the blocks of odd rank; the shell planes on
+        // the outer halos of the first and the second to last block
+        {
+            const int K = m == 0 ? 0 : (m == KC - 2 ? 8 : ((m & 1) && m < KC - 2 ? (int)(m + 1) / 2 : -1));
+            const int lp = m == 0 ? 0 : (m == KC - 2 ? 2 : 1);
+            for (int s = threadIdx.x; K >= 0 && s < 81; s += TC) {
+                const int J = s / 9, I = s - J * 9, pf = lp * C.PL + 2 * J * 17 + 2 * I;
+                const bool in = I > 0 && J > 0 && K > 0 && I < 8 && J < 8 && K < 8;
+                const float rv = in ? xfer::weighted_restrict(C.r, pf, 17, C.PL, T.kind) : 0.0f;
+                const float wv = in && T.approx == 1 ? xfer::weighted_restrict(C.e, pf, 17, C.PL, T.kind) : C.e[pf];
+                store_remote(tsm + V9.orr + 81 * K + s, 0, rv);
+                store_remote(tsm + V9.ow + 81 * K + s, 0, wv);
+                store_remote(tsm + V9.oe + 81 * K + s, 0, wv);
+            }
+        }
+        cluster_barrier();
+        if (m == 0) {
+            tail_coarse_rhs(T, tsm, 0);
+            tail_cycle(T, tsm, &ev);
+        }
+        cluster_barrier();
+        {   // 9^3 -> 17^3: plane k = m + 1 lies on or between coarse planes K0 = k / 2 and K0 + 1
+            const int k = (int)m + 1, K0 = k >> 1;
+            for (int t = threadIdx.x; t < 162; t += TC) {
+                const int s = t < 81 ? t : t - 81, p = 81 * min(K0 + (t < 81 ? 0 : 1), 8) + s;
+                d[t] = load_remote(tsm + V9.oe + p, 0) - load_remote(tsm + V9.ow + p, 0);
+            }
+            __syncthreads();
+            for (int t = threadIdx.x; t < C.M2; t += TC) {
+                int lq, i, j;
+                if (!C.interior(t, &lq, &i, &j)) continue;
+                const int s = j * 17 + i;
+                C.put(C.e, 1, s, C.e[C.PL + s] + cluster_prolong<9>(d, d + 81, i, j, k & 1));
+            }
+        }
+        cluster_barrier();
+        C.smooth(T.nu2, A.l17.pairs, &ev);
+        if (A.top33) {   // fine plane 2m + 1 between coarse planes m and m + 1, plane 2m + 2 on coarse plane m + 1
+            for (int t = threadIdx.x; t < 2 * C.PL; t += TC) d[t] = C.e[t] - w17[t];
+            __syncthreads();
+            for (int t = threadIdx.x; t < 2 * F.M2; t += TC) {
+                int lq, i, j;
+                if (!F.interior(t, &lq, &i, &j)) continue;
+                const int s = j * 33 + i;
+                const float v = lq == 1 ? cluster_prolong<17>(d, d + C.PL, i, j, 1)
+                                        : cluster_prolong<17>(d + C.PL, d, i, j, 0);
+                F.put(F.e, lq, s, F.e[lq * F.PL + s] + v);
+            }
+            cluster_barrier();
+            F.smooth(T.nu2, A.l33.pairs, &ev);
+        }
+    }
+    if (A.top33) F.store(A.l33.e);
+    else C.store(A.l17.e);
+    if (T.events && ev) atomicAdd(T.events, ev);
+}
 
 // FP64 <-> FP32 copies of whole grids (the FP32 mode's iterate and data).
 __global__ void k_f64_to_f32(const double* __restrict__ u, float* __restrict__ e, long long m)
@@ -1772,20 +2174,50 @@ int tail_smem_bytes(const int* ns, int nlev)
     return f * (int)sizeof(float);
 }
 
-// Default largest level of the fused tail: at 17^3 one SM's serial colour
+// Largest level of the single-block tail: at 17^3 one SM's serial colour
 // phases take longer than the launches they replace, at 9^3 and below the
-// launches cost more (measured on whole solves from 33^3 to 257^3).
-constexpr int kTailDefault = 9;
-std::atomic<int> g_tail_max{kTailDefault};
+// launches cost more (measured on whole solves from 33^3 to 257^3).  By
+// default the cluster takes the levels up to 33^3 (measured per cycle beside
+// k_corr_vcycle_cluster); a bound set by hand leaves it out.
+constexpr int kTailDefault = 9, kClusterDefault = 33;
+std::atomic<int> g_tail_max{kClusterDefault};
 
-int corr_tail_max_n() { return g_tail_max.load(std::memory_order_relaxed); }
+int corr_tail_max_n()
+{
+    const int m = g_tail_max.load(std::memory_order_relaxed);
+    return m == kClusterDefault ? kTailDefault : m;
+}
+
+int corr_cluster_max_n() { return g_tail_max.load(std::memory_order_relaxed) == kClusterDefault ? kClusterDefault : 0; }
 
 bool set_corr_tail(int max_n)
 {
-    if (max_n == 1) max_n = kTailDefault;
-    if (!(max_n == 0 || max_n == 3 || max_n == 5 || max_n == 9 || max_n == kTailMaxN)) return false;
+    if (max_n == 1) max_n = kClusterDefault;
+    else if (!(max_n == 0 || max_n == 3 || max_n == 5 || max_n == 9 || max_n == kTailMaxN)) return false;
     g_tail_max.store(max_n, std::memory_order_relaxed);
     return true;
+}
+
+static void fill_tail(TailArgs* A, const TailSpec* lv, int nlev, int nu1, int nu2, int kind, int approx,
+                      int coarse_sweeps, unsigned long long* events)
+{
+    A->nlev = nlev;
+    for (int l = 0; l < nlev; ++l) {
+        const double h = lv[l].h;
+        A->lev[l].n = lv[l].n;
+        A->lev[l].pairs = corr_smooth_choice(lv[l].n) == CORR_PAIRS;
+        A->lev[l].inv_h2 = (float)(1.0 / (h * h));
+        A->lev[l].h2half = (float)(0.5 * h * h);
+        A->lev[l].e = lv[l].e;
+        A->lev[l].b = (const float*)lv[l].bstore;
+        A->lev[l].rhs = lv[l].rhs_cm;
+    }
+    A->nu1 = nu1;
+    A->nu2 = nu2;
+    A->kind = kind;
+    A->approx = approx;
+    A->coarse_sweeps = coarse_sweeps;
+    A->events = events;
 }
 
 cudaError_t launch_corr_vcycle_tail(const TailSpec* lv, int nlev, int nu1, int nu2, int kind, int approx,
@@ -1793,28 +2225,74 @@ cudaError_t launch_corr_vcycle_tail(const TailSpec* lv, int nlev, int nu1, int n
 {
     if (nlev < 1 || nlev > 4) return cudaErrorInvalidValue;
     TailArgs A;
-    A.nlev = nlev;
     int ns[4];
-    for (int l = 0; l < nlev; ++l) {
-        const double h = lv[l].h;
-        A.lev[l].n = ns[l] = lv[l].n;
-        A.lev[l].pairs = corr_smooth_choice(lv[l].n) == CORR_PAIRS;
-        A.lev[l].inv_h2 = (float)(1.0 / (h * h));
-        A.lev[l].h2half = (float)(0.5 * h * h);
-        A.lev[l].e = lv[l].e;
-        A.lev[l].b = (const float*)lv[l].bstore;
-        A.lev[l].rhs = lv[l].rhs_cm;
-    }
-    A.nu1 = nu1;
-    A.nu2 = nu2;
-    A.kind = kind;
-    A.approx = approx;
-    A.coarse_sweeps = coarse_sweeps;
-    A.events = events;
+    for (int l = 0; l < nlev; ++l) ns[l] = lv[l].n;
+    fill_tail(&A, lv, nlev, nu1, nu2, kind, approx, coarse_sweeps, events);
     set_tail_offsets(&A);
     count_launches(1);
     k_corr_vcycle_tail<<<1, TT, tail_smem_bytes(ns, nlev), s>>>(A);
     return cudaGetLastError();
+}
+
+static_assert(TC == TT, "the cluster's first block runs the tail's block body");
+
+static int cluster_smem_bytes()
+{
+    return (kClusterFloats33 + kClusterFloats17 + tail_level_floats(9, false) + tail_level_floats(5, false) +
+            tail_level_floats(3, false)) * (int)sizeof(float);
+}
+
+cudaError_t launch_corr_vcycle_cluster(const TailSpec* lv, int nlev, int cycles, int nu1, int nu2, int kind,
+                                       int approx, int coarse_sweeps, unsigned long long* events, cudaStream_t s)
+{
+    ClusterArgs A{};
+    A.top33 = lv[0].n == 33;
+    const int t = A.top33 ? 2 : 1;   // the tail's first level
+    if (nlev - t < 1 || nlev - t > 3 || lv[t].n != 9 || lv[t - 1].n != 17) return cudaErrorInvalidValue;
+    auto level = [](const TailSpec& v) {
+        return ClusterLevel{(float)(1.0 / (v.h * v.h)), (float)(0.5 * v.h * v.h),
+                            corr_smooth_choice(v.n) == CORR_PAIRS, v.e, (const float*)v.bstore, v.rhs_cm};
+    };
+    if (A.top33) A.l33 = level(lv[0]);
+    A.l17 = level(lv[t - 1]);
+    fill_tail(&A.tail, lv + t, nlev - t, nu1, nu2, kind, approx, coarse_sweeps, events);
+    set_tail_offsets(&A.tail, false);
+    A.cycles = cycles;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(KC);
+    cfg.blockDim = dim3(TC);
+    cfg.dynamicSmemBytes = (size_t)cluster_smem_bytes();
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = KC;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    count_launches(1);
+    return cudaLaunchKernelEx(&cfg, k_corr_vcycle_cluster, A);
+}
+
+bool prepare_corr_cluster()
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(KC);
+    cfg.blockDim = dim3(TC);
+    cfg.dynamicSmemBytes = (size_t)cluster_smem_bytes();
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = KC;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int clusters = 0;
+    const bool ok = cudaFuncSetAttribute(k_corr_vcycle_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         cluster_smem_bytes()) == cudaSuccess &&
+                    cudaFuncSetAttribute(k_corr_vcycle_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
+                        cudaSuccess &&
+                    cudaOccupancyMaxActiveClusters(&clusters, k_corr_vcycle_cluster, &cfg) == cudaSuccess && clusters > 0;
+    if (!ok) (void)cudaGetLastError();
+    return ok;
 }
 
 cudaError_t prepare_coarsest_f64();

@@ -127,3 +127,41 @@ def test_tail_sizes_outside_the_level_sizes_are_refused():
         with pytest.raises(M.MAError):
             M.ma_set_corr_tail(bad)
     assert M.ma_set_vcycle_tail(True) is None and M.ma_set_corr_tail(True) is None
+
+
+@pytest.mark.parametrize("n,precision,kw", [
+    (17, M.MA_MIXED, {}), (33, M.MA_MIXED, {}), (65, M.MA_MIXED, {}), (33, M.MA_FP32, {}), (129, M.MA_FP32, {}),
+    (33, M.MA_MIXED, dict(coarsest_n=5)), (17, M.MA_MIXED, dict(coarsest_n=9)), (33, M.MA_MIXED, dict(coarsest_n=9)),
+    (33, M.MA_MIXED, dict(coarsest_n=17)), (9, M.MA_MIXED, {}),
+    (33, M.MA_MIXED, dict(nu1=1, nu2=3)), (17, M.MA_MIXED, dict(nu1=0, nu2=2)), (33, M.MA_MIXED, dict(nu1=2, nu2=0)),
+    (33, M.MA_MIXED, dict(restrict_kind=M.MA_HALF_WEIGHTING, approx_restrict=M.MA_APPROX_INJECTION, coarse_sweeps=4)),
+    (65, M.MA_FP32, dict(approx_restrict=M.MA_APPROX_INJECTION, inner_cycles=1))])
+@pytest.mark.parametrize("pairs", [True, False])
+def test_cluster_cycle_is_bitwise_the_level_by_level_cycle(n, precision, kw, pairs):
+    """The levels up to 33^3 in one cluster launch (the default) against every
+    level by its own launches, from the Dirichlet data on (the first cycles are
+    far from convergence): iterate, residuals, cycles and root events, sweeping
+    in colour pairs and in ascending order."""
+    pr = P.make("exp", n)
+    out = []
+    try:
+        for v in (17, 33):
+            M.ma_set_corr_tuning(v, M.MA_CORR_PAIRS if pairs else M.MA_CORR_BY_COLOUR, -1)
+        for tail in (True, False):
+            M.ma_set_corr_tail(tail)
+            H = M.Hierarchy(M.make_desc(n, precision=precision, **kw))
+            H.set_rhs_bc(dev(pr.f), dev(pr.initial()))
+            for init in (M.MA_INIT_FMG, M.MA_INIT_ZERO):
+                r = H.solve(tol=1e-11, max_cycles=6, init=init, raise_on_error=False)
+                u = torch.empty_like(dev(pr.f))
+                H.get_solution(u)
+                out.append((host(u), r))
+            H.close()
+    finally:
+        M.ma_set_corr_tail(True)
+        for v in (17, 33):
+            M.ma_set_corr_tuning(v, -1, -1)
+    for (u, r), (v, q) in zip(out[:2], out[2:]):
+        assert np.array_equal(u, v, equal_nan=True)
+        assert (r.cycles, r.status, r.nonconvex_root_events) == (q.cycles, q.status, q.nonconvex_root_events)
+        assert r.res == q.res or (np.isnan(r.res) and np.isnan(q.res))
