@@ -249,13 +249,18 @@ cudaError_t refresh_base(ma_hierarchy* H, int apply, int l0)
 }
 
 // First level of the cycles from l0 that the cluster launch takes (33^3 or
-// 17^3, down to the coarsest grid, which is 9^3 or smaller), or -1.
+// 17^3 sweeping in colour pairs, down to the coarsest grid, which is 9^3 or
+// smaller), or -1.
 int cluster_level(const ma_hierarchy* H, int l0)
 {
     if (!H->corr_cluster || H->lev[H->L - 1].n > 9) return -1;
-    for (int l = l0; l < H->L; ++l)
-        if (H->lev[l].n <= ma::corr_cluster_max_n()) return H->lev[l].n >= 17 ? l : -1;
-    return -1;
+    int lc = -1;
+    for (int l = H->L - 1; l >= l0 && H->lev[l].n <= ma::corr_cluster_max_n(); --l) {
+        if (H->lev[l].n < 17) continue;
+        if (ma::corr_smooth_choice(H->lev[l].n) != ma::CORR_PAIRS) break;
+        lc = l;
+    }
+    return lc;
 }
 
 // One cycle from level l0; lc >= 0: `cluster` runs the levels from lc down.

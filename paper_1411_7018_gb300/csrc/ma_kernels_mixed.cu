@@ -1418,28 +1418,36 @@ __global__ void __launch_bounds__(TT, 1) k_corr_vcycle_tail(TailArgs A) { corr_t
 // Correction V-cycles from a level of 33^3 or 17^3 down to the coarsest grid
 // and back in one cluster of 16 thread blocks.  Level by level those two grids
 // take 16 colour-pair launches and 4 transfers each a cycle, 1.8 us and more
-// apiece whatever their work; here a phase is a cluster barrier.
+// apiece whatever their work.
 //
 // A block owns planes of k: at 33^3 the odd plane 2m + 1 and the even plane
 // 2m + 2 (m its rank), at 17^3 the plane m + 1, in shared memory with one
-// plane of its neighbours on either side.  A phase updates the even planes'
-// colour and the odd planes' colour of a pair (at most 481 points a block,
-// one a thread), and each new value also goes to the neighbour block that
-// holds its plane as a halo.  Points of the pair's other colour, which a
-// neighbour may be writing into the halo meanwhile, are not in the stencil.
+// plane of its neighbours on either side, and their B and rhs.  A phase
+// updates the even planes' colour and the odd planes' colour of a pair (at
+// most 481 points a block, one a thread), and each new value also goes to the
+// neighbour block that holds its plane as a halo.  Points of the pair's other
+// colour, which a neighbour may be writing into the halo meanwhile, are not in
+// the stencil.
+//
+// Phases are ordered between neighbours only, by the data itself: a value is
+// sent with st.async, which counts its bytes on an mbarrier of the receiver,
+// and a block goes on when its own threads are through (a block barrier) and
+// the bytes that its neighbours send in the phase have come.  A cluster
+// barrier with release and acquire took 540 cycles a phase, most of them its
+// fences.  Two mbarriers in turn suffice: every block sends to both neighbours
+// in every phase, so none is more than a phase ahead, and a neighbour that is
+// ahead writes only values whose readers have sent theirs.
 // Coarse plane K = m + 1 of the 17^3 grid sits on the block's own fine plane
 // 2m + 2, so restriction and prolongation stay inside the block but for the
 // halo of r.  The levels up to 9^3 run as the single-block tail does, in the
-// first block.  Every point runs the arithmetic of the separate kernels: the
-// same bits.  B, which nothing here writes, is read from global memory one
-// phase ahead.
+// first block.  Every point runs the arithmetic of the separate kernels in
+// colour-pair order: the same bits.
 // ---------------------------------------------------------------------------
 constexpr int KC = 16;      // blocks of the cluster
 constexpr int TC = 512;     // threads of a block
 
 struct ClusterLevel {
     float inv_h2, h2half;
-    int pairs;
     float* e;             // global, natural layout (top level: read and written back)
     const float* b;       // global colour-major B
     const float* rhs;     // global colour-major rhs (top level: read)
@@ -1482,13 +1490,53 @@ __device__ __forceinline__ float load_remote(const float* smem, unsigned rank)
     return v;
 }
 
+// A value into block `rank`'s shared memory, its 4 bytes counted there on the
+// mbarrier at the place of `bar`.
+__device__ __forceinline__ void send_async(float* smem, unsigned bar, unsigned rank, float v)
+{
+    unsigned a = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("{\n.reg .b32 ra, rb;\nmapa.shared::cluster.u32 ra, %0, %2;\nmapa.shared::cluster.u32 rb, %1, %2;\n"
+                 "st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.f32 [ra], %3, [rb];\n}" ::"r"(a),
+                 "r"(bar), "r"(rank), "f"(v)
+                 : "memory");
+}
+
+// The phases' order between neighbours: phase number t of the launch uses
+// mbarrier t & 1 for the (t >> 1)-th time.
+struct PhaseSync {
+    unsigned bar;      // shared address of the two mbarriers
+    unsigned t;
+    bool lost;         // a wait ran out (another block of the cluster never came): the result is void
+
+    __device__ __forceinline__ unsigned now() const { return bar + 8 * (t & 1); }
+    __device__ __forceinline__ void expect(unsigned bytes) const
+    {
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(now()), "r"(bytes) : "memory");
+    }
+    __device__ __forceinline__ void wait()
+    {
+        const unsigned b = now(), parity = (t >> 1) & 1;
+        unsigned done = 0;
+        for (int spin = 0; spin < (1 << 20) && !done && !lost; ++spin)
+            asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+                         "selp.u32 %0, 1, 0, p;\n}"
+                         : "=r"(done)
+                         : "r"(b), "r"(parity)
+                         : "memory");
+        lost = lost || !done;
+        ++t;
+    }
+};
+
 // One level of the cluster: N points a side, P planes a block (local planes
 // 1 .. P; 0 and P + 1 are the neighbours').  Local plane q is plane m P + q.
 template <int N, int P>
 struct Slab {
     static constexpr int PL = N * N, A = (N - 3) / 2, B = (N - 1) / 2, M2 = (N - 2) * (N - 2);
-    float *e, *r, *rh;          // [P + 2][N][N], the same, [P][M2]
-    const float* b;             // global colour-major B
+    static constexpr int NT = P == 1 ? 64 : TC;   // threads that a phase's points fill: at most B^2, or A^2 + B^2
+    static constexpr int FLOATS = 2 * (P + 2) * PL + 7 * P * M2;
+    static_assert(P == 1 ? B * B <= NT : A * A + B * B <= NT, "one point a thread");
+    float *e, *r, *rh, *b;      // [P + 2][N][N], the same, [P][M2], [P][6][M2]; colours in order inside a plane
     unsigned m;                 // block rank
     float inv_h2, h2half;
 
@@ -1500,10 +1548,9 @@ struct Slab {
     {
         return ((c & 1) ? A * ((c & 2) ? B : A) : 0) + ((c & 2) ? (A + B) * A : 0);
     }
-    static __device__ __forceinline__ int offset(int c) { return (int)cm_offset(N, c); }
 
     // A new value of local plane q at in-plane place s, and its copies in the
-    // neighbours' halos.
+    // neighbours' halos (ordered by the next cluster barrier).
     __device__ __forceinline__ void put(float* f, int q, int s, float v) const
     {
         f[q * PL + s] = v;
@@ -1512,40 +1559,47 @@ struct Slab {
     }
 
     struct Pt {
-        int q, s, cnt;      // local plane, in-plane place, points of the colour
-        const float *b, *r;
+        int q, s, u;      // local plane, place in the plane, slot of its B and rhs
     };
 
-    // Point t of a phase that sweeps colour ce of even planes and colour co of
-    // odd ones (-1: none).
-    __device__ __forceinline__ bool locate(int ce, int co, int t, Pt* X) const
+    // Point t of the phase that sweeps colour c of the even planes and c ^ 7 of the odd ones.
+    __device__ __forceinline__ bool locate(int c, int t, Pt* X) const
     {
-        int q, c;
         const int np = planes();
+        int q = 1, k;
         if (P == 1) {
-            q = 1;
-            c = ((m + 1) & 1) ? co : ce;
-            if (np < 1 || c < 0) return false;
-        } else {            // local plane 1 is odd, 2 even
-            const int no = co >= 0 && np >= 1 ? ni(co) * nj(co) : 0;
-            q = 1;
-            c = co;
-            if (t >= no) {
+            if (np < 1) return false;
+            k = (int)m + 1;
+            if (k & 1) c ^= 7;
+        } else {          // local plane 1 is odd, 2 even
+            const int no = ni(c ^ 7) * nj(c ^ 7);
+            if (t < no) {
+                c ^= 7;
+            } else {
                 t -= no;
                 q = 2;
-                c = ce;
-                if (c < 0 || np < 2) return false;
+                if (np < 2) return false;
             }
         }
         if (t >= ni(c) * nj(c)) return false;
-        const int d = ni(c), y = (c & 1) ? t / B : t / A, x = t - y * d;
-        const int k = (int)m * P + q, kk = (k - ((k & 1) ? 1 : 2)) >> 1;
+        const int y = (c & 1) ? t / B : t / A, x = t - y * ni(c);
         X->q = q;
         X->s = (((c & 2) ? 1 : 2) + 2 * y) * N + ((c & 1) ? 1 : 2) + 2 * x;
-        X->cnt = d * nj(c) * ((c & 4) ? B : A);
-        X->b = b + 6 * offset(c) + kk * (d * nj(c)) + t;
-        X->r = rh + (q - 1) * M2 + in_plane(c) + t;
+        X->u = in_plane(c) + t;
         return true;
+    }
+
+    // Bytes that the neighbours send in that phase: the last plane of the block before, the first of the one after.
+    __device__ __forceinline__ unsigned bytes(int c) const
+    {
+        auto plane = [&](int k) -> unsigned {
+            if (k < 1 || k > N - 2) return 0u;
+            const int d = (k & 1) ? c ^ 7 : c;
+            return 4u * (unsigned)(ni(d) * nj(d));
+        };
+        const int k0 = (int)m * P;
+        // P = 1: the last block owns no interior plane and sends one word to keep its turn
+        return plane(k0) + (P == 1 && m == KC - 2 ? 4u : plane(k0 + P + 1));
     }
 
     // Interior point t of the block's planes in natural order.
@@ -1557,67 +1611,74 @@ struct Slab {
         *i = 1 + u - y * (N - 2);
         return p < planes();
     }
-    // B and the rhs slot of the interior point (i, j) of local plane q
-    __device__ __forceinline__ S3f base(int q, int i, int j, int* slot) const
+    // slot of its B and rhs
+    static __device__ __forceinline__ int slot(int i, int j)
     {
-        const int k = (int)m * P + q;
-        const int c = (i & 1) | ((j & 1) << 1) | ((k & 1) << 2);
-        const int u = ((j - 1) >> 1) * ni(c) + ((i - 1) >> 1), pl = ni(c) * nj(c);
-        *slot = (q - 1) * M2 + in_plane(c) + u;
-        return load_b(b + 6 * offset(c) + ((k - 1) >> 1) * pl + u, pl * ((c & 4) ? B : A));
+        const int c = (i & 1) | ((j & 1) << 1);
+        return in_plane(c) + ((j - 1) >> 1) * ni(c) + ((i - 1) >> 1);
     }
 
+    __device__ __forceinline__ S3f base(int q, int u) const { return load_b_sm(b + (q - 1) * 6 * M2 + u, M2); }
     __device__ __forceinline__ S3f hess(const float* f, int q, int s) const
     {
         return corr_hess_sm(f, q * PL + s, N, PL, f[q * PL + s], inv_h2);
     }
 
-    // nsw sweeps; every phase ends with the cluster's barrier.
-    __device__ __forceinline__ void smooth(int nsw, int pairs, unsigned long long* ev) const
+    // nsw sweeps in colour pairs.  Every thread of the block enters; ends with a block barrier.
+    __device__ __forceinline__ void smooth(int nsw, PhaseSync& S, float* word, unsigned long long* ev) const
     {
-        const int per = pairs ? 4 : 7, nq = nsw * per;
-        // ascending: 0, 1, 2, (3, 4), 5, 6, 7
-        auto even = [&](int w) { return pairs ? w : (w <= 3 ? w : -1); };
-        auto odd = [&](int w) { return pairs ? w ^ 7 : (w >= 3 ? w + 1 : -1); };
-        Pt cur, nxt;
-        S3f Bc = {0, 0, 0, 0, 0, 0}, Bn = Bc;
-        float rc = 0.0f, rn = 0.0f;
-        bool on = nq > 0 && locate(even(0), odd(0), threadIdx.x, &cur);
-        if (on) {
-            Bc = load_b(cur.b, cur.cnt);
-            rc = *cur.r;
-        }
-        int w = 0;
-        for (int t = 0; t < nq; ++t) {
-            w = w + 1 == per ? 0 : w + 1;
-            const bool onn = t + 1 < nq && locate(even(w), odd(w), threadIdx.x, &nxt);
-            if (onn) {
-                Bn = load_b(nxt.b, nxt.cnt);
-                rn = *nxt.r;
-            }
+        if ((int)threadIdx.x < NT) {
+            Pt cur, nxt;
+            S3f Bc = {0, 0, 0, 0, 0, 0}, Bn = Bc;
+            float rc = 0.0f, rn = 0.0f;
+            bool on = nsw > 0 && locate(0, threadIdx.x, &cur);
             if (on) {
-                const float e0 = e[cur.q * PL + cur.s];
-                const S3f K = hess(e, cur.q, cur.s);
-                bool nonconvex = false;
-                put(e, cur.q, cur.s, fmaf(h2half, corr_root(Bc, K, rc, &nonconvex), e0));
-                *ev += nonconvex ? 1ull : 0ull;
+                Bc = base(cur.q, cur.u);
+                rc = rh[(cur.q - 1) * M2 + cur.u];
             }
-            cluster_barrier();
-            on = onn;
-            cur = nxt;
-            Bc = Bn;
-            rc = rn;
+            for (int t = 0; t < 4 * nsw; ++t) {
+                if (threadIdx.x == 0) {
+                    S.expect(bytes(t & 3));
+                    if (P == 1 && m == KC - 1) send_async(word, S.now(), m - 1, 0.0f);
+                }
+                const bool onn = t + 1 < 4 * nsw && locate((t + 1) & 3, threadIdx.x, &nxt);
+                if (onn) {   // B and rhs of the next phase, which nothing writes
+                    Bn = base(nxt.q, nxt.u);
+                    rn = rh[(nxt.q - 1) * M2 + nxt.u];
+                }
+                if (on) {
+                    float* p = e + cur.q * PL + cur.s;
+                    const float e0 = *p;
+                    const S3f K = hess(e, cur.q, cur.s);
+                    bool nonconvex = false;
+                    const float v = fmaf(h2half, corr_root(Bc, K, rc, &nonconvex), e0);
+                    *p = v;
+                    if (cur.q == 1 && m > 0) send_async(e + (P + 1) * PL + cur.s, S.now(), m - 1, v);
+                    if (cur.q == P && m + 1 < KC) send_async(e + cur.s, S.now(), m + 1, v);
+                    *ev += nonconvex ? 1ull : 0ull;
+                }
+                if (P == 1) asm volatile("bar.sync 2, 64;" ::: "memory");
+                else __syncthreads();
+                S.wait();
+                on = onn;
+                cur = nxt;
+                Bc = Bn;
+                rc = rn;
+            }
+        } else {
+            S.t += 4 * nsw;
         }
+        __syncthreads();
     }
 
     // r = rhs - N(e) on the block's planes, with halos.
     __device__ __forceinline__ void residual() const
     {
         for (int t = threadIdx.x; t < P * M2; t += TC) {
-            int q, i, j, slot;
+            int q, i, j;
             if (!interior(t, &q, &i, &j)) continue;
-            const S3f Bm = base(q, i, j, &slot);
-            put(r, q, j * N + i, rh[slot] - delta_det(Bm, hess(e, q, j * N + i)));
+            const int u = slot(i, j);
+            put(r, q, j * N + i, rh[(q - 1) * M2 + u] - delta_det(base(q, u), hess(e, q, j * N + i)));
         }
         cluster_barrier();
     }
@@ -1626,36 +1687,41 @@ struct Slab {
     __device__ __forceinline__ void coarse_rhs(const float* w) const
     {
         for (int t = threadIdx.x; t < P * M2; t += TC) {
-            int q, i, j, slot;
+            int q, i, j;
             if (!interior(t, &q, &i, &j)) continue;
-            const S3f Bm = base(q, i, j, &slot);
-            rh[slot] = delta_det(Bm, hess(w, q, j * N + i)) + r[q * PL + j * N + i];
+            const int u = slot(i, j);
+            rh[(q - 1) * M2 + u] = delta_det(base(q, u), hess(w, q, j * N + i)) + r[q * PL + j * N + i];
         }
         __syncthreads();
     }
 
-    // The top level's iterate and right-hand side from global memory.
-    __device__ __forceinline__ void load(const float* ge, const float* grhs) const
+    // B of the block's planes from the colour-major store, and at the level the
+    // cycle enters (ge not null) its iterate and right-hand side.
+    __device__ __forceinline__ void load(const float* gb, const float* ge, const float* grhs) const
     {
+        for (int t = threadIdx.x; t < P * M2; t += TC) {
+            int q, i, j;
+            if (!interior(t, &q, &i, &j)) continue;
+            const int k = (int)m * P + q, c = (i & 1) | ((j & 1) << 1) | ((k & 1) << 2), u = slot(i, j);
+            const int pl = ni(c) * nj(c), at = ((k - 1) >> 1) * pl + u - in_plane(c), off = (int)cm_offset(N, c);
+            const S3f Bm = load_b(gb + 6 * off + at, pl * ((c & 4) ? B : A));
+            float* d = b + (q - 1) * 6 * M2 + u;
+            d[0] = Bm.xx; d[M2] = Bm.yy; d[2 * M2] = Bm.zz; d[3 * M2] = Bm.xy; d[4 * M2] = Bm.xz; d[5 * M2] = Bm.yz;
+            if (ge) rh[(q - 1) * M2 + u] = grhs[off + at];
+        }
+        if (!ge) return;
         for (int t = threadIdx.x; t < (P + 2) * PL; t += TC) {
             const int k = (int)m * P + t / PL;
             e[t] = k < N ? ge[k * PL + t % PL] : 0.0f;
         }
-        for (int t = threadIdx.x; t < P * M2; t += TC) {
-            int q, i, j;
-            if (!interior(t, &q, &i, &j)) continue;
-            const int k = (int)m * P + q, c = (i & 1) | ((j & 1) << 1) | ((k & 1) << 2);
-            const int u = ((j - 1) >> 1) * ni(c) + ((i - 1) >> 1);
-            rh[(q - 1) * M2 + in_plane(c) + u] = grhs[offset(c) + ((k - 1) >> 1) * (ni(c) * nj(c)) + u];
-        }
     }
 
-    __device__ __forceinline__ void store(float* ge) const
+    __device__ __forceinline__ void store(float* ge, bool lost) const
     {
         for (int t = threadIdx.x; t < P * M2; t += TC) {
             int q, i, j;
             if (!interior(t, &q, &i, &j)) continue;
-            ge[((int)m * P + q) * PL + j * N + i] = e[q * PL + j * N + i];
+            ge[((int)m * P + q) * PL + j * N + i] = lost ? __int_as_float(0x7fffffff) : e[q * PL + j * N + i];
         }
     }
 };
@@ -1680,12 +1746,13 @@ __device__ __forceinline__ float cluster_prolong(const float* dlo, const float* 
     return (i & 1) ? (line(I) + line(I + 1)) * 0.5f : line(I);
 }
 
-constexpr int kClusterFloats33 = 2 * 4 * 33 * 33 + 2 * 31 * 31;
-constexpr int kClusterFloats17 = 3 * 3 * 17 * 17 + 15 * 15 + 2 * 17 * 17;
+constexpr int kClusterFloats = Slab<33, 2>::FLOATS + Slab<17, 1>::FLOATS + 5 * 17 * 17;   // and w, and two planes of d
 
 __global__ void __launch_bounds__(TC, 1) k_corr_vcycle_cluster(const __grid_constant__ ClusterArgs A)
 {
     extern __shared__ float csm[];
+    __shared__ alignas(8) unsigned long long bars[2];
+    __shared__ float word;
     const unsigned m = cluster_rank();
     float* q = csm;
     auto take = [&](int f) {
@@ -1694,25 +1761,30 @@ __global__ void __launch_bounds__(TC, 1) k_corr_vcycle_cluster(const __grid_cons
         return p;
     };
     Slab<33, 2> F;
-    F.e = take(4 * 33 * 33); F.r = take(4 * 33 * 33); F.rh = take(2 * 31 * 31);
-    F.b = A.l33.b; F.m = m; F.inv_h2 = A.l33.inv_h2; F.h2half = A.l33.h2half;
+    F.e = take(4 * F.PL); F.r = take(4 * F.PL); F.rh = take(2 * F.M2); F.b = take(12 * F.M2);
+    F.m = m; F.inv_h2 = A.l33.inv_h2; F.h2half = A.l33.h2half;
     Slab<17, 1> C;
-    C.e = take(3 * 17 * 17);
-    float* w17 = take(3 * 17 * 17);
-    C.r = take(3 * 17 * 17); C.rh = take(15 * 15);
-    C.b = A.l17.b; C.m = m; C.inv_h2 = A.l17.inv_h2; C.h2half = A.l17.h2half;
-    float* d = take(2 * 17 * 17);   // planes of e_H - w_H
+    C.e = take(3 * C.PL); C.r = take(3 * C.PL); C.rh = take(C.M2); C.b = take(6 * C.M2);
+    C.m = m; C.inv_h2 = A.l17.inv_h2; C.h2half = A.l17.h2half;
+    float* w17 = take(3 * C.PL);
+    float* d = take(2 * C.PL);      // planes of e_H - w_H
     float* tsm = q;                 // first block: the levels from 9^3 down
     const TailArgs& T = A.tail;
     const TailLevel& V9 = T.lev[0];
     unsigned long long ev = 0;
-    if (A.top33) F.load(A.l33.e, A.l33.rhs);
-    else C.load(A.l17.e, A.l17.rhs);
+    PhaseSync S{(unsigned)__cvta_generic_to_shared(bars), 0u, false};
+    if (threadIdx.x == 0) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(S.bar) : "memory");
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(S.bar + 8) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (A.top33) F.load(A.l33.b, A.l33.e, A.l33.rhs);
+    C.load(A.l17.b, A.top33 ? nullptr : A.l17.e, A.l17.rhs);
     if (m == 0) tail_load_base(T, tsm);
-    cluster_barrier();   // every block is running before its memory is written from another
+    cluster_barrier();   // every block is running and its mbarriers are set before another writes to it
     for (int cyc = 0; cyc < A.cycles; ++cyc) {
         if (A.top33) {
-            F.smooth(T.nu1, A.l33.pairs, &ev);
+            F.smooth(T.nu1, S, &word, &ev);
             F.residual();
             // coarse plane K = m + 1 on the block's fine plane 2m + 2, and plane 0 in the first block
             for (int t = threadIdx.x; t < (m == 0 ? 2 : 1) * C.PL; t += TC) {
@@ -1733,7 +1805,7 @@ __global__ void __launch_bounds__(TC, 1) k_corr_vcycle_cluster(const __grid_cons
             cluster_barrier();
             C.coarse_rhs(w17);
         }
-        C.smooth(T.nu1, A.l17.pairs, &ev);
+        C.smooth(T.nu1, S, &word, &ev);
         C.residual();
         // plane K of the 9^3 grid sits on fine plane 2K: local plane 1 of the blocks of odd rank; the shell planes on
         // the outer halos of the first and the second to last block
@@ -1771,7 +1843,7 @@ __global__ void __launch_bounds__(TC, 1) k_corr_vcycle_cluster(const __grid_cons
             }
         }
         cluster_barrier();
-        C.smooth(T.nu2, A.l17.pairs, &ev);
+        C.smooth(T.nu2, S, &word, &ev);
         if (A.top33) {   // fine plane 2m + 1 between coarse planes m and m + 1, plane 2m + 2 on coarse plane m + 1
             for (int t = threadIdx.x; t < 2 * C.PL; t += TC) d[t] = C.e[t] - w17[t];
             __syncthreads();
@@ -1784,11 +1856,13 @@ __global__ void __launch_bounds__(TC, 1) k_corr_vcycle_cluster(const __grid_cons
                 F.put(F.e, lq, s, F.e[lq * F.PL + s] + v);
             }
             cluster_barrier();
-            F.smooth(T.nu2, A.l33.pairs, &ev);
+            F.smooth(T.nu2, S, &word, &ev);
         }
     }
-    if (A.top33) F.store(A.l33.e);
-    else C.store(A.l17.e);
+    const bool lost = __syncthreads_or(S.lost);
+    if (A.top33) F.store(A.l33.e, lost);
+    else C.store(A.l17.e, lost);
+    cluster_barrier();   // no block leaves while another may still write to it
     if (T.events && ev) atomicAdd(T.events, ev);
 }
 
@@ -2238,7 +2312,7 @@ static_assert(TC == TT, "the cluster's first block runs the tail's block body");
 
 static int cluster_smem_bytes()
 {
-    return (kClusterFloats33 + kClusterFloats17 + tail_level_floats(9, false) + tail_level_floats(5, false) +
+    return (kClusterFloats + tail_level_floats(9, false) + tail_level_floats(5, false) +
             tail_level_floats(3, false)) * (int)sizeof(float);
 }
 
@@ -2250,8 +2324,8 @@ cudaError_t launch_corr_vcycle_cluster(const TailSpec* lv, int nlev, int cycles,
     const int t = A.top33 ? 2 : 1;   // the tail's first level
     if (nlev - t < 1 || nlev - t > 3 || lv[t].n != 9 || lv[t - 1].n != 17) return cudaErrorInvalidValue;
     auto level = [](const TailSpec& v) {
-        return ClusterLevel{(float)(1.0 / (v.h * v.h)), (float)(0.5 * v.h * v.h),
-                            corr_smooth_choice(v.n) == CORR_PAIRS, v.e, (const float*)v.bstore, v.rhs_cm};
+        return ClusterLevel{(float)(1.0 / (v.h * v.h)), (float)(0.5 * v.h * v.h), v.e, (const float*)v.bstore,
+                            v.rhs_cm};
     };
     if (A.top33) A.l33 = level(lv[0]);
     A.l17 = level(lv[t - 1]);
