@@ -44,32 +44,42 @@ struct S3f {
     float xx, yy, zz, xy, xz, yz;
 };
 
-// Scaled Hessian (divided by h^2) from a difference functor d(di, dj, dk) =
-// value at the offset minus the centre value; every user builds B and K
-// through this one routine, in the same order of operations.
-template <typename D>
-__device__ __forceinline__ S3f hess_from_diff(D d, float inv_h2)
+// Scaled Hessian (divided by h^2) from the stencil's values v(di, dj, dk);
+// sub(a, b) takes their differences.  Every sum is one of differences of
+// neighbours or to the centre, which lose no digits of the values' common
+// part; every user builds B and K through this one routine, in the same order
+// of operations.  The products are kept from contraction into the sums that
+// follow, which could differ from kernel to kernel.
+__device__ __forceinline__ float sub(float a, float b) { return a - b; }
+
+template <typename V>
+__device__ __forceinline__ S3f hess_of(V v, float inv_h2)
 {
     S3f B;
     const float q = 0.25f * inv_h2;
-    B.xx = (d(1, 0, 0) + d(-1, 0, 0)) * inv_h2;
-    B.yy = (d(0, 1, 0) + d(0, -1, 0)) * inv_h2;
-    B.zz = (d(0, 0, 1) + d(0, 0, -1)) * inv_h2;
-    B.xy = ((d(1, 1, 0) + d(-1, -1, 0)) - (d(-1, 1, 0) + d(1, -1, 0))) * q;
-    B.xz = ((d(1, 0, 1) + d(-1, 0, -1)) - (d(-1, 0, 1) + d(1, 0, -1))) * q;
-    B.yz = ((d(0, 1, 1) + d(0, -1, -1)) - (d(0, 1, -1) + d(0, -1, 1))) * q;
+    const auto c = v(0, 0, 0);
+    B.xx = __fmul_rn(sub(v(1, 0, 0), c) + sub(v(-1, 0, 0), c), inv_h2);
+    B.yy = __fmul_rn(sub(v(0, 1, 0), c) + sub(v(0, -1, 0), c), inv_h2);
+    B.zz = __fmul_rn(sub(v(0, 0, 1), c) + sub(v(0, 0, -1), c), inv_h2);
+    B.xy = __fmul_rn(sub(v(1, 1, 0), v(-1, 1, 0)) - sub(v(1, -1, 0), v(-1, -1, 0)), q);
+    B.xz = __fmul_rn(sub(v(1, 0, 1), v(-1, 0, 1)) - sub(v(1, 0, -1), v(-1, 0, -1)), q);
+    B.yz = __fmul_rn(sub(v(0, 1, 1), v(0, -1, 1)) - sub(v(0, 1, -1), v(0, -1, -1)), q);
     return B;
 }
 
 // B = D^2_h u from the hi/lo split of u in global memory.
+struct HiLo {
+    float hi, lo;
+};
+__device__ __forceinline__ float sub(HiLo a, HiLo b) { return (a.hi - b.hi) + (a.lo - b.lo); }
+
 __device__ __forceinline__ S3f base_hess(const float* __restrict__ hi, const float* __restrict__ lo, long long p,
                                          long long sy, long long sz, float inv_h2)
 {
-    const float vh = hi[p], vl = lo[p];
-    return hess_from_diff(
-        [&](int di, int dj, int dk) -> float {
+    return hess_of(
+        [&](int di, int dj, int dk) -> HiLo {
             const long long o = p + di + dj * sy + dk * sz;
-            return (__ldg(hi + o) - vh) + (__ldg(lo + o) - vl);
+            return {__ldg(hi + o), __ldg(lo + o)};
         },
         inv_h2);
 }
@@ -78,67 +88,89 @@ __device__ __forceinline__ S3f base_hess(const float* __restrict__ hi, const flo
 // fixed order, so that every kernel that inlines them (by-colour and plane
 // sweeps, residuals, the fused tail) rounds identically: the compiler may
 // otherwise contract a*b + c*d either way depending on the surrounding code.
-__device__ __forceinline__ float mdiff(float a, float b, float c, float d) { return fmaf(a, b, -(c * d)); }   // ab - cd
-
-__device__ __forceinline__ float det3(const S3f& A)
+__device__ __forceinline__ float mdiff(float a, float b, float c, float d)   // ab - cd
 {
-    const float c1 = mdiff(A.yy, A.zz, A.yz, A.yz);
-    const float c2 = mdiff(A.xy, A.zz, A.xz, A.yz);
-    const float c3 = mdiff(A.xy, A.yz, A.yy, A.xz);
-    return fmaf(A.xz, c3, fmaf(A.xx, c1, -(A.xy * c2)));
+    return fmaf(a, b, -__fmul_rn(c, d));
 }
 
-// tr(cof(A) X) for symmetric A, X.
-__device__ __forceinline__ float cof_dot(const S3f& A, const S3f& X)
+__device__ __forceinline__ S3f cofactors(const S3f& A)
 {
-    const float cxx = mdiff(A.yy, A.zz, A.yz, A.yz);
-    const float cyy = mdiff(A.xx, A.zz, A.xz, A.xz);
-    const float czz = mdiff(A.xx, A.yy, A.xy, A.xy);
-    const float cxy = mdiff(A.xz, A.yz, A.xy, A.zz);
-    const float cxz = mdiff(A.xy, A.yz, A.xz, A.yy);
-    const float cyz = mdiff(A.xy, A.xz, A.xx, A.yz);
-    const float diag = fmaf(czz, X.zz, fmaf(cyy, X.yy, cxx * X.xx));
-    const float off = fmaf(cyz, X.yz, fmaf(cxz, X.xz, cxy * X.xy));
-    return fmaf(2.0f, off, diag);
+    return {mdiff(A.yy, A.zz, A.yz, A.yz), mdiff(A.xx, A.zz, A.xz, A.xz), mdiff(A.xx, A.yy, A.xy, A.xy),
+            mdiff(A.xz, A.yz, A.xy, A.zz), mdiff(A.xy, A.yz, A.xz, A.yy), mdiff(A.xy, A.xz, A.xx, A.yz)};
 }
 
-// N = det(B + K) - det(B) by the 3x3 expansion.
-__device__ __forceinline__ float delta_det(const S3f& B, const S3f& K)
+// N = det(B + K) - det(B) by the 3x3 expansion tr(cof(B) K) + tr(cof(K) B) +
+// det(K), cB = cof(B).  With det(K) = K.xx k.xx + K.xy k.xy + K.xz k.xz (k =
+// cof(K)) the last two are one sum over k.
+__device__ __forceinline__ float delta_det(const S3f& B, const S3f& cB, const S3f& K)
 {
-    return cof_dot(B, K) + cof_dot(K, B) + det3(K);
+    const S3f k = cofactors(K);
+    const float first = fmaf(cB.zz, K.zz, fmaf(cB.yy, K.yy, __fmul_rn(cB.xx, K.xx)));
+    float off = fmaf(cB.yz, K.yz, fmaf(cB.xz, K.xz, __fmul_rn(cB.xy, K.xy)));
+    off = fmaf(k.yz, B.yz, off);
+    float rest = __fmul_rn(k.xx, B.xx + K.xx);
+    rest = fmaf(k.yy, B.yy, rest);
+    rest = fmaf(k.zz, B.zz, rest);
+    rest = fmaf(k.xy, B.xy + (B.xy + K.xy), rest);
+    rest = fmaf(k.xz, B.xz + (B.xz + K.xz), rest);
+    return fmaf(2.0f, off, first + rest);
 }
+
+__device__ __forceinline__ float delta_det(const S3f& B, const S3f& K) { return delta_det(B, cofactors(B), K); }
 
 // Smallest-root update of the correction problem at one point, z with
-// e_new = e0 + h^2 z / 2.  Fast path: FP32 Newton on
-// F(z) = det(G - zI) - det(B) - r from z = 0 (its first step is z = F(0) / M)
-// when G = B + K is positive definite and not near-degenerate, and the
-// target det(B) + r = det(G) - F(0) is clearly positive (Theorem 2.2: then F
-// is decreasing and convex left of the smallest eigenvalue of G, which lies
-// right of z = 0, and has its one root there; with a target <= 0 Eq.
-// (realroots) asks for the smallest real root elsewhere, which only the FP64
-// path finds and counts).  It stops once a step is at most 1e-4 |z|: Newton
-// converges quadratically there, so the step just taken leaves an error of
-// order (1e-4)^2 |z|, below FP32 resolution.  Returns false (z unset) when
-// the point needs the FP64 path.
+// e_new = e0 + h^2 z / 2.  Fast path: FP32 solution of
+// F(z) = det(G - zI) - det(B) - r = c - M z + T z^2 - z^3 near z = 0 when
+// G = B + K is positive definite and not near-degenerate, and the target
+// det(B) + r is clearly positive (Theorem 2.2: then F is decreasing and convex
+// left of the smallest eigenvalue of G, which lies right of z = 0, and has its
+// one root there; with a target <= 0 Eq. (realroots) asks for the smallest real
+// root elsewhere, which only the FP64 path finds and counts).
+//
+// A correction is mostly small against the Hessian, and then z = c / M is
+// nearly the root: with one reciprocal of M the iteration
+// z <- (c + z^2 (T - z)) / M contracts by 2 T z / M, a chain of four
+// operations a step where Newton's has a division.  It stops when the step
+// times that rate is at most 6e-8 |z|.  From T z > 0.03 M on Newton from
+// there, which stops once a step is at most 1e-4 |z|: it converges
+// quadratically, so the step just taken leaves an error of order (1e-4)^2 |z|,
+// below FP32 resolution.  Returns false (z unset) when the point needs the
+// FP64 path.
 __device__ __forceinline__ bool corr_root_fast(const S3f& B, const S3f& K, float r, float* zout)
 {
+    const S3f cB = cofactors(B);
+    const float N = delta_det(B, cB, K);
+    const float detB = fmaf(B.xz, cB.xz, fmaf(B.xy, cB.xy, __fmul_rn(B.xx, cB.xx)));
     S3f G;
     G.xx = B.xx + K.xx; G.yy = B.yy + K.yy; G.zz = B.zz + K.zz;
     G.xy = B.xy + K.xy; G.xz = B.xz + K.xz; G.yz = B.yz + K.yz;
-    const float c = delta_det(B, K) - r;   // F(0)
+    const float c = N - r;   // F(0)
     const float T = G.xx + G.yy + G.zz;
     const float m2 = mdiff(G.xx, G.yy, G.xy, G.xy);
     const float M = m2 + mdiff(G.xx, G.zz, G.xz, G.xz) + mdiff(G.yy, G.zz, G.yz, G.yz);
-    const float dG = det3(G);
-    const bool pd = G.xx > 0.0f && m2 > 0.0f && dG > 0.0f;
+    const bool pd = G.xx > 0.0f && m2 > 0.0f && detB + N > 0.0f;
     // with a positive diagonal, |G| summed entrywise is T + |off-diagonals|
     const float scale = T + fabsf(G.xy) + fabsf(G.xz) + fabsf(G.yz);
-    if (!(pd && M > 0.05f * (scale * scale))) return false;
-    // the target det(B) + r, far enough above 0 that FP32 rounding of the
-    // two determinants cannot flip its sign (margin 1e-5 scale^3)
-    if (!(dG - c > 1e-5f * (scale * scale * scale))) return false;
-    // F(z) = c - z M + z^2 T - z^3 = c - z (M - z (T - z));  M(z) = -F'(z)
-    float z = __fdividef(c, M);
+    const float scale2 = __fmul_rn(scale, scale);
+    if (!(pd && M > __fmul_rn(0.05f, scale2))) return false;
+    // the target, far enough above 0 that FP32 rounding of the two
+    // determinants cannot flip its sign (margin 1e-5 scale^3)
+    if (!(detB + r > __fmul_rn(1e-5f, __fmul_rn(scale2, scale)))) return false;
+    const float iM = __fdividef(1.0f, M);
+    float z = __fmul_rn(c, iM);
+    if (fabsf(__fmul_rn(T, z)) <= __fmul_rn(0.03f, M)) {
+        const float enough = __fmul_rn(3e-8f, M);
+        for (int it = 0; it < 8; ++it) {
+            const float zn = __fmul_rn(fmaf(__fmul_rn(z, z), T - z, c), iM);
+            const float dz = zn - z;
+            z = zn;
+            if (__fmul_rn(fabsf(dz), T) <= enough) {
+                *zout = z;
+                return isfinite(z);
+            }
+        }
+    }
+    // F(z) = c - z (M - z (T - z));  M(z) = -F'(z)
     const float T2 = 2.0f * T;
     for (int it = 0; it < 30; ++it) {
         const float F = fmaf(-z, fmaf(-z, T - z, M), c);
@@ -405,11 +437,14 @@ __device__ __forceinline__ void smooth_corr_block(float* e, const float* __restr
         v[0][2][1] = __ldg(q + (sy - sz));
         v[2][0][1] = __ldg(q + (sz - sy));
         e0 = v[1][1][1];
-        K = hess_from_diff([&](int di, int dj, int dk) -> float { return v[dk + 1][dj + 1][di + 1] - e0; }, inv_h2);
+        K = hess_of([&](int di, int dj, int dk) -> float { return v[dk + 1][dj + 1][di + 1]; }, inv_h2);
     } else {
         e0 = q[0];
-        K = hess_from_diff([&](int di, int dj, int dk) -> float { return __ldg(q + (di + dj * sy + dk * sz)) - e0; },
-                           inv_h2);
+        K = hess_of(
+            [&](int di, int dj, int dk) -> float {
+                return di == 0 && dj == 0 && dk == 0 ? e0 : __ldg(q + (di + dj * sy + dk * sz));
+            },
+            inv_h2);
     }
     bool nonconvex = false;
     const float z = corr_root(B, K, __ldcs(rc + idx), &nonconvex);
@@ -649,9 +684,9 @@ __device__ __forceinline__ unsigned colour_phase(float* sp, const float* __restr
         const float rr = __ldcs(rq + rel);
         const int sc = s0 + 2 * b * PW + a;
         const float e0 = sp[sc];
-        const S3f K = hess_from_diff(
+        const S3f K = hess_of(
             [&](int di, int dj, int dk) -> float {
-                return sp[sc + dk * PW * PW + dj * PW + (di > 0 ? DXP : (di < 0 ? DXM : 0))] - e0;
+                return sp[sc + dk * PW * PW + dj * PW + (di > 0 ? DXP : (di < 0 ? DXM : 0))];
             },
             inv_h2);
         if (SMOOTH) {
@@ -680,9 +715,9 @@ __device__ __forceinline__ unsigned colour_phase(float* sp, const float* __restr
         const S3f B = load_b(bq + rel, cnt);
         const int sc = s0 + 2 * b2 * PW + a2;
         const float e0 = sp[sc];
-        const S3f K = hess_from_diff(
+        const S3f K = hess_of(
             [&](int di, int dj, int dk) -> float {
-                return sp[sc + dk * PW * PW + dj * PW + (di > 0 ? DXP : (di < 0 ? DXM : 0))] - e0;
+                return sp[sc + dk * PW * PW + dj * PW + (di > 0 ? DXP : (di < 0 ? DXM : 0))];
             },
             inv_h2);
         bool nonconvex = false;
@@ -847,12 +882,11 @@ __device__ __forceinline__ void residual_corr_col_block(const float* __restrict_
         const float Nc_e = __shfl_down_sync(FULL, Nc, 1), Nc_w = __shfl_up_sync(FULL, Nc, 1);
         const float Sc_e = __shfl_down_sync(FULL, Sc, 1), Sc_w = __shfl_up_sync(FULL, Sc, 1);
         if (act) {
-            const float e0 = Cc;
-            const S3f K = hess_from_diff(
+            const S3f K = hess_of(
                 [&](int di, int dj, int dk) -> float {
                     float v;
                     if (dk == 0) {
-                        if (dj == 0) v = di > 0 ? Cc_e : Cc_w;
+                        if (dj == 0) v = di > 0 ? Cc_e : (di < 0 ? Cc_w : Cc);
                         else if (dj > 0) v = di > 0 ? Nc_e : (di < 0 ? Nc_w : Nc);
                         else v = di > 0 ? Sc_e : (di < 0 ? Sc_w : Sc);
                     } else if (dk > 0) {
@@ -862,7 +896,7 @@ __device__ __forceinline__ void residual_corr_col_block(const float* __restrict_
                         if (dj == 0) v = di > 0 ? Cm_e : (di < 0 ? Cm_w : Cm);
                         else v = dj > 0 ? Nm : Sm;
                     }
-                    return v - e0;
+                    return v;
                 },
                 inv_h2);
             if constexpr (CRHS) {
@@ -944,9 +978,7 @@ __device__ __forceinline__ void coarse_rhs_corr_block(const float* __restrict__ 
     const long long sy = n, sz = (long long)n * n;
     const CmPos c = cm_pos(i, j, k, n);
     const S3f B = load_b(bstore + 6 * c.off + c.idx, c.cnt);
-    const float e0 = w[p];
-    const S3f K = hess_from_diff(
-        [&](int di, int dj, int dk) -> float { return __ldg(w + p + di + dj * sy + dk * sz) - e0; }, inv_h2);
+    const S3f K = hess_of([&](int di, int dj, int dk) -> float { return __ldg(w + p + di + dj * sy + dk * sz); }, inv_h2);
     rhs_cm[c.off + c.idx] = delta_det(B, K) + resc[p];
 }
 
@@ -969,8 +1001,11 @@ __global__ void __launch_bounds__(BX * BY) k_coarse_rhs_corr(const float* __rest
 
 __device__ __forceinline__ S3f corr_hess_sm(const float* e, int p, int sy, int sz, float e0, float inv_h2)
 {
-    return hess_from_diff([&](int di, int dj, int dk) -> float { return e[p + di + dj * sy + dk * sz] - e0; },
-                          inv_h2);
+    return hess_of(
+        [&](int di, int dj, int dk) -> float {
+            return di == 0 && dj == 0 && dk == 0 ? e0 : e[p + di + dj * sy + dk * sz];
+        },
+        inv_h2);
 }
 
 // Index arithmetic of a grid of n <= 17 points a side.  t / d as
