@@ -130,13 +130,16 @@ __device__ __forceinline__ float delta_det(const S3f& B, const S3f& K) { return 
 // A correction is mostly small against the Hessian, and then z = c / M is
 // nearly the root: with one reciprocal of M the iteration
 // z <- (c + z^2 (T - z)) / M contracts by 2 T z / M, a chain of four
-// operations a step where Newton's has a division.  It stops when the step
-// times that rate is at most 6e-8 |z|.  From T z > 0.03 M on Newton from
-// there, which stops once a step is at most 1e-4 |z|: it converges
-// quadratically, so the step just taken leaves an error of order (1e-4)^2 |z|,
-// below FP32 resolution.  Returns false (z unset) when the point needs the
-// FP64 path.
-__device__ __forceinline__ bool corr_root_fast(const S3f& B, const S3f& K, float r, float* zout)
+// operations a step where Newton's has a division.  Two steps are taken, and
+// their result where T z <= 0.03 M and the second step times that rate is at
+// most 6e-8 |z|: no branch, one test.  Returns false (z unset) when the point
+// needs corr_root_rest.
+struct CorrCoef {
+    float c, T, M, scale;
+    bool ok;   // G positive definite, not near-degenerate, the target clearly positive
+};
+
+__device__ __forceinline__ CorrCoef corr_coef(const S3f& B, const S3f& K, float r)
 {
     const S3f cB = cofactors(B);
     const float N = delta_det(B, cB, K);
@@ -144,40 +147,47 @@ __device__ __forceinline__ bool corr_root_fast(const S3f& B, const S3f& K, float
     S3f G;
     G.xx = B.xx + K.xx; G.yy = B.yy + K.yy; G.zz = B.zz + K.zz;
     G.xy = B.xy + K.xy; G.xz = B.xz + K.xz; G.yz = B.yz + K.yz;
-    const float c = N - r;   // F(0)
-    const float T = G.xx + G.yy + G.zz;
+    CorrCoef R;
+    R.c = N - r;   // F(0)
+    R.T = G.xx + G.yy + G.zz;
     const float m2 = mdiff(G.xx, G.yy, G.xy, G.xy);
-    const float M = m2 + mdiff(G.xx, G.zz, G.xz, G.xz) + mdiff(G.yy, G.zz, G.yz, G.yz);
-    const bool pd = G.xx > 0.0f && m2 > 0.0f && detB + N > 0.0f;
+    R.M = m2 + mdiff(G.xx, G.zz, G.xz, G.xz) + mdiff(G.yy, G.zz, G.yz, G.yz);
     // with a positive diagonal, |G| summed entrywise is T + |off-diagonals|
-    const float scale = T + fabsf(G.xy) + fabsf(G.xz) + fabsf(G.yz);
-    const float scale2 = __fmul_rn(scale, scale);
-    if (!(pd && M > __fmul_rn(0.05f, scale2))) return false;
-    // the target, far enough above 0 that FP32 rounding of the two
+    R.scale = R.T + fabsf(G.xy) + fabsf(G.xz) + fabsf(G.yz);
+    const float scale2 = __fmul_rn(R.scale, R.scale);
+    // the target det(B) + r far enough above 0 that FP32 rounding of the two
     // determinants cannot flip its sign (margin 1e-5 scale^3)
-    if (!(detB + r > __fmul_rn(1e-5f, __fmul_rn(scale2, scale)))) return false;
-    const float iM = __fdividef(1.0f, M);
-    float z = __fmul_rn(c, iM);
-    if (fabsf(__fmul_rn(T, z)) <= __fmul_rn(0.03f, M)) {
-        const float enough = __fmul_rn(3e-8f, M);
-        for (int it = 0; it < 8; ++it) {
-            const float zn = __fmul_rn(fmaf(__fmul_rn(z, z), T - z, c), iM);
-            const float dz = zn - z;
-            z = zn;
-            if (__fmul_rn(fabsf(dz), T) <= enough) {
-                *zout = z;
-                return isfinite(z);
-            }
-        }
-    }
+    R.ok = (G.xx > 0.0f) & (m2 > 0.0f) & (detB + N > 0.0f) & (R.M > __fmul_rn(0.05f, scale2)) &
+           (detB + r > __fmul_rn(1e-5f, __fmul_rn(scale2, R.scale)));
+    return R;
+}
+
+__device__ __forceinline__ bool corr_root_fast(const S3f& B, const S3f& K, float r, float* zout)
+{
+    const CorrCoef R = corr_coef(B, K, r);
+    const float iM = __fdividef(1.0f, R.M);
+    const float z0 = __fmul_rn(R.c, iM);
+    const float z1 = __fmul_rn(fmaf(__fmul_rn(z0, z0), R.T - z0, R.c), iM);
+    const float z2 = __fmul_rn(fmaf(__fmul_rn(z1, z1), R.T - z1, R.c), iM);
+    *zout = z2;
+    return R.ok & (fabsf(__fmul_rn(R.T, z0)) <= __fmul_rn(0.03f, R.M)) &
+           (__fmul_rn(fabsf(z2 - z1), R.T) <= __fmul_rn(3e-8f, R.M));
+}
+
+// FP32 Newton on F from z = c / M, for the larger corrections: it stops once a
+// step is at most 1e-4 |z|, and converging quadratically leaves an error of
+// order (1e-4)^2 |z|, below FP32 resolution.
+__device__ __forceinline__ bool corr_root_newton(const CorrCoef& R, float* zout)
+{
     // F(z) = c - z (M - z (T - z));  M(z) = -F'(z)
-    const float T2 = 2.0f * T;
+    const float T2 = 2.0f * R.T;
+    float z = __fdividef(R.c, R.M);
     for (int it = 0; it < 30; ++it) {
-        const float F = fmaf(-z, fmaf(-z, T - z, M), c);
-        const float Mz = fmaf(-z, fmaf(-3.0f, z, T2), M);
+        const float F = fmaf(-z, fmaf(-z, R.T - z, R.M), R.c);
+        const float Mz = fmaf(-z, fmaf(-3.0f, z, T2), R.M);
         const float dz = __fdividef(F, Mz);
         z += dz;
-        if (fabsf(dz) <= fmaf(1e-4f, fabsf(z), 1e-12f * scale)) {
+        if (fabsf(dz) <= fmaf(1e-4f, fabsf(z), 1e-12f * R.scale)) {
             *zout = z;
             return isfinite(z);
         }
@@ -229,15 +239,18 @@ __device__ __forceinline__ CorrCubic corr_cubic(const S3f& B, const S3f& K, floa
 __device__ __forceinline__ double corr_F(const CorrCubic& C, double z) { return C.c - z * (C.M - z * (C.T - z)); }
 __device__ __forceinline__ double corr_Mz(const CorrCubic& C, double z) { return C.M - z * (2.0 * C.T - 3.0 * z); }
 
-// FP64 path (near-degenerate or indefinite G, or no FP32 convergence).
-// tot > 0: F is decreasing and convex left of the smallest eigenvalue of G
+// The points corr_root_fast leaves: Newton in FP32, else the FP64 path
+// (near-degenerate or indefinite G, or no FP32 convergence).  tot > 0: F is decreasing and convex left of the smallest eigenvalue of G
 // and has its unique root there; monotone Newton from the Gershgorin bound
 // minus tot^(1/3), where F >= 0.  tot <= 0: Eq. (realroots) taken
 // literally, the smallest real root of the cubic, bracketed between the
 // Gershgorin bounds and the stationary points of det(G - zI) and found by
 // bisection (smallest_root_nonpositive), counted in *nonconvex.
-__device__ __noinline__ float corr_root_slow(S3f B, S3f K, float r, bool* nonconvex)
+__device__ __noinline__ float corr_root_rest(S3f B, S3f K, float r, bool* nonconvex)
 {
+    const CorrCoef R = corr_coef(B, K, r);
+    float z32;
+    if (R.ok && corr_root_newton(R, &z32)) return z32;
     const CorrCubic C = corr_cubic(B, K, r);
     if (C.tot > 0.0) {
         const double g0 = C.g[0] - fabs(C.g[3]) - fabs(C.g[4]);
@@ -268,7 +281,7 @@ __device__ __forceinline__ float corr_root(const S3f& B, const S3f& K, float r, 
 {
     float z;
     if (corr_root_fast(B, K, r, &z)) return z;
-    return corr_root_slow(B, K, r, nonconvex);
+    return corr_root_rest(B, K, r, nonconvex);
 }
 
 __host__ __device__ __forceinline__ int colour_count(int n, int parity) { return parity ? (n - 1) / 2 : (n - 3) / 2; }
@@ -721,7 +734,7 @@ __device__ __forceinline__ unsigned colour_phase(float* sp, const float* __restr
             },
             inv_h2);
         bool nonconvex = false;
-        const float z = corr_root_slow(B, K, __ldcs(rq + rel), &nonconvex);
+        const float z = corr_root_rest(B, K, __ldcs(rq + rel), &nonconvex);
         sp[sc] = fmaf(h2half, z, e0);
         // count each point once: halo points are the neighbouring block's
         const int i2 = R.ilo + 2 * a2, j2 = R.jlo + 2 * b2;
@@ -1008,16 +1021,16 @@ __device__ __forceinline__ S3f corr_hess_sm(const float* e, int p, int sy, int s
         inv_h2);
 }
 
-// Index arithmetic of a grid of n <= 17 points a side.  t / d as
+// Index arithmetic of a grid of n = 3, 5, 9 or 17 points a side.  t / d as
 // t (65536 / d + 1) >> 16: exact for t d <= 65536.
 struct SmallGrid {
-    int n, a, b, ma, mb, mi, mn;   // a, b: interior indices of parity 0, 1; m*: reciprocals of a, b, n - 2, n
+    int n, a, b, ma, mi, mn, lb;   // a, b = 2^lb: interior indices of parity 0, 1; m*: reciprocals of a, n - 2, n
     __device__ __forceinline__ explicit SmallGrid(int n_) : n(n_), a((n_ - 3) / 2), b((n_ - 1) / 2)
     {
-        ma = a > 0 ? 65536 / a + 1 : 0;
-        mb = 65536 / b + 1;
-        mi = 65536 / (n - 2) + 1;
-        mn = 65536 / n + 1;
+        lb = n == 3 ? 0 : (n == 5 ? 1 : (n == 9 ? 2 : 3));
+        ma = n == 17 ? 65536 / 7 + 1 : (n == 9 ? 65536 / 3 + 1 : 65537);
+        mi = n == 17 ? 65536 / 15 + 1 : (n == 9 ? 65536 / 7 + 1 : (n == 5 ? 65536 / 3 + 1 : 65537));
+        mn = n == 17 ? 65536 / 17 + 1 : (n == 9 ? 65536 / 9 + 1 : (n == 5 ? 65536 / 5 + 1 : 65536 / 3 + 1));
     }
     __device__ __forceinline__ int count(int c) const
     {
@@ -1032,8 +1045,8 @@ struct SmallGrid {
     __device__ __forceinline__ int point(int c, int t) const
     {
         const bool pi = c & 1, pj = c & 2, pk = c & 4;
-        const int y0 = (t * (pi ? mb : ma)) >> 16, x = t - y0 * (pi ? b : a);
-        const int z = (y0 * (pj ? mb : ma)) >> 16, y = y0 - z * (pj ? b : a);
+        const int y0 = pi ? t >> lb : (t * ma) >> 16, x = t - y0 * (pi ? b : a);
+        const int z = pj ? y0 >> lb : (y0 * ma) >> 16, y = y0 - z * (pj ? b : a);
         return (((pk ? 1 : 2) + 2 * z) * n + (pj ? 1 : 2) + 2 * y) * n + (pi ? 1 : 2) + 2 * x;
     }
     // interior point q in natural order: (i, j, k), its linear index returned
@@ -1056,11 +1069,26 @@ struct SmallGrid {
     }
 };
 
-__device__ __forceinline__ S3f load_b_sm(const float* b, int cnt)
+// B in shared memory is component-major over the grid's mi = (n - 2)^3 slots in
+// colour order: the six entries of a slot lie mi apart.
+__device__ __forceinline__ S3f load_b_sm(const float* b, int mi)
 {
     S3f B;
-    B.xx = b[0]; B.yy = b[cnt]; B.zz = b[2 * cnt]; B.xy = b[3 * cnt]; B.xz = b[4 * cnt]; B.yz = b[5 * cnt];
+    B.xx = b[0]; B.yy = b[mi]; B.zz = b[2 * mi]; B.xy = b[3 * mi]; B.xz = b[4 * mi]; B.yz = b[5 * mi];
     return B;
+}
+
+__device__ __forceinline__ void stage_b_sm(float* sb, const float* __restrict__ bstore, const SmallGrid& G)
+{
+    const int mi = (G.n - 2) * (G.n - 2) * (G.n - 2);
+    for (int q = threadIdx.x; q < mi; q += blockDim.x) {
+        int i, j, k, cnt, off;
+        G.interior(q, &i, &j, &k);
+        const int t = G.slot(i, j, k, &cnt, &off);
+        const S3f B = load_b(bstore + 6 * off + t, cnt);
+        float* d = sb + off + t;
+        d[0] = B.xx; d[mi] = B.yy; d[2 * mi] = B.zz; d[3 * mi] = B.xy; d[4 * mi] = B.xz; d[5 * mi] = B.yz;
+    }
 }
 
 // Warps that run a grid's colour phases, and their barrier: one warp up to
@@ -1074,79 +1102,89 @@ __device__ __forceinline__ void phase_barrier(int n)
     else __syncthreads();
 }
 
-// Visits the points of a phase sequence: phase q (0 .. nq - 1) holds colour
-// first(q) and, where it is not negative, colour second(q).  body(p, B, r,
-// slot_colour...) updates one point.  NT threads of the block enter.
-template <typename First, typename Second, typename Body>
-__device__ __forceinline__ void run_phases(const SmallGrid& G, const float* sb, const float* sr, int nq, int nt,
-                                           First first, Second second, Body body)
+// Phase q of a sweep: in colour pairs (c, c ^ 7) for c = 0 .. 3, or in
+// ascending order in 7 phases: colours 3 and 4 differ in all three parities,
+// so they are independent and share one.
+__device__ __forceinline__ int phases_of(bool pairs) { return pairs ? 4 : 7; }
+__device__ __forceinline__ int phase_first(bool pairs, int q) { return pairs || q <= 3 ? q : q + 1; }
+__device__ __forceinline__ int phase_second(bool pairs, int q) { return pairs ? q ^ 7 : (q == 3 ? 4 : -1); }
+
+// Linear index and slot of a phase's point t, packed; -1 where it has none.
+__device__ __forceinline__ int phase_point(const SmallGrid& G, bool pairs, int q, int t)
 {
-    struct Pt {
-        int p, cnt;
-        const float *b, *r;
-    };
-    const int tid = threadIdx.x;
-    auto locate = [&](int q, int t, Pt* P) -> bool {
-        int c = first(q);
-        const int d = second(q), nc = G.count(c);
-        if (t >= nc) {
-            if (d < 0) return false;
-            t -= nc;
-            c = d;
-            if (t >= G.count(d)) return false;
-        }
-        const int off = G.offset(c);
-        P->cnt = G.count(c);
-        P->p = G.point(c, t);
-        P->b = sb + 6 * off + t;
-        P->r = sr + off + t;
-        return true;
-    };
-    if (G.n <= 9) {   // at most one point a thread: its B and rhs one phase ahead
-        Pt cur, nxt;
+    int c = phase_first(pairs, q);
+    const int d = phase_second(pairs, q), nc = G.count(c);
+    if (t >= nc) {
+        if (d < 0) return -1;
+        t -= nc;
+        c = d;
+        if (t >= G.count(d)) return -1;
+    }
+    return G.point(c, t) | (G.offset(c) + t) << 16;
+}
+
+// The points of grids up to 9^3, at most one a thread in each phase, worked
+// out once: entry [phase][thread].
+constexpr int kPhaseTab = 7 * 128;
+
+__device__ __forceinline__ void fill_phase_tab(int* tab, int n, bool pairs)
+{
+    if (n > 9 || n < 5) return;
+    const SmallGrid G(n);
+    const int lt = n <= 5 ? 5 : 7;   // log2 of the threads
+    for (int x = threadIdx.x; x < phases_of(pairs) << lt; x += blockDim.x)
+        tab[x] = phase_point(G, pairs, x >> lt, x & ((1 << lt) - 1));
+}
+
+// nsw sweeps over a grid in shared memory: body(p, B, r) updates one point.
+// The grid's phase threads enter.
+template <typename Body>
+__device__ __forceinline__ void run_sweeps(const SmallGrid& G, const int* tab, const float* sb, const float* sr,
+                                           bool pairs, int nsw, int nt, Body body)
+{
+    const int tid = threadIdx.x, per = phases_of(pairs), nq = nsw * per, mi = (G.n - 2) * (G.n - 2) * (G.n - 2);
+    if (G.n <= 9) {   // the next phase's B and rhs, which no phase writes, one phase ahead; its place two ahead
+        int w = 1;
+        int cur = tab[tid], nxt = tab[nt + tid];
         S3f B = {0, 0, 0, 0, 0, 0}, Bn = B;
         float r = 0.0f, rn = 0.0f;
-        bool on = locate(0, tid, &cur);
-        if (on) {
-            B = load_b_sm(cur.b, cur.cnt);
-            r = *cur.r;
+        if (cur >= 0) {
+            B = load_b_sm(sb + (cur >> 16), mi);
+            r = sr[cur >> 16];
         }
         for (int q = 0; q < nq; ++q) {
-            const bool onn = q + 1 < nq && locate(q + 1, tid, &nxt);
-            if (onn) {
-                Bn = load_b_sm(nxt.b, nxt.cnt);
-                rn = *nxt.r;
+            w = w + 1 == per ? 0 : w + 1;
+            const int nn = tab[w * nt + tid];
+            if (nxt >= 0) {
+                Bn = load_b_sm(sb + (nxt >> 16), mi);
+                rn = sr[nxt >> 16];
             }
-            if (on) body(cur.p, B, r);
+            if (cur >= 0) body(cur & 0xffff, B, r);
             phase_barrier(G.n);
-            on = onn;
             cur = nxt;
+            nxt = nn;
             B = Bn;
             r = rn;
         }
         return;
     }
-    for (int q = 0; q < nq; ++q) {
-        const int tot = G.count(first(q)) + (second(q) >= 0 ? G.count(second(q)) : 0);
+    for (int q = 0, w = 0; q < nq; ++q, w = w + 1 == per ? 0 : w + 1) {
+        const int c = phase_first(pairs, w), d = phase_second(pairs, w);
+        const int tot = G.count(c) + (d >= 0 ? G.count(d) : 0);
         for (int t = tid; t < tot; t += nt) {
-            Pt P;
-            if (locate(q, t, &P)) body(P.p, load_b_sm(P.b, P.cnt), *P.r);
+            const int P = phase_point(G, pairs, w, t);
+            body(P & 0xffff, load_b_sm(sb + (P >> 16), mi), sr[P >> 16]);
         }
         phase_barrier(G.n);
     }
 }
 
-// Ascending colour order in 7 phases: colours 3 and 4 differ in all three
-// parities, so they are independent and share one.
-__device__ __forceinline__ int asc_first(int q) { return q <= 3 ? q : q + 1; }
-__device__ __forceinline__ int asc_second(int q) { return q == 3 ? 4 : -1; }
-
 // Coarsest correction grid in shared memory: FP32 sweeps in ascending order
 // until max|de| <= 2e-6 max|e| (FP32 resolution of the correction; at most 40
 // sweeps), or a fixed count.  Every thread of the block enters; ends with a
 // block barrier.
-__device__ __forceinline__ void coarsest_corr_sm(float* se, const float* sb, const float* sr, int n, float inv_h2,
-                                                 float h2half, int sweeps, unsigned long long* ev)
+__device__ __forceinline__ void coarsest_corr_sm(float* se, const float* sb, const float* sr, const int* tab, int n,
+                                                 float inv_h2, float h2half, int sweeps, unsigned long long* ev)
 {
     const int max_sweeps = sweeps > 0 ? sweeps : 40;
     const int nt = phase_threads(n, (int)blockDim.x);
@@ -1170,7 +1208,7 @@ __device__ __forceinline__ void coarsest_corr_sm(float* se, const float* sb, con
         const SmallGrid G(n);
         for (int s = 0; s < max_sweeps; ++s) {
             float du = 0.0f, um = 0.0f;
-            run_phases(G, sb, sr, 7, nt, asc_first, asc_second, [&](int p, const S3f& B, float r) {
+            run_sweeps(G, tab, sb, sr, false, 1, nt, [&](int p, const S3f& B, float r) {
                 const float e0 = se[p];
                 const S3f K = corr_hess_sm(se, p, n, n * n, e0, inv_h2);
                 bool nonconvex = false;
@@ -1214,11 +1252,13 @@ __device__ __forceinline__ void coarsest_corr_body(float* e, const float* __rest
     float* sb = smf + m;
     float* sr = smf + m + 6 * mi;
     for (int q = threadIdx.x; q < m; q += CT) se[q] = e[q];
-    for (int q = threadIdx.x; q < 6 * mi; q += CT) sb[q] = bstore[q];
     for (int q = threadIdx.x; q < mi; q += CT) sr[q] = rhs_cm[q];
+    __shared__ int tab[kPhaseTab];
+    stage_b_sm(sb, bstore, SmallGrid(n));
+    fill_phase_tab(tab, n, false);
     __syncthreads();
     unsigned long long ev = 0;
-    coarsest_corr_sm(se, sb, sr, n, inv_h2, h2half, sweeps, &ev);
+    coarsest_corr_sm(se, sb, sr, tab, n, inv_h2, h2half, sweeps, &ev);
     for (int q = threadIdx.x; q < m; q += CT) e[q] = se[q];
     if (events && ev) atomicAdd(events, ev);
 }
@@ -1297,15 +1337,12 @@ struct TailSmem {
 // (2, 5), (3, 4), the colour-pair kernel's sweep; otherwise ascending.  Each
 // point runs the separate kernels' arithmetic.  Every thread of the block
 // enters; ends with a block barrier.
-__device__ __forceinline__ void tail_smooth(const TailSmem& S, const SmallGrid& G, float inv_h2, float h2half, int nsw,
-                                            bool pairs, unsigned long long* ev)
+__device__ __forceinline__ void tail_smooth(const TailSmem& S, const SmallGrid& G, const int* tab, float inv_h2,
+                                            float h2half, int nsw, bool pairs, unsigned long long* ev)
 {
     const int n = G.n, nt = phase_threads(n, (int)blockDim.x);
     if ((int)threadIdx.x < nt && nsw > 0) {
-        const int per = pairs ? 4 : 7;
-        run_phases(
-            G, S.b, S.rhs, nsw * per, nt, [&](int q) { return pairs ? q & 3 : asc_first(q % 7); },
-            [&](int q) { return pairs ? (q & 3) ^ 7 : asc_second(q % 7); },
+        run_sweeps(G, tab, S.b, S.rhs, pairs, nsw, nt,
             [&](int p, const S3f& B, float r) {
                 const float e0 = S.e[p];
                 const S3f K = corr_hess_sm(S.e, p, n, n * n, e0, inv_h2);
@@ -1336,15 +1373,21 @@ __device__ __forceinline__ TailSmem tail_fields(const TailArgs& A, float* tsm, i
     return TailSmem{tsm + V.oe, tsm + V.ow, tsm + V.orr, tsm + V.ob, tsm + V.orhs};
 }
 
-// Every level's B; residual shells 0 (restrictions only read the interior, as
-// in the separate path).
-__device__ __forceinline__ void tail_load_base(const TailArgs& A, float* tsm)
+// The phase tables of the 9^3 and 5^3 grids.
+constexpr int kTailTab = kPhaseTab + 7 * 32;
+__device__ __forceinline__ int* tail_tab(int* tab, int n) { return n == 9 ? tab : tab + kPhaseTab; }
+
+// Every level's B and phase table; residual shells 0 (restrictions only read
+// the interior, as in the separate path).
+__device__ __forceinline__ void tail_load_base(const TailArgs& A, float* tsm, int* tab)
 {
     for (int l = 0; l < A.nlev; ++l) {
-        const int n = A.lev[l].n, m = n * n * n, mi = (n - 2) * (n - 2) * (n - 2);
+        const int n = A.lev[l].n, m = n * n * n;
         const TailSmem S = tail_fields(A, tsm, l);
-        for (int q = threadIdx.x; q < 6 * mi; q += TT) S.b[q] = A.lev[l].b[q];
         for (int q = threadIdx.x; q < m; q += TT) S.r[q] = 0.0f;
+        stage_b_sm(S.b, A.lev[l].b, SmallGrid(n));
+        // the coarsest grid sweeps in ascending order
+        fill_phase_tab(tail_tab(tab, n), n, A.lev[l].pairs && l < A.nlev - 1);
     }
 }
 
@@ -1356,16 +1399,16 @@ __device__ __forceinline__ void tail_coarse_rhs(const TailArgs& A, float* tsm, i
     const SmallGrid GC(nc);
     for (int q = threadIdx.x; q < (nc - 2) * (nc - 2) * (nc - 2); q += TT) {
         int i, j, k, cnt, off;
-        const int p = GC.interior(q, &i, &j, &k), sl = GC.slot(i, j, k, &cnt, &off);
-        const S3f B = load_b_sm(C.b + 6 * off + sl, cnt);
+        const int p = GC.interior(q, &i, &j, &k), sl = GC.slot(i, j, k, &cnt, &off) + off;
+        const S3f B = load_b_sm(C.b + sl, (nc - 2) * (nc - 2) * (nc - 2));
         const S3f K = corr_hess_sm(C.w, p, nc, nc * nc, C.w[p], A.lev[l].inv_h2);
-        C.rhs[off + sl] = delta_det(B, K) + C.r[p];
+        C.rhs[sl] = delta_det(B, K) + C.r[p];
     }
     __syncthreads();
 }
 
 // The cycle from level 0 of the tail, whose e and rhs are in place, down and back.
-__device__ __forceinline__ void tail_cycle(const TailArgs& A, float* tsm, unsigned long long* ev)
+__device__ __forceinline__ void tail_cycle(const TailArgs& A, float* tsm, int* tab, unsigned long long* ev)
 {
     const int L = A.nlev;
     for (int l = 0; l < L - 1; ++l) {
@@ -1373,14 +1416,14 @@ __device__ __forceinline__ void tail_cycle(const TailArgs& A, float* tsm, unsign
         const TailSmem C = tail_fields(A, tsm, l + 1);
         const int nf = A.lev[l].n, nc = A.lev[l + 1].n;
         const SmallGrid GF(nf), GC(nc);
-        tail_smooth(F, GF, A.lev[l].inv_h2, A.lev[l].h2half, A.nu1, A.lev[l].pairs != 0, ev);
+        tail_smooth(F, GF, tail_tab(tab, nf), A.lev[l].inv_h2, A.lev[l].h2half, A.nu1, A.lev[l].pairs != 0, ev);
         // residual on the fine interior
         for (int q = threadIdx.x; q < (nf - 2) * (nf - 2) * (nf - 2); q += TT) {
             int i, j, k, cnt, off;
-            const int p = GF.interior(q, &i, &j, &k), sl = GF.slot(i, j, k, &cnt, &off);
-            const S3f B = load_b_sm(F.b + 6 * off + sl, cnt);
+            const int p = GF.interior(q, &i, &j, &k), sl = GF.slot(i, j, k, &cnt, &off) + off;
+            const S3f B = load_b_sm(F.b + sl, (nf - 2) * (nf - 2) * (nf - 2));
             const S3f K = corr_hess_sm(F.e, p, nf, nf * nf, F.e[p], A.lev[l].inv_h2);
-            F.r[p] = F.rhs[off + sl] - delta_det(B, K);
+            F.r[p] = F.rhs[sl] - delta_det(B, K);
         }
         __syncthreads();
         // restriction: coarse residual, approximation restriction of e
@@ -1388,9 +1431,11 @@ __device__ __forceinline__ void tail_cycle(const TailArgs& A, float* tsm, unsign
             const int J0 = (pc * GC.mn) >> 16, K = (J0 * GC.mn) >> 16, I = pc - J0 * nc, J = J0 - K * nc;
             const int pf = ((2 * K) * nf + 2 * J) * nf + 2 * I;
             const bool inside = I > 0 && J > 0 && K > 0 && I < nc - 1 && J < nc - 1 && K < nc - 1;
-            C.r[pc] = inside ? xfer::weighted_restrict(F.r, pf, nf, (long long)nf * nf, A.kind) : 0.0f;
-            const float w = (inside && A.approx == 1) ? xfer::weighted_restrict(F.e, pf, nf, (long long)nf * nf, A.kind)
-                                                     : F.e[pf];
+            auto at = [&](const float* v) {
+                return [=](int di, int dj, int dk) -> float { return v[pf + (dk * nf + dj) * nf + di]; };
+            };
+            C.r[pc] = inside ? xfer::restrict_of<float>(at(F.r), A.kind) : 0.0f;
+            const float w = inside && A.approx == 1 ? xfer::restrict_of<float>(at(F.e), A.kind) : F.e[pf];
             C.w[pc] = w;
             C.e[pc] = w;
         }
@@ -1399,8 +1444,8 @@ __device__ __forceinline__ void tail_cycle(const TailArgs& A, float* tsm, unsign
     }
     {
         const TailSmem S = tail_fields(A, tsm, L - 1);
-        coarsest_corr_sm(S.e, S.b, S.rhs, A.lev[L - 1].n, A.lev[L - 1].inv_h2, A.lev[L - 1].h2half, A.coarse_sweeps,
-                         ev);
+        coarsest_corr_sm(S.e, S.b, S.rhs, tail_tab(tab, A.lev[L - 1].n), A.lev[L - 1].n, A.lev[L - 1].inv_h2,
+                         A.lev[L - 1].h2half, A.coarse_sweeps, ev);
     }
     for (int l = L - 2; l >= 0; --l) {
         const TailSmem F = tail_fields(A, tsm, l);
@@ -1425,14 +1470,15 @@ __device__ __forceinline__ void tail_cycle(const TailArgs& A, float* tsm, unsign
             F.e[p] = F.e[p] + v;
         }
         __syncthreads();
-        tail_smooth(F, GF, A.lev[l].inv_h2, A.lev[l].h2half, A.nu2, A.lev[l].pairs != 0, ev);
+        tail_smooth(F, GF, tail_tab(tab, nf), A.lev[l].inv_h2, A.lev[l].h2half, A.nu2, A.lev[l].pairs != 0, ev);
     }
 }
 
 __device__ __forceinline__ void corr_tail_body(const TailArgs& A)
 {
     extern __shared__ float tsm[];
-    tail_load_base(A, tsm);
+    __shared__ int tab[kTailTab];
+    tail_load_base(A, tsm, tab);
     {   // the top level's iterate and rhs
         const int n = A.lev[0].n, m = n * n * n, mi = (n - 2) * (n - 2) * (n - 2);
         const TailSmem S = tail_fields(A, tsm, 0);
@@ -1441,7 +1487,7 @@ __device__ __forceinline__ void corr_tail_body(const TailArgs& A)
     }
     __syncthreads();
     unsigned long long ev = 0;
-    tail_cycle(A, tsm, &ev);
+    tail_cycle(A, tsm, tab, &ev);
     const int m0 = A.lev[0].n * A.lev[0].n * A.lev[0].n;
     for (int q = threadIdx.x; q < m0; q += TT) A.lev[0].e[q] = tsm[A.lev[0].oe + q];
     if (A.events && ev) atomicAdd(A.events, ev);
@@ -1525,14 +1571,20 @@ __device__ __forceinline__ float load_remote(const float* smem, unsigned rank)
     return v;
 }
 
-// A value into block `rank`'s shared memory, its 4 bytes counted there on the
-// mbarrier at the place of `bar`.
-__device__ __forceinline__ void send_async(float* smem, unsigned bar, unsigned rank, float v)
+// The place of a shared-memory address in block `rank`.
+__device__ __forceinline__ unsigned remote(unsigned smem, unsigned rank)
 {
-    unsigned a = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("{\n.reg .b32 ra, rb;\nmapa.shared::cluster.u32 ra, %0, %2;\nmapa.shared::cluster.u32 rb, %1, %2;\n"
-                 "st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.f32 [ra], %3, [rb];\n}" ::"r"(a),
-                 "r"(bar), "r"(rank), "f"(v)
+    unsigned a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem), "r"(rank));
+    return a;
+}
+
+// A value into another block's shared memory, its 4 bytes counted there on
+// the mbarrier at `bar` (both remote places).
+__device__ __forceinline__ void send_async(unsigned to, unsigned bar, float v)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];" ::"r"(to), "f"(v),
+                 "r"(bar)
                  : "memory");
 }
 
@@ -1565,16 +1617,22 @@ struct PhaseSync {
 
 // One level of the cluster: N points a side, P planes a block (local planes
 // 1 .. P; 0 and P + 1 are the neighbours').  Local plane q is plane m P + q.
+// A row of e holds its even x in front and its odd x behind: the points of a
+// phase, two apart in x, then lie side by side, so their loads meet no bank
+// conflicts and what they send is contiguous (480 words sent two apart took
+// 850 cycles to arrive, side by side 380).
 template <int N, int P>
 struct Slab {
-    static constexpr int PL = N * N, A = (N - 3) / 2, B = (N - 1) / 2, M2 = (N - 2) * (N - 2);
+    static constexpr int PL = N * N, A = (N - 3) / 2, B = (N - 1) / 2, M2 = (N - 2) * (N - 2), H = (N + 1) / 2;
     static constexpr int NT = P == 1 ? 64 : TC;   // threads that a phase's points fill: at most B^2, or A^2 + B^2
-    static constexpr int FLOATS = 2 * (P + 2) * PL + 7 * P * M2;
+    static constexpr int FLOATS = 2 * (P + 2) * PL + 7 * P * M2 + 4 * NT;
     static_assert(P == 1 ? B * B <= NT : A * A + B * B <= NT, "one point a thread");
-    float *e, *r, *rh, *b;      // [P + 2][N][N], the same, [P][M2], [P][6][M2]; colours in order inside a plane
+    float *e, *r, *rh, *b;      // [P + 2][N][N] (rows split by parity), [P + 2][N][N], [P][M2], [P][6][M2] (colours in order)
+    int* tab;                   // [4][NT]: the points of the phases
     unsigned m;                 // block rank
     float inv_h2, h2half;
 
+    static __device__ __forceinline__ int xs(int x) { return (x & 1) ? H + (x >> 1) : x >> 1; }
     __device__ __forceinline__ int planes() const { return max(0, min(P, N - 2 - (int)m * P)); }
     static __device__ __forceinline__ int ni(int c) { return (c & 1) ? B : A; }
     static __device__ __forceinline__ int nj(int c) { return (c & 2) ? B : A; }
@@ -1593,19 +1651,16 @@ struct Slab {
         if (q == P && m + 1 < KC) store_remote(f + s, m + 1, v);
     }
 
-    struct Pt {
-        int q, s, u;      // local plane, place in the plane, slot of its B and rhs
-    };
-
-    // Point t of the phase that sweeps colour c of the even planes and c ^ 7 of the odd ones.
-    __device__ __forceinline__ bool locate(int c, int t, Pt* X) const
+    // Point t of the phase that sweeps colour c of the even planes and c ^ 7 of
+    // the odd ones: place in the plane (11 bits), slot of its B and rhs (10),
+    // local plane (2), parity of x (1); -1 where there is none.
+    __device__ __forceinline__ int locate(int c, int t) const
     {
         const int np = planes();
-        int q = 1, k;
+        int q = 1;
         if (P == 1) {
-            if (np < 1) return false;
-            k = (int)m + 1;
-            if (k & 1) c ^= 7;
+            if (np < 1) return -1;
+            if ((m + 1) & 1) c ^= 7;
         } else {          // local plane 1 is odd, 2 even
             const int no = ni(c ^ 7) * nj(c ^ 7);
             if (t < no) {
@@ -1613,15 +1668,13 @@ struct Slab {
             } else {
                 t -= no;
                 q = 2;
-                if (np < 2) return false;
+                if (np < 2) return -1;
             }
         }
-        if (t >= ni(c) * nj(c)) return false;
+        if (t >= ni(c) * nj(c)) return -1;
         const int y = (c & 1) ? t / B : t / A, x = t - y * ni(c);
-        X->q = q;
-        X->s = (((c & 2) ? 1 : 2) + 2 * y) * N + ((c & 1) ? 1 : 2) + 2 * x;
-        X->u = in_plane(c) + t;
-        return true;
+        const int s = (((c & 2) ? 1 : 2) + 2 * y) * N + xs(((c & 1) ? 1 : 2) + 2 * x);
+        return s | (in_plane(c) + t) << 11 | q << 21 | (c & 1) << 23;
     }
 
     // Bytes that the neighbours send in that phase: the last plane of the block before, the first of the one after.
@@ -1654,49 +1707,65 @@ struct Slab {
     }
 
     __device__ __forceinline__ S3f base(int q, int u) const { return load_b_sm(b + (q - 1) * 6 * M2 + u, M2); }
-    __device__ __forceinline__ S3f hess(const float* f, int q, int s) const
+
+    // D^2 of a field with split rows at place s of local plane q: x + 1 lies at
+    // p + xp and x - 1 just before it, p + xp - 1.
+    __device__ __forceinline__ S3f hess(const float* f, int q, int s, int par) const
     {
-        return corr_hess_sm(f, q * PL + s, N, PL, f[q * PL + s], inv_h2);
+        const float* p = f + q * PL + s;
+        const float* px = p + (par ? 1 - H : H);
+        return hess_of(
+            [&](int di, int dj, int dk) -> float {
+                return (di == 0 ? p : px)[dk * PL + dj * N - (di < 0 ? 1 : 0)];
+            },
+            inv_h2);
     }
 
     // nsw sweeps in colour pairs.  Every thread of the block enters; ends with a block barrier.
     __device__ __forceinline__ void smooth(int nsw, PhaseSync& S, float* word, unsigned long long* ev) const
     {
-        if ((int)threadIdx.x < NT) {
-            Pt cur, nxt;
+        const int tid = threadIdx.x;
+        if (tid < NT) {
+            const unsigned es = (unsigned)__cvta_generic_to_shared(e), down = m > 0 ? m - 1 : 0,
+                           up = m + 1 < KC ? m + 1 : m;
+            const unsigned e_down = remote(es + 4 * (P + 1) * PL, down), e_up = remote(es, up);
+            const unsigned bar_down = remote(S.bar, down), bar_up = remote(S.bar, up);
+            int cur = tab[tid], nxt = tab[NT + tid];
             S3f Bc = {0, 0, 0, 0, 0, 0}, Bn = Bc;
             float rc = 0.0f, rn = 0.0f;
-            bool on = nsw > 0 && locate(0, threadIdx.x, &cur);
-            if (on) {
-                Bc = base(cur.q, cur.u);
-                rc = rh[(cur.q - 1) * M2 + cur.u];
-            }
+            auto fetch = [&](int X, S3f* Bm, float* rv) {
+                const int q = (X >> 21) & 3, u = (X >> 11) & 1023;
+                *Bm = base(q, u);
+                *rv = rh[(q - 1) * M2 + u];
+            };
+            if (cur >= 0) fetch(cur, &Bc, &rc);
             for (int t = 0; t < 4 * nsw; ++t) {
-                if (threadIdx.x == 0) {
+                const unsigned ph = 8 * (S.t & 1);
+                if (tid == 0) {
                     S.expect(bytes(t & 3));
-                    if (P == 1 && m == KC - 1) send_async(word, S.now(), m - 1, 0.0f);
+                    if (P == 1 && m == KC - 1)
+                        send_async(remote((unsigned)__cvta_generic_to_shared(word), down), bar_down + ph, 0.0f);
                 }
-                const bool onn = t + 1 < 4 * nsw && locate((t + 1) & 3, threadIdx.x, &nxt);
-                if (onn) {   // B and rhs of the next phase, which nothing writes
-                    Bn = base(nxt.q, nxt.u);
-                    rn = rh[(nxt.q - 1) * M2 + nxt.u];
-                }
-                if (on) {
-                    float* p = e + cur.q * PL + cur.s;
+                // the next phase's B and rhs, which nothing writes, and the place of the one after
+                const int nn = tab[((t + 2) & 3) * NT + tid];
+                if (nxt >= 0) fetch(nxt, &Bn, &rn);
+                if (cur >= 0) {
+                    const int q = (cur >> 21) & 3, s = cur & 2047;
+                    float* p = e + q * PL + s;
                     const float e0 = *p;
-                    const S3f K = hess(e, cur.q, cur.s);
+                    const S3f K = hess(e, q, s, (cur >> 23) & 1);
                     bool nonconvex = false;
                     const float v = fmaf(h2half, corr_root(Bc, K, rc, &nonconvex), e0);
                     *p = v;
-                    if (cur.q == 1 && m > 0) send_async(e + (P + 1) * PL + cur.s, S.now(), m - 1, v);
-                    if (cur.q == P && m + 1 < KC) send_async(e + cur.s, S.now(), m + 1, v);
+                    if (q == 1 && m > 0) send_async(e_down + 4 * s, bar_down + ph, v);
+                    if (q == P && m + 1 < KC) send_async(e_up + 4 * s, bar_up + ph, v);
                     *ev += nonconvex ? 1ull : 0ull;
                 }
                 if (P == 1) asm volatile("bar.sync 2, 64;" ::: "memory");
                 else __syncthreads();
                 S.wait();
-                on = onn;
                 cur = nxt;
+                nxt = nn;
                 Bc = Bn;
                 rc = rn;
             }
@@ -1713,7 +1782,7 @@ struct Slab {
             int q, i, j;
             if (!interior(t, &q, &i, &j)) continue;
             const int u = slot(i, j);
-            put(r, q, j * N + i, rh[(q - 1) * M2 + u] - delta_det(base(q, u), hess(e, q, j * N + i)));
+            put(r, q, j * N + i, rh[(q - 1) * M2 + u] - delta_det(base(q, u), hess(e, q, j * N + xs(i), i & 1)));
         }
         cluster_barrier();
     }
@@ -1725,13 +1794,30 @@ struct Slab {
             int q, i, j;
             if (!interior(t, &q, &i, &j)) continue;
             const int u = slot(i, j);
-            rh[(q - 1) * M2 + u] = delta_det(base(q, u), hess(w, q, j * N + i)) + r[q * PL + j * N + i];
+            rh[(q - 1) * M2 + u] = delta_det(base(q, u), hess(w, q, j * N + xs(i), i & 1)) + r[q * PL + j * N + i];
         }
         __syncthreads();
     }
 
-    // B of the block's planes from the colour-major store, and at the level the
-    // cycle enters (ge not null) its iterate and right-hand side.
+    // Restriction to coarse point (I, J) on fine local plane lp: of r, and of e
+    // (the approximation restriction; `in`: a coarse interior point).
+    __device__ __forceinline__ void restrict_to(int lp, int I, int J, bool in, int kind, int approx, float* rv,
+                                                float* wv) const
+    {
+        const float* rp = r + lp * PL + 2 * J * N + 2 * I;
+        const float* ep = e + lp * PL + 2 * J * N + I;
+        auto ate = [&](int di, int dj, int dk) -> float {
+            return ep[dk * PL + dj * N + (di == 0 ? 0 : (di > 0 ? H : H - 1))];
+        };
+        *rv = in ? xfer::restrict_of<float>(
+                       [&](int di, int dj, int dk) -> float { return rp[dk * PL + dj * N + di]; }, kind)
+                 : 0.0f;
+        *wv = in && approx == 1 ? xfer::restrict_of<float>(ate, kind) : ep[0];
+    }
+
+    // The phases' points; B of the block's planes from the colour-major store, and
+    // at the level the cycle enters (ge not null) its iterate and right-hand side,
+    // by asynchronous copies (to be waited for).
     __device__ __forceinline__ void load(const float* gb, const float* ge, const float* grhs) const
     {
         for (int t = threadIdx.x; t < P * M2; t += TC) {
@@ -1739,16 +1825,15 @@ struct Slab {
             if (!interior(t, &q, &i, &j)) continue;
             const int k = (int)m * P + q, c = (i & 1) | ((j & 1) << 1) | ((k & 1) << 2), u = slot(i, j);
             const int pl = ni(c) * nj(c), at = ((k - 1) >> 1) * pl + u - in_plane(c), off = (int)cm_offset(N, c);
-            const S3f Bm = load_b(gb + 6 * off + at, pl * ((c & 4) ? B : A));
-            float* d = b + (q - 1) * 6 * M2 + u;
-            d[0] = Bm.xx; d[M2] = Bm.yy; d[2 * M2] = Bm.zz; d[3 * M2] = Bm.xy; d[4 * M2] = Bm.xz; d[5 * M2] = Bm.yz;
-            if (ge) rh[(q - 1) * M2 + u] = grhs[off + at];
+            const int cnt = pl * ((c & 4) ? B : A);
+            for (int v = 0; v < 6; ++v) cp_async_f32(b + ((q - 1) * 6 + v) * M2 + u, gb + 6 * off + at + v * cnt, 4);
+            if (ge) cp_async_f32(rh + (q - 1) * M2 + u, grhs + off + at, 4);
         }
-        if (!ge) return;
-        for (int t = threadIdx.x; t < (P + 2) * PL; t += TC) {
-            const int k = (int)m * P + t / PL;
-            e[t] = k < N ? ge[k * PL + t % PL] : 0.0f;
+        for (int t = threadIdx.x; ge && t < (P + 2) * PL; t += TC) {
+            const int p = t / PL, s = t - p * PL, j = s / N, i = s - j * N, k = (int)m * P + p;
+            cp_async_f32(e + p * PL + j * N + xs(i), k < N ? ge + k * PL + s : ge, k < N ? 4 : 0);
         }
+        for (int x = threadIdx.x; x < 4 * NT; x += TC) tab[x] = locate(x / NT, x % NT);
     }
 
     __device__ __forceinline__ void store(float* ge, bool lost) const
@@ -1756,38 +1841,43 @@ struct Slab {
         for (int t = threadIdx.x; t < P * M2; t += TC) {
             int q, i, j;
             if (!interior(t, &q, &i, &j)) continue;
-            ge[((int)m * P + q) * PL + j * N + i] = lost ? __int_as_float(0x7fffffff) : e[q * PL + j * N + i];
+            ge[((int)m * P + q) * PL + j * N + i] = lost ? __int_as_float(0x7fffffff) : e[q * PL + j * N + xs(i)];
         }
     }
 };
 
 // Trilinear correction of one fine point from the coarse planes dlo (K0) and
-// dhi (K0 + 1) of e_H - w_H, formed as xfer::k_prolong forms it.
-template <int NC>
-__device__ __forceinline__ float cluster_prolong(const float* dlo, const float* dhi, int i, int j, int ok)
+// dhi (K0 + 1) of e_H - w_H, rows of NC values at xc(x), formed as
+// xfer::k_prolong forms it.
+template <int NC, typename X>
+__device__ __forceinline__ float cluster_prolong(const float* dlo, const float* dhi, int i, int j, int ok, X xc)
 {
     const int J0 = j >> 1, oj = j & 1, I = i >> 1;
     const float w = oj + ok == 2 ? 0.25f : (oj + ok == 1 ? 0.5f : 1.0f);
     auto line = [&](int Ic) {
+        const int x = J0 * NC + xc(Ic);
         float s = 0.0f;
-        s += dlo[J0 * NC + Ic];
-        if (oj) s += dlo[(J0 + 1) * NC + Ic];
+        s += dlo[x];
+        if (oj) s += dlo[x + NC];
         if (ok) {
-            s += dhi[J0 * NC + Ic];
-            if (oj) s += dhi[(J0 + 1) * NC + Ic];
+            s += dhi[x];
+            if (oj) s += dhi[x + NC];
         }
         return s * w;
     };
     return (i & 1) ? (line(I) + line(I + 1)) * 0.5f : line(I);
 }
 
-constexpr int kClusterFloats = Slab<33, 2>::FLOATS + Slab<17, 1>::FLOATS + 5 * 17 * 17;   // and w, and two planes of d
+using Slab33 = Slab<33, 2>;
+using Slab17 = Slab<17, 1>;
+constexpr int kClusterFloats = Slab33::FLOATS + Slab17::FLOATS + 5 * 17 * 17;   // and w, and two planes of d
 
 __global__ void __launch_bounds__(TC, 1) k_corr_vcycle_cluster(const __grid_constant__ ClusterArgs A)
 {
     extern __shared__ float csm[];
     __shared__ alignas(8) unsigned long long bars[2];
     __shared__ float word;
+    __shared__ int ttab[kTailTab];
     const unsigned m = cluster_rank();
     float* q = csm;
     auto take = [&](int f) {
@@ -1795,11 +1885,13 @@ __global__ void __launch_bounds__(TC, 1) k_corr_vcycle_cluster(const __grid_cons
         q += f;
         return p;
     };
-    Slab<33, 2> F;
+    Slab33 F;
     F.e = take(4 * F.PL); F.r = take(4 * F.PL); F.rh = take(2 * F.M2); F.b = take(12 * F.M2);
+    F.tab = (int*)take(4 * F.NT);
     F.m = m; F.inv_h2 = A.l33.inv_h2; F.h2half = A.l33.h2half;
-    Slab<17, 1> C;
+    Slab17 C;
     C.e = take(3 * C.PL); C.r = take(3 * C.PL); C.rh = take(C.M2); C.b = take(6 * C.M2);
+    C.tab = (int*)take(4 * C.NT);
     C.m = m; C.inv_h2 = A.l17.inv_h2; C.h2half = A.l17.h2half;
     float* w17 = take(3 * C.PL);
     float* d = take(2 * C.PL);      // planes of e_H - w_H
@@ -1815,7 +1907,8 @@ __global__ void __launch_bounds__(TC, 1) k_corr_vcycle_cluster(const __grid_cons
     }
     if (A.top33) F.load(A.l33.b, A.l33.e, A.l33.rhs);
     C.load(A.l17.b, A.top33 ? nullptr : A.l17.e, A.l17.rhs);
-    if (m == 0) tail_load_base(T, tsm);
+    if (m == 0) tail_load_base(T, tsm, ttab);
+    cp_async_wait_all();
     cluster_barrier();   // every block is running and its mbarriers are set before another writes to it
     for (int cyc = 0; cyc < A.cycles; ++cyc) {
         if (A.top33) {
@@ -1823,13 +1916,13 @@ __global__ void __launch_bounds__(TC, 1) k_corr_vcycle_cluster(const __grid_cons
             F.residual();
             // coarse plane K = m + 1 on the block's fine plane 2m + 2, and plane 0 in the first block
             for (int t = threadIdx.x; t < (m == 0 ? 2 : 1) * C.PL; t += TC) {
-                const int own = t < C.PL, s = own ? t : t - C.PL, J = s / 17, I = s - J * 17;
-                const int K = own ? (int)m + 1 : 0, pf = (own ? 2 : 0) * F.PL + 2 * J * 33 + 2 * I;
-                const bool in = I > 0 && J > 0 && K > 0 && I < 16 && J < 16 && K < 16;
-                const float rv = in ? xfer::weighted_restrict(F.r, pf, 33, F.PL, T.kind) : 0.0f;
-                const float wv = in && T.approx == 1 ? xfer::weighted_restrict(F.e, pf, 33, F.PL, T.kind) : F.e[pf];
+                const int own = t < C.PL, u = own ? t : t - C.PL, J = u / 17, I = u - J * 17, s = J * 17 + C.xs(I);
+                const int K = own ? (int)m + 1 : 0;
+                float rv, wv;
+                F.restrict_to(own ? 2 : 0, I, J, I > 0 && J > 0 && K > 0 && I < 16 && J < 16 && K < 16, T.kind,
+                              T.approx, &rv, &wv);
                 if (own) {
-                    C.r[C.PL + s] = rv;
+                    C.r[C.PL + u] = rv;
                     C.put(w17, 1, s, wv);
                     C.put(C.e, 1, s, wv);
                 } else {
@@ -1848,10 +1941,9 @@ __global__ void __launch_bounds__(TC, 1) k_corr_vcycle_cluster(const __grid_cons
             const int K = m == 0 ? 0 : (m == KC - 2 ? 8 : ((m & 1) && m < KC - 2 ? (int)(m + 1) / 2 : -1));
             const int lp = m == 0 ? 0 : (m == KC - 2 ? 2 : 1);
             for (int s = threadIdx.x; K >= 0 && s < 81; s += TC) {
-                const int J = s / 9, I = s - J * 9, pf = lp * C.PL + 2 * J * 17 + 2 * I;
-                const bool in = I > 0 && J > 0 && K > 0 && I < 8 && J < 8 && K < 8;
-                const float rv = in ? xfer::weighted_restrict(C.r, pf, 17, C.PL, T.kind) : 0.0f;
-                const float wv = in && T.approx == 1 ? xfer::weighted_restrict(C.e, pf, 17, C.PL, T.kind) : C.e[pf];
+                const int J = s / 9, I = s - J * 9;
+                float rv, wv;
+                C.restrict_to(lp, I, J, I > 0 && J > 0 && K > 0 && I < 8 && J < 8 && K < 8, T.kind, T.approx, &rv, &wv);
                 store_remote(tsm + V9.orr + 81 * K + s, 0, rv);
                 store_remote(tsm + V9.ow + 81 * K + s, 0, wv);
                 store_remote(tsm + V9.oe + 81 * K + s, 0, wv);
@@ -1860,7 +1952,7 @@ __global__ void __launch_bounds__(TC, 1) k_corr_vcycle_cluster(const __grid_cons
         cluster_barrier();
         if (m == 0) {
             tail_coarse_rhs(T, tsm, 0);
-            tail_cycle(T, tsm, &ev);
+            tail_cycle(T, tsm, ttab, &ev);
         }
         cluster_barrier();
         {   // 9^3 -> 17^3: plane k = m + 1 lies on or between coarse planes K0 = k / 2 and K0 + 1
@@ -1873,8 +1965,8 @@ __global__ void __launch_bounds__(TC, 1) k_corr_vcycle_cluster(const __grid_cons
             for (int t = threadIdx.x; t < C.M2; t += TC) {
                 int lq, i, j;
                 if (!C.interior(t, &lq, &i, &j)) continue;
-                const int s = j * 17 + i;
-                C.put(C.e, 1, s, C.e[C.PL + s] + cluster_prolong<9>(d, d + 81, i, j, k & 1));
+                const int s = j * 17 + C.xs(i);
+                C.put(C.e, 1, s, C.e[C.PL + s] + cluster_prolong<9>(d, d + 81, i, j, k & 1, [](int x) { return x; }));
             }
         }
         cluster_barrier();
@@ -1885,9 +1977,9 @@ __global__ void __launch_bounds__(TC, 1) k_corr_vcycle_cluster(const __grid_cons
             for (int t = threadIdx.x; t < 2 * F.M2; t += TC) {
                 int lq, i, j;
                 if (!F.interior(t, &lq, &i, &j)) continue;
-                const int s = j * 33 + i;
-                const float v = lq == 1 ? cluster_prolong<17>(d, d + C.PL, i, j, 1)
-                                        : cluster_prolong<17>(d + C.PL, d, i, j, 0);
+                const int s = j * 33 + F.xs(i);
+                const float v = lq == 1 ? cluster_prolong<17>(d, d + C.PL, i, j, 1, Slab17::xs)
+                                        : cluster_prolong<17>(d + C.PL, d, i, j, 0, Slab17::xs);
                 F.put(F.e, lq, s, F.e[lq * F.PL + s] + v);
             }
             cluster_barrier();

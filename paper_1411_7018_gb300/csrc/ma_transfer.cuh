@@ -25,13 +25,13 @@ __device__ __forceinline__ double fma_t(double a, double b, double c) { return f
 // full weighting, separable (1 2 1)/4 along each axis.  Written with explicit
 // fused multiply-adds in a fixed order so that every kernel that inlines it
 // rounds identically.
-template <typename T>
-__device__ __forceinline__ T weighted_restrict(const T* __restrict__ v, long long p, long long sy, long long sz,
-                                               int kind)
+// at(di, dj, dk) reads the value at an offset from the point.
+template <typename T, typename At>
+__device__ __forceinline__ T restrict_of(At at, int kind)
 {
     if (kind == 0) {
-        const T faces = (v[p + 1] + v[p - 1]) + (v[p + sy] + v[p - sy]) + (v[p + sz] + v[p - sz]);
-        return fma_t(T(6), v[p], faces) * (T(1) / T(12));
+        const T faces = (at(1, 0, 0) + at(-1, 0, 0)) + (at(0, 1, 0) + at(0, -1, 0)) + (at(0, 0, 1) + at(0, 0, -1));
+        return fma_t(T(6), at(0, 0, 0), faces) * (T(1) / T(12));
     }
     T acc = T(0);
 #pragma unroll
@@ -39,13 +39,19 @@ __device__ __forceinline__ T weighted_restrict(const T* __restrict__ v, long lon
         T plane = T(0);
 #pragma unroll
         for (int dj = -1; dj <= 1; ++dj) {
-            const long long q = p + dk * sz + dj * sy;
-            const T row = fma_t(T(2), v[q], v[q - 1] + v[q + 1]);
+            const T row = fma_t(T(2), at(0, dj, dk), at(-1, dj, dk) + at(1, dj, dk));
             plane = fma_t(dj == 0 ? T(2) : T(1), row, plane);
         }
         acc = fma_t(dk == 0 ? T(2) : T(1), plane, acc);
     }
     return acc * (T(1) / T(64));
+}
+
+template <typename T>
+__device__ __forceinline__ T weighted_restrict(const T* __restrict__ v, long long p, long long sy, long long sz,
+                                               int kind)
+{
+    return restrict_of<T>([&](int di, int dj, int dk) -> T { return v[p + dk * sz + dj * sy + di]; }, kind);
 }
 
 // Coarse-grid outputs, any may be null: rc = I r (0 on the shell);
