@@ -1052,7 +1052,6 @@ ma_status batch_describe(ma_hierarchy* const* hs, int count, std::vector<ma::Bat
     p->coarse_sweeps = d0.coarse_sweeps;
     p->inner = d0.inner_cycles > 0 ? d0.inner_cycles : 3;
     p->tail_max = ma::corr_tail_max_n();
-    p->vtail_max = ma::vcycle_tail_max_n();
     p->fmg_interp = d0.fmg_interp;
     return MA_OK;
 }

@@ -172,7 +172,6 @@ struct BatchInstance {
 struct BatchParams {
     int nu1, nu2, kind, approx, coarse_sweeps, inner;
     int tail_max;          // largest level of the fused correction tail
-    int vtail_max;         // largest level of the fused FP64 tail (the FMG V-cycles)
     int fmg_interp;        // MA_FMG_TRILINEAR | MA_FMG_CUBIC
 };
 struct BatchPlan;
@@ -181,15 +180,14 @@ struct BLaunch;
 struct TableBuilder;
 }  // namespace batched
 // The FP64 part of the batched start (ma_kernels_f64.cu): the partials of
-// the norms of f, and the FMG pass of Algorithm 2 with its FP64 V-cycles
-// below the finest level, all hierarchies sharing the coarsest grid size so
-// that every FMG step runs on one level size; and the launcher of its ops.
+// the norms of f, and the FMG pass of Algorithm 2, all hierarchies sharing the
+// coarsest grid size so that every FMG step runs on one level size; and the
+// launcher of its ops.
 void emit_rhs_partials_f64(batched::TableBuilder& T, const BatchInstance* in, int count);
-// level_step, when given, replaces the FP64 V-cycle of each FMG level below
-// the finest: it receives (instance index, level) for the instances that
-// have that level.
+// level_step runs the cycle of each FMG level below the finest: it receives
+// (instance index, level) for the instances that have that level.
 void emit_fmg_f64(batched::TableBuilder& T, const BatchInstance* in, int count, const BatchParams& p,
-                  const std::function<void(const std::vector<std::pair<int, int>>&)>& level_step = nullptr);
+                  const std::function<void(const std::vector<std::pair<int, int>>&)>& level_step);
 cudaError_t batch_launch_f64(const char* tables, const batched::BLaunch& L, const int* active, cudaStream_t s);
 // Bytes of the device job tables of a batch.
 size_t batch_tables_bytes(const BatchInstance* in, int count, const BatchParams& p);

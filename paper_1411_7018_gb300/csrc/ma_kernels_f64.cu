@@ -23,13 +23,23 @@
 #include "ma_point.cuh"
 #include "ma_transfer.cuh"
 #include "ma_residual.cuh"
+#include "ma_small_grid.cuh"
 #include "ma_smooth_f2.cuh"
 
 namespace ma {
 
 namespace {
 
+using namespace small;
+
 constexpr int BX = 32, BY = 4;
+
+// Grids of kF2MinN points a side and more take the two-float forms of the
+// point update, the residual and the coarse right-hand side; the one unknown of
+// a 3^3 grid, which FP64 solves to a few ulps of the root, does not.
+constexpr int kF2MinN = 5;
+// ... with det3's sums unnormalised from here up, where its error stays below an ulp of u
+constexpr int kUnormMinN = 33;
 
 __device__ __forceinline__ long long lin(int i, int j, int k, int n)
 {
@@ -84,16 +94,13 @@ cudaError_t launch_colour(double* u, const double* rhs, int n, double h6, unsign
 }
 
 // ---------------------------------------------------------------------------
-// The same sweep with the point update of ma_smooth_f2.cuh, on grids of
-// kF2MinN points a side and more.  Below, the colours of a level fill few
-// warps and the fused tail (which shares those sizes) runs the FP64 form.
-// Colours 3 and 4 follow each other in the order and differ in all three
+// The same sweep with the point update of ma_smooth_f2.cuh.  Colours 3 and 4 follow each other in the order and differ in all three
 // parities, a corner offset the stencil lacks, so they are independent and one
 // launch sweeps both: blocks with z below nk0 take colour C, the rest colour
 // D.  NN > 0 fixes the grid size at compile time for the sizes that stream
 // from HBM: the 18 neighbour offsets become immediates of the loads.
 // ---------------------------------------------------------------------------
-template <int C, int NN>
+template <int C, int NN, bool UNORM>
 __device__ __forceinline__ void smooth_f2_block(double* u, const double* __restrict__ rhs, int n_rt,
                                                 const smoothf2::Params& P, unsigned long long* events, int bz)
 {
@@ -102,16 +109,16 @@ __device__ __forceinline__ void smooth_f2_block(double* u, const double* __restr
     const int j = ((C & 2) ? 1 : 2) + 2 * (int)(blockIdx.y * BY + threadIdx.y);
     const int k = ((C & 4) ? 1 : 2) + 2 * bz;
     if (i > n - 2 || j > n - 2 || k > n - 2) return;
-    smoothf2::point<long long>(u, rhs, lin(i, j, k, n), n, (long long)n * n, P, events);
+    smoothf2::point<UNORM, long long>(u, rhs, lin(i, j, k, n), n, (long long)n * n, P, events);
 }
 
-template <int C, int D, int NN>
+template <int C, int D, int NN, bool UNORM>
 __global__ void __launch_bounds__(BX * BY) k_smooth_f2(double* u, const double* __restrict__ rhs, int n,
                                                         smoothf2::Params P, unsigned long long* events, int nk0)
 {
     const int bz = blockIdx.z;
-    if (C == D || bz < nk0) smooth_f2_block<C, NN>(u, rhs, n, P, events, bz);
-    else smooth_f2_block<D, NN>(u, rhs, n, P, events, bz - nk0);
+    if (C == D || bz < nk0) smooth_f2_block<C, NN, UNORM>(u, rhs, n, P, events, bz);
+    else smooth_f2_block<D, NN, UNORM>(u, rhs, n, P, events, bz - nk0);
 }
 
 template <int C, int D>
@@ -124,15 +131,15 @@ cudaError_t launch_smooth_f2(double* u, const double* rhs, int n, const smoothf2
     const dim3 grid((ni + BX - 1) / BX, (nj + BY - 1) / BY, nk), blk(BX, BY);
     count_launches(1);
     switch (n) {
-    case 129: k_smooth_f2<C, D, 129><<<grid, blk, 0, s>>>(u, rhs, n, P, ev, nk0); break;
-    case 257: k_smooth_f2<C, D, 257><<<grid, blk, 0, s>>>(u, rhs, n, P, ev, nk0); break;
-    case 513: k_smooth_f2<C, D, 513><<<grid, blk, 0, s>>>(u, rhs, n, P, ev, nk0); break;
-    default: k_smooth_f2<C, D, 0><<<grid, blk, 0, s>>>(u, rhs, n, P, ev, nk0); break;
+    case 129: k_smooth_f2<C, D, 129, true><<<grid, blk, 0, s>>>(u, rhs, n, P, ev, nk0); break;
+    case 257: k_smooth_f2<C, D, 257, true><<<grid, blk, 0, s>>>(u, rhs, n, P, ev, nk0); break;
+    case 513: k_smooth_f2<C, D, 513, true><<<grid, blk, 0, s>>>(u, rhs, n, P, ev, nk0); break;
+    default:
+        if (n < kUnormMinN) k_smooth_f2<C, D, 0, false><<<grid, blk, 0, s>>>(u, rhs, n, P, ev, nk0);
+        else k_smooth_f2<C, D, 0, true><<<grid, blk, 0, s>>>(u, rhs, n, P, ev, nk0);
     }
     return cudaGetLastError();
 }
-
-constexpr int kF2MinN = 33;
 
 // ---------------------------------------------------------------------------
 // Block reduction of (max |x|, sum x^2) in a fixed order (deterministic).
@@ -212,20 +219,45 @@ __global__ void __launch_bounds__(BX * BY) k_coarse_rhs(const double* __restrict
     coarse_rhs_block(wc, rc, bc, nc, inv_H6, blockIdx);
 }
 
-// out = r + det(D^2_h u) (SIGN = 1, the coarse right-hand side) or r - det
-// (SIGN = -1, the residual without norms) inside and 0 on the shell, with exact
-// integer second differences and a two-float determinant (resid::gather_f2): one
-// point a thread, the grid size at compile time for the sizes of a hierarchy's
-// larger levels.  The FP64 forms of the two were bound by the FP64 pipe
-// (257^3: 754 us residual, 800 us right-hand side); this one by issue, 254 us
-// at 257^3, 36 against 98 at 129^3, 8.4 against 22 at 65^3, 3.8 against 7.2 at
-// 33^3 (Example 4, graph replay).  Runs of planes a thread, as the residual
-// with norms walks them, keep more values live (76 registers for 64): 297 us.
-template <int NN, int SIGN>
+// r + det(D^2_h u) (SIGN = 1, the coarse right-hand side) or r - det (SIGN = -1,
+// the residual) at a point, with exact integer second differences and a
+// two-float determinant; ld as gather_f2_of takes it.
+template <int SIGN, bool UNORM, typename Idx, typename Ld>
+__device__ __forceinline__ double operator_of(Ld ld, Idx sy, Idx sz, double rv, double inv_h6)
+{
+    using namespace resid;
+    f2::F2 H[6];
+    long long b0;
+    if (gather_f2_of<Idx>(ld, sy, sz, 0, H, &b0)) {
+        const float ih = (float)(SIGN * inv_h6);
+        const f2::F2 d = f2::mul(f2::det3<UNORM>(H[0], H[1], H[2], H[3], H[4], H[5]),
+                                 f2::F2{ih, (float)(SIGN * inv_h6 - (double)ih)});
+        const f2::F2 v = f2::add(f2::from_f64(rv), d);
+        return f2d(v.hi) + f2d(v.lo);
+    }
+    const HessS G = gather_hess_of([&](Idx o) { return __longlong_as_double(ld(o)); }, sy, sz, __longlong_as_double(b0));
+    return fma(SIGN * det0(G), inv_h6, rv);
+}
+
+// At a point of a grid in shared memory (q points at it).
+template <int SIGN, bool UNORM>
+__device__ __forceinline__ double operator_point(const double* q, int sy, int sz, double rv, double inv_h6)
+{
+    return operator_of<SIGN, UNORM, int>([q](int o) -> long long { return __double_as_longlong(q[o]); }, sy, sz, rv,
+                                         inv_h6);
+}
+
+// Over a grid, 0 on the shell: one point a thread, the grid size at compile time
+// for the sizes of a hierarchy's larger levels.  The FP64 forms of the two were
+// bound by the FP64 pipe (257^3: 754 us residual, 800 us right-hand side); this
+// one by issue, 252 us at 257^3, 36 against 98 at 129^3, 8.3 against 22 at 65^3,
+// 3.8 against 7.2 at 33^3 (Example 4, graph replay).  Runs of planes a thread,
+// as the residual with norms walks them, keep more values live (76 registers
+// for 64): 297 us.
+template <int NN, int SIGN, bool UNORM>
 __global__ void __launch_bounds__(BX * BY) k_operator_f2(const double* __restrict__ u, const double* __restrict__ r,
                                                          double* __restrict__ out, int n_rt, double inv_h6)
 {
-    using namespace resid;
     const int n = NN > 0 ? NN : n_rt;
     const int i = blockIdx.x * BX + threadIdx.x;
     const int j = blockIdx.y * BY + threadIdx.y;
@@ -236,19 +268,9 @@ __global__ void __launch_bounds__(BX * BY) k_operator_f2(const double* __restric
         out[p] = 0.0;
         return;
     }
-    f2::F2 H[6];
-    long long b0;
-    const double rv = __ldg(r + p);
-    if (gather_f2<long long>(u, p, n, sz, 0, H, &b0)) {
-        const float ih = (float)(SIGN * inv_h6);
-        const f2::F2 d = f2::mul(f2::det3<true>(H[0], H[1], H[2], H[3], H[4], H[5]),
-                                 f2::F2{ih, (float)(SIGN * inv_h6 - (double)ih)});
-        const f2::F2 v = f2::add(f2::from_f64(rv), d);
-        out[p] = f2d(v.hi) + f2d(v.lo);
-        return;
-    }
-    const HessS G = gather_hess(u, p, n, sz, __longlong_as_double(b0));
-    out[p] = fma(SIGN * det0(G), inv_h6, rv);
+    const long long* q = reinterpret_cast<const long long*>(u) + p;
+    out[p] = operator_of<SIGN, UNORM, long long>([q](long long o) -> long long { return __ldg(q + o); }, n, sz,
+                                                 __ldg(r + p), inv_h6);
 }
 
 template <int SIGN>
@@ -256,12 +278,14 @@ cudaError_t launch_operator_f2(const double* u, const double* r, double* out, in
 {
     const dim3 g = xfer::grid_of(n), b(BX, BY);
     switch (n) {
-    case 33: k_operator_f2<33, SIGN><<<g, b, 0, s>>>(u, r, out, n, inv_h6); break;
-    case 65: k_operator_f2<65, SIGN><<<g, b, 0, s>>>(u, r, out, n, inv_h6); break;
-    case 129: k_operator_f2<129, SIGN><<<g, b, 0, s>>>(u, r, out, n, inv_h6); break;
-    case 257: k_operator_f2<257, SIGN><<<g, b, 0, s>>>(u, r, out, n, inv_h6); break;
-    case 513: k_operator_f2<513, SIGN><<<g, b, 0, s>>>(u, r, out, n, inv_h6); break;
-    default: k_operator_f2<0, SIGN><<<g, b, 0, s>>>(u, r, out, n, inv_h6); break;
+    case 33: k_operator_f2<33, SIGN, true><<<g, b, 0, s>>>(u, r, out, n, inv_h6); break;
+    case 65: k_operator_f2<65, SIGN, true><<<g, b, 0, s>>>(u, r, out, n, inv_h6); break;
+    case 129: k_operator_f2<129, SIGN, true><<<g, b, 0, s>>>(u, r, out, n, inv_h6); break;
+    case 257: k_operator_f2<257, SIGN, true><<<g, b, 0, s>>>(u, r, out, n, inv_h6); break;
+    case 513: k_operator_f2<513, SIGN, true><<<g, b, 0, s>>>(u, r, out, n, inv_h6); break;
+    default:
+        if (n < kUnormMinN) k_operator_f2<0, SIGN, false><<<g, b, 0, s>>>(u, r, out, n, inv_h6);
+        else k_operator_f2<0, SIGN, true><<<g, b, 0, s>>>(u, r, out, n, inv_h6);
     }
     return cudaGetLastError();
 }
@@ -285,112 +309,255 @@ __global__ void k_copy_rhs_bc(const double* __restrict__ f, const double* __rest
 }
 
 // ---------------------------------------------------------------------------
-// Coarsest grid: one thread block sweeps the whole grid in shared memory.
+// Grids of n <= 17 in one thread block (ma_small_grid.cuh): sweeps, the
+// coarsest solve, the fused tail.  From 5^3 up the points take the two-float
+// forms, as the separate launches do: one warp's chain of 47 FP64 operations
+// holds its scheduler's FP64 unit for about 3000 cycles a phase, the two-float
+// chain takes about 1100.
 // ---------------------------------------------------------------------------
 constexpr int COARSE_THREADS = 256;
 
-__device__ __forceinline__ HessS gather_hess_plain(const double* u, int p, int sy, int sz, double v0)
+struct Grid64 {
+    double* u;
+    const double* rhs;
+    const int* tab;          // phase table (ascending order), n <= 9
+    smoothf2::Params P;
+};
+
+// nsw sweeps in ascending order; each(p, old, new) sees every update.  The
+// grid's phase threads enter.
+template <typename Each>
+__device__ __forceinline__ void run_sweeps64(const SmallGrid& G, const Grid64& S, int nsw, int nt,
+                                             unsigned long long* ev, Each each)
 {
-    const double* q = u + p;
-    const double a = q[1] + q[-1];
-    const double b = q[sy] + q[-sy];
-    const double c = q[sz] + q[-sz];
-    const double r4 = (q[sy + 1] + q[-sy - 1]) - (q[sy - 1] + q[-sy + 1]);
-    const double s4 = (q[sz + 1] + q[-sz - 1]) - (q[sz - 1] + q[-sz + 1]);
-    const double t4 = (q[sz + sy] + q[-sz - sy]) - (q[sy - sz] + q[-sy + sz]);
-    HessS H;
-    const double m8v = -8.0 * v0;
-    H.A = fma(4.0, a, m8v);
-    H.B = fma(4.0, b, m8v);
-    H.C = fma(4.0, c, m8v);
-    H.R = r4;
-    H.S = s4;
-    H.T = t4;
-    return H;
+    const int n = G.n, tid = threadIdx.x;
+    auto update = [&](int p) {
+        const double v0 = S.u[p];
+        bool nonconvex = false;
+        const double v = smoothf2::point_sm(S.u + p, n, n * n, S.rhs[p], S.P, &nonconvex);
+        S.u[p] = v;
+        *ev += nonconvex ? 1ull : 0ull;
+        each(v0, v);
+    };
+    if (n <= 9) {
+        int cur = S.tab[tid];
+        for (int q = 0, w = 0; q < 7 * nsw; ++q) {
+            w = w == 6 ? 0 : w + 1;
+            const int nxt = S.tab[w * nt + tid];
+            if (cur >= 0) update(cur & 0xffff);
+            phase_barrier(n);
+            cur = nxt;
+        }
+        return;
+    }
+    for (int q = 0, w = 0; q < 7 * nsw; ++q, w = w == 6 ? 0 : w + 1) {
+        const int c = phase_first(false, w), d = phase_second(false, w);
+        const int tot = G.count(c) + (d >= 0 ? G.count(d) : 0);
+        for (int t = tid; t < tot; t += nt) update(phase_point(G, false, w, t) & 0xffff);
+        phase_barrier(n);
+    }
 }
 
-__device__ __forceinline__ void coarsest64_body(double* u, const double* __restrict__ rhs, int n, double h6, int sweeps,
-                                                unsigned long long* events)
+// Newton's method on the 5^3 grid (27 unknowns) by one warp, from the current
+// iterate: the sweeps converge by a factor of 0.6, 40 - 70 of them to 1e-14,
+// each 7 phases long.  Lane = interior point.  The residuals and their FP32
+// Jacobian come from the two-float Hessian; the Jacobian is inverted in place
+// (Gauss-Jordan) and kept while an iteration cuts the residual tenfold.  Only
+// an iterate whose points are all positive definite, with positive right-hand
+// sides, is touched, and if the residual does not fall it is put back and
+// false returned; the caller's sweeps then decide as they would have.
+// J: 27 x kJ floats.
+constexpr int kJ = 29;   // an odd stride: a lane's row and a column of it meet no bank conflicts
+
+__device__ __forceinline__ bool newton5(double* u, const double* rhs, const smoothf2::Params& P, float* J)
+{
+    using namespace resid;
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const bool on = lane < 27;
+    const int a = on ? lane : 0;
+    const int i = 1 + a % 3, j = 1 + (a / 3) % 3, k = 1 + a / 9, p = (k * 5 + j) * 5 + i;
+    const double b = rhs[p], start = u[p];
+    const f2::F2 r6 = f2::mul(f2::from_f64(b), f2::F2{P.chi, P.clo});
+    float last = 0.0f;
+    bool moved = false;
+    for (int it = 0; it < 24; ++it) {
+        f2::F2 H[6];
+        long long b0;
+        bool ok = gather_f2_of<int>([&](int o) -> long long { return __double_as_longlong(u[p + o]); }, 5, 25, P.kexp,
+                                    H, &b0) &&
+                  __double_as_longlong(b) > 0;
+        float g = 0.0f;
+        if (ok) {
+            const f2::F2 d = f2::det3(H[0], H[1], H[2], H[3], H[4], H[5]);
+            const f2::F2 e = f2::add(d, f2::neg(r6));
+            g = e.hi + e.lo;
+            HessSf F;
+            F.A = H[0].hi; F.B = H[1].hi; F.C = H[2].hi;
+            F.R = H[3].hi; F.S = H[4].hi; F.T = H[5].hi;
+            const float scale = fabsf(F.A) + fabsf(F.B) + fabsf(F.C) + fabsf(F.R) + fabsf(F.S) + fabsf(F.T);
+            ok = is_pd<HessSf, float>(F, d.hi) && minors_shift_f(F, 0.0f) > 0.05f * scale * scale &&
+                 scale > 9.5e-7f && scale < 1.0e9f && isfinite(g);
+        }
+        float worst = fabsf(g);
+        for (int o = 16; o > 0; o >>= 1) worst = fmaxf(worst, __shfl_xor_sync(FULL, worst, o));
+        if (__any_sync(FULL, on && !ok) || (moved && !(worst < last))) {
+            // not a point Newton can be trusted from; or round-off: the residual no longer falls
+            const bool settled = moved && worst <= 1e-11f * fabsf(r6.hi);
+            if (moved && !__all_sync(FULL, !on || settled)) {
+                __syncwarp();
+                if (on) u[p] = start;
+                __syncwarp();
+                return false;
+            }
+            return moved;
+        }
+        if (worst == 0.0f) return true;
+        if (!moved || worst > 0.1f * last) {
+            // row of the Jacobian: the cofactors times the stencil's weights, 2^k taken out
+            const float A = H[0].hi, B = H[1].hi, C = H[2].hi, R = H[3].hi, S = H[4].hi, T = H[5].hi;
+            const float cA = B * C - T * T, cB = A * C - S * S, cC = A * B - R * R;
+            const float cR = S * T - R * C, cS = R * T - S * B, cT = R * S - T * A;
+            float* row = J + lane * kJ;
+            if (on) {
+                for (int c = 0; c < 27; ++c) row[c] = 0.0f;
+                auto add = [&](int di, int dj, int dk, float w) {
+                    const int x = i + di, y = j + dj, z = k + dk;
+                    if (x >= 1 && x <= 3 && y >= 1 && y <= 3 && z >= 1 && z <= 3)
+                        row[(x - 1) + 3 * (y - 1) + 9 * (z - 1)] = w;
+                };
+                add(0, 0, 0, -8.0f * (cA + cB + cC));
+                add(1, 0, 0, 4.0f * cA); add(-1, 0, 0, 4.0f * cA);
+                add(0, 1, 0, 4.0f * cB); add(0, -1, 0, 4.0f * cB);
+                add(0, 0, 1, 4.0f * cC); add(0, 0, -1, 4.0f * cC);
+                add(1, 1, 0, 2.0f * cR); add(-1, -1, 0, 2.0f * cR); add(1, -1, 0, -2.0f * cR); add(-1, 1, 0, -2.0f * cR);
+                add(1, 0, 1, 2.0f * cS); add(-1, 0, -1, 2.0f * cS); add(1, 0, -1, -2.0f * cS); add(-1, 0, 1, -2.0f * cS);
+                add(0, 1, 1, 2.0f * cT); add(0, -1, -1, 2.0f * cT); add(0, 1, -1, -2.0f * cT); add(0, -1, 1, -2.0f * cT);
+            }
+            __syncwarp();
+            for (int q = 0; q < 27; ++q) {   // in-place Gauss-Jordan; no pivoting: the matrix is near a definite one
+                const float piv = __fdividef(1.0f, J[q * kJ + q]);
+                const float f = on ? row[q] : 0.0f;
+                __syncwarp();
+                if (lane < 27) J[q * kJ + lane] = lane == q ? piv : J[q * kJ + lane] * piv;   // the pivot's row
+                __syncwarp();
+                if (on && lane != q) {
+#pragma unroll 9
+                    for (int c = 0; c < 27; ++c) row[c] = c == q ? -f * piv : fmaf(-f, J[q * kJ + c], row[c]);
+                }
+                __syncwarp();
+            }
+        }
+        float d = 0.0f;
+        for (int c = 0; c < 27; ++c) {
+            const float gc = __shfl_sync(FULL, g, c);
+            if (on) d = fmaf(-J[lane * kJ + c], gc, d);
+        }
+        if (on) u[p] = fma(8.0 * P.kz, f2d(d), u[p]);
+        __syncwarp();
+        last = worst;
+        moved = true;
+    }
+    return true;
+}
+
+// The coarsest grid in shared memory: sweeps until max |du| <= 1e-14 max |u| (at
+// most 100), or a fixed count; on 5^3 Newton's method first, again after every
+// eighth sweep where it could not start.  On 3^3 the one unknown's root with a
+// Newton step in FP64 (smallest_root_precise).  Every thread of the block
+// enters; ends with a block barrier.  J: 27 kJ floats.
+__device__ __forceinline__ void coarsest64_sm(const Grid64& S, int n, int sweeps, float* J, unsigned long long* ev)
+{
+    const int max_sweeps = sweeps > 0 ? sweeps : 100;
+    const int nt = phase_threads(n, (int)blockDim.x);
+    __shared__ double red[32][2];
+    if (n == 3) {
+        if (threadIdx.x == 0) {
+            double v = S.u[13];
+            for (int s = 0; s < max_sweeps; ++s) {
+                const double v0 = v;
+                const HessS H = gather_hess_of([&](int o) { return S.u[13 + o]; }, 3, 9, v0);
+                bool nonconvex = false;
+                const double z = smallest_root_precise(H, __dmul_rn(S.P.h6, S.rhs[13]), &nonconvex);
+                v = fma(0.125, z, v0);
+                *ev += nonconvex ? 1ull : 0ull;
+                if (sweeps == 0 && fabs(v - v0) <= 1e-14 * fabs(v)) break;
+            }
+            S.u[13] = v;
+        }
+    } else if ((int)threadIdx.x < nt) {
+        const SmallGrid G(n);
+        bool solved = false;
+        for (int s = 0; s < max_sweeps; ++s) {
+            if (n == 5 && sweeps == 0 && !solved && (s & 7) == 0) solved = newton5(S.u, S.rhs, S.P, J);
+            double du = 0.0, um = 0.0;
+            run_sweeps64(G, S, 1, nt, ev, [&](double v0, double v) {
+                du = fmax(du, fabs(v - v0));
+                um = fmax(um, fabs(v));
+            });
+            if (sweeps > 0) continue;
+            for (int o = 16; o > 0; o >>= 1) {
+                du = fmax(du, __shfl_xor_sync(0xffffffffu, du, o));
+                um = fmax(um, __shfl_xor_sync(0xffffffffu, um, o));
+            }
+            if (nt > 32) {
+                if ((threadIdx.x & 31) == 0) { red[threadIdx.x >> 5][0] = du; red[threadIdx.x >> 5][1] = um; }
+                phase_barrier(n);
+                du = um = 0.0;
+                for (int w = 0; w < nt / 32; ++w) { du = fmax(du, red[w][0]); um = fmax(um, red[w][1]); }
+                phase_barrier(n);   // red is free again
+            }
+            if (du <= 1e-14 * um) break;
+        }
+    }
+    __syncthreads();
+}
+
+__device__ __forceinline__ void coarsest64_body(double* u, const double* __restrict__ rhs, int n,
+                                                const smoothf2::Params& P, int sweeps, unsigned long long* events)
 {
     extern __shared__ double sm[];
+    __shared__ int tab[kPhaseTab];
+    __shared__ float J[27 * kJ];
     const int m = n * n * n;
     double* su = sm;
     double* sr = sm + m;
-    __shared__ double red[COARSE_THREADS / 32][2];
-    __shared__ int stop;
     for (int q = threadIdx.x; q < m; q += COARSE_THREADS) { su[q] = u[q]; sr[q] = rhs[q]; }
+    fill_phase_tab(tab, n, false);
     __syncthreads();
-    const int max_sweeps = sweeps > 0 ? sweeps : 100;
     unsigned long long ev = 0;
-    for (int s = 0; s < max_sweeps; ++s) {
-        double du = 0.0, um = 0.0;
-        for (int c = 0; c < 8; ++c) {
-            const int pi = c & 1, pj = (c >> 1) & 1, pk = (c >> 2) & 1;
-            const int ni = colour_count(n, pi), nj = colour_count(n, pj), nk = colour_count(n, pk);
-            const int cnt = (ni > 0 && nj > 0 && nk > 0) ? ni * nj * nk : 0;
-            for (int t = threadIdx.x; t < cnt; t += COARSE_THREADS) {
-                const int i = (pi ? 1 : 2) + 2 * (t % ni);
-                const int j = (pj ? 1 : 2) + 2 * ((t / ni) % nj);
-                const int k = (pk ? 1 : 2) + 2 * (t / (ni * nj));
-                const int p = (k * n + j) * n + i;
-                const double v0 = su[p];
-                const HessS H = gather_hess_plain(su, p, n, n * n, v0);
-                bool nonconvex = false;
-                const double z = smallest_root_precise(H, __dmul_rn(h6, sr[p]), &nonconvex);
-                const double v = fma(0.125, z, v0);
-                su[p] = v;
-                du = fmax(du, fabs(v - v0));
-                um = fmax(um, fabs(v));
-                ev += nonconvex ? 1ull : 0ull;
-            }
-            __syncthreads();
-        }
-        if (sweeps > 0) continue;
-        // converged when max |du| <= 1e-14 max |u| over this sweep's updates
-        for (int o = 16; o > 0; o >>= 1) {
-            du = fmax(du, __shfl_down_sync(0xffffffffu, du, o));
-            um = fmax(um, __shfl_down_sync(0xffffffffu, um, o));
-        }
-        if ((threadIdx.x & 31) == 0) { red[threadIdx.x >> 5][0] = du; red[threadIdx.x >> 5][1] = um; }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double a = 0.0, b = 0.0;
-            for (int w = 0; w < COARSE_THREADS / 32; ++w) { a = fmax(a, red[w][0]); b = fmax(b, red[w][1]); }
-            stop = (a <= 1e-14 * b) ? 1 : 0;
-        }
-        __syncthreads();
-        if (stop) break;
-    }
+    coarsest64_sm(Grid64{su, sr, tab, P}, n, sweeps, J, &ev);
     for (int q = threadIdx.x; q < m; q += COARSE_THREADS) u[q] = su[q];
     if (events && ev) atomicAdd(events, ev);
 }
 
 __global__ void __launch_bounds__(COARSE_THREADS) k_coarsest(double* u, const double* __restrict__ rhs, int n,
-                                                             double h6, int sweeps, unsigned long long* events)
+                                                             smoothf2::Params P, int sweeps,
+                                                             unsigned long long* events)
 {
-    coarsest64_body(u, rhs, n, h6, sweeps, events);
+    coarsest64_body(u, rhs, n, P, sweeps, events);
 }
 
 // ---------------------------------------------------------------------------
 // The tail of an FP64 V-cycle in one block: every level with n <= 17, from
 // the level the cycle enters there down to the coarsest grid and back, with
 // u, w, r and rhs of those levels in shared memory.  Each step repeats the
-// per-point arithmetic of its separate kernel -- the colour sweeps of
-// k_smooth_colour, the residual of resid::k_residual_col (its column
-// grouping of the cross differences), the restriction of xfer::k_restrict,
-// the tau-corrected right-hand side of k_coarse_rhs, the coarsest solve of
-// k_coarsest, the prolongation of xfer::k_prolong -- so the result is the
-// same bits; it replaces the ~100 launches these latency-bound levels take
-// (8 colour launches per sweep) by one.  FMG runs such a cycle from every
-// level, so it pays most there.
+// per-point arithmetic of its separate kernel -- the colour sweeps, the
+// residual and the tau-corrected right-hand side, the restriction of
+// xfer::k_restrict, the coarsest solve of k_coarsest, the prolongation of
+// xfer::k_prolong -- so the result is the same bits; it replaces the ~100
+// launches these latency-bound levels take by one.  FMG runs such a cycle
+// from every level, so it pays most there.
 // ---------------------------------------------------------------------------
 constexpr int T64 = 512;
 
 struct Tail64Level {
     int n;
-    double h6, inv_h6;   // 64 h^6 (the 4 Hs scaling) and its reciprocal
+    double inv_h6;       // 1 / (64 h^6)
+    smoothf2::Params P;
     double* u;           // global iterate (read on the top level, written back there)
     const double* rhs;   // global right-hand side (read on the top level)
+    int ou, ow, orr, orhs;   // places of the level's fields in shared memory, in doubles
 };
 
 struct Tail64Args {
@@ -406,55 +573,34 @@ __host__ __device__ inline int tail64_level_doubles(int n, bool top)
     return m /* u */ + (top ? 0 : m) /* w */ + m /* r */ + m /* rhs */;
 }
 
+inline void set_tail64_offsets(Tail64Args* A)
+{
+    int q = 0;
+    for (int l = 0; l < A->nlev; ++l) {
+        Tail64Level& V = A->lev[l];
+        const int m = V.n * V.n * V.n;
+        V.ou = q; q += m;
+        V.ow = q; q += l > 0 ? m : 0;
+        V.orr = q; q += m;
+        V.orhs = q; q += m;
+    }
+}
+
 struct Tail64Smem {
     double *u, *w, *r, *rhs;
 };
 
-__device__ __forceinline__ void tail64_smooth(const Tail64Smem& S, int n, double h6, int nsw, unsigned long long* ev)
+__device__ __forceinline__ Tail64Smem tail64_fields(const Tail64Args& A, double* sm, int l)
 {
-    for (int sw = 0; sw < nsw; ++sw) {
-        for (int c = 0; c < 8; ++c) {
-            const int pi = c & 1, pj = (c >> 1) & 1, pk = (c >> 2) & 1;
-            const int ni = colour_count(n, pi), nj = colour_count(n, pj), nk = colour_count(n, pk);
-            const int cnt = (ni > 0 && nj > 0 && nk > 0) ? ni * nj * nk : 0;
-            for (int t = threadIdx.x; t < cnt; t += T64) {
-                const int i = (pi ? 1 : 2) + 2 * (t % ni);
-                const int j = (pj ? 1 : 2) + 2 * ((t / ni) % nj);
-                const int k = (pk ? 1 : 2) + 2 * (t / (ni * nj));
-                const int p = (k * n + j) * n + i;
-                const double v0 = S.u[p];
-                const HessS H = gather_hess_plain(S.u, p, n, n * n, v0);
-                bool nonconvex = false;
-                const double z = smallest_root(H, __dmul_rn(h6, S.rhs[p]), &nonconvex);
-                S.u[p] = fma(0.125, z, v0);
-                *ev += nonconvex ? 1ull : 0ull;
-            }
-            __syncthreads();
-        }
-    }
+    const Tail64Level& V = A.lev[l];
+    return Tail64Smem{sm + V.ou, sm + V.ow, sm + V.orr, sm + V.orhs};
 }
 
-// rhs - det(D^2_h u) at interior point p, the cross differences grouped as
-// the column-marching residual kernel forms them.
-__device__ __forceinline__ double tail64_residual(const double* u, int p, int n, double rhs, double inv_h6)
+__device__ __forceinline__ void tail64_smooth(const Grid64& S, int n, int nsw, unsigned long long* ev)
 {
-    const int sy = n, sz = n * n;
-    const double* q = u + p;
-    const double a = q[1] + q[-1];
-    const double b = q[sy] + q[-sy];
-    const double c = q[sz] + q[-sz];
-    const double r4 = (q[sy + 1] - q[sy - 1]) - (q[-sy + 1] - q[-sy - 1]);
-    const double dxc = q[sz + 1] - q[sz - 1], dxa = q[-sz + 1] - q[-sz - 1];
-    const double dyc = q[sz + sy] - q[sz - sy], dya = q[-sz + sy] - q[-sz - sy];
-    HessS H;
-    const double m8v = -8.0 * q[0];
-    H.A = fma(4.0, a, m8v);
-    H.B = fma(4.0, b, m8v);
-    H.C = fma(4.0, c, m8v);
-    H.R = r4;
-    H.S = dxc - dxa;
-    H.T = dyc - dya;
-    return fma(-det0(H), inv_h6, rhs);
+    const int nt = phase_threads(n, T64);
+    if ((int)threadIdx.x < nt && nsw > 0) run_sweeps64(SmallGrid(n), S, nsw, nt, ev, [](double, double) {});
+    __syncthreads();
 }
 
 __device__ __forceinline__ double tail64_line(const double* uc, const double* wc, int nc, int Ic, int J0, int K0,
@@ -472,116 +618,84 @@ __device__ __forceinline__ double tail64_line(const double* uc, const double* wc
 __device__ __forceinline__ void vcycle_tail_body(const Tail64Args& A)
 {
     extern __shared__ double t64sm[];
-    Tail64Smem S[4];
+    __shared__ int tab[kTailTab];
+    __shared__ float J[27 * kJ];
+    // inputs: the top level's iterate and right-hand side
     {
-        double* q = t64sm;
-        for (int l = 0; l < A.nlev; ++l) {
-            const int m = A.lev[l].n * A.lev[l].n * A.lev[l].n;
-            S[l].u = q; q += m;
-            S[l].w = l > 0 ? q : nullptr; q += l > 0 ? m : 0;
-            S[l].r = q; q += m;
-            S[l].rhs = q; q += m;
-        }
+        const Tail64Smem S = tail64_fields(A, t64sm, 0);
+        const int m = A.lev[0].n * A.lev[0].n * A.lev[0].n;
+        for (int q = threadIdx.x; q < m; q += T64) { S.u[q] = A.lev[0].u[q]; S.rhs[q] = A.lev[0].rhs[q]; }
     }
-    // inputs: the top level's iterate and right-hand side; residual shells 0
-    // (the restriction reads only the interior, as in the separate path)
-    for (int l = 0; l < A.nlev; ++l) {
-        const int m = A.lev[l].n * A.lev[l].n * A.lev[l].n;
-        for (int q = threadIdx.x; q < m; q += T64) S[l].r[q] = 0.0;
-        if (l == 0)
-            for (int q = threadIdx.x; q < m; q += T64) { S[0].u[q] = A.lev[0].u[q]; S[0].rhs[q] = A.lev[0].rhs[q]; }
-    }
+    for (int l = 0; l < A.nlev; ++l) fill_phase_tab(tail_tab(tab, A.lev[l].n), A.lev[l].n, false);
     __syncthreads();
     unsigned long long ev = 0;
     const int L = A.nlev;
+    auto grid = [&](int l) {
+        const Tail64Smem S = tail64_fields(A, t64sm, l);
+        return Grid64{S.u, S.rhs, tail_tab(tab, A.lev[l].n), A.lev[l].P};
+    };
     for (int l = 0; l < L - 1; ++l) {
-        const Tail64Smem& F = S[l];
-        const Tail64Smem& C = S[l + 1];
-        const int nf = A.lev[l].n, nc = A.lev[l + 1].n;
-        tail64_smooth(F, nf, A.lev[l].h6, A.nu1, &ev);                                       // (2)
+        const Tail64Smem F = tail64_fields(A, t64sm, l);
+        const Tail64Smem C = tail64_fields(A, t64sm, l + 1);
+        const int nf = A.lev[l].n, nc = A.lev[l + 1].n, ni = nc - 2;
+        const SmallGrid GF(nf), GC(nc);
+        tail64_smooth(grid(l), nf, A.nu1, &ev);                                              // (2)
         for (int q = threadIdx.x; q < (nf - 2) * (nf - 2) * (nf - 2); q += T64) {        // (3)
-            const int i = 1 + q % (nf - 2), j = 1 + (q / (nf - 2)) % (nf - 2), k = 1 + q / ((nf - 2) * (nf - 2));
-            const int p = (k * nf + j) * nf + i;
-            F.r[p] = tail64_residual(F.u, p, nf, F.rhs[p], A.lev[l].inv_h6);
+            int i, j, k;
+            const int p = GF.interior(q, &i, &j, &k);
+            F.r[p] = operator_point<-1, false>(F.u + p, nf, nf * nf, F.rhs[p], A.lev[l].inv_h6);
         }
         __syncthreads();
-        for (int pc = threadIdx.x; pc < nc * nc * nc; pc += T64) {                        // (3)-(4)
-            const int I = pc % nc, J = (pc / nc) % nc, K = pc / (nc * nc);
-            const int pf = ((2 * K) * nf + 2 * J) * nf + 2 * I;
-            const bool inside = I > 0 && J > 0 && K > 0 && I < nc - 1 && J < nc - 1 && K < nc - 1;
-            C.r[pc] = inside ? xfer::weighted_restrict(F.r, pf, nf, (long long)nf * nf, A.kind) : 0.0;
-            const double w = (inside && A.approx == 1) ? xfer::weighted_restrict(F.u, pf, nf, (long long)nf * nf, A.kind)
-                                                      : F.u[pf];
+        // (3)-(4): the interior's two restrictions side by side (both are FP64 sums), the shell's injection
+        for (int q = threadIdx.x; q < 2 * ni * ni * ni; q += T64) {
+            const bool of_u = q >= ni * ni * ni;
+            int I, Jc, K;
+            const int pc = GC.interior(of_u ? q - ni * ni * ni : q, &I, &Jc, &K);
+            const double* v = (of_u ? F.u : F.r) + ((2 * K) * nf + 2 * Jc) * nf + 2 * I;
+            const double x = of_u && A.approx != 1
+                                 ? v[0]
+                                 : xfer::restrict_of<double>(
+                                       [&](int di, int dj, int dk) -> double { return v[(dk * nf + dj) * nf + di]; },
+                                       A.kind);
+            if (of_u) {
+                C.w[pc] = x;
+                C.u[pc] = x;
+            } else {
+                C.r[pc] = x;
+            }
+        }
+        for (int pc = threadIdx.x; pc < nc * nc * nc; pc += T64) {
+            const int J0 = (pc * GC.mn) >> 16, K = (J0 * GC.mn) >> 16, I = pc - J0 * nc, Jc = J0 - K * nc;
+            if (I > 0 && Jc > 0 && K > 0 && I < nc - 1 && Jc < nc - 1 && K < nc - 1) continue;
+            const double w = F.u[((2 * K) * nf + 2 * Jc) * nf + 2 * I];
             C.w[pc] = w;
             C.u[pc] = w;
         }
         __syncthreads();
-        for (int p = threadIdx.x; p < nc * nc * nc; p += T64) {                           // (5)
-            const int I = p % nc, J = (p / nc) % nc, K = p / (nc * nc);
-            double b = 0.0;
-            if (I > 0 && J > 0 && K > 0 && I < nc - 1 && J < nc - 1 && K < nc - 1) {
-                const HessS H = gather_hess_plain(C.w, p, nc, nc * nc, C.w[p]);
-                b = fma(det0(H), A.lev[l + 1].inv_h6, C.r[p]);
+        for (int q = threadIdx.x; q < ni * ni * ni; q += T64) {                            // (5)
+            int i, j, k;
+            const int p = GC.interior(q, &i, &j, &k);
+            if (nc >= kF2MinN) {
+                C.rhs[p] = operator_point<1, false>(C.w + p, nc, nc * nc, C.r[p], A.lev[l + 1].inv_h6);
+            } else {
+                const HessS H = gather_hess_of([&](int o) { return C.w[p + o]; }, nc, nc * nc, C.w[p]);
+                C.rhs[p] = fma(det0(H), A.lev[l + 1].inv_h6, C.r[p]);
             }
-            C.rhs[p] = b;
         }
         __syncthreads();
     }
-    {   // (1) coarsest grid: sweeps until max|du| <= 1e-14 max|u| (at most 100), or a fixed count
-        const Tail64Smem& Bt = S[L - 1];
-        const int n = A.lev[L - 1].n;
-        const double h6 = A.lev[L - 1].h6;
-        __shared__ double red[T64 / 32][2];
-        __shared__ int stop;
-        const int max_sweeps = A.coarse_sweeps > 0 ? A.coarse_sweeps : 100;
-        for (int s = 0; s < max_sweeps; ++s) {
-            double du = 0.0, um = 0.0;
-            for (int c = 0; c < 8; ++c) {
-                const int pi = c & 1, pj = (c >> 1) & 1, pk = (c >> 2) & 1;
-                const int ni = colour_count(n, pi), nj = colour_count(n, pj), nk = colour_count(n, pk);
-                const int cnt = (ni > 0 && nj > 0 && nk > 0) ? ni * nj * nk : 0;
-                for (int t = threadIdx.x; t < cnt; t += T64) {
-                    const int i = (pi ? 1 : 2) + 2 * (t % ni);
-                    const int j = (pj ? 1 : 2) + 2 * ((t / ni) % nj);
-                    const int k = (pk ? 1 : 2) + 2 * (t / (ni * nj));
-                    const int p = (k * n + j) * n + i;
-                    const double v0 = Bt.u[p];
-                    const HessS H = gather_hess_plain(Bt.u, p, n, n * n, v0);
-                    bool nonconvex = false;
-                    const double z = smallest_root_precise(H, __dmul_rn(h6, Bt.rhs[p]), &nonconvex);
-                    const double v = fma(0.125, z, v0);
-                    Bt.u[p] = v;
-                    du = fmax(du, fabs(v - v0));
-                    um = fmax(um, fabs(v));
-                    ev += nonconvex ? 1ull : 0ull;
-                }
-                __syncthreads();
-            }
-            if (A.coarse_sweeps > 0) continue;
-            for (int o = 16; o > 0; o >>= 1) {
-                du = fmax(du, __shfl_down_sync(0xffffffffu, du, o));
-                um = fmax(um, __shfl_down_sync(0xffffffffu, um, o));
-            }
-            if ((threadIdx.x & 31) == 0) { red[threadIdx.x >> 5][0] = du; red[threadIdx.x >> 5][1] = um; }
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                double a = 0.0, b = 0.0;
-                for (int w = 0; w < T64 / 32; ++w) { a = fmax(a, red[w][0]); b = fmax(b, red[w][1]); }
-                stop = (a <= 1e-14 * b) ? 1 : 0;
-            }
-            __syncthreads();
-            if (stop) break;
-        }
-    }
+    coarsest64_sm(grid(L - 1), A.lev[L - 1].n, A.coarse_sweeps, J, &ev);                     // (1)
     for (int l = L - 2; l >= 0; --l) {
-        const Tail64Smem& F = S[l];
-        const Tail64Smem& C = S[l + 1];
+        const Tail64Smem F = tail64_fields(A, t64sm, l);
+        const Tail64Smem C = tail64_fields(A, t64sm, l + 1);
         const int nf = A.lev[l].n, nc = A.lev[l + 1].n;
+        const SmallGrid GF(nf);
         // (7)-(8) u_h += I(u_H - w_H) on the fine interior, each value formed as xfer::k_prolong forms it
         for (int q = threadIdx.x; q < (nf - 2) * (nf - 2) * (nf - 2); q += T64) {
-            const int i = 1 + q % (nf - 2), j = 1 + (q / (nf - 2)) % (nf - 2), k = 1 + q / ((nf - 2) * (nf - 2));
+            int i, j, k;
+            const int p = GF.interior(q, &i, &j, &k);
             const int J0 = j >> 1, K0 = k >> 1, oj = j & 1, ok = k & 1;
-            const double w = 1.0 / (double)(1 << (oj + ok));
+            const double w = oj + ok == 2 ? 0.25 : (oj + ok == 1 ? 0.5 : 1.0);
             double v;
             if (i & 1) {
                 const int I = i >> 1;
@@ -591,18 +705,17 @@ __device__ __forceinline__ void vcycle_tail_body(const Tail64Args& A)
             } else {
                 v = tail64_line(C.u, C.w, nc, i >> 1, J0, K0, oj, ok, w);
             }
-            const int p = (k * nf + j) * nf + i;
             F.u[p] = F.u[p] + v;
         }
         __syncthreads();
-        tail64_smooth(F, nf, A.lev[l].h6, A.nu2, &ev);                                      // (9)
+        tail64_smooth(grid(l), nf, A.nu2, &ev);                                             // (9)
     }
     const int m0 = A.lev[0].n * A.lev[0].n * A.lev[0].n;
-    for (int q = threadIdx.x; q < m0; q += T64) A.lev[0].u[q] = S[0].u[q];
+    for (int q = threadIdx.x; q < m0; q += T64) A.lev[0].u[q] = t64sm[A.lev[0].ou + q];
     if (A.events && ev) atomicAdd(A.events, ev);
 }
 
-__global__ void __launch_bounds__(T64, 1) k_vcycle_tail(Tail64Args A) { vcycle_tail_body(A); }
+__global__ void __launch_bounds__(T64, 1) k_vcycle_tail(const __grid_constant__ Tail64Args A) { vcycle_tail_body(A); }
 
 int tail64_smem_bytes(const int* ns, int nlev)
 {
@@ -626,77 +739,7 @@ using batched::split_block;
 using batched::TableBuilder;
 
 enum F64OpId {
-    F_SMOOTH0 = batched::kF64Ops,   // .. + 7
-    F_RESID = batched::kF64Ops + 8, F_RESTRICT, F_COARSE_RHS, F_PROLONG, F_CUBIC0, F_CUBIC1, F_CUBIC2, F_INJECT,
-    F_ZERO, F_COARSEST, F_TAIL, F_NORMPART
-};
-
-struct Smooth64Job {
-    int inst, n, gx, gy;
-    double h6;
-    double* u;
-    const double* rhs;
-    unsigned long long* events;
-};
-
-template <int C>
-struct OpSmooth64 {
-    static constexpr int NT = BX * BY, MINB = 1;
-    using Job = Smooth64Job;
-    static __device__ __forceinline__ void run(const Job& J, int q)
-    {
-        smooth_colour_block<C & 1, (C >> 1) & 1, (C >> 2) & 1>(J.u, J.rhs, J.n, J.h6, J.events,
-                                                               split_block(q, J.gx, J.gy));
-    }
-};
-
-struct OpResid64 {
-    static constexpr int NT = resid::RX * resid::RY, MINB = 1;
-    struct Job {
-        int inst, n, kchunk, gx, gy, gz;
-        double inv_h6;
-        const double* u;
-        const double* rhs;
-        double* r;
-    };
-    static __device__ __forceinline__ void run(const Job& J, int q)
-    {
-        resid::residual_col_block<resid::NaturalF64Out>(J.u, J.rhs, resid::NaturalF64Out{J.r}, J.n, J.inv_h6, nullptr,
-                                                        J.kchunk, split_block(q, J.gx, J.gy),
-                                                        make_uint3((unsigned)J.gx, (unsigned)J.gy, (unsigned)J.gz));
-    }
-};
-
-struct OpRestrict64 {
-    static constexpr int NT = BX * BY, MINB = 1;
-    struct Job {
-        int inst, nf, nc, kind, approx, gx, gy;
-        const double* uf;
-        const double* rf;
-        double* wc;
-        double* uc;
-        double* rc;
-    };
-    static __device__ __forceinline__ void run(const Job& J, int q)
-    {
-        xfer::restrict_block<double>(J.uf, J.rf, J.nf, J.wc, J.uc, J.rc, J.nc, J.kind, J.approx,
-                                     split_block(q, J.gx, J.gy));
-    }
-};
-
-struct OpCoarseRhs64 {
-    static constexpr int NT = BX * BY, MINB = 1;
-    struct Job {
-        int inst, nc, gx, gy;
-        double inv_H6;
-        const double* wc;
-        const double* rc;
-        double* bc;
-    };
-    static __device__ __forceinline__ void run(const Job& J, int q)
-    {
-        coarse_rhs_block(J.wc, J.rc, J.bc, J.nc, J.inv_H6, split_block(q, J.gx, J.gy));
-    }
+    F_PROLONG = batched::kF64Ops, F_CUBIC0, F_CUBIC1, F_CUBIC2, F_INJECT, F_ZERO, F_COARSEST, F_NORMPART
 };
 
 // add != 0: uf += I(uc - wc); add == 0: uf = I(uc) (trilinear)
@@ -759,24 +802,15 @@ struct OpCoarsest64 {
     static constexpr int NT = COARSE_THREADS, MINB = 1;
     struct Job {
         int inst, n, sweeps;
-        double h6;
+        smoothf2::Params P;
         double* u;
         const double* rhs;
         unsigned long long* events;
     };
     static __device__ __forceinline__ void run(const Job& J, int)
     {
-        coarsest64_body(J.u, J.rhs, J.n, J.h6, J.sweeps, J.events);
+        coarsest64_body(J.u, J.rhs, J.n, J.P, J.sweeps, J.events);
     }
-};
-
-struct OpTail64 {
-    static constexpr int NT = T64, MINB = 1;
-    struct Job {
-        int inst;
-        Tail64Args A;
-    };
-    static __device__ __forceinline__ void run(const Job& J, int) { vcycle_tail_body(J.A); }
 };
 
 struct OpNormPart64 {
@@ -793,151 +827,7 @@ struct OpNormPart64 {
     }
 };
 
-inline double pow6h(double h)
-{
-    const double h2 = h * h;
-    return 64.0 * h2 * h2 * h2;
-}
-
 dim3 grid2(int n) { return dim3((n + BX - 1) / BX, (n + BY - 1) / BY, n); }
-
-// An entry of a batched FP64 V-cycle: instance (index into the array) and the
-// level its cycle starts from.
-struct VEntry {
-    int b, l0;
-};
-
-void emit_smooth64(TableBuilder& T, const BatchInstance* in, const std::vector<VEntry>& E, const std::vector<int>& lev,
-                   int nsweeps)
-{
-    for (int sw = 0; sw < nsweeps; ++sw)
-        for (int c = 0; c < 8; ++c) {
-            std::vector<Smooth64Job> jobs;
-            std::vector<int> blocks;
-            for (size_t q = 0; q < E.size(); ++q) {
-                if (lev[q] < 0) continue;
-                const BatchInstance& I = in[E[q].b];
-                const BatchLevel& F = I.lev[lev[q]];
-                const int ni = colour_count(F.n, c & 1), nj = colour_count(F.n, (c >> 1) & 1),
-                          nk = colour_count(F.n, (c >> 2) & 1);
-                if (ni <= 0 || nj <= 0 || nk <= 0) continue;
-                Smooth64Job J{I.id, F.n, (ni + BX - 1) / BX, (nj + BY - 1) / BY, pow6h(F.h), F.u, F.rhs, I.events};
-                jobs.push_back(J);
-                blocks.push_back(J.gx * J.gy * nk);
-            }
-            T.emit(F_SMOOTH0 + c, jobs, blocks, 0);
-        }
-}
-
-// Algorithm 1 from level l0 of each entry down to the coarsest grid and
-// back, with the fused FP64 tail: the launches of vcycle_from, depth by
-// depth relative to l0.
-void emit_vcycle64(TableBuilder& T, const BatchInstance* in, const std::vector<VEntry>& E, const BatchParams& p)
-{
-    if (E.empty()) return;
-    std::vector<int> lt(E.size()), fused(E.size());
-    int R = 0;
-    for (size_t q = 0; q < E.size(); ++q) {
-        const BatchInstance& I = in[E[q].b];
-        int t = I.L - 1;
-        while (t > E[q].l0 && I.lev[t - 1].n <= p.vtail_max) --t;
-        fused[q] = I.lev[t].n <= p.vtail_max;
-        lt[q] = fused[q] ? t : I.L - 1;
-        R = std::max(R, lt[q] - E[q].l0);
-    }
-    auto level_at = [&](int r) {
-        std::vector<int> lev(E.size(), -1);
-        for (size_t q = 0; q < E.size(); ++q)
-            if (r < lt[q] - E[q].l0) lev[q] = E[q].l0 + r;
-        return lev;
-    };
-    for (int r = 0; r < R; ++r) {
-        const std::vector<int> lev = level_at(r);
-        emit_smooth64(T, in, E, lev, p.nu1);
-        std::vector<OpResid64::Job> rj;
-        std::vector<OpRestrict64::Job> sj;
-        std::vector<OpCoarseRhs64::Job> cj;
-        std::vector<int> rb, sb, cb;
-        for (size_t q = 0; q < E.size(); ++q) {
-            if (lev[q] < 0) continue;
-            const BatchInstance& I = in[E[q].b];
-            const BatchLevel& F = I.lev[lev[q]];
-            const BatchLevel& C = I.lev[lev[q] + 1];
-            const dim3 g = reduce_grid(F.n);
-            const int kchunk = (F.n + (int)g.z - 1) / (int)g.z;
-            rj.push_back(OpResid64::Job{I.id, F.n, kchunk, (int)g.x, (int)g.y, (int)g.z, 1.0 / pow6h(F.h), F.u, F.rhs,
-                                        F.r});
-            rb.push_back((int)(g.x * g.y * g.z));
-            const dim3 gc = grid2(C.n);
-            sj.push_back(OpRestrict64::Job{I.id, F.n, C.n, p.kind, p.approx, (int)gc.x, (int)gc.y, F.u, F.r, C.w, C.u,
-                                           C.r});
-            sb.push_back((int)(gc.x * gc.y * gc.z));
-            cj.push_back(OpCoarseRhs64::Job{I.id, C.n, (int)gc.x, (int)gc.y, 1.0 / pow6h(C.h), C.w, C.r, C.rhs});
-            cb.push_back((int)(gc.x * gc.y * gc.z));
-        }
-        T.emit(F_RESID, rj, rb, 0);
-        T.emit(F_RESTRICT, sj, sb, 0);
-        T.emit(F_COARSE_RHS, cj, cb, 0);
-    }
-    {
-        std::vector<OpTail64::Job> tj;
-        std::vector<OpCoarsest64::Job> kj;
-        std::vector<int> tb, kb;
-        int tsmem = 0, ksmem = 0;
-        for (size_t q = 0; q < E.size(); ++q) {
-            const BatchInstance& I = in[E[q].b];
-            if (fused[q]) {
-                OpTail64::Job J;
-                std::memset(&J, 0, sizeof J);
-                J.inst = I.id;
-                Tail64Args& A = J.A;
-                A.nlev = I.L - lt[q];
-                int ns[4] = {0, 0, 0, 0};
-                for (int v = 0; v < A.nlev; ++v) {
-                    const BatchLevel& V = I.lev[lt[q] + v];
-                    ns[v] = V.n;
-                    A.lev[v].n = V.n;
-                    A.lev[v].h6 = pow6h(V.h);
-                    A.lev[v].inv_h6 = 1.0 / pow6h(V.h);
-                    A.lev[v].u = V.u;
-                    A.lev[v].rhs = V.rhs;
-                }
-                A.nu1 = p.nu1;
-                A.nu2 = p.nu2;
-                A.kind = p.kind;
-                A.approx = p.approx;
-                A.coarse_sweeps = p.coarse_sweeps;
-                A.events = I.events;
-                tsmem = std::max(tsmem, tail64_smem_bytes(ns, A.nlev));
-                tj.push_back(J);
-                tb.push_back(1);
-            } else {
-                const BatchLevel& V = I.lev[I.L - 1];
-                kj.push_back(OpCoarsest64::Job{I.id, V.n, p.coarse_sweeps, pow6h(V.h), V.u, V.rhs, I.events});
-                kb.push_back(1);
-                ksmem = std::max(ksmem, (int)(2 * sizeof(double) * (size_t)V.n * V.n * V.n));
-            }
-        }
-        T.emit(F_TAIL, tj, tb, tsmem);
-        T.emit(F_COARSEST, kj, kb, ksmem);
-    }
-    for (int r = R - 1; r >= 0; --r) {
-        const std::vector<int> lev = level_at(r);
-        std::vector<OpProlong64::Job> pj;
-        std::vector<int> pb;
-        for (size_t q = 0; q < E.size(); ++q) {
-            if (lev[q] < 0) continue;
-            const BatchInstance& I = in[E[q].b];
-            const BatchLevel& F = I.lev[lev[q]];
-            const BatchLevel& C = I.lev[lev[q] + 1];
-            const dim3 g = xfer::prolong_grid(F.n);
-            pj.push_back(OpProlong64::Job{I.id, C.n, F.n, 1, (int)g.x, (int)g.y, C.u, C.w, F.u});
-            pb.push_back((int)(g.x * g.y * g.z));
-        }
-        T.emit(F_PROLONG, pj, pb, 0);
-        emit_smooth64(T, in, E, lev, p.nu2);
-    }
-}
 
 }  // namespace
 
@@ -987,7 +877,8 @@ void emit_fmg_f64(TableBuilder& T, const BatchInstance* in, int count, const Bat
             const dim3 g = grid2(V.n);
             zj.push_back(OpZero64::Job{in[b].id, V.n, (int)g.x, (int)g.y, V.u});
             zb.push_back((int)(g.x * g.y * g.z));
-            kj.push_back(OpCoarsest64::Job{in[b].id, V.n, p.coarse_sweeps, pow6h(V.h), V.u, V.rhs, in[b].events});
+            kj.push_back(OpCoarsest64::Job{in[b].id, V.n, p.coarse_sweeps, smoothf2::make_params(V.h), V.u, V.rhs,
+                                           in[b].events});
             kb.push_back(1);
             ksmem = std::max(ksmem, (int)(2 * sizeof(double) * (size_t)V.n * V.n * V.n));
         }
@@ -999,7 +890,7 @@ void emit_fmg_f64(TableBuilder& T, const BatchInstance* in, int count, const Bat
         std::vector<OpProlong64::Job> lj;
         std::vector<CubicJob> c0, c1, c2;
         std::vector<int> lb, b0, b1, b2;
-        std::vector<VEntry> E;
+        std::vector<std::pair<int, int>> E;
         for (int b = 0; b < count; ++b) {
             const int l = in[b].L - 1 - j;
             if (l < 0) continue;
@@ -1023,19 +914,13 @@ void emit_fmg_f64(TableBuilder& T, const BatchInstance* in, int count, const Bat
                 lj.push_back(OpProlong64::Job{in[b].id, nc, nf, 0, (int)g.x, (int)g.y, C.u, nullptr, F.u});
                 lb.push_back((int)(g.x * g.y * g.z));
             }
-            if (l >= 1) E.push_back(VEntry{b, l});
+            if (l >= 1) E.emplace_back(b, l);
         }
         T.emit(F_PROLONG, lj, lb, 0);
         T.emit(F_CUBIC0, c0, b0, 0);
         T.emit(F_CUBIC1, c1, b1, 0);
         T.emit(F_CUBIC2, c2, b2, 0);
-        if (level_step) {
-            std::vector<std::pair<int, int>> steps;
-            for (const VEntry& v : E) steps.emplace_back(v.b, v.l0);
-            if (!steps.empty()) level_step(steps);
-        } else {
-            emit_vcycle64(T, in, E, p);
-        }
+        if (!E.empty()) level_step(E);
     }
 }
 
@@ -1044,17 +929,6 @@ cudaError_t batch_launch_f64(const char* tables, const batched::BLaunch& L, cons
     using batched::launch;
     const dim3 b2(BX, BY);
     switch (L.op) {
-    case F_SMOOTH0 + 0: return launch<OpSmooth64<0>>(tables, L, b2, active, s);
-    case F_SMOOTH0 + 1: return launch<OpSmooth64<1>>(tables, L, b2, active, s);
-    case F_SMOOTH0 + 2: return launch<OpSmooth64<2>>(tables, L, b2, active, s);
-    case F_SMOOTH0 + 3: return launch<OpSmooth64<3>>(tables, L, b2, active, s);
-    case F_SMOOTH0 + 4: return launch<OpSmooth64<4>>(tables, L, b2, active, s);
-    case F_SMOOTH0 + 5: return launch<OpSmooth64<5>>(tables, L, b2, active, s);
-    case F_SMOOTH0 + 6: return launch<OpSmooth64<6>>(tables, L, b2, active, s);
-    case F_SMOOTH0 + 7: return launch<OpSmooth64<7>>(tables, L, b2, active, s);
-    case F_RESID: return launch<OpResid64>(tables, L, dim3(resid::RX, resid::RY), active, s);
-    case F_RESTRICT: return launch<OpRestrict64>(tables, L, b2, active, s);
-    case F_COARSE_RHS: return launch<OpCoarseRhs64>(tables, L, b2, active, s);
     case F_PROLONG: return launch<OpProlong64>(tables, L, b2, active, s);
     case F_CUBIC0: return launch<OpCubic<0>>(tables, L, b2, active, s);
     case F_CUBIC1: return launch<OpCubic<1>>(tables, L, b2, active, s);
@@ -1062,7 +936,6 @@ cudaError_t batch_launch_f64(const char* tables, const batched::BLaunch& L, cons
     case F_INJECT: return launch<OpInject64>(tables, L, b2, active, s);
     case F_ZERO: return launch<OpZero64>(tables, L, b2, active, s);
     case F_COARSEST: return launch<OpCoarsest64>(tables, L, dim3(COARSE_THREADS), active, s);
-    case F_TAIL: return launch<OpTail64>(tables, L, dim3(T64), active, s);
     case F_NORMPART: return launch<OpNormPart64>(tables, L, b2, active, s);
     default: return cudaErrorInvalidValue;
     }
@@ -1082,8 +955,8 @@ static inline double pow6(double h) { const double h2 = h * h; return 64.0 * h2 
 cudaError_t launch_smooth(double* u, const double* rhs, int n, double h, int nsweeps,
                           unsigned long long* events, cudaStream_t s)
 {
-    smoothf2::Params P;
-    if (n >= kF2MinN && smoothf2::make_params(h, &P)) {
+    const smoothf2::Params P = smoothf2::make_params(h);
+    if (n >= kF2MinN && P.kexp != smoothf2::kNone) {
         for (int sw = 0; sw < nsweeps; ++sw) {
             cudaError_t e;
             if ((e = launch_smooth_f2<0, 0>(u, rhs, n, P, events, s)) != cudaSuccess) return e;
@@ -1127,8 +1000,13 @@ cudaError_t launch_residual(const double* u, const double* rhs, double* r, int n
     const int kchunk = (n + (int)g.z - 1) / (int)g.z;
     if (n >= kF2MinN) {
         if (!partials) return launch_operator_f2<-1>(u, rhs, r, n, 1.0 / pow6(h), s);
-        resid::launch_k_residual_f2(resid::grid_for(n, g.z), s, u, rhs, resid::NaturalF2Out<true>{r}, n, 1.0 / pow6(h),
-                                    partials, kchunk);
+        const dim3 gk = resid::grid_for(n, g.z);
+        if (n < kUnormMinN)
+            resid::launch_k_residual_f2(gk, s, u, rhs, resid::NaturalF2Out<false>{r}, n, 1.0 / pow6(h), partials,
+                                        kchunk);
+        else
+            resid::launch_k_residual_f2(gk, s, u, rhs, resid::NaturalF2Out<true>{r}, n, 1.0 / pow6(h), partials,
+                                        kchunk);
         return cudaGetLastError();
     }
     resid::k_residual_col<resid::NaturalF64Out><<<resid::grid_for(n, g.z), dim3(resid::RX, resid::RY), 0, s>>>(
@@ -1258,7 +1136,7 @@ cudaError_t launch_coarsest(double* u, const double* rhs, int n, double h, int s
 {
     const size_t smem = 2 * sizeof(double) * (size_t)n * n * n;
     count_launches(1);
-    k_coarsest<<<1, COARSE_THREADS, smem, s>>>(u, rhs, n, pow6(h), sweeps, events);
+    k_coarsest<<<1, COARSE_THREADS, smem, s>>>(u, rhs, n, smoothf2::make_params(h), sweeps, events);
     return cudaGetLastError();
 }
 
@@ -1283,17 +1161,18 @@ cudaError_t launch_vcycle_tail(const TailSpec64* lv, int nlev, int nu1, int nu2,
                                int coarse_sweeps, unsigned long long* events, cudaStream_t s)
 {
     if (nlev < 1 || nlev > 4) return cudaErrorInvalidValue;
-    Tail64Args A;
+    Tail64Args A{};
     A.nlev = nlev;
     int ns[4];
     for (int l = 0; l < nlev; ++l) {
         if (lv[l].n > 17 || (l > 0 && lv[l].n != (lv[l - 1].n + 1) / 2)) return cudaErrorInvalidValue;
         A.lev[l].n = ns[l] = lv[l].n;
-        A.lev[l].h6 = pow6(lv[l].h);
         A.lev[l].inv_h6 = 1.0 / pow6(lv[l].h);
+        A.lev[l].P = smoothf2::make_params(lv[l].h);
         A.lev[l].u = lv[l].u;
         A.lev[l].rhs = lv[l].rhs;
     }
+    set_tail64_offsets(&A);
     A.nu1 = nu1;
     A.nu2 = nu2;
     A.kind = kind;
@@ -1312,9 +1191,6 @@ cudaError_t prepare_coarsest_f64()
     if (e != cudaSuccess) return e;
     const int tail_ns[4] = {17, 9, 5, 3};
     if ((e = cudaFuncSetAttribute(k_vcycle_tail, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  tail64_smem_bytes(tail_ns, 4))) != cudaSuccess)
-        return e;
-    if ((e = cudaFuncSetAttribute(batched::k_batched<OpTail64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   tail64_smem_bytes(tail_ns, 4))) != cudaSuccess)
         return e;
     return cudaFuncSetAttribute(batched::k_batched<OpCoarsest64>, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -30,6 +30,7 @@
 #include "ma_point.cuh"
 #include "ma_transfer.cuh"
 #include "ma_residual.cuh"
+#include "ma_small_grid.cuh"
 
 namespace ma {
 
@@ -39,6 +40,7 @@ using xfer::BX;
 using xfer::BY;
 using xfer::grid_of;
 using xfer::lin;
+using namespace small;
 
 struct S3f {
     float xx, yy, zz, xy, xz, yz;
@@ -1003,14 +1005,7 @@ __global__ void __launch_bounds__(BX * BY) k_coarse_rhs_corr(const float* __rest
     coarse_rhs_corr_block(w, bstore, resc, rhs_cm, n, inv_h2, blockIdx);
 }
 
-// ---- correction grids in one block's shared memory ---------------------------
-// A sweep of a small grid is a chain of colour phases, each as long as one
-// point's dependent chain (loads, Hessian, the Newton steps of the root) and a
-// barrier; the points of a phase fill few warps.  So a phase runs on no more
-// warps than it has points for (a whole block's barrier, and idle warps at
-// it, cost more than the phase), a point's position comes from multiplications
-// by reciprocals in place of integer divisions, and its B and rhs, which no
-// phase writes, are loaded one phase ahead.
+// ---- correction grids in one block's shared memory (ma_small_grid.cuh) ---------
 
 __device__ __forceinline__ S3f corr_hess_sm(const float* e, int p, int sy, int sz, float e0, float inv_h2)
 {
@@ -1020,54 +1015,6 @@ __device__ __forceinline__ S3f corr_hess_sm(const float* e, int p, int sy, int s
         },
         inv_h2);
 }
-
-// Index arithmetic of a grid of n = 3, 5, 9 or 17 points a side.  t / d as
-// t (65536 / d + 1) >> 16: exact for t d <= 65536.
-struct SmallGrid {
-    int n, a, b, ma, mi, mn, lb;   // a, b = 2^lb: interior indices of parity 0, 1; m*: reciprocals of a, n - 2, n
-    __device__ __forceinline__ explicit SmallGrid(int n_) : n(n_), a((n_ - 3) / 2), b((n_ - 1) / 2)
-    {
-        lb = n == 3 ? 0 : (n == 5 ? 1 : (n == 9 ? 2 : 3));
-        ma = n == 17 ? 65536 / 7 + 1 : (n == 9 ? 65536 / 3 + 1 : 65537);
-        mi = n == 17 ? 65536 / 15 + 1 : (n == 9 ? 65536 / 7 + 1 : (n == 5 ? 65536 / 3 + 1 : 65537));
-        mn = n == 17 ? 65536 / 17 + 1 : (n == 9 ? 65536 / 9 + 1 : (n == 5 ? 65536 / 5 + 1 : 65536 / 3 + 1));
-    }
-    __device__ __forceinline__ int count(int c) const
-    {
-        return ((c & 1) ? b : a) * ((c & 2) ? b : a) * ((c & 4) ? b : a);
-    }
-    __device__ __forceinline__ int offset(int c) const   // cm_offset
-    {
-        const int sj = (c & 2) ? b : a, sk = (c & 4) ? b : a;
-        return ((c & 4) ? (a + b) * (a + b) * a : 0) + ((c & 2) ? (a + b) * a * sk : 0) + ((c & 1) ? a * sj * sk : 0);
-    }
-    // linear index of point t of colour c
-    __device__ __forceinline__ int point(int c, int t) const
-    {
-        const bool pi = c & 1, pj = c & 2, pk = c & 4;
-        const int y0 = pi ? t >> lb : (t * ma) >> 16, x = t - y0 * (pi ? b : a);
-        const int z = pj ? y0 >> lb : (y0 * ma) >> 16, y = y0 - z * (pj ? b : a);
-        return (((pk ? 1 : 2) + 2 * z) * n + (pj ? 1 : 2) + 2 * y) * n + (pi ? 1 : 2) + 2 * x;
-    }
-    // interior point q in natural order: (i, j, k), its linear index returned
-    __device__ __forceinline__ int interior(int q, int* i, int* j, int* k) const
-    {
-        const int y0 = (q * mi) >> 16, z = (y0 * mi) >> 16;
-        *i = 1 + q - y0 * (n - 2);
-        *j = 1 + y0 - z * (n - 2);
-        *k = 1 + z;
-        return (*k * n + *j) * n + *i;
-    }
-    // colour-major slot and colour count of interior point (i, j, k)
-    __device__ __forceinline__ int slot(int i, int j, int k, int* cnt, int* off) const
-    {
-        const int c = (i & 1) | ((j & 1) << 1) | ((k & 1) << 2);
-        const int ni = (i & 1) ? b : a, nj = (j & 1) ? b : a;
-        *cnt = count(c);
-        *off = offset(c);
-        return (((k - 1) >> 1) * nj + ((j - 1) >> 1)) * ni + ((i - 1) >> 1);
-    }
-};
 
 // B in shared memory is component-major over the grid's mi = (n - 2)^3 slots in
 // colour order: the six entries of a slot lie mi apart.
@@ -1089,51 +1036,6 @@ __device__ __forceinline__ void stage_b_sm(float* sb, const float* __restrict__ 
         float* d = sb + off + t;
         d[0] = B.xx; d[mi] = B.yy; d[2 * mi] = B.zz; d[3 * mi] = B.xy; d[4 * mi] = B.xz; d[5 * mi] = B.yz;
     }
-}
-
-// Warps that run a grid's colour phases, and their barrier: one warp up to
-// 5^3 (at most 9 points a phase), four up to 9^3 (at most 91), the block above.
-__device__ __forceinline__ int phase_threads(int n, int block) { return n <= 5 ? 32 : (n <= 9 ? 128 : block); }
-
-__device__ __forceinline__ void phase_barrier(int n)
-{
-    if (n <= 5) __syncwarp();
-    else if (n <= 9) asm volatile("bar.sync 1, 128;" ::: "memory");
-    else __syncthreads();
-}
-
-// Phase q of a sweep: in colour pairs (c, c ^ 7) for c = 0 .. 3, or in
-// ascending order in 7 phases: colours 3 and 4 differ in all three parities,
-// so they are independent and share one.
-__device__ __forceinline__ int phases_of(bool pairs) { return pairs ? 4 : 7; }
-__device__ __forceinline__ int phase_first(bool pairs, int q) { return pairs || q <= 3 ? q : q + 1; }
-__device__ __forceinline__ int phase_second(bool pairs, int q) { return pairs ? q ^ 7 : (q == 3 ? 4 : -1); }
-
-// Linear index and slot of a phase's point t, packed; -1 where it has none.
-__device__ __forceinline__ int phase_point(const SmallGrid& G, bool pairs, int q, int t)
-{
-    int c = phase_first(pairs, q);
-    const int d = phase_second(pairs, q), nc = G.count(c);
-    if (t >= nc) {
-        if (d < 0) return -1;
-        t -= nc;
-        c = d;
-        if (t >= G.count(d)) return -1;
-    }
-    return G.point(c, t) | (G.offset(c) + t) << 16;
-}
-
-// The points of grids up to 9^3, at most one a thread in each phase, worked
-// out once: entry [phase][thread].
-constexpr int kPhaseTab = 7 * 128;
-
-__device__ __forceinline__ void fill_phase_tab(int* tab, int n, bool pairs)
-{
-    if (n > 9 || n < 5) return;
-    const SmallGrid G(n);
-    const int lt = n <= 5 ? 5 : 7;   // log2 of the threads
-    for (int x = threadIdx.x; x < phases_of(pairs) << lt; x += blockDim.x)
-        tab[x] = phase_point(G, pairs, x >> lt, x & ((1 << lt) - 1));
 }
 
 // nsw sweeps over a grid in shared memory: body(p, B, r) updates one point.
@@ -1372,10 +1274,6 @@ __device__ __forceinline__ TailSmem tail_fields(const TailArgs& A, float* tsm, i
     const TailLevel& V = A.lev[l];
     return TailSmem{tsm + V.oe, tsm + V.ow, tsm + V.orr, tsm + V.ob, tsm + V.orhs};
 }
-
-// The phase tables of the 9^3 and 5^3 grids.
-constexpr int kTailTab = kPhaseTab + 7 * 32;
-__device__ __forceinline__ int* tail_tab(int* tab, int n) { return n == 9 ? tab : tab + kPhaseTab; }
 
 // Every level's B and phase table; residual shells 0 (restrictions only read
 // the interior, as in the separate path).

@@ -66,16 +66,15 @@ struct HessSf {
 // sums, so no 1/4 scalings are spent; callers use det(4 Hs) = 64 det(Hs) and
 // v = v0 + zeta4 / 8.  Neighbour loads go through the read-only path: no
 // launch writes a point and reads it as a neighbour.
-__device__ __forceinline__ HessS gather_hess(const double* __restrict__ u, long long p, long long sy,
-                                             long long sz, double v0)
+template <typename Idx, typename Ld>
+__device__ __forceinline__ HessS gather_hess_of(Ld ld, Idx sy, Idx sz, double v0)
 {
-    const double* q = u + p;
-    const double a = __ldg(q + 1) + __ldg(q - 1);
-    const double b = __ldg(q + sy) + __ldg(q - sy);
-    const double c = __ldg(q + sz) + __ldg(q - sz);
-    const double r4 = (__ldg(q + sy + 1) + __ldg(q - sy - 1)) - (__ldg(q + sy - 1) + __ldg(q - sy + 1));
-    const double s4 = (__ldg(q + sz + 1) + __ldg(q - sz - 1)) - (__ldg(q + sz - 1) + __ldg(q - sz + 1));
-    const double t4 = (__ldg(q + sz + sy) + __ldg(q - sz - sy)) - (__ldg(q + sy - sz) + __ldg(q - sy + sz));
+    const double a = ld(1) + ld(-1);
+    const double b = ld(sy) + ld(-sy);
+    const double c = ld(sz) + ld(-sz);
+    const double r4 = (ld(sy + 1) + ld(-sy - 1)) - (ld(sy - 1) + ld(1 - sy));
+    const double s4 = (ld(sz + 1) + ld(-sz - 1)) - (ld(sz - 1) + ld(1 - sz));
+    const double t4 = (ld(sz + sy) + ld(-sz - sy)) - (ld(sy - sz) + ld(sz - sy));
     HessS H;
     const double m8v = -8.0 * v0;
     H.A = fma(4.0, a, m8v);
@@ -85,6 +84,13 @@ __device__ __forceinline__ HessS gather_hess(const double* __restrict__ u, long 
     H.S = s4;
     H.T = t4;
     return H;
+}
+
+__device__ __forceinline__ HessS gather_hess(const double* __restrict__ u, long long p, long long sy,
+                                             long long sz, double v0)
+{
+    const double* q = u + p;
+    return gather_hess_of([q](long long o) { return __ldg(q + o); }, sy, sz, v0);
 }
 
 // det(Hs - z I) by cofactor expansion along the first row.

@@ -305,25 +305,19 @@ struct ResF2 {
     f2::F2 H[6];   // 4 h^2 D^2_h u: xx, yy, zz, xy, xz, yz
 };
 
-// H = 2^kexp 4 h^2 D^2_h u at interior point p, formed exactly in int64 and
-// held as two-float values; false (H unset) where the stencil's largest value
-// is zero, huge or tiny.  -20 <= kexp <= 40 keeps every scaled unit inside
-// FP32's range.
-template <typename Idx>
-__device__ __forceinline__ bool gather_f2(const double* __restrict__ u, Idx p, Idx sy, Idx sz, int kexp, f2::F2* H,
-                                          long long* centre)
+// H = 2^kexp 4 h^2 D^2_h u at a point, formed exactly in int64 and held as
+// two-float values; ld(o) gives the bits of the value at offset o from the
+// point, sy and sz are the offsets of a step in j and k.  false (H unset) where
+// the stencil's largest value is zero, huge or tiny.  -20 <= kexp <= 40 keeps
+// every scaled unit inside FP32's range.
+template <typename Idx, typename Ld>
+__device__ __forceinline__ bool gather_f2_of(Ld ld, Idx sy, Idx sz, int kexp, f2::F2* H, long long* centre)
 {
-    const long long* q = reinterpret_cast<const long long*>(u) + p;
-    const long long b0 = __ldg(q);
-    const long long bxp = __ldg(q + 1), bxm = __ldg(q - 1);
-    const long long byp = __ldg(q + sy), bym = __ldg(q - sy);
-    const long long bzp = __ldg(q + sz), bzm = __ldg(q - sz);
-    const long long rpp = __ldg(q + (sy + 1)), rmm = __ldg(q - (sy + 1)), rpm = __ldg(q + (sy - 1)),
-                    rmp = __ldg(q - (sy - 1));
-    const long long spp = __ldg(q + (sz + 1)), smm = __ldg(q - (sz + 1)), spm = __ldg(q + (sz - 1)),
-                    smp = __ldg(q - (sz - 1));
-    const long long tpp = __ldg(q + (sz + sy)), tmm = __ldg(q - (sz + sy)), tpm = __ldg(q + (sz - sy)),
-                    tmp = __ldg(q - (sz - sy));
+    const long long b0 = ld(0);
+    const long long bxp = ld(1), bxm = ld(-1), byp = ld(sy), bym = ld(-sy), bzp = ld(sz), bzm = ld(-sz);
+    const long long rpp = ld(sy + 1), rmm = ld(-sy - 1), rpm = ld(sy - 1), rmp = ld(1 - sy);
+    const long long spp = ld(sz + 1), smm = ld(-sz - 1), spm = ld(sz - 1), smp = ld(1 - sz);
+    const long long tpp = ld(sz + sy), tmm = ld(-sz - sy), tpm = ld(sz - sy), tmp = ld(sy - sz);
     *centre = b0;
     // one sign and one exponent: the top 12 bits of every pattern equal b0's
     const unsigned h0 = (unsigned)(b0 >> 32);
@@ -352,29 +346,40 @@ __device__ __forceinline__ bool gather_f2(const double* __restrict__ u, Idx p, I
         // to 2^-7 of the largest value, truncated by less than 2^-7 of its
         // ulp below (a sum in FP64 rounds by half of one); four of them fit
         // int64.
-        auto ex = [](long long b) { return (int)((b >> 52) & 0x7ff); };
-#define MA_F2_MM(v) E = max(E, ex(v))
+        auto mag = [](long long b) { return (unsigned)(b >> 32) & 0x7fffffffu; };
+        unsigned top = mag(b0);
+#define MA_F2_MM(v) top = max(top, mag(v))
         MA_F2_MM(bxp); MA_F2_MM(bxm); MA_F2_MM(byp); MA_F2_MM(bym); MA_F2_MM(bzp); MA_F2_MM(bzm);
         MA_F2_MM(rpp); MA_F2_MM(rmm); MA_F2_MM(rpm); MA_F2_MM(rmp);
         MA_F2_MM(spp); MA_F2_MM(smm); MA_F2_MM(spm); MA_F2_MM(smp);
         MA_F2_MM(tpp); MA_F2_MM(tmm); MA_F2_MM(tpm); MA_F2_MM(tmp);
 #undef MA_F2_MM
+        E = (int)(top >> 20);
         if (E < f2::kMinE || E > f2::kMaxE) return false;
-        auto sg = [E, ex](long long b) -> long long {
-            const int e = ex(b);
-            const long long m = (b & 0x000FFFFFFFFFFFFFll) | (e > 0 ? 0x0010000000000000ll : 0ll);
-            const long long v = (m << 7) >> min(E - e, 63);
-            return b < 0 ? -v : v;
+        // (zeros and denormals shift out with the rest: E exceeds 63 by far)
+        auto fix = [E](long long b) -> long long {
+            const long long m = (b & 0x000FFFFFFFFFFFFFll) | 0x0010000000000000ll;
+            return (m << 7) >> min(E - (int)((b >> 52) & 0x7ff), 63);
         };
-        const long long m0 = sg(b0);
-        A = (sg(bxp) - m0) + (sg(bxm) - m0);
-        B = (sg(byp) - m0) + (sg(bym) - m0);
-        C = (sg(bzp) - m0) + (sg(bzm) - m0);
-        R = (sg(rpp) - sg(rmp)) - (sg(rpm) - sg(rmm));
-        S = (sg(spp) - sg(smp)) - (sg(spm) - sg(smm));
-        T = (sg(tpp) - sg(tmp)) - (sg(tpm) - sg(tmm));
+        auto sums = [&](auto g) {
+            const long long m0 = g(b0);
+            A = (g(bxp) - m0) + (g(bxm) - m0);
+            B = (g(byp) - m0) + (g(bym) - m0);
+            C = (g(bzp) - m0) + (g(bzm) - m0);
+            R = (g(rpp) - g(rmp)) - (g(rpm) - g(rmm));
+            S = (g(spp) - g(smp)) - (g(spm) - g(smm));
+            T = (g(tpp) - g(tmp)) - (g(tpm) - g(tmm));
+        };
+        if (!__any_sync(__activemask(), (int)diff < 0)) {   // one sign each: the unit carries it
+            sums(fix);
+        } else {
+            sums([&](long long b) {
+                const long long v = fix(b), neg = b >> 63;
+                return (v ^ neg) - neg;
+            });
+            sign = 0;
+        }
         E -= 7;
-        sign = 0;
     }
     const float unit = __int_as_float(((E - 1075 + 127 + kexp) << 23) | sign);
     const float unit4 = 4.0f * unit;
@@ -401,6 +406,16 @@ __device__ __forceinline__ bool gather_f2(const double* __restrict__ u, Idx p, I
         H[5] = f2::from_i64(T, unit);
     }
     return true;
+}
+
+// The same at interior point p of a grid in global memory, through the
+// read-only path (no launch writes a point and reads it as a neighbour).
+template <typename Idx>
+__device__ __forceinline__ bool gather_f2(const double* __restrict__ u, Idx p, Idx sy, Idx sz, int kexp, f2::F2* H,
+                                          long long* centre)
+{
+    const long long* q = reinterpret_cast<const long long*>(u) + p;
+    return gather_f2_of<Idx>([q](Idx o) -> long long { return __ldg(q + o); }, sy, sz, kexp, H, centre);
 }
 
 template <bool UNORM = false>

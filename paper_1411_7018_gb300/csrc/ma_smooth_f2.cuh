@@ -39,35 +39,39 @@ struct Params {
     double h6;      // 64 h^6, the right-hand side's factor of the FP64 form
     double kz;      // 2^-k / 8: z to the change of u
     float chi, clo; // (2^k 4 h^2)^3 as two floats
-    int kexp;       // k
+    int kexp;       // k, or kNone: outside gather_f2's range, every point takes the FP64 form
 };
+constexpr int kNone = 1 << 20;
 
-// false: k would leave gather_f2's range, the grid keeps the FP64 form.
-inline bool make_params(double h, Params* P)
+
+inline Params make_params(double h)
 {
+    Params P{};
     const double h2 = h * h;
+    P.h6 = 64.0 * h2 * h2 * h2;
     int e = 0;
     const double m = frexp(4.0 * h2, &e);   // 4 h^2 = m 2^e, m in [1/2, 1)
-    P->kexp = m < 0.70710678118654752 ? 1 - e : -e;
-    if (P->kexp < -20 || P->kexp > 40) return false;
-    const double q = ldexp(4.0 * h2, P->kexp), c = q * q * q;
-    P->h6 = 64.0 * h2 * h2 * h2;
-    P->kz = ldexp(0.125, -P->kexp);
-    P->chi = (float)c;
-    P->clo = (float)(c - (double)P->chi);
-    return true;
+    P.kexp = m < 0.70710678118654752 ? 1 - e : -e;
+    if (P.kexp < -20 || P.kexp > 40) {
+        P.kexp = kNone;
+        return P;
+    }
+    const double q = ldexp(4.0 * h2, P.kexp), c = q * q * q;
+    P.kz = ldexp(0.125, -P.kexp);
+    P.chi = (float)c;
+    P.clo = (float)(c - (double)P.chi);
+    return P;
 }
 
-// The FP64 form, for the points the fast path leaves.
-static __device__ __noinline__ void point_f64(double* u, const double* __restrict__ rhs, long long p, long long sy,
-                                              long long sz, double h6, unsigned long long* events)
+// The new centre value by the FP64 form, for the points the fast path leaves;
+// q points at the centre.
+static __device__ __noinline__ double point_f64(const double* q, long long sy, long long sz, double rhs6,
+                                                bool* nonconvex)
 {
-    const double v0 = u[p];
-    const HessS H = gather_hess(u, p, sy, sz, v0);
-    bool nonconvex = false;
-    const double z = smallest_root(H, __dmul_rn(h6, rhs[p]), &nonconvex);
-    u[p] = fma(0.125, z, v0);
-    if (nonconvex && events) atomicAdd(events, 1ull);
+    auto at = [&](long long o) { return q[o]; };
+    const double v0 = at(0);
+    const HessS H = gather_hess_of(at, sy, sz, v0);
+    return fma(0.125, smallest_root(H, rhs6, nonconvex), v0);
 }
 
 // a - z as two floats, z one float
@@ -77,41 +81,69 @@ __device__ __forceinline__ resid::f2::F2 shift(resid::f2::F2 a, float z)
     return resid::f2::fast_two_sum(s.hi, s.lo + a.lo);
 }
 
-template <typename Idx>
-__device__ __forceinline__ void point(double* u, const double* __restrict__ rhs, Idx p, Idx sy, Idx sz,
-                                      const Params& P, unsigned long long* events)
+// The new centre value; ld as gather_f2_of takes it, b the right-hand side.
+// false: the point needs the FP64 form.  UNORM: det3's sums unnormalised, which
+// saves 15 operations and leaves the root's residual to about 2^-45 of the
+// entries' cube in place of 2^-46; that is below an ulp of u from 33^3 up.
+template <bool UNORM, typename Idx, typename Ld>
+__device__ __forceinline__ bool update(Ld ld, Idx sy, Idx sz, double b, const Params& P, double* v)
 {
     using namespace resid;
     f2::F2 H[6];
     long long b0;
-    const double b = __ldg(rhs + p);
     // rhs > 0 by its bits (NaN passes and fails to converge below)
-    if (gather_f2<Idx>(u, p, sy, sz, P.kexp, H, &b0) && __double_as_longlong(b) > 0) {
-        const f2::F2 r6 = f2::mul(f2::from_f64(b), f2::F2{P.chi, P.clo});
-        HessSf F;
-        F.A = H[0].hi; F.B = H[1].hi; F.C = H[2].hi;
-        F.R = H[3].hi; F.S = H[4].hi; F.T = H[5].hi;
-        const float scale = fabsf(F.A) + fabsf(F.B) + fabsf(F.C) + fabsf(F.R) + fabsf(F.S) + fabsf(F.T);
-        const float d0 = det_shift_f(F, 0.0f);
-        float z = is_pd<HessSf, float>(F, d0) ? 0.0f : gershgorin_low<HessSf, float>(F) - cbrtf(r6.hi);
-        bool conv = false;
-        for (int it = 0; it < 60; ++it) {
-            const float dz = __fdividef(det_shift_f(F, z) - r6.hi, minors_shift_f(F, z));
-            z += dz;
-            if (!isfinite(z)) break;
-            if (fabsf(dz) <= 2e-6f * scale) { conv = true; break; }
-        }
-        const float m = minors_shift_f(F, z);
-        // the scale's window keeps the cube's low parts inside FP32's range
-        if (conv && m > 0.05f * scale * scale && r6.hi > 0.0f && scale > 9.5e-7f && scale < 1.0e9f) {
-            const f2::F2 d = f2::det3<true>(shift(H[0], z), shift(H[1], z), shift(H[2], z), H[3], H[4], H[5]);
-            const f2::F2 g = f2::add_u(d, f2::neg(r6));
-            const float dz = __fdividef(g.hi + g.lo, m);
-            u[p] = fma(P.kz, f2d(z) + f2d(dz), __longlong_as_double(b0));
-            return;
-        }
+    if (!gather_f2_of<Idx>(ld, sy, sz, P.kexp, H, &b0) || __double_as_longlong(b) <= 0) return false;
+    const f2::F2 r6 = f2::mul(f2::from_f64(b), f2::F2{P.chi, P.clo});
+    HessSf F;
+    F.A = H[0].hi; F.B = H[1].hi; F.C = H[2].hi;
+    F.R = H[3].hi; F.S = H[4].hi; F.T = H[5].hi;
+    const float scale = fabsf(F.A) + fabsf(F.B) + fabsf(F.C) + fabsf(F.R) + fabsf(F.S) + fabsf(F.T);
+    // FP32 Newton on c - M z + T z^2 - z^3 = det(F - z I) - r6: from 0 when F is
+    // positive definite, else from left of the root
+    const float d0 = det_shift_f(F, 0.0f), c = d0 - r6.hi, T = F.A + F.B + F.C, M = minors_shift_f(F, 0.0f);
+    float z = is_pd<HessSf, float>(F, d0) ? 0.0f : gershgorin_low<HessSf, float>(F) - cbrtf(r6.hi);
+    bool conv = false;
+    for (int it = 0; it < 60; ++it) {
+        const float dz = __fdividef(fmaf(-z, fmaf(-z, T - z, M), c), fmaf(-z, fmaf(-3.0f, z, 2.0f * T), M));
+        z += dz;
+        if (!isfinite(z)) break;
+        if (fabsf(dz) <= 2e-6f * scale) { conv = true; break; }
     }
-    point_f64(u, rhs, p, sy, sz, P.h6, events);
+    const float m = fmaf(-z, fmaf(-3.0f, z, 2.0f * T), M);
+    // the scale's window keeps the cube's low parts inside FP32's range
+    if (!(conv && m > 0.05f * scale * scale && r6.hi > 0.0f && scale > 9.5e-7f && scale < 1.0e9f)) return false;
+    const f2::F2 d = f2::det3<UNORM>(shift(H[0], z), shift(H[1], z), shift(H[2], z), H[3], H[4], H[5]);
+    const f2::F2 g = UNORM ? f2::add_u(d, f2::neg(r6)) : f2::add(d, f2::neg(r6));
+    const float dz = __fdividef(g.hi + g.lo, m);
+    *v = fma(P.kz, f2d(z) + f2d(dz), __longlong_as_double(b0));
+    return true;
+}
+
+// A point of a grid in global memory, in place.
+template <bool UNORM, typename Idx>
+__device__ __forceinline__ void point(double* u, const double* __restrict__ rhs, Idx p, Idx sy, Idx sz,
+                                      const Params& P, unsigned long long* events)
+{
+    const long long* q = reinterpret_cast<const long long*>(u) + p;
+    const double b = __ldg(rhs + p);
+    double v;
+    if (update<UNORM, Idx>([q](Idx o) -> long long { return __ldg(q + o); }, sy, sz, b, P, &v)) {
+        u[p] = v;   // (one store after both forms: 10 % slower at 257^3)
+        return;
+    }
+    bool nonconvex = false;
+    u[p] = point_f64(u + p, sy, sz, __dmul_rn(P.h6, b), &nonconvex);
+    if (nonconvex && events) atomicAdd(events, 1ull);
+}
+
+// A point of a grid in shared memory: its new value.
+__device__ __forceinline__ double point_sm(const double* q, int sy, int sz, double b, const Params& P, bool* nonconvex)
+{
+    double v;
+    if (P.kexp != kNone &&
+        update<false, int>([q](int o) -> long long { return __double_as_longlong(q[o]); }, sy, sz, b, P, &v))
+        return v;
+    return point_f64(q, sy, sz, __dmul_rn(P.h6, b), nonconvex);
 }
 
 }  // namespace smoothf2

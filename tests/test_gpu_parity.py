@@ -527,3 +527,30 @@ def test_two_float_residual_and_coarse_rhs_match_oracle(name, n):
     shell = np.ones_like(gb, bool)
     shell[1:-1, 1:-1, 1:-1] = False
     assert np.all(got[shell] == 0.0) and np.all(gb[shell] == 0.0)
+
+
+@pytest.mark.parametrize("start", ["near", "zero", "nonpositive"])
+@pytest.mark.parametrize("name,length", [("exp", 1.0), ("sine", np.pi), ("cosine", 1.0), ("exp", 1e-3), ("exp", 1e-7)])
+def test_coarsest_5_converges_to_the_swept_solution(name, length, start):
+    """The 5^3 coarsest solve (Newton's method, checked by a sweep) against the
+    oracle's sweeps to 1e-14: from near the solution, from a zero interior (far
+    from convex: sweeps first) and with right-hand sides <= 0 (sweeps only).  The
+    sweeps contract by about 0.6, so stopping at a change of 1e-14 leaves up to
+    2.5e-14 of max|u| on either side; 1e-12 is the bound the other coarsest
+    solves are held to."""
+    n = 5
+    pr = P.make(name, n)
+    scale = (length / (np.pi if name == "sine" else 1.0)) ** 2
+    h = length / (n - 1)
+    u0, f = scale * (pr.initial() if start == "zero" else perturbed(name, n, 1e-3)[1]), pr.f.copy()
+    if start == "nonpositive":
+        f[2, 2, 2] = -0.1 * f[2, 2, 2]
+    ref = u0.copy()
+    for _ in range(100):
+        prev = ref.copy()
+        O.gs_sweep(ref, f, h)
+        if np.max(np.abs(ref - prev)) <= 1e-14 * np.max(np.abs(ref)):
+            break
+    u = dev(u0)
+    M.ma_coarsest_solve(u, dev(f), n, h, 0)
+    assert np.max(np.abs(host(u) - ref)) <= 1e-12 * np.max(np.abs(ref))
