@@ -222,13 +222,13 @@ __global__ void __launch_bounds__(BX * BY) k_coarse_rhs(const double* __restrict
 // r + det(D^2_h u) (SIGN = 1, the coarse right-hand side) or r - det (SIGN = -1,
 // the residual) at a point, with exact integer second differences and a
 // two-float determinant; ld as gather_f2_of takes it.
-template <int SIGN, bool UNORM, typename Idx, typename Ld>
+template <int SIGN, bool UNORM, bool SMALL, typename Idx, typename Ld>
 __device__ __forceinline__ double operator_of(Ld ld, Idx sy, Idx sz, double rv, double inv_h6)
 {
     using namespace resid;
     f2::F2 H[6];
     long long b0;
-    if (gather_f2_of<Idx>(ld, sy, sz, 0, H, &b0)) {
+    if (gather_f2_of<SMALL, Idx>(ld, sy, sz, 0, H, &b0)) {
         const float ih = (float)(SIGN * inv_h6);
         const f2::F2 d = f2::mul(f2::det3<UNORM>(H[0], H[1], H[2], H[3], H[4], H[5]),
                                  f2::F2{ih, (float)(SIGN * inv_h6 - (double)ih)});
@@ -243,7 +243,7 @@ __device__ __forceinline__ double operator_of(Ld ld, Idx sy, Idx sz, double rv, 
 template <int SIGN, bool UNORM>
 __device__ __forceinline__ double operator_point(const double* q, int sy, int sz, double rv, double inv_h6)
 {
-    return operator_of<SIGN, UNORM, int>([q](int o) -> long long { return __double_as_longlong(q[o]); }, sy, sz, rv,
+    return operator_of<SIGN, UNORM, true, int>([q](int o) -> long long { return __double_as_longlong(q[o]); }, sy, sz, rv,
                                          inv_h6);
 }
 
@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(BX * BY) k_operator_f2(const double* __restric
         return;
     }
     const long long* q = reinterpret_cast<const long long*>(u) + p;
-    out[p] = operator_of<SIGN, UNORM, long long>([q](long long o) -> long long { return __ldg(q + o); }, n, sz,
+    out[p] = operator_of<SIGN, UNORM, !UNORM, long long>([q](long long o) -> long long { return __ldg(q + o); }, n, sz,
                                                  __ldg(r + p), inv_h6);
 }
 
@@ -362,11 +362,12 @@ __device__ __forceinline__ void run_sweeps64(const SmallGrid& G, const Grid64& S
 // iterate: the sweeps converge by a factor of 0.6, 40 - 70 of them to 1e-14,
 // each 7 phases long.  Lane = interior point.  The residuals and their FP32
 // Jacobian come from the two-float Hessian; the Jacobian is inverted in place
-// (Gauss-Jordan) and kept while an iteration cuts the residual tenfold.  Only
+// (Gauss-Jordan) and kept while an iteration cuts the residual fourfold.  Only
 // an iterate whose points are all positive definite, with positive right-hand
-// sides, is touched, and if the residual does not fall it is put back and
-// false returned; the caller's sweeps then decide as they would have.
-// J: 27 x kJ floats.
+// sides, is touched, and if the residual does not fall it is put back.  True
+// when the changes that a sweep would make (each point's residual over its
+// derivative) are at most 1e-14 max |u|, the sweeps' own rule; otherwise the
+// caller's sweeps decide as they would have.  J: 27 x kJ floats.
 constexpr int kJ = 29;   // an odd stride: a lane's row and a column of it meet no bank conflicts
 
 __device__ __forceinline__ bool newton5(double* u, const double* rhs, const smoothf2::Params& P, float* J)
@@ -384,10 +385,10 @@ __device__ __forceinline__ bool newton5(double* u, const double* rhs, const smoo
     for (int it = 0; it < 24; ++it) {
         f2::F2 H[6];
         long long b0;
-        bool ok = gather_f2_of<int>([&](int o) -> long long { return __double_as_longlong(u[p + o]); }, 5, 25, P.kexp,
+        bool ok = gather_f2_of<true, int>([&](int o) -> long long { return __double_as_longlong(u[p + o]); }, 5, 25, P.kexp,
                                     H, &b0) &&
                   __double_as_longlong(b) > 0;
-        float g = 0.0f;
+        float g = 0.0f, m = 0.0f;
         if (ok) {
             const f2::F2 d = f2::det3(H[0], H[1], H[2], H[3], H[4], H[5]);
             const f2::F2 e = f2::add(d, f2::neg(r6));
@@ -396,24 +397,25 @@ __device__ __forceinline__ bool newton5(double* u, const double* rhs, const smoo
             F.A = H[0].hi; F.B = H[1].hi; F.C = H[2].hi;
             F.R = H[3].hi; F.S = H[4].hi; F.T = H[5].hi;
             const float scale = fabsf(F.A) + fabsf(F.B) + fabsf(F.C) + fabsf(F.R) + fabsf(F.S) + fabsf(F.T);
-            ok = is_pd<HessSf, float>(F, d.hi) && minors_shift_f(F, 0.0f) > 0.05f * scale * scale &&
-                 scale > 9.5e-7f && scale < 1.0e9f && isfinite(g);
+            m = minors_shift_f(F, 0.0f);
+            ok = is_pd<HessSf, float>(F, d.hi) && m > 0.05f * scale * scale && scale > 9.5e-7f &&
+                 scale < 1.0e9f && isfinite(g);
         }
         float worst = fabsf(g);
         for (int o = 16; o > 0; o >>= 1) worst = fmaxf(worst, __shfl_xor_sync(FULL, worst, o));
         if (__any_sync(FULL, on && !ok) || (moved && !(worst < last))) {
-            // not a point Newton can be trusted from; or round-off: the residual no longer falls
-            const bool settled = moved && worst <= 1e-11f * fabsf(r6.hi);
-            if (moved && !__all_sync(FULL, !on || settled)) {
+            // not a point Newton can be trusted from, or the residual no longer falls: round-off, or put it back
+            if (moved && !__all_sync(FULL, !on || worst <= 1e-11f * fabsf(r6.hi))) {
                 __syncwarp();
                 if (on) u[p] = start;
                 __syncwarp();
                 return false;
             }
-            return moved;
+            double big = on ? fabs(__longlong_as_double(b0)) : 0.0;
+            for (int o = 16; o > 0; o >>= 1) big = fmax(big, __shfl_xor_sync(FULL, big, o));
+            return moved && __all_sync(FULL, !on || fabsf(g) * (float)P.kz <= 1e-14f * (float)big * m);
         }
-        if (worst == 0.0f) return true;
-        if (!moved || worst > 0.1f * last) {
+        if (!moved || worst > 0.25f * last) {
             // row of the Jacobian: the cofactors times the stencil's weights, 2^k taken out
             const float A = H[0].hi, B = H[1].hi, C = H[2].hi, R = H[3].hi, S = H[4].hi, T = H[5].hi;
             const float cA = B * C - T * T, cB = A * C - S * S, cC = A * B - R * R;
@@ -458,12 +460,12 @@ __device__ __forceinline__ bool newton5(double* u, const double* rhs, const smoo
         last = worst;
         moved = true;
     }
-    return true;
+    return false;
 }
 
 // The coarsest grid in shared memory: sweeps until max |du| <= 1e-14 max |u| (at
 // most 100), or a fixed count; on 5^3 Newton's method first, again after every
-// eighth sweep where it could not start.  On 3^3 the one unknown's root with a
+// eighth sweep where it did not finish.  On 3^3 the one unknown's root with a
 // Newton step in FP64 (smallest_root_precise).  Every thread of the block
 // enters; ends with a block barrier.  J: 27 kJ floats.
 __device__ __forceinline__ void coarsest64_sm(const Grid64& S, int n, int sweeps, float* J, unsigned long long* ev)
@@ -487,9 +489,8 @@ __device__ __forceinline__ void coarsest64_sm(const Grid64& S, int n, int sweeps
         }
     } else if ((int)threadIdx.x < nt) {
         const SmallGrid G(n);
-        bool solved = false;
         for (int s = 0; s < max_sweeps; ++s) {
-            if (n == 5 && sweeps == 0 && !solved && (s & 7) == 0) solved = newton5(S.u, S.rhs, S.P, J);
+            if (n == 5 && sweeps == 0 && (s & 7) == 0 && newton5(S.u, S.rhs, S.P, J)) break;
             double du = 0.0, um = 0.0;
             run_sweeps64(G, S, 1, nt, ev, [&](double v0, double v) {
                 du = fmax(du, fabs(v - v0));
@@ -603,15 +604,16 @@ __device__ __forceinline__ void tail64_smooth(const Grid64& S, int n, int nsw, u
     __syncthreads();
 }
 
-__device__ __forceinline__ double tail64_line(const double* uc, const double* wc, int nc, int Ic, int J0, int K0,
-                                              int oj, int ok, double w)
+// d: the coarse values u_H - w_H
+__device__ __forceinline__ double tail64_line(const double* d, int nc, int Ic, int J0, int K0, int oj, int ok, double w)
 {
-    double s = 0.0;
-    for (int dk = 0; dk <= ok; ++dk)
-        for (int dj = 0; dj <= oj; ++dj) {
-            const int q = ((K0 + dk) * nc + (J0 + dj)) * nc + Ic;
-            s += uc[q] - wc[q];
-        }
+    const double* q = d + (K0 * nc + J0) * nc + Ic;
+    double s = 0.0 + q[0];
+    if (oj) s += q[nc];
+    if (ok) {
+        s += q[nc * nc];
+        if (oj) s += q[nc * nc + nc];
+    }
     return s * w;
 }
 
@@ -691,6 +693,8 @@ __device__ __forceinline__ void vcycle_tail_body(const Tail64Args& A)
         const int nf = A.lev[l].n, nc = A.lev[l + 1].n;
         const SmallGrid GF(nf);
         // (7)-(8) u_h += I(u_H - w_H) on the fine interior, each value formed as xfer::k_prolong forms it
+        for (int q = threadIdx.x; q < nc * nc * nc; q += T64) C.w[q] = C.u[q] - C.w[q];
+        __syncthreads();
         for (int q = threadIdx.x; q < (nf - 2) * (nf - 2) * (nf - 2); q += T64) {
             int i, j, k;
             const int p = GF.interior(q, &i, &j, &k);
@@ -699,11 +703,11 @@ __device__ __forceinline__ void vcycle_tail_body(const Tail64Args& A)
             double v;
             if (i & 1) {
                 const int I = i >> 1;
-                const double a = tail64_line(C.u, C.w, nc, I, J0, K0, oj, ok, w);
-                const double b = tail64_line(C.u, C.w, nc, I + 1, J0, K0, oj, ok, w);
+                const double a = tail64_line(C.w, nc, I, J0, K0, oj, ok, w);
+                const double b = tail64_line(C.w, nc, I + 1, J0, K0, oj, ok, w);
                 v = (a + b) * 0.5;
             } else {
-                v = tail64_line(C.u, C.w, nc, i >> 1, J0, K0, oj, ok, w);
+                v = tail64_line(C.w, nc, i >> 1, J0, K0, oj, ok, w);
             }
             F.u[p] = F.u[p] + v;
         }

@@ -310,7 +310,9 @@ struct ResF2 {
 // point, sy and sz are the offsets of a step in j and k.  false (H unset) where
 // the stencil's largest value is zero, huge or tiny.  -20 <= kexp <= 40 keeps
 // every scaled unit inside FP32's range.
-template <typename Idx, typename Ld>
+// SMALL: for the smaller grids, where most warps meet a change of binade: the
+// general form at once.
+template <bool SMALL = false, typename Idx, typename Ld>
 __device__ __forceinline__ bool gather_f2_of(Ld ld, Idx sy, Idx sz, int kexp, f2::F2* H, long long* centre)
 {
     const long long b0 = ld(0);
@@ -332,7 +334,7 @@ __device__ __forceinline__ bool gather_f2_of(Ld ld, Idx sy, Idx sz, int kexp, f2
     int sign = (int)(h0 & 0x80000000u);   // the ulp of the binade, negated for negative values
     // a quarter of the diagonal entries, and the off-diagonal ones, in ulps
     long long A, B, C, R, S, T;
-    if ((diff >> 20) == 0) {
+    if (!SMALL && (diff >> 20) == 0) {
         if (E < f2::kMinE || E > f2::kMaxE) return false;
         A = (bxp - b0) + (bxm - b0);
         B = (byp - b0) + (bym - b0);
@@ -347,13 +349,12 @@ __device__ __forceinline__ bool gather_f2_of(Ld ld, Idx sy, Idx sz, int kexp, f2
         // ulp below (a sum in FP64 rounds by half of one); four of them fit
         // int64.
         auto mag = [](long long b) { return (unsigned)(b >> 32) & 0x7fffffffu; };
-        unsigned top = mag(b0);
-#define MA_F2_MM(v) top = max(top, mag(v))
-        MA_F2_MM(bxp); MA_F2_MM(bxm); MA_F2_MM(byp); MA_F2_MM(bym); MA_F2_MM(bzp); MA_F2_MM(bzm);
-        MA_F2_MM(rpp); MA_F2_MM(rmm); MA_F2_MM(rpm); MA_F2_MM(rmp);
-        MA_F2_MM(spp); MA_F2_MM(smm); MA_F2_MM(spm); MA_F2_MM(smp);
-        MA_F2_MM(tpp); MA_F2_MM(tmm); MA_F2_MM(tpm); MA_F2_MM(tmp);
-#undef MA_F2_MM
+        auto max4 = [&](long long a, long long b, long long c, long long d) {
+            return max(max(mag(a), mag(b)), max(mag(c), mag(d)));
+        };
+        const unsigned top = max(max(max(max4(bxp, bxm, byp, bym), max4(bzp, bzm, b0, b0)),
+                                     max(max4(rpp, rmm, rpm, rmp), max4(spp, smm, spm, smp))),
+                                 max4(tpp, tmm, tpm, tmp));
         E = (int)(top >> 20);
         if (E < f2::kMinE || E > f2::kMaxE) return false;
         // (zeros and denormals shift out with the rest: E exceeds 63 by far)
@@ -389,7 +390,7 @@ __device__ __forceinline__ bool gather_f2_of(Ld ld, Idx sy, Idx sz, int kexp, f2
 #define MA_F2_HW(x) big |= (int)((x) >> 32) ^ (int)((x) >> 63)
     MA_F2_HW(A); MA_F2_HW(B); MA_F2_HW(C); MA_F2_HW(R); MA_F2_HW(S); MA_F2_HW(T);
 #undef MA_F2_HW
-    if (big < (1 << 13)) {
+    if (!SMALL && big < (1 << 13)) {
         const float u23 = 8388608.0f * unit, u423 = 8388608.0f * unit4;
         H[0] = f2::from_i45(A, unit4, u423);
         H[1] = f2::from_i45(B, unit4, u423);
@@ -415,7 +416,7 @@ __device__ __forceinline__ bool gather_f2(const double* __restrict__ u, Idx p, I
                                           long long* centre)
 {
     const long long* q = reinterpret_cast<const long long*>(u) + p;
-    return gather_f2_of<Idx>([q](Idx o) -> long long { return __ldg(q + o); }, sy, sz, kexp, H, centre);
+    return gather_f2_of<false, Idx>([q](Idx o) -> long long { return __ldg(q + o); }, sy, sz, kexp, H, centre);
 }
 
 template <bool UNORM = false>

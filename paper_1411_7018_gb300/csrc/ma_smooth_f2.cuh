@@ -19,8 +19,9 @@
 // whatever the step; the local equation det(H - z I) = (2^k 4 h^2)^3 rhs has the
 // root of Eq. (realroots) at v = v0 + z / (8 2^k).
 //
-// The root is found as smallest_root finds it: Newton in FP32 on the rounded
-// entries, then one Newton correction whose residual is evaluated to about 2^-45
+// The root is found as smallest_root finds it: in FP32 on the rounded entries
+// (by the iteration of corr_root_fast where it is small, else by Newton from 0,
+// or from left of it where the matrix is not positive definite), then one Newton correction whose residual is evaluated to about 2^-45
 // of the entries' cube (in FP64 there), with the FP32 derivative.  The second
 // differences it starts from are exact, where the FP64 gather rounds the
 // neighbour sums to 2^-53 |u|, so from 17^3 up the result lies closer to the
@@ -85,29 +86,36 @@ __device__ __forceinline__ resid::f2::F2 shift(resid::f2::F2 a, float z)
 // false: the point needs the FP64 form.  UNORM: det3's sums unnormalised, which
 // saves 15 operations and leaves the root's residual to about 2^-45 of the
 // entries' cube in place of 2^-46; that is below an ulp of u from 33^3 up.
-template <bool UNORM, typename Idx, typename Ld>
+template <bool UNORM, bool SMALL, typename Idx, typename Ld>
 __device__ __forceinline__ bool update(Ld ld, Idx sy, Idx sz, double b, const Params& P, double* v)
 {
     using namespace resid;
     f2::F2 H[6];
     long long b0;
     // rhs > 0 by its bits (NaN passes and fails to converge below)
-    if (!gather_f2_of<Idx>(ld, sy, sz, P.kexp, H, &b0) || __double_as_longlong(b) <= 0) return false;
+    if (!gather_f2_of<SMALL, Idx>(ld, sy, sz, P.kexp, H, &b0) || __double_as_longlong(b) <= 0) return false;
     const f2::F2 r6 = f2::mul(f2::from_f64(b), f2::F2{P.chi, P.clo});
     HessSf F;
     F.A = H[0].hi; F.B = H[1].hi; F.C = H[2].hi;
     F.R = H[3].hi; F.S = H[4].hi; F.T = H[5].hi;
     const float scale = fabsf(F.A) + fabsf(F.B) + fabsf(F.C) + fabsf(F.R) + fabsf(F.S) + fabsf(F.T);
-    // FP32 Newton on c - M z + T z^2 - z^3 = det(F - z I) - r6: from 0 when F is
-    // positive definite, else from left of the root
+    // the FP32 root of c - M z + T z^2 - z^3 = det(F - z I) - r6
     const float d0 = det_shift_f(F, 0.0f), c = d0 - r6.hi, T = F.A + F.B + F.C, M = minors_shift_f(F, 0.0f);
-    float z = is_pd<HessSf, float>(F, d0) ? 0.0f : gershgorin_low<HessSf, float>(F) - cbrtf(r6.hi);
-    bool conv = false;
-    for (int it = 0; it < 60; ++it) {
-        const float dz = __fdividef(fmaf(-z, fmaf(-z, T - z, M), c), fmaf(-z, fmaf(-3.0f, z, 2.0f * T), M));
-        z += dz;
-        if (!isfinite(z)) break;
-        if (fabsf(dz) <= 2e-6f * scale) { conv = true; break; }
+    const bool pd = is_pd<HessSf, float>(F, d0);
+    const float tol = 2e-6f * scale;
+    // a root that is small against the entries: two steps of z <- (c + z^2 (T - z)) / M, one reciprocal
+    const float iM = __fdividef(1.0f, M), z0 = __fmul_rn(c, iM);
+    const float z1 = __fmul_rn(fmaf(__fmul_rn(z0, z0), T - z0, c), iM);
+    float z = __fmul_rn(fmaf(__fmul_rn(z1, z1), T - z1, c), iM);
+    bool conv = pd && M > 0.05f * scale * scale && fabsf(T * z0) <= 0.05f * M && fabsf(z - z1) <= tol;
+    if (!conv) {
+        z = pd ? 0.0f : gershgorin_low<HessSf, float>(F) - cbrtf(r6.hi);
+        for (int it = 0; it < 60; ++it) {
+            const float dz = __fdividef(fmaf(-z, fmaf(-z, T - z, M), c), fmaf(-z, fmaf(-3.0f, z, 2.0f * T), M));
+            z += dz;
+            if (!isfinite(z)) break;
+            if (fabsf(dz) <= tol) { conv = true; break; }
+        }
     }
     const float m = fmaf(-z, fmaf(-3.0f, z, 2.0f * T), M);
     // the scale's window keeps the cube's low parts inside FP32's range
@@ -127,7 +135,7 @@ __device__ __forceinline__ void point(double* u, const double* __restrict__ rhs,
     const long long* q = reinterpret_cast<const long long*>(u) + p;
     const double b = __ldg(rhs + p);
     double v;
-    if (update<UNORM, Idx>([q](Idx o) -> long long { return __ldg(q + o); }, sy, sz, b, P, &v)) {
+    if (update<UNORM, !UNORM, Idx>([q](Idx o) -> long long { return __ldg(q + o); }, sy, sz, b, P, &v)) {
         u[p] = v;   // (one store after both forms: 10 % slower at 257^3)
         return;
     }
@@ -141,7 +149,7 @@ __device__ __forceinline__ double point_sm(const double* q, int sy, int sz, doub
 {
     double v;
     if (P.kexp != kNone &&
-        update<false, int>([q](int o) -> long long { return __double_as_longlong(q[o]); }, sy, sz, b, P, &v))
+        update<false, true, int>([q](int o) -> long long { return __double_as_longlong(q[o]); }, sy, sz, b, P, &v))
         return v;
     return point_f64(q, sy, sz, __dmul_rn(P.h6, b), nonconvex);
 }
