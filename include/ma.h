@@ -313,17 +313,27 @@ ma_status ma_probe_phase_chain(float *a_dev, float *b_dev, size_t n, int phases,
 ma_status ma_smooth(double *u_dev, const double *rhs_dev, int n, double h, int nsweeps,
                     unsigned long long *events_dev, ma_stream_t stream);
 
+/* The same sweeps as the cycles of a hierarchy run them: from 5^3 up the
+ * second differences are exact integer differences of the values' bit
+ * patterns and the determinant is taken in two-float (hi + lo FP32)
+ * arithmetic, two FP64 operations a point.  Agrees with ma_smooth to the
+ * rounding of its FP64 sums (a few 2^-53 |u|) and lies closer to the exact
+ * update; the smallest-root rule and the events are the same. */
+ma_status ma_smooth_f2(double *u_dev, const double *rhs_dev, int n, double h, int nsweeps,
+                       unsigned long long *events_dev, ma_stream_t stream);
+
 /* r = rhs - det(D^2_h u) on the interior and 0 on the shell (Algorithm 1
  * step 3, the operator of Eq. MA_discrete). */
 ma_status ma_residual(const double *u_dev, const double *rhs_dev, double *r_dev, int n, double h,
                       ma_stream_t stream);
 
 /* The same residual (Algorithm 1 step 3, Eq. MA_discrete) as the fine-grid
- * residual of MA_MIXED solves computes it, without FP64 arithmetic: where the
- * 19 stencil values of a point share one sign and one binade, the second
- * differences are exact integer differences of their bit patterns, and the
- * determinant and rhs - det are taken in two-float (hi + lo FP32)
- * arithmetic, about 48 significant bits; elsewhere the FP64 evaluation of
+ * residual of MA_MIXED solves computes it, without FP64 arithmetic: the second
+ * differences are integer differences, of the 19 stencil values' bit patterns
+ * where they share one sign and one binade (exact), of fixed-point values with 7
+ * bits to spare otherwise, and the determinant and rhs - det are taken in
+ * two-float (hi + lo FP32) arithmetic, about 48 significant bits; a stencil
+ * whose largest value is zero, huge or tiny takes the FP64 evaluation of
  * ma_residual.  Same layout and arguments as ma_residual; asynchronous. */
 ma_status ma_residual_f2(const double *u_dev, const double *rhs_dev, double *r_dev, int n, double h,
                          ma_stream_t stream);

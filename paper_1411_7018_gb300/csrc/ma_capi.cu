@@ -1393,6 +1393,15 @@ ma_status ma_smooth(double* u, const double* rhs, int n, double h, int nsweeps, 
 {
     if (!u || !rhs || !valid_step_grid(n) || !(h > 0.0) || nsweeps < 0)
         return fail(MA_ERR_INVALID_ARG, "ma_smooth: bad arguments");
+    MA_CK(ma::launch_smooth_f64(u, rhs, n, h, nsweeps, events, (cudaStream_t)stream));
+    return MA_OK;
+}
+
+ma_status ma_smooth_f2(double* u, const double* rhs, int n, double h, int nsweeps, unsigned long long* events,
+                       ma_stream_t stream)
+{
+    if (!u || !rhs || !valid_step_grid(n) || !(h > 0.0) || nsweeps < 0)
+        return fail(MA_ERR_INVALID_ARG, "ma_smooth_f2: bad arguments");
     MA_CK(ma::launch_smooth(u, rhs, n, h, nsweeps, events, (cudaStream_t)stream));
     return MA_OK;
 }
@@ -1400,7 +1409,7 @@ ma_status ma_smooth(double* u, const double* rhs, int n, double h, int nsweeps, 
 ma_status ma_residual(const double* u, const double* rhs, double* r, int n, double h, ma_stream_t stream)
 {
     if (!u || !rhs || !r || !valid_step_grid(n) || !(h > 0.0)) return fail(MA_ERR_INVALID_ARG, "ma_residual: bad arguments");
-    MA_CK(ma::launch_residual(u, rhs, r, n, h, nullptr, (cudaStream_t)stream));
+    MA_CK(ma::launch_residual_f64(u, rhs, r, n, h, nullptr, (cudaStream_t)stream));
     return MA_OK;
 }
 

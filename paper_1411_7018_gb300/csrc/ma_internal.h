@@ -23,6 +23,12 @@ unsigned long long launch_count();
 void set_last_error(const char* msg);
 
 // FP64 kernels (ma_kernels_f64.cu).  All grids are n^3 doubles, [k][j][i].
+// launch_smooth and launch_residual, which the cycles run, take the two-float
+// forms from 5^3 up; the _f64 ones are FP64 throughout.
+cudaError_t launch_smooth_f64(double* u, const double* rhs, int n, double h, int nsweeps,
+                              unsigned long long* events, cudaStream_t s);
+cudaError_t launch_residual_f64(const double* u, const double* rhs, double* r, int n, double h,
+                                double* partials, cudaStream_t s);
 cudaError_t launch_smooth(double* u, const double* rhs, int n, double h, int nsweeps,
                           unsigned long long* events, cudaStream_t s);
 cudaError_t launch_residual(const double* u, const double* rhs, double* r, int n, double h,

@@ -362,9 +362,12 @@ __device__ __forceinline__ void run_sweeps64(const SmallGrid& G, const Grid64& S
 // iterate: the sweeps converge by a factor of 0.6, 40 - 70 of them to 1e-14,
 // each 7 phases long.  Lane = interior point.  The residuals and their FP32
 // Jacobian come from the two-float Hessian; the Jacobian is inverted in place
-// (Gauss-Jordan) and kept while an iteration cuts the residual fourfold.  Only
-// an iterate whose points are all positive definite, with positive right-hand
-// sides, is touched, and if the residual does not fall it is put back.  True
+// (Gauss-Jordan) and kept while an iteration cuts the residual fourfold.  It
+// starts from an iterate whose points are all positive definite, with positive
+// right-hand sides; where they are not positive definite (FMG's zero interior)
+// from the solution of the Poisson equation with right-hand side
+// 3 rhs^(1/3), which a convex solution exceeds and mostly lies near.  If the
+// residual does not fall the iterate is put back.  True
 // when the changes that a sweep would make (each point's residual over its
 // derivative) are at most 1e-14 max |u|, the sweeps' own rule; otherwise the
 // caller's sweeps decide as they would have.  J: 27 x kJ floats.
@@ -381,13 +384,13 @@ __device__ __forceinline__ bool newton5(double* u, const double* rhs, const smoo
     const double b = rhs[p], start = u[p];
     const f2::F2 r6 = f2::mul(f2::from_f64(b), f2::F2{P.chi, P.clo});
     float last = 0.0f;
-    bool moved = false;
+    bool moved = false, laplace = false;
     for (int it = 0; it < 24; ++it) {
         f2::F2 H[6];
         long long b0;
-        bool ok = gather_f2_of<true, int>([&](int o) -> long long { return __double_as_longlong(u[p + o]); }, 5, 25, P.kexp,
-                                    H, &b0) &&
-                  __double_as_longlong(b) > 0;
+        auto ld = [&](int o) -> long long { return __double_as_longlong(u[p + o]); };
+        const bool usable = gather_f2_of<true, int>(ld, 5, 25, P.kexp, H, &b0) && __double_as_longlong(b) > 0;
+        bool ok = usable;
         float g = 0.0f, m = 0.0f;
         if (ok) {
             const f2::F2 d = f2::det3(H[0], H[1], H[2], H[3], H[4], H[5]);
@@ -403,9 +406,11 @@ __device__ __forceinline__ bool newton5(double* u, const double* rhs, const smoo
         }
         float worst = fabsf(g);
         for (int o = 16; o > 0; o >>= 1) worst = fmaxf(worst, __shfl_xor_sync(FULL, worst, o));
-        if (__any_sync(FULL, on && !ok) || (moved && !(worst < last))) {
+        const bool bad = __any_sync(FULL, on && !ok);
+        const bool start_laplace = bad && !moved && !laplace && __all_sync(FULL, !on || usable);
+        if (!start_laplace && (bad || (moved && !(worst < last)))) {
             // not a point Newton can be trusted from, or the residual no longer falls: round-off, or put it back
-            if (moved && !__all_sync(FULL, !on || worst <= 1e-11f * fabsf(r6.hi))) {
+            if ((bad && laplace) || (moved && !__all_sync(FULL, !on || worst <= 1e-11f * fabsf(r6.hi)))) {
                 __syncwarp();
                 if (on) u[p] = start;
                 __syncwarp();
@@ -415,11 +420,13 @@ __device__ __forceinline__ bool newton5(double* u, const double* rhs, const smoo
             for (int o = 16; o > 0; o >>= 1) big = fmax(big, __shfl_xor_sync(FULL, big, o));
             return moved && __all_sync(FULL, !on || fabsf(g) * (float)P.kz <= 1e-14f * (float)big * m);
         }
+        if (start_laplace) g = H[0].hi + H[1].hi + H[2].hi - 3.0f * cbrtf(r6.hi);
         if (!moved || worst > 0.25f * last) {
             // row of the Jacobian: the cofactors times the stencil's weights, 2^k taken out
             const float A = H[0].hi, B = H[1].hi, C = H[2].hi, R = H[3].hi, S = H[4].hi, T = H[5].hi;
-            const float cA = B * C - T * T, cB = A * C - S * S, cC = A * B - R * R;
-            const float cR = S * T - R * C, cS = R * T - S * B, cT = R * S - T * A;
+            const bool lp = start_laplace;
+            const float cA = lp ? 1.0f : B * C - T * T, cB = lp ? 1.0f : A * C - S * S, cC = lp ? 1.0f : A * B - R * R;
+            const float cR = lp ? 0.0f : S * T - R * C, cS = lp ? 0.0f : R * T - S * B, cT = lp ? 0.0f : R * S - T * A;
             float* row = J + lane * kJ;
             if (on) {
                 for (int c = 0; c < 27; ++c) row[c] = 0.0f;
@@ -457,6 +464,10 @@ __device__ __forceinline__ bool newton5(double* u, const double* rhs, const smoo
         }
         if (on) u[p] = fma(8.0 * P.kz, f2d(d), u[p]);
         __syncwarp();
+        if (start_laplace) {
+            laplace = true;
+            continue;
+        }
         last = worst;
         moved = true;
     }
@@ -490,7 +501,8 @@ __device__ __forceinline__ void coarsest64_sm(const Grid64& S, int n, int sweeps
     } else if ((int)threadIdx.x < nt) {
         const SmallGrid G(n);
         for (int s = 0; s < max_sweeps; ++s) {
-            if (n == 5 && sweeps == 0 && (s & 7) == 0 && newton5(S.u, S.rhs, S.P, J)) break;
+            if (n == 5 && sweeps == 0 && (s & 7) == 0 && S.P.kexp != smoothf2::kNone && newton5(S.u, S.rhs, S.P, J))
+                break;
             double du = 0.0, um = 0.0;
             run_sweeps64(G, S, 1, nt, ev, [&](double v0, double v) {
                 du = fmax(du, fabs(v - v0));
@@ -973,6 +985,12 @@ cudaError_t launch_smooth(double* u, const double* rhs, int n, double h, int nsw
         }
         return cudaSuccess;
     }
+    return launch_smooth_f64(u, rhs, n, h, nsweeps, events, s);
+}
+
+cudaError_t launch_smooth_f64(double* u, const double* rhs, int n, double h, int nsweeps,
+                              unsigned long long* events, cudaStream_t s)
+{
     const double h6 = pow6(h);
     for (int sw = 0; sw < nsweeps; ++sw) {
         cudaError_t e;
@@ -999,10 +1017,10 @@ int norm_partial_count(int n) { return residual_partial_count(n); }
 cudaError_t launch_residual(const double* u, const double* rhs, double* r, int n, double h,
                             double* partials, cudaStream_t s)
 {
-    count_launches(1);
-    const dim3 g = reduce_grid(n);
-    const int kchunk = (n + (int)g.z - 1) / (int)g.z;
     if (n >= kF2MinN) {
+        const dim3 g = reduce_grid(n);
+        const int kchunk = (n + (int)g.z - 1) / (int)g.z;
+        count_launches(1);
         if (!partials) return launch_operator_f2<-1>(u, rhs, r, n, 1.0 / pow6(h), s);
         const dim3 gk = resid::grid_for(n, g.z);
         if (n < kUnormMinN)
@@ -1013,6 +1031,15 @@ cudaError_t launch_residual(const double* u, const double* rhs, double* r, int n
                                         kchunk);
         return cudaGetLastError();
     }
+    return launch_residual_f64(u, rhs, r, n, h, partials, s);
+}
+
+cudaError_t launch_residual_f64(const double* u, const double* rhs, double* r, int n, double h, double* partials,
+                                cudaStream_t s)
+{
+    count_launches(1);
+    const dim3 g = reduce_grid(n);
+    const int kchunk = (n + (int)g.z - 1) / (int)g.z;
     resid::k_residual_col<resid::NaturalF64Out><<<resid::grid_for(n, g.z), dim3(resid::RX, resid::RY), 0, s>>>(
         u, rhs, resid::NaturalF64Out{r}, n, 1.0 / pow6(h), partials, kchunk);
     return cudaGetLastError();

@@ -78,6 +78,7 @@ _SIGS = {
     "ma_hierarchy_info": [_vp, C.POINTER(C.c_int), C.POINTER(C.c_int), C.POINTER(C.c_size_t)],
     "ma_destroy_hierarchy": [_vp],
     "ma_smooth": [_vp, _vp, C.c_int, C.c_double, C.c_int, _vp, _vp],
+    "ma_smooth_f2": [_vp, _vp, C.c_int, C.c_double, C.c_int, _vp, _vp],
     "ma_residual": [_vp, _vp, _vp, C.c_int, C.c_double, _vp],
     "ma_residual_f2": [_vp, _vp, _vp, C.c_int, C.c_double, _vp],
     "ma_restrict_residual": [_vp, C.c_int, _vp, C.c_int, _vp],
@@ -343,6 +344,10 @@ def ma_last_error_string() -> str:
 
 def ma_smooth(u, rhs, n: int, h: float, nsweeps: int = 1, events=None, stream=None) -> None:
     _check(load().ma_smooth(_ptr(u), _ptr(rhs), n, h, nsweeps, _ptr(events), _stream(stream)))
+
+
+def ma_smooth_f2(u, rhs, n: int, h: float, nsweeps: int = 1, events=None, stream=None) -> None:
+    _check(load().ma_smooth_f2(_ptr(u), _ptr(rhs), n, h, nsweeps, _ptr(events), _stream(stream)))
 
 
 def ma_residual(u, rhs, r, n: int, h: float, stream=None) -> None:

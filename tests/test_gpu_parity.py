@@ -459,10 +459,10 @@ def test_single_level_hierarchy_solves(n, precision):
 
 
 # ---------------------------------------------------------------------------
-# the two-float forms of the FP64 kernels (grids from 33^3 up)
+# the two-float forms of the FP64 kernels
 # ---------------------------------------------------------------------------
 
-@pytest.mark.parametrize("n", [33, 37, 67])   # the smallest grid that takes them, and ragged ones
+@pytest.mark.parametrize("n", [5, 9, 17, 33, 37, 67, 129])   # each form: small, runtime and compile-time sizes
 @pytest.mark.parametrize("length,shift", [(1.0, 0.0), (1e-3, 0.0), (1e3, 0.0), (1e-7, 0.0), (1.0, -1.5), (1.0, -40.0),
                                           (1.0, 1e7)])
 def test_smooth_in_two_floats_over_scales_signs_and_binades(n, length, shift):
@@ -485,7 +485,7 @@ def test_smooth_in_two_floats_over_scales_signs_and_binades(n, length, shift):
     ev_ref = O.gs_sweep(ref, f, h) + O.gs_sweep(ref, f, h)
     u = dev(u0)
     ev = torch.zeros(1, dtype=torch.int64, device="cuda")
-    M.ma_smooth(u, dev(f), n, h, 2, events=ev)
+    M.ma_smooth_f2(u, dev(f), n, h, 2, events=ev)
     got = host(u)
     assert int(ev.item()) == ev_ref
     assert np.max(np.abs(got - ref)) <= 1e-12 * np.max(np.abs(ref))
@@ -503,7 +503,7 @@ def test_smooth_in_two_floats_from_a_zero_interior(n):
     ev_ref = O.gs_sweep(ref, f, pr.h)
     u = dev(u0)
     ev = torch.zeros(1, dtype=torch.int64, device="cuda")
-    M.ma_smooth(u, dev(f), n, pr.h, 1, events=ev)
+    M.ma_smooth_f2(u, dev(f), n, pr.h, 1, events=ev)
     assert int(ev.item()) == ev_ref
     assert np.max(np.abs(host(u) - ref)) <= 1e-12 * np.max(np.abs(ref))
 
@@ -516,7 +516,7 @@ def test_two_float_residual_and_coarse_rhs_match_oracle(name, n):
     is the larger part of it), and 0 on the shell."""
     pr, u0 = perturbed(name, n, 1e-6)
     r = torch.full_like(dev(u0), 7.0)
-    M.ma_residual(dev(u0), dev(pr.f), r, n, pr.h)
+    M.ma_residual_f2(dev(u0), dev(pr.f), r, n, pr.h)
     got, ref = host(r), O.residual(u0, pr.f, pr.h)
     assert np.max(np.abs(got - ref)) <= _residual_bound(u0, pr.h, name)
     r0 = 1e-3 * np.random.default_rng(n).standard_normal((n, n, n))
