@@ -389,7 +389,12 @@ __device__ __forceinline__ bool newton5(double* u, const double* rhs, const smoo
         f2::F2 H[6];
         long long b0;
         auto ld = [&](int o) -> long long { return __double_as_longlong(u[p + o]); };
-        const bool usable = gather_f2_of<true, int>(ld, 5, 25, P.kexp, H, &b0) && __double_as_longlong(b) > 0;
+        bool usable = gather_f2_of<true, int>(ld, 5, 25, P.kexp, H, &b0);
+        if (!usable && ((ld(0) | ld(1) | ld(-1) | ld(5) | ld(-5) | ld(25) | ld(-25)) << 1) == 0) {
+            usable = true;   // a zero interior's centre: no Hessian there, which is a Laplacian of 0
+            H[0] = H[1] = H[2] = H[3] = H[4] = H[5] = f2::F2{0.0f, 0.0f};
+        }
+        usable = usable && __double_as_longlong(b) > 0;
         bool ok = usable;
         float g = 0.0f, m = 0.0f;
         if (ok) {
