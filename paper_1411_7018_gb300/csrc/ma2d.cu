@@ -7,7 +7,22 @@
 // whose smaller root v = ((a + b) - sqrt((a - b)^2 + 4 r^2 + 4 h^4 f)) / 4 is
 // the convex one (Section 2).  A negative discriminant (possible only for a
 // coarse right-hand side < 0) has no real root; the vertex (a + b)/4 is taken
-// and counted.  FP64 throughout: the 2D point update is ~20 FP64 operations.
+// and counted.
+//
+// The point update is ~20 FP64 operations and an FP64 square root, and FP64
+// issues at 1/64 of the FP32 rate, so from 5^2 up it is taken in two floats, as
+// the 3D FP64 smoother takes it (ma_smooth_f2.cuh): the second differences
+// A = a - 2 v0, B = b - 2 v0 and 4 r at the current centre v0 are exact
+// integers (or fixed-point values with 7 bits to spare where the stencil
+// changes binade), the root z = 2 (v - v0) of (A - z)(B - z) - r^2 = h^4 f comes
+// from FP32, and one Newton correction takes its residual to about 2^-46.  The
+// square of the scaled entries stays in FP32's range by a power of two 2^k next
+// to 1 / h^2.  Points with an ill-conditioned root (discriminant small against
+// the entries) or values that are zero, huge or tiny take the FP64 form.  Per
+// launch of a 1025^2 FMG solve with three cycles (all levels together): a phase
+// 4.6 -> 3.9 us, the residual with norms of 1025^2 17.6 us.  The whole solve:
+// 5.23 -> 2.11 ms, 812 -> 355 launches, with the small levels in one block
+// (k_vcycle_tail2) and the cycle as a graph.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -19,7 +34,9 @@
 
 #include "ma.h"
 #include "ma2d.h"
+#include "ma_hier.h"
 #include "ma_internal.h"
+#include "ma_residual.cuh"
 
 namespace {
 
@@ -50,6 +67,263 @@ __device__ __forceinline__ double s_h(const double* u, int n, int i, int j, doub
     sums2(u, n, i, j, a, b, r);
     const double v = u[(long long)j * n + i];
     return ((a - 2.0 * v) * inv_h2) * ((b - 2.0 * v) * inv_h2) - (r * inv_h2) * (r * inv_h2);
+}
+
+// ---- two-float forms -----------------------------------------------------------
+
+struct Params2 {
+    double h4;        // h^4
+    double kz;        // 2^-k / 2: z to the change of v
+    double inv_h2;
+    float chi, clo;   // (2^k h^2)^2 as two floats
+    float ihi, ilo;   // its inverse
+    int kexp;         // k, or kNone: the FP64 form everywhere
+};
+constexpr int kNone = 1 << 20;
+// Grids that take the two-float forms.  Above 4097^2 the rounding of the FP64
+// forms (eps |u| / h^2, 1e-8 of D^2 u) shows in the solution itself: after the FMG
+// pass at 8193^2 it is 5e-11 from the two-float one, a twentieth of the scheme's
+// error (1.059e-9 against 1.114e-9 for u = exp((x^2 + y^2) / 2)), and grids of
+// that size keep the FP64 values.
+constexpr int kF2Min2 = 5, kF2Max2 = 4097;
+__host__ __device__ constexpr bool takes_f2(int n) { return n >= kF2Min2 && n <= kF2Max2; }
+
+Params2 make_params2(double h)
+{
+    Params2 P{};
+    const double h2 = h * h;
+    P.h4 = h2 * h2;
+    P.inv_h2 = 1.0 / h2;
+    int e = 0;
+    const double m = std::frexp(h2, &e);   // h^2 = m 2^e, m in [1/2, 1)
+    P.kexp = m < 0.70710678118654752 ? 1 - e : -e;
+    if (P.kexp < -18 || P.kexp > 40) {
+        P.kexp = kNone;
+        return P;
+    }
+    const double q = std::ldexp(h2, P.kexp), c = q * q;
+    P.kz = std::ldexp(0.5, -P.kexp);
+    P.chi = (float)c;
+    P.clo = (float)(c - (double)P.chi);
+    P.ihi = (float)(1.0 / c);
+    P.ilo = (float)(1.0 / c - (double)P.ihi);
+    return P;
+}
+
+using F2 = ma::resid::f2::F2;
+
+// 2^kexp (a - 2 v0, b - 2 v0, r) at a point as two floats; ld(o) gives the bits
+// of the value at offset o, sy the offset of a step in j.  false where the
+// stencil's largest value is zero, huge or tiny.
+template <typename Idx, typename Ld>
+__device__ __forceinline__ bool gather2_f2(Ld ld, Idx sy, int kexp, F2* H, long long* centre)
+{
+    namespace f2 = ma::resid::f2;
+    const long long c = ld(0), xp = ld(1), xm = ld(-1), yp = ld(sy), ym = ld(-sy);
+    const long long pp = ld(sy + 1), mp = ld(sy - 1), pm = ld(1 - sy), mm = ld(-sy - 1);
+    *centre = c;
+    const unsigned h0 = (unsigned)(c >> 32);
+    auto dif = [h0](long long v) { return (unsigned)(v >> 32) ^ h0; };
+    const unsigned diff = dif(xp) | dif(xm) | dif(yp) | dif(ym) | dif(pp) | dif(mp) | dif(pm) | dif(mm);
+    int E = (int)((h0 >> 20) & 0x7ff), sign = (int)(h0 & 0x80000000u);
+    long long A, B, Rx;
+    if ((diff >> 20) == 0) {
+        if (E < f2::kMinE || E > f2::kMaxE) return false;
+        A = (xp - c) + (xm - c);
+        B = (yp - c) + (ym - c);
+        Rx = (pp - mp) - (pm - mm);
+    } else {
+        auto mag = [](long long b) { return (unsigned)(b >> 32) & 0x7fffffffu; };
+        const unsigned top = max(max(max(mag(c), max(mag(xp), mag(xm))), max(mag(yp), mag(ym))),
+                                 max(max(mag(pp), mag(mp)), max(mag(pm), mag(mm))));
+        E = (int)(top >> 20);
+        if (E < f2::kMinE || E > f2::kMaxE) return false;
+        auto fix = [E](long long b) -> long long {
+            const long long m = (b & 0x000FFFFFFFFFFFFFll) | 0x0010000000000000ll;
+            const long long v = (m << 7) >> min(E - (int)((b >> 52) & 0x7ff), 63), neg = b >> 63;
+            return (v ^ neg) - neg;
+        };
+        const long long m0 = fix(c);
+        A = (fix(xp) - m0) + (fix(xm) - m0);
+        B = (fix(yp) - m0) + (fix(ym) - m0);
+        Rx = (fix(pp) - fix(mp)) - (fix(pm) - fix(mm));
+        E -= 7;
+        sign = 0;
+    }
+    const float unit = __int_as_float(((E - 1075 + 127 + kexp) << 23) | sign), unit4 = 0.25f * unit;
+    const int big = ((int)(A >> 32) ^ (int)(A >> 63)) | ((int)(B >> 32) ^ (int)(B >> 63)) |
+                    ((int)(Rx >> 32) ^ (int)(Rx >> 63));
+    if (big < (1 << 13)) {
+        const float u23 = 8388608.0f * unit;
+        H[0] = f2::from_i45(A, unit, u23);
+        H[1] = f2::from_i45(B, unit, u23);
+        H[2] = f2::from_i45(Rx, unit4, 0.25f * u23);
+    } else {
+        H[0] = f2::from_i64(A, unit);
+        H[1] = f2::from_i64(B, unit);
+        H[2] = f2::from_i64(Rx, unit4);
+    }
+    return true;
+}
+
+// The new centre value; false: the point needs the FP64 form.
+template <typename Idx, typename Ld>
+__device__ __forceinline__ bool update2(Ld ld, Idx sy, double b, const Params2& P, double* v)
+{
+    namespace f2 = ma::resid::f2;
+    F2 H[3];
+    long long c;
+    if (!gather2_f2<Idx>(ld, sy, P.kexp, H, &c)) return false;
+    const F2 r4 = f2::mul(f2::from_f64(b), F2{P.chi, P.clo});
+    const float A = H[0].hi, B = H[1].hi, Rr = H[2].hi, T = A + B, D = A - B;
+    const float scale = fabsf(A) + fabsf(B) + fabsf(Rr);
+    const float disc = fmaf(D, D, 4.0f * fmaf(Rr, Rr, r4.hi));
+    const float sq = disc * rsqrtf(disc);
+    // a discriminant well above its rounding; the scale's window keeps the products' low parts in FP32's range
+    if (!(disc > 4e-4f * scale * scale && scale > 9.5e-7f && scale < 1.0e9f && isfinite(sq))) return false;
+    const float g0 = fmaf(A, B, -fmaf(Rr, Rr, r4.hi));
+    const float z = T > 0.0f ? __fdividef(2.0f * g0, T + sq) : 0.5f * (T - sq);
+    auto shift = [z](F2 a) {
+        const F2 s = f2::two_sum(a.hi, -z);
+        return f2::fast_two_sum(s.hi, s.lo + a.lo);
+    };
+    const F2 g = f2::add(f2::add(f2::mul_u(shift(H[0]), shift(H[1])), f2::neg(f2::mul_u(H[2], H[2]))), f2::neg(r4));
+    const float dz = __fdividef(g.hi + g.lo, fmaf(-2.0f, z, T));
+    *v = fma(P.kz, ma::f2d(z) + ma::f2d(dz), __longlong_as_double(c));
+    return true;
+}
+
+// rv + S_h(u) (SIGN = 1) or rv - S_h(u) (SIGN = -1).
+template <int SIGN, typename Idx, typename Ld>
+__device__ __forceinline__ double operator2(Ld ld, Idx sy, double rv, const Params2& P)
+{
+    namespace f2 = ma::resid::f2;
+    F2 H[3];
+    long long c;
+    if (P.kexp != kNone && gather2_f2<Idx>(ld, sy, P.kexp, H, &c)) {
+        const float scale = fabsf(H[0].hi) + fabsf(H[1].hi) + fabsf(H[2].hi);
+        if ((scale > 1.0e-11f && scale < 1.0e15f) || scale == 0.0f) {   // the products' low parts in FP32's range
+            F2 d = f2::mul(f2::add(f2::mul_u(H[0], H[1]), f2::neg(f2::mul_u(H[2], H[2]))), F2{P.ihi, P.ilo});
+            if (SIGN < 0) d = f2::neg(d);
+            const F2 v = f2::add(f2::from_f64(rv), d);
+            return ma::f2d(v.hi) + ma::f2d(v.lo);
+        }
+    }
+    auto at = [&](Idx o) { return __longlong_as_double(ld(o)); };
+    const double v = at(0), a = at(1) + at(-1), b = at(sy) + at(-sy);
+    const double r = 0.25 * ((at(sy + 1) - at(sy - 1)) - (at(1 - sy) - at(-sy - 1)));
+    const double S = ((a - 2.0 * v) * P.inv_h2) * ((b - 2.0 * v) * P.inv_h2) - (r * P.inv_h2) * (r * P.inv_h2);
+    return SIGN > 0 ? S + rv : rv - S;
+}
+
+// The FP64 form of a point's new value, out of line.
+__device__ __noinline__ double point2_f64(const double* u, int n, int i, int j, double h4, double rhs, bool* neg)
+{
+    double a, b, r;
+    sums2(u, n, i, j, a, b, r);
+    return quad_root(a, b, r, h4, rhs, neg);
+}
+
+// The new value of point (i, j); RO: the grid is only read by the launch.
+template <bool RO>
+__device__ __forceinline__ double point2(const double* u, int n, int i, int j, double b, const Params2& P,
+                                         unsigned long long* events)
+{
+    const long long* q = reinterpret_cast<const long long*>(u) + (long long)j * n + i;
+    double v;
+    if (P.kexp != kNone &&
+        update2<int>([q](int o) -> long long { return RO ? __ldg(q + o) : q[o]; }, n, b, P, &v))
+        return v;
+    bool neg = false;
+    v = point2_f64(u, n, i, j, P.h4, b, &neg);
+    if (neg && events) atomicAdd(events, 1ull);
+    return v;
+}
+
+// The red-black and four-colour phases below with this point update.
+__global__ void __launch_bounds__(TX * TY) k_rb_f2(const double* __restrict__ src, double* __restrict__ dst,
+                                                    const double* __restrict__ rhs, int n, Params2 P, int colour,
+                                                    unsigned long long* events)
+{
+    const int i0 = 2 * (int)(blockIdx.x * TX + threadIdx.x), j = blockIdx.y * TY + threadIdx.y;
+    if (i0 >= n || j >= n) return;
+    const long long row = (long long)j * n;
+    const int ic = i0 + ((j + colour) & 1);   // (ic + j) & 1 == colour
+    const int io = ic == i0 ? i0 + 1 : i0;
+    if (io < n) dst[row + io] = __ldg(src + row + io);
+    if (ic >= n) return;
+    dst[row + ic] = ic > 0 && j > 0 && ic < n - 1 && j < n - 1
+                        ? point2<true>(src, n, ic, j, __ldg(rhs + row + ic), P, events)
+                        : __ldg(src + row + ic);
+}
+
+__global__ void __launch_bounds__(TX * TY) k_c4_f2(double* u, const double* __restrict__ rhs, int n, Params2 P, int pi,
+                                                    int pj, unsigned long long* events)
+{
+    const int i = (pi ? 1 : 2) + 2 * (int)(blockIdx.x * TX + threadIdx.x);
+    const int j = (pj ? 1 : 2) + 2 * (int)(blockIdx.y * TY + threadIdx.y);
+    if (i > n - 2 || j > n - 2) return;
+    const long long p = (long long)j * n + i;
+    u[p] = point2<false>(u, n, i, j, __ldg(rhs + p), P, events);
+}
+
+// out = r + S(u) (SIGN = 1, the coarse right-hand side) or r - S(u) (SIGN = -1,
+// the residual without norms) inside, 0 on the boundary.
+template <int SIGN>
+__global__ void __launch_bounds__(TX * TY) k_operator2(const double* __restrict__ u, const double* __restrict__ r,
+                                                        double* __restrict__ out, int n, Params2 P)
+{
+    const int i = blockIdx.x * TX + threadIdx.x, j = blockIdx.y * TY + threadIdx.y;
+    if (i >= n || j >= n) return;
+    const long long p = (long long)j * n + i;
+    const long long* q = reinterpret_cast<const long long*>(u) + p;
+    out[p] = i > 0 && j > 0 && i < n - 1 && j < n - 1
+                 ? operator2<SIGN, int>([q](int o) -> long long { return __ldg(q + o); }, n, __ldg(r + p), P)
+                 : 0.0;
+}
+
+// (max |.|, sum of squares) of a block's threads, in a fixed order, into its slot.
+__device__ __forceinline__ void reduce2(double m, double s, double* partials)
+{
+    __shared__ double sm[TX * TY / 32][2];
+    for (int o = 16; o > 0; o >>= 1) {
+        m = fmax(m, __shfl_down_sync(0xffffffffu, m, o));
+        s += __shfl_down_sync(0xffffffffu, s, o);
+    }
+    const int t = threadIdx.y * TX + threadIdx.x;
+    if ((t & 31) == 0) { sm[t >> 5][0] = m; sm[t >> 5][1] = s; }
+    __syncthreads();
+    if (t == 0) {
+        for (int w = 1; w < TX * TY / 32; ++w) { m = fmax(m, sm[w][0]); s += sm[w][1]; }
+        const int slot = blockIdx.y * gridDim.x + blockIdx.x;
+        partials[2 * slot] = m;
+        partials[2 * slot + 1] = s;
+    }
+}
+
+// The norms' partials of the residual r - S(u) (u not null) or of r itself over
+// the interior: each thread takes NROW rows TY apart before the block's
+// reduction, whose FP64 shuffles cost more than a point.
+constexpr int NROW = 8;
+template <bool RESIDUAL>
+__global__ void __launch_bounds__(TX * TY) k_partials2(const double* __restrict__ u, const double* __restrict__ r,
+                                                        int n, Params2 P, double* partials)
+{
+    const int i = blockIdx.x * TX + threadIdx.x;
+    double m = 0.0, s = 0.0;
+    for (int w = 0; w < NROW; ++w) {
+        const int j = (blockIdx.y * NROW + w) * TY + threadIdx.y;
+        if (i < 1 || j < 1 || i > n - 2 || j > n - 2) continue;
+        const long long p = (long long)j * n + i;
+        double v = __ldg(r + p);
+        if (RESIDUAL) {
+            const long long* q = reinterpret_cast<const long long*>(u) + p;
+            v = operator2<-1, int>([q](int o) -> long long { return __ldg(q + o); }, n, v, P);
+        }
+        m = fmax(m, fabs(v));
+        s = fma(v, v, s);
+    }
+    reduce2(m, s, partials);
 }
 
 // Red-black phase: dst = src with the points of one colour (i + j parity)
@@ -93,64 +367,14 @@ __global__ void __launch_bounds__(TX * TY) k_c4_phase(double* u, const double* _
     if (neg && events) atomicAdd(events, 1ull);
 }
 
-// r = rhs - S_h(u) inside, 0 on the boundary; per-block (max |r|, sum r^2).
+// r = rhs - S_h(u) inside, 0 on the boundary.
 __global__ void __launch_bounds__(TX * TY) k_resid2(const double* __restrict__ u, const double* __restrict__ rhs,
-                                                     double* __restrict__ res, int n, double inv_h2,
-                                                     double* partials)
+                                                     double* __restrict__ res, int n, double inv_h2)
 {
     const int i = blockIdx.x * TX + threadIdx.x, j = blockIdx.y * TY + threadIdx.y;
-    double m = 0.0, s = 0.0;
-    if (i < n && j < n) {
-        const long long p = (long long)j * n + i;
-        double v = 0.0;
-        if (i > 0 && j > 0 && i < n - 1 && j < n - 1) {
-            v = rhs[p] - s_h(u, n, i, j, inv_h2);
-            m = fabs(v);
-            s = v * v;
-        }
-        if (res) res[p] = v;
-    }
-    if (!partials) return;
-    __shared__ double sm[TX * TY / 32][2];
-    for (int o = 16; o > 0; o >>= 1) {
-        m = fmax(m, __shfl_down_sync(0xffffffffu, m, o));
-        s += __shfl_down_sync(0xffffffffu, s, o);
-    }
-    const int t = threadIdx.y * TX + threadIdx.x;
-    if ((t & 31) == 0) { sm[t >> 5][0] = m; sm[t >> 5][1] = s; }
-    __syncthreads();
-    if (t == 0) {
-        for (int w = 1; w < TX * TY / 32; ++w) { m = fmax(m, sm[w][0]); s += sm[w][1]; }
-        const int slot = blockIdx.y * gridDim.x + blockIdx.x;
-        partials[2 * slot] = m;
-        partials[2 * slot + 1] = s;
-    }
-}
-
-// Per-block (max |v|, sum v^2) over the interior of v.
-__global__ void __launch_bounds__(TX * TY) k_norm_partials2(const double* __restrict__ v, int n, double* partials)
-{
-    const int i = blockIdx.x * TX + threadIdx.x, j = blockIdx.y * TY + threadIdx.y;
-    double m = 0.0, s = 0.0;
-    if (i > 0 && j > 0 && i < n - 1 && j < n - 1) {
-        const double x = v[(long long)j * n + i];
-        m = fabs(x);
-        s = x * x;
-    }
-    __shared__ double sm[TX * TY / 32][2];
-    for (int o = 16; o > 0; o >>= 1) {
-        m = fmax(m, __shfl_down_sync(0xffffffffu, m, o));
-        s += __shfl_down_sync(0xffffffffu, s, o);
-    }
-    const int t = threadIdx.y * TX + threadIdx.x;
-    if ((t & 31) == 0) { sm[t >> 5][0] = m; sm[t >> 5][1] = s; }
-    __syncthreads();
-    if (t == 0) {
-        for (int w = 1; w < TX * TY / 32; ++w) { m = fmax(m, sm[w][0]); s += sm[w][1]; }
-        const int slot = blockIdx.y * gridDim.x + blockIdx.x;
-        partials[2 * slot] = m;
-        partials[2 * slot + 1] = s;
-    }
+    if (i >= n || j >= n) return;
+    const long long p = (long long)j * n + i;
+    res[p] = i > 0 && j > 0 && i < n - 1 && j < n - 1 ? rhs[p] - s_h(u, n, i, j, inv_h2) : 0.0;
 }
 
 // out2 = (max, sqrt(h^2 sum)) from the partials (one block).
@@ -262,83 +486,218 @@ __global__ void __launch_bounds__(TX * TY) k_prolong2(const double* __restrict__
     uf[p] = add ? uf[p] + v : v;
 }
 
-// b = S_H(w) + r inside, 0 on the boundary (Algorithm 1 step 5).
-__global__ void __launch_bounds__(TX * TY) k_coarse_rhs2(const double* __restrict__ w, const double* __restrict__ r,
-                                                          double* __restrict__ b, int nc, double inv_h2)
+// ---- small grids in one block ---------------------------------------------------
+// A level of 33^2 points or fewer is bound by its launches (8 phases and 4
+// transfers a cycle, 1.5 - 2 us each); one block runs those levels of a cycle in
+// shared memory, a phase on the warps that it fills.  At 65^2 one block's phases
+// (2000 points) take as long as the launches.  A cycle from 33^2: 62 us, 52
+// launches before.
+
+// Colour phases of a grid of n = 2^k + 1 <= 33 points a side: slots of a phase
+// (at most one a thread), the threads that hold them and their barrier.
+struct Small2 {
+    int n, S, ls;   // S = 2^ls = (n - 1) / 2 points of a row's colour at most
+    __device__ __forceinline__ explicit Small2(int n_) : n(n_), S((n_ - 1) / 2)
+    {
+        ls = n == 33 ? 4 : (n == 17 ? 3 : (n == 9 ? 2 : (n == 5 ? 1 : 0)));
+    }
+    __device__ __forceinline__ int threads() const { return n <= 9 ? 32 : (n <= 17 ? 128 : 512); }
+    __device__ __forceinline__ void barrier() const
+    {
+        if (n <= 9) __syncwarp();
+        else if (n <= 17) asm volatile("bar.sync 1, 128;" ::: "memory");
+        else asm volatile("bar.sync 2, 512;" ::: "memory");
+    }
+    // point t of a phase: red-black colour q, or four-colour class q
+    __device__ __forceinline__ bool point(int ordering, int q, int t, int* i, int* j) const
+    {
+        const int s = t & (S - 1), row = t >> ls;
+        if (ordering == MA2D_COLOUR4) {
+            *i = ((q & 1) ? 1 : 2) + 2 * s;
+            *j = ((q & 2) ? 1 : 2) + 2 * row;
+        } else {
+            *j = 1 + row;
+            *i = (((1 + *j) & 1) == q ? 1 : 2) + 2 * s;
+        }
+        return *i <= n - 2 && *j <= n - 2;
+    }
+};
+
+// nsw sweeps; each(old, new) sees every update.  The grid's threads enter.
+template <typename Each>
+__device__ __forceinline__ void sweeps2_sm(double* u, const double* rhs, const Small2& G, int ordering,
+                                           const Params2& P, int nsw, Each each)
 {
-    const int I = blockIdx.x * TX + threadIdx.x, J = blockIdx.y * TY + threadIdx.y;
-    if (I >= nc || J >= nc) return;
-    const long long p = (long long)J * nc + I;
-    b[p] = (I > 0 && J > 0 && I < nc - 1 && J < nc - 1) ? s_h(w, nc, I, J, inv_h2) + r[p] : 0.0;
+    const int phases = ordering == MA2D_COLOUR4 ? 4 : 2;
+    for (int q = 0, w = 0; q < nsw * phases; ++q, w = w + 1 == phases ? 0 : w + 1) {
+        int i, j;
+        const bool on = G.point(ordering, w, threadIdx.x, &i, &j);
+        const int p = j * G.n + i;
+        double v = 0.0, v0 = 0.0;
+        if (on) {
+            v0 = u[p];
+            v = point2<false>(u, G.n, i, j, rhs[p], P, nullptr);
+        }
+        G.barrier();   // red-black: every point of the colour from the old values
+        if (on) {
+            u[p] = v;
+            each(v0, v);
+        }
+        G.barrier();
+    }
 }
 
-// Coarsest grid (n <= 17): one block, the grid in shared memory; sweeps > 0
-// fixed sweeps, else until max|du| <= 1e-14 max|u| (at most 100).
-constexpr int CT2 = 256;
-__global__ void __launch_bounds__(CT2) k_coarsest2(double* u, const double* __restrict__ rhs, int n, double h4,
-                                                   int sweeps, int ordering, unsigned long long* events)
+// Coarsest grid (n <= 17): fixed sweeps, or until max |du| <= 1e-14 max |u| over
+// the whole grid (boundary included; at most 100).  Every thread of the block
+// enters; ends with a block barrier.
+__device__ __forceinline__ void coarsest2_sm(double* u, const double* rhs, int n, int sweeps, int ordering,
+                                             const Params2& P)
+{
+    const Small2 G(n);
+    __shared__ double red[4][2];
+    if (n == 3) {   // one unknown, whose root does not depend on it
+        if (threadIdx.x == 0) {
+            bool neg = false;
+            u[4] = point2_f64(u, 3, 1, 1, P.h4, rhs[4], &neg);
+        }
+    } else if ((int)threadIdx.x < G.threads()) {
+        const int max_sweeps = sweeps > 0 ? sweeps : 100;
+        double bmax = 0.0;
+        for (int q = threadIdx.x; q < n * n && sweeps == 0; q += G.threads()) {
+            const int i = q % n, j = q / n;
+            if (i == 0 || j == 0 || i == n - 1 || j == n - 1) bmax = fmax(bmax, fabs(u[q]));
+        }
+        for (int s = 0; s < max_sweeps; ++s) {
+            double du = 0.0, um = bmax;
+            sweeps2_sm(u, rhs, G, ordering, P, 1, [&](double v0, double v) {
+                du = fmax(du, fabs(v - v0));
+                um = fmax(um, fabs(v));
+            });
+            if (sweeps > 0) continue;
+            for (int o = 16; o > 0; o >>= 1) {
+                du = fmax(du, __shfl_xor_sync(0xffffffffu, du, o));
+                um = fmax(um, __shfl_xor_sync(0xffffffffu, um, o));
+            }
+            if (G.threads() > 32) {
+                if ((threadIdx.x & 31) == 0) { red[threadIdx.x >> 5][0] = du; red[threadIdx.x >> 5][1] = um; }
+                G.barrier();
+                for (int w = 0; w < 4; ++w) { du = fmax(du, red[w][0]); um = fmax(um, red[w][1]); }
+                G.barrier();   // red is free again
+            }
+            if (du <= 1e-14 * um) break;
+        }
+    }
+    __syncthreads();
+}
+
+constexpr int kTail2MaxN = 33, kTail2Levels = 5;
+constexpr int CT2 = 128, TT2 = 512;
+
+__global__ void __launch_bounds__(CT2) k_coarsest2(double* u, const double* __restrict__ rhs, int n, Params2 P,
+                                                   int sweeps, int ordering)
 {
     __shared__ double su[17 * 17];
     __shared__ double sr[17 * 17];
-    __shared__ double red[CT2 / 32][2];
-    __shared__ int stop;
-    const int m = n * n;
-    // the stopping test compares with max |u| over the whole grid, boundary
-    // included (boundary values do not change)
-    double bmax = 0.0;
-    for (int q = threadIdx.x; q < m; q += CT2) {
+    for (int q = threadIdx.x; q < n * n; q += CT2) {
         su[q] = u[q];
         sr[q] = rhs[q];
-        const int i = q % n, j = q / n;
-        if (i == 0 || j == 0 || i == n - 1 || j == n - 1) bmax = fmax(bmax, fabs(su[q]));
     }
     __syncthreads();
-    unsigned long long ev = 0;
-    const int phases = ordering == MA2D_COLOUR4 ? 4 : 2;
-    const int max_sweeps = sweeps > 0 ? sweeps : 100;
-    for (int s = 0; s < max_sweeps; ++s) {
-        double du = 0.0, um = bmax;
-        for (int ph = 0; ph < phases; ++ph) {
-            // each thread takes at most two points per phase (n <= 17: <= 225 interior)
-            double nv[2];
-            int np[2], cnt = 0;
-            for (int q = threadIdx.x; q < (n - 2) * (n - 2); q += CT2) {
-                const int i = 1 + q % (n - 2), j = 1 + q / (n - 2);
-                const bool mine = ordering == MA2D_COLOUR4 ? (((i & 1) | ((j & 1) << 1)) == ph) : (((i + j) & 1) == ph);
-                if (!mine) continue;
-                double a, b, r;
-                sums2(su, n, i, j, a, b, r);
-                bool neg = false;
-                nv[cnt] = quad_root(a, b, r, h4, sr[j * n + i], &neg);
-                np[cnt] = j * n + i;
-                ++cnt;
-                ev += neg ? 1 : 0;
-            }
-            __syncthreads();   // red-black: every point of the colour from the old values
-            for (int c = 0; c < cnt; ++c) {
-                du = fmax(du, fabs(nv[c] - su[np[c]]));
-                su[np[c]] = nv[c];
-                um = fmax(um, fabs(nv[c]));
-            }
-            __syncthreads();
+    coarsest2_sm(su, sr, n, sweeps, ordering, P);
+    for (int q = threadIdx.x; q < n * n; q += CT2) u[q] = su[q];
+}
+
+struct Tail2Level {
+    int n;
+    Params2 P;
+    double* u;           // global iterate (read on the top level, written back there)
+    const double* rhs;   // global right-hand side (read on the top level)
+};
+
+struct Tail2Args {
+    int nlev;
+    Tail2Level lev[kTail2Levels];
+    int nu1, nu2, kind, approx, coarse_sweeps, ordering;
+};
+
+constexpr int kTail2Doubles = 3 * 33 * 33 + 4 * (17 * 17 + 9 * 9 + 5 * 5 + 3 * 3);
+
+// One V-cycle over levels of n <= 33 down to the coarsest grid and back.
+__global__ void __launch_bounds__(TT2) k_vcycle_tail2(const __grid_constant__ Tail2Args A)
+{
+    __shared__ double sm[kTail2Doubles];
+    // level l's u, r, rhs and (below the top) w, one after the other
+    auto at = [&](int l) {
+        int o = 0;
+        for (int q = 0; q < l; ++q) o += (q > 0 ? 4 : 3) * A.lev[q].n * A.lev[q].n;
+        return sm + o;
+    };
+    {
+        const int m = A.lev[0].n * A.lev[0].n;
+        for (int q = threadIdx.x; q < m; q += TT2) {
+            sm[q] = A.lev[0].u[q];
+            sm[2 * m + q] = A.lev[0].rhs[q];
         }
-        if (sweeps > 0) continue;
-        for (int o = 16; o > 0; o >>= 1) {
-            du = fmax(du, __shfl_down_sync(0xffffffffu, du, o));
-            um = fmax(um, __shfl_down_sync(0xffffffffu, um, o));
-        }
-        if ((threadIdx.x & 31) == 0) { red[threadIdx.x >> 5][0] = du; red[threadIdx.x >> 5][1] = um; }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double a = 0.0, b = 0.0;
-            for (int w = 0; w < CT2 / 32; ++w) { a = fmax(a, red[w][0]); b = fmax(b, red[w][1]); }
-            stop = a <= 1e-14 * b;
-        }
-        __syncthreads();
-        if (stop) break;
     }
-    for (int q = threadIdx.x; q < m; q += CT2) u[q] = su[q];
-    if (events && ev) atomicAdd(events, ev);
+    __syncthreads();
+    const int L = A.nlev;
+    for (int l = 0; l < L - 1; ++l) {
+        const int n = A.lev[l].n, m = n * n, nc = A.lev[l + 1].n, mc = nc * nc;
+        double *u = at(l), *r = u + m, *rhs = u + 2 * m;
+        double *uc = at(l + 1), *rc = uc + mc, *bc = uc + 2 * mc, *wc = uc + 3 * mc;
+        const Small2 G(n);
+        if ((int)threadIdx.x < G.threads())
+            sweeps2_sm(u, rhs, G, A.ordering, A.lev[l].P, A.nu1, [](double, double) {});
+        __syncthreads();
+        for (int t = threadIdx.x; t < (n - 2) * (n - 2); t += TT2) {
+            const int j = 1 + t / (n - 2), i = 1 + t - (j - 1) * (n - 2), p = j * n + i;
+            const long long* q = reinterpret_cast<const long long*>(u) + p;
+            r[p] = operator2<-1, int>([q](int o) -> long long { return q[o]; }, n, rhs[p], A.lev[l].P);
+        }
+        __syncthreads();
+        for (int t = threadIdx.x; t < mc; t += TT2) {
+            const int J = t / nc, I = t - J * nc;
+            const bool inside = I > 0 && J > 0 && I < nc - 1 && J < nc - 1;
+            rc[t] = inside ? restrict_at2(r, n, 2 * I, 2 * J, A.kind) : 0.0;
+            const double w = inside && A.approx == MA_APPROX_WEIGHTED ? restrict_at2(u, n, 2 * I, 2 * J, A.kind)
+                                                                      : u[2 * J * n + 2 * I];
+            wc[t] = w;
+            uc[t] = w;
+        }
+        __syncthreads();
+        for (int t = threadIdx.x; t < (nc - 2) * (nc - 2); t += TT2) {
+            const int j = 1 + t / (nc - 2), i = 1 + t - (j - 1) * (nc - 2), p = j * nc + i;
+            const long long* q = reinterpret_cast<const long long*>(wc) + p;
+            bc[p] = operator2<1, int>([q](int o) -> long long { return q[o]; }, nc, rc[p], A.lev[l + 1].P);
+        }
+        __syncthreads();
+    }
+    {
+        const int n = A.lev[L - 1].n;
+        double* u = at(L - 1);
+        coarsest2_sm(u, u + 2 * n * n, n, A.coarse_sweeps, A.ordering, A.lev[L - 1].P);
+    }
+    for (int l = L - 2; l >= 0; --l) {
+        const int n = A.lev[l].n, m = n * n, nc = A.lev[l + 1].n, mc = nc * nc;
+        double *u = at(l), *uc = at(l + 1), *wc = uc + 3 * mc;
+        for (int t = threadIdx.x; t < mc; t += TT2) wc[t] = uc[t] - wc[t];
+        __syncthreads();
+        for (int t = threadIdx.x; t < (n - 2) * (n - 2); t += TT2) {
+            const int j = 1 + t / (n - 2), i = 1 + t - (j - 1) * (n - 2);
+            const int I = i >> 1, J = j >> 1, oi = i & 1, oj = j & 1;
+            double s = 0.0;
+            for (int b = 0; b <= oj; ++b)
+                for (int a = 0; a <= oi; ++a) s += wc[(J + b) * nc + I + a];
+            u[j * n + i] += s * (oi + oj == 2 ? 0.25 : (oi + oj == 1 ? 0.5 : 1.0));
+        }
+        __syncthreads();
+        const Small2 G(n);
+        if ((int)threadIdx.x < G.threads())
+            sweeps2_sm(u, u + 2 * m, G, A.ordering, A.lev[l].P, A.nu2, [](double, double) {});
+        __syncthreads();
+    }
+    const int m = A.lev[0].n * A.lev[0].n;
+    for (int q = threadIdx.x; q < m; q += TT2) A.lev[0].u[q] = sm[q];
 }
 
 // rhs = f, u = g; flag = 1 if f is not finite and > 0 inside.
@@ -363,14 +722,17 @@ __global__ void __launch_bounds__(TX * TY) k_zero_interior2(double* u, int n)
 }
 
 dim3 grid2(int nx, int ny) { return dim3((nx + TX - 1) / TX, (ny + TY - 1) / TY); }
-int partial_count2(int n) { const dim3 g = grid2(n, n); return (int)(g.x * g.y); }
+dim3 partial_grid2(int n) { return dim3((n + TX - 1) / TX, (n + TY * NROW - 1) / (TY * NROW)); }
+int partial_count2(int n) { const dim3 g = partial_grid2(n); return (int)(g.x * g.y); }
 
 // ---- launchers ---------------------------------------------------------------
 
-cudaError_t smooth2(double* u, double* t, const double* rhs, int n, double h, int nsweeps, int ordering,
+// f2: the two-float forms (the cycles); otherwise FP64 throughout.
+cudaError_t smooth2(double* u, double* t, const double* rhs, int n, double h, int nsweeps, int ordering, bool f2,
                     unsigned long long* ev, cudaStream_t s)
 {
-    const double h4 = h * h * h * h;
+    const Params2 P = make_params2(h);
+    f2 = f2 && takes_f2(n) && P.kexp != kNone;
     for (int sw = 0; sw < nsweeps; ++sw) {
         if (ordering == MA2D_COLOUR4) {
             for (int c = 0; c < 4; ++c) {
@@ -378,13 +740,19 @@ cudaError_t smooth2(double* u, double* t, const double* rhs, int n, double h, in
                 const int ni = pi ? (n - 1) / 2 : (n - 3) / 2, nj = pj ? (n - 1) / 2 : (n - 3) / 2;
                 if (ni <= 0 || nj <= 0) continue;
                 ma::count_launches(1);
-                k_c4_phase<<<grid2(ni, nj), dim3(TX, TY), 0, s>>>(u, rhs, n, h4, pi, pj, ev);
+                if (f2) k_c4_f2<<<grid2(ni, nj), dim3(TX, TY), 0, s>>>(u, rhs, n, P, pi, pj, ev);
+                else k_c4_phase<<<grid2(ni, nj), dim3(TX, TY), 0, s>>>(u, rhs, n, P.h4, pi, pj, ev);
             }
         } else {
             ma::count_launches(2);
-            const dim3 g = grid2((n + 1) / 2, n);
-            k_rb_phase<<<g, dim3(TX, TY), 0, s>>>(u, t, rhs, n, h4, 0, ev);
-            k_rb_phase<<<g, dim3(TX, TY), 0, s>>>(t, u, rhs, n, h4, 1, ev);
+            const dim3 g = grid2((n + 1) / 2, n), b(TX, TY);
+            if (f2) {
+                k_rb_f2<<<g, b, 0, s>>>(u, t, rhs, n, P, 0, ev);
+                k_rb_f2<<<g, b, 0, s>>>(t, u, rhs, n, P, 1, ev);
+            } else {
+                k_rb_phase<<<g, b, 0, s>>>(u, t, rhs, n, P.h4, 0, ev);
+                k_rb_phase<<<g, b, 0, s>>>(t, u, rhs, n, P.h4, 1, ev);
+            }
         }
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
@@ -392,11 +760,13 @@ cudaError_t smooth2(double* u, double* t, const double* rhs, int n, double h, in
     return cudaSuccess;
 }
 
-cudaError_t residual2(const double* u, const double* rhs, double* r, int n, double h, double* partials,
-                      cudaStream_t s)
+template <int SIGN>
+cudaError_t operator2_launch(const double* u, const double* r, double* out, int n, double h, cudaStream_t s)
 {
+    Params2 P = make_params2(h);
+    if (!takes_f2(n)) P.kexp = kNone;
     ma::count_launches(1);
-    k_resid2<<<grid2(n, n), dim3(TX, TY), 0, s>>>(u, rhs, r, n, 1.0 / (h * h), partials);
+    k_operator2<SIGN><<<grid2(n, n), dim3(TX, TY), 0, s>>>(u, r, out, n, P);
     return cudaGetLastError();
 }
 
@@ -405,6 +775,18 @@ cudaError_t norm_final2(const double* partials, int count, double h, double* out
     ma::count_launches(1);
     k_norm_final2<<<1, 1024, 0, s>>>(partials, count, h, out2);
     return cudaGetLastError();
+}
+
+// Norms of the residual rhs - S(u) into out2, or (u null) of rhs.
+cudaError_t norms2(const double* u, const double* rhs, int n, double h, double* partials, double* out2, cudaStream_t s)
+{
+    Params2 P = make_params2(h);
+    if (!takes_f2(n)) P.kexp = kNone;
+    ma::count_launches(1);
+    if (u) k_partials2<true><<<partial_grid2(n), dim3(TX, TY), 0, s>>>(u, rhs, n, P, partials);
+    else k_partials2<false><<<partial_grid2(n), dim3(TX, TY), 0, s>>>(nullptr, rhs, n, P, partials);
+    const cudaError_t e = cudaGetLastError();
+    return e != cudaSuccess ? e : norm_final2(partials, partial_count2(n), h, out2, s);
 }
 
 thread_local char g_err2[512] = "";
@@ -446,6 +828,9 @@ struct ma2d_hierarchy {
     int* flag = nullptr;
     double* host = nullptr;       // pinned, 4 doubles
     cudaStream_t s = nullptr;
+    cudaStream_t cap = nullptr;   // private stream the graphs are captured on
+    ma::GraphSlot g_init[9];      // per initial iterate and reference of the stopping rule: start and first norms
+    ma::GraphSlot g_cycle;        // one cycle and its norms
 };
 
 namespace {
@@ -517,9 +902,30 @@ size_t layout2(ma2d_hierarchy* H, const ma2d_desc* d, char* base)
 cudaError_t coarsest_solve2(ma2d_hierarchy* H, int l)
 {
     auto& B = H->lev[l];
-    const double h4 = B.h * B.h * B.h * B.h;
     ma::count_launches(1);
-    k_coarsest2<<<1, CT2, 0, H->s>>>(B.u, B.rhs, B.n, h4, H->d.coarse_sweeps, H->d.ordering, nullptr);
+    k_coarsest2<<<1, CT2, 0, H->s>>>(B.u, B.rhs, B.n, make_params2(B.h), H->d.coarse_sweeps, H->d.ordering);
+    return cudaGetLastError();
+}
+
+// The levels from l down to the coarsest grid (n <= 33) in one launch.
+cudaError_t tail2(ma2d_hierarchy* H, int l)
+{
+    const ma2d_desc& d = H->d;
+    Tail2Args A{};
+    A.nlev = H->L - l;
+    for (int q = 0; q < A.nlev; ++q) {
+        auto& V = H->lev[l + q];
+        A.lev[q] = Tail2Level{V.n, make_params2(V.h), V.u, V.rhs};
+        if (!takes_f2(V.n)) A.lev[q].P.kexp = kNone;
+    }
+    A.nu1 = d.nu1;
+    A.nu2 = d.nu2;
+    A.kind = d.restrict_kind;
+    A.approx = d.approx_restrict;
+    A.coarse_sweeps = d.coarse_sweeps;
+    A.ordering = d.ordering;
+    ma::count_launches(1);
+    k_vcycle_tail2<<<1, TT2, 0, H->s>>>(A);
     return cudaGetLastError();
 }
 
@@ -529,27 +935,36 @@ cudaError_t vcycle2_from(ma2d_hierarchy* H, int l0)
     cudaStream_t s = H->s;
     const ma2d_desc& d = H->d;
     cudaError_t e;
-    for (int l = l0; l < H->L - 1; ++l) {
+    int lt = l0;
+    while (H->lev[lt].n > kTail2MaxN) ++lt;   // the coarsest grid has n <= 17
+    for (int l = l0; l < lt; ++l) {
         auto& F = H->lev[l];
         auto& C = H->lev[l + 1];
-        if ((e = smooth2(F.u, H->t, F.rhs, F.n, F.h, d.nu1, d.ordering, nullptr, s)) != cudaSuccess) return e;
-        if ((e = residual2(F.u, F.rhs, F.r, F.n, F.h, nullptr, s)) != cudaSuccess) return e;
-        ma::count_launches(2);
+        if ((e = smooth2(F.u, H->t, F.rhs, F.n, F.h, d.nu1, d.ordering, true, nullptr, s)) != cudaSuccess) return e;
+        if ((e = operator2_launch<-1>(F.u, F.rhs, F.r, F.n, F.h, s)) != cudaSuccess) return e;
+        ma::count_launches(1);
         k_restrict2<<<grid2(C.n, C.n), dim3(TX, TY), 0, s>>>(F.u, F.r, F.n, C.w, C.u, C.r, C.n, d.restrict_kind,
                                                              d.approx_restrict);
-        k_coarse_rhs2<<<grid2(C.n, C.n), dim3(TX, TY), 0, s>>>(C.w, C.r, C.rhs, C.n, 1.0 / (C.h * C.h));
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if ((e = operator2_launch<1>(C.w, C.r, C.rhs, C.n, C.h, s)) != cudaSuccess) return e;
     }
-    if ((e = coarsest_solve2(H, H->L - 1)) != cudaSuccess) return e;
-    for (int l = H->L - 2; l >= l0; --l) {
+    if ((e = tail2(H, lt)) != cudaSuccess) return e;
+    for (int l = lt - 1; l >= l0; --l) {
         auto& F = H->lev[l];
         auto& C = H->lev[l + 1];
         ma::count_launches(1);
         k_prolong2<<<grid2(F.n, F.n), dim3(TX, TY), 0, s>>>(C.u, C.w, C.n, F.u, F.n, 1, 0);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        if ((e = smooth2(F.u, H->t, F.rhs, F.n, F.h, d.nu2, d.ordering, nullptr, s)) != cudaSuccess) return e;
+        if ((e = smooth2(F.u, H->t, F.rhs, F.n, F.h, d.nu2, d.ordering, true, nullptr, s)) != cudaSuccess) return e;
     }
     return cudaSuccess;
+}
+
+cudaError_t zero_interior2(double* u, int n, cudaStream_t s)
+{
+    ma::count_launches(1);
+    k_zero_interior2<<<grid2(n, n), dim3(TX, TY), 0, s>>>(u, n);
+    return cudaGetLastError();
 }
 
 // Algorithm 2 (2D).
@@ -565,8 +980,7 @@ cudaError_t fmg2(ma2d_hierarchy* H)
         k_inject2<<<grid2(C.n, C.n), dim3(TX, TY), 0, s>>>(F.u, F.n, C.u, C.n);
     }
     auto& B = H->lev[H->L - 1];
-    ma::count_launches(1);
-    k_zero_interior2<<<grid2(B.n, B.n), dim3(TX, TY), 0, s>>>(B.u, B.n);
+    if ((e = zero_interior2(B.u, B.n, s)) != cudaSuccess) return e;
     if ((e = coarsest_solve2(H, H->L - 1)) != cudaSuccess) return e;
     for (int l = H->L - 2; l >= 0; --l) {
         auto& F = H->lev[l];
@@ -580,17 +994,55 @@ cudaError_t fmg2(ma2d_hierarchy* H)
     return cudaSuccess;
 }
 
-// Residual norms of the finest level into out[slot], out[slot + 1]; reads
-// them back when readback != 0 (blocks).
-ma_status fine_norms2(ma2d_hierarchy* H, int slot, double* mx, double* l2)
+// Runs body() as a CUDA graph captured once on the hierarchy's private stream
+// and replayed on its own: one graph launch in place of the hundreds of launches
+// of a cycle or an FMG pass, which left the GPU idle a third of a 1025^2 solve.
+template <typename Body>
+cudaError_t run_graph2(ma2d_hierarchy* H, ma::GraphSlot& gs, Body body)
 {
-    auto& F = H->lev[0];
-    CK2(residual2(F.u, F.rhs, F.r, F.n, F.h, H->partials, H->s));
-    CK2(norm_final2(H->partials, H->npartials, F.h, H->out + slot, H->s));
+    if (!gs.exec) {
+        const unsigned long long before = ma::launch_count();
+        cudaError_t e = cudaStreamBeginCapture(H->cap, cudaStreamCaptureModeThreadLocal);
+        if (e != cudaSuccess) return e;
+        cudaStream_t user = H->s;
+        H->s = H->cap;
+        const cudaError_t eb = body();
+        H->s = user;
+        cudaGraph_t g = nullptr;
+        e = cudaStreamEndCapture(H->cap, &g);
+        const unsigned long long captured = ma::launch_count() - before;
+        ma::uncount_launches(captured);   // captured, not run
+        if (eb != cudaSuccess || e != cudaSuccess) {
+            if (g) cudaGraphDestroy(g);
+            return eb != cudaSuccess ? eb : e;
+        }
+        e = cudaGraphInstantiate(&gs.exec, g, 0);
+        if (e != cudaSuccess) {
+            cudaGraphDestroy(g);
+            gs.exec = nullptr;
+            return e;
+        }
+        gs.graph = g;
+        gs.launches = captured;
+    }
+    ma::count_launches(gs.launches);
+    return cudaGraphLaunch(gs.exec, H->s);
+}
+
+void drop_graph2(ma::GraphSlot& gs)
+{
+    if (gs.exec) cudaGraphExecDestroy(gs.exec);
+    if (gs.graph) cudaGraphDestroy(gs.graph);
+    gs = ma::GraphSlot();
+}
+
+// Reads the norms in out back to the host (blocks): the residual's max and L2.
+ma_status read_norms2(ma2d_hierarchy* H, double* mx, double* l2)
+{
     CK2(cudaMemcpyAsync(H->host, H->out, 4 * sizeof(double), cudaMemcpyDeviceToHost, H->s));
     CK2(cudaStreamSynchronize(H->s));
-    *mx = H->host[slot];
-    *l2 = H->host[slot + 1];
+    *mx = H->host[0];
+    *l2 = H->host[1];
     return MA_OK;
 }
 
@@ -626,7 +1078,9 @@ ma_status ma2d_create_hierarchy(const ma2d_desc* desc, void* ws, size_t bytes, m
     }
     H->s = (cudaStream_t)stream;
     cudaError_t e = cudaMallocHost((void**)&H->host, 4 * sizeof(double));
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&H->cap, cudaStreamNonBlocking);
     if (e != cudaSuccess) {
+        if (H->host) cudaFreeHost(H->host);
         delete H;
         return fail2(MA_ERR_CUDA, "create: %s", cudaGetErrorString(e));
     }
@@ -638,6 +1092,9 @@ ma_status ma2d_destroy_hierarchy(ma2d_hierarchy* H)
 {
     if (!H) return MA_OK;
     cudaError_t e = cudaStreamSynchronize(H->s);
+    for (ma::GraphSlot& g : H->g_init) drop_graph2(g);
+    drop_graph2(H->g_cycle);
+    if (H->cap) cudaStreamDestroy(H->cap);
     if (H->host) cudaFreeHost(H->host);
     delete H;
     if (e != cudaSuccess) return fail2(MA_ERR_CUDA, "destroy: %s", cudaGetErrorString(e));
@@ -673,33 +1130,25 @@ ma_status ma2d_solve(ma2d_hierarchy* H, const ma_solve_opts* o, ma_solve_result*
         o->init < MA_INIT_FMG || o->init > MA_INIT_KEEP || o->relative < MA_REL_NONE || o->relative > MA_REL_INITIAL)
         return fail2(MA_ERR_INVALID_ARG, "bad solve options");
     std::memset(res, 0, sizeof *res);
-    auto& F = H->lev[0];
-    double mx = 0.0, l2 = 0.0, scale = 1.0;
-    if (o->relative == MA_REL_INITIAL) {
-        if (o->init != MA_INIT_KEEP) {
-            ma::count_launches(1);
-            k_zero_interior2<<<grid2(F.n, F.n), dim3(TX, TY), 0, H->s>>>(F.u, F.n);
+    // the norms of the reference, the initial iterate and its residual norms as one graph
+    CK2(run_graph2(H, H->g_init[3 * o->init + o->relative], [&]() -> cudaError_t {
+        auto& F = H->lev[0];
+        cudaError_t e = cudaSuccess;
+        if (o->relative == MA_REL_INITIAL) {
+            if (o->init != MA_INIT_KEEP) e = zero_interior2(F.u, F.n, H->s);
+            if (e == cudaSuccess) e = norms2(F.u, F.rhs, F.n, F.h, H->partials, H->out + 2, H->s);
+        } else if (o->relative == MA_REL_RHS) {
+            e = norms2(nullptr, F.rhs, F.n, F.h, H->partials, H->out + 2, H->s);
         }
-        ma_status st = fine_norms2(H, 2, &mx, &l2);
-        if (st != MA_OK) return st;
-        scale = o->norm == MA_NORM_MAX ? mx : l2;
-    } else if (o->relative == MA_REL_RHS) {
-        ma::count_launches(2);
-        k_norm_partials2<<<grid2(F.n, F.n), dim3(TX, TY), 0, H->s>>>(F.rhs, F.n, H->partials);
-        k_norm_final2<<<1, 1024, 0, H->s>>>(H->partials, H->npartials, F.h, H->out + 2);
-        CK2(cudaGetLastError());
-        CK2(cudaMemcpyAsync(H->host, H->out, 4 * sizeof(double), cudaMemcpyDeviceToHost, H->s));
-        CK2(cudaStreamSynchronize(H->s));
-        scale = o->norm == MA_NORM_MAX ? H->host[2] : H->host[3];
-    }
-    if (!(scale > 0.0)) scale = 1.0;
-    if (o->init == MA_INIT_FMG) CK2(fmg2(H));
-    if (o->init == MA_INIT_ZERO) {
-        ma::count_launches(1);
-        k_zero_interior2<<<grid2(F.n, F.n), dim3(TX, TY), 0, H->s>>>(F.u, F.n);
-    }
-    ma_status st = fine_norms2(H, 0, &mx, &l2);
+        if (e == cudaSuccess && o->init == MA_INIT_FMG) e = fmg2(H);
+        if (e == cudaSuccess && o->init == MA_INIT_ZERO) e = zero_interior2(F.u, F.n, H->s);
+        return e != cudaSuccess ? e : norms2(F.u, F.rhs, F.n, F.h, H->partials, H->out, H->s);
+    }));
+    double mx = 0.0, l2 = 0.0, scale = 1.0;
+    ma_status st = read_norms2(H, &mx, &l2);
     if (st != MA_OK) return st;
+    if (o->relative != MA_REL_NONE) scale = o->norm == MA_NORM_MAX ? H->host[2] : H->host[3];
+    if (!(scale > 0.0)) scale = 1.0;
     double rel = (o->norm == MA_NORM_MAX ? mx : l2) / scale;
     res->res0 = rel;
     int stagnant = 0;
@@ -707,9 +1156,13 @@ ma_status ma2d_solve(ma2d_hierarchy* H, const ma_solve_opts* o, ma_solve_result*
     // sum of squares does not, so both are checked
     while (std::isfinite(rel) && std::isfinite(l2) && rel > o->tol && res->cycles < o->max_cycles &&
            stagnant < ma::kFloorStagnantCycles) {
-        CK2(vcycle2_from(H, 0));
+        CK2(run_graph2(H, H->g_cycle, [&]() -> cudaError_t {
+            auto& F = H->lev[0];
+            const cudaError_t e = vcycle2_from(H, 0);
+            return e != cudaSuccess ? e : norms2(F.u, F.rhs, F.n, F.h, H->partials, H->out, H->s);
+        }));
         res->cycles += 1;
-        if ((st = fine_norms2(H, 0, &mx, &l2)) != MA_OK) return st;
+        if ((st = read_norms2(H, &mx, &l2)) != MA_OK) return st;
         const double nrel = (o->norm == MA_NORM_MAX ? mx : l2) / scale;
         stagnant = nrel > 0.8 * rel ? stagnant + 1 : 0;
         rel = nrel;
@@ -742,14 +1195,16 @@ ma_status ma2d_smooth(double* u, const double* rhs, int n, double h, int nsweeps
     if (!u || !rhs || !valid_n2(n) || !(h > 0.0) || nsweeps < 0 ||
         (ordering != MA2D_REDBLACK && ordering != MA2D_COLOUR4) || (ordering == MA2D_REDBLACK && !scratch))
         return fail2(MA_ERR_INVALID_ARG, "ma2d_smooth: bad arguments");
-    CK2(smooth2(u, scratch, rhs, n, h, nsweeps, ordering, events, (cudaStream_t)stream));
+    CK2(smooth2(u, scratch, rhs, n, h, nsweeps, ordering, false, events, (cudaStream_t)stream));
     return MA_OK;
 }
 
 ma_status ma2d_residual(const double* u, const double* rhs, double* r, int n, double h, ma_stream_t stream)
 {
     if (!u || !rhs || !r || !valid_n2(n) || !(h > 0.0)) return fail2(MA_ERR_INVALID_ARG, "ma2d_residual: bad arguments");
-    CK2(residual2(u, rhs, r, n, h, nullptr, (cudaStream_t)stream));
+    ma::count_launches(1);
+    k_resid2<<<grid2(n, n), dim3(TX, TY), 0, (cudaStream_t)stream>>>(u, rhs, r, n, 1.0 / (h * h));
+    CK2(cudaGetLastError());
     return MA_OK;
 }
 

@@ -144,3 +144,31 @@ def test_table1_reproduced_on_the_gpu_up_to_8192():
         # 5 %, plus half a unit of the table's second significant digit
         half_unit = 0.05 * 10.0 ** np.floor(np.log10(err))
         assert abs(e - err) <= 0.05 * err + half_unit, (ex, N, e, err)
+
+
+@pytest.mark.parametrize("scale,shift", [(1.0, 0.0), (2.0 ** -12, 0.0), (1.0, -1.3)])
+@pytest.mark.parametrize("n,opts", [
+    (3, dict()), (5, dict()), (9, dict(coarsest_n=5)), (17, dict(coarsest_n=17)), (33, dict()),
+    (65, dict(ordering=2, coarsest_n=9, coarse_sweeps=2, nu1=1, nu2=3)),
+    (33, dict(ordering=2, approx_restrict=0)), (129, dict(coarsest_n=17, coarse_sweeps=3, restrict_kind=1)),
+])
+def test_cycles_from_a_zero_interior_match_oracle(n, opts, scale, shift):
+    """Two cycles over small grids (those of one block, and above), their options, and
+    values that cross zero and binades.  Every form rounds a point's change to 2^-40 of
+    its differences or to eps |u| in the oracle, and a cycle passes such errors on
+    without growth: 1e-11 of max |u| stands over both, a phase or point left out is
+    1e-4 and more."""
+    pr = P2.make2d("ex1", n)
+    g = scale * (pr.initial() + shift)
+    g[1:-1, 1:-1] = 0.0
+    f = scale * scale * pr.f
+    H = M.Hierarchy2D(M.make_desc2d(n, **opts))
+    H.set_rhs_bc(dev(f), dev(g))
+    H.solve(tol=0.0, max_cycles=2, init=M.MA_INIT_ZERO, raise_on_error=False)
+    u = torch.empty((n, n), dtype=torch.float64, device="cuda")
+    H.get_solution(u)
+    got = host(u)
+    H.close()
+    ref = g.copy()
+    O2.solve(ref, f, pr.h, tol=0.0, max_cycles=2, init_fmg=False, params=O2.Params2D(**opts))
+    assert np.max(np.abs(got - ref)) <= 1e-11 * np.max(np.abs(ref))
