@@ -109,7 +109,7 @@ __device__ __forceinline__ void smooth_f2_block(double* u, const double* __restr
     const int j = ((C & 2) ? 1 : 2) + 2 * (int)(blockIdx.y * BY + threadIdx.y);
     const int k = ((C & 4) ? 1 : 2) + 2 * bz;
     if (i > n - 2 || j > n - 2 || k > n - 2) return;
-    smoothf2::point<UNORM, long long>(u, rhs, lin(i, j, k, n), n, (long long)n * n, P, events);
+    smoothf2::point<UNORM, UNORM ? resid::kDirect : resid::kSmall, long long>(u, rhs, lin(i, j, k, n), n, (long long)n * n, P, events);
 }
 
 template <int C, int D, int NN, bool UNORM>
@@ -140,6 +140,156 @@ cudaError_t launch_smooth_f2(double* u, const double* rhs, int n, const smoothf2
     }
     return cudaGetLastError();
 }
+
+// ---------------------------------------------------------------------------
+// Sweeps of a 33^3 grid in one cluster of 16 thread blocks.  A phase there is
+// one point's dependent chain (3400 cycles with the general gather, of which
+// 1900 the gather) and a launch: 7 launches a sweep, 2.7 us each.  Two sweeps in
+// one launch: 38 -> 29 us.  Block m holds planes 2m .. 2m + 3 of u in shared memory
+// and owns the middle two, an odd and an even one; a point's new value also
+// goes to the neighbour that holds its plane, and a cluster barrier ends the
+// phase.  Rows are kept with the even i first, so that the points of a phase
+// are contiguous.  Same point update in the same order as the launches, whose
+// gather may take the other exact form.
+// ---------------------------------------------------------------------------
+namespace sweep33 {
+
+constexpr int N = 33, KC = 16, TC = 512;
+constexpr int RS = 34, PS = N * RS;      // row: 17 even places, then 16 odd ones
+constexpr int kSmem = 6 * PS * (int)sizeof(double);
+
+__device__ __forceinline__ int place(int i) { return (i & 1) * 17 + (i >> 1); }
+
+// The value at offset o = di + N dj + N^2 dk of a point, all in -1 .. 1: q is
+// the point's row, x its place and xm, xp those of i - 1 and i + 1.
+struct At {
+    const double* q;
+    int x, xm, xp;
+    __device__ __forceinline__ double operator()(int o) const
+    {
+        const int w = o + 1 + N + N * N, di = w % N - 1, dj = w / N % N - 1, dk = w / (N * N) - 1;
+        return q[dk * PS + dj * RS + (di == 0 ? x : (di < 0 ? xm : xp))];
+    }
+};
+
+__device__ __noinline__ double point_f64(At at, double rhs6, bool* nonconvex)
+{
+    const double v0 = at(0);
+    const HessS H = gather_hess_of(at, N, N * N, v0);
+    return fma(0.125, smallest_root(H, rhs6, nonconvex), v0);
+}
+
+__device__ __forceinline__ unsigned rank()
+{
+    unsigned r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+
+__device__ __forceinline__ void barrier()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+__device__ __forceinline__ void store_remote(const double* smem, unsigned block, double v)
+{
+    unsigned a = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("mapa.shared::cluster.u32 %0, %0, %1;\n" : "+r"(a) : "r"(block));
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
+
+__global__ void __launch_bounds__(TC, 1) k_sweeps(double* u, const double* __restrict__ rhs, smoothf2::Params P,
+                                                  int nsweeps, unsigned long long* events)
+{
+    extern __shared__ double csm[];
+    double *su = csm, *sr = csm + 4 * PS;
+    const int m = (int)rank();
+    for (int t = threadIdx.x; t < 4 * N * N; t += TC) {
+        const int lp = t / (N * N), r = t - lp * N * N, j = r / N, i = r - j * N, k = 2 * m + lp;
+        if (k >= N) continue;
+        const int at = j * RS + place(i);
+        su[lp * PS + at] = u[k * N * N + r];
+        if (lp == 1 || lp == 2) sr[(lp - 1) * PS + at] = __ldg(rhs + k * N * N + r);
+    }
+    barrier();   // every block is running before another writes to it
+    const int half = threadIdx.x >> 8, a = threadIdx.x & 15, b = (threadIdx.x >> 4) & 15;
+    unsigned long long ev = 0;
+    for (int q = 0, w = 0; q < 7 * nsweeps; ++q, w = w == 6 ? 0 : w + 1) {
+        const int c = half == 0 ? phase_first(false, w) : phase_second(false, w);
+        const int i = ((c & 1) ? 1 : 2) + 2 * a, j = ((c & 2) ? 1 : 2) + 2 * b, lp = (c & 4) ? 1 : 2;
+        if (c >= 0 && i <= N - 2 && j <= N - 2 && 2 * m + lp <= N - 2) {
+            const At at{su + lp * PS + j * RS, place(i), place(i - 1), place(i + 1)};
+            const double bv = sr[(lp - 1) * PS + j * RS + at.x];
+            double v;
+            if (!smoothf2::update<true, resid::kSmall, int>(
+                    [&](int o) -> long long { return __double_as_longlong(at(o)); }, N, N * N, bv, P, &v)) {
+                bool nonconvex = false;
+                v = point_f64(at, __dmul_rn(P.h6, bv), &nonconvex);
+                ev += nonconvex ? 1 : 0;
+            }
+            double* p = su + lp * PS + j * RS + at.x;
+            *p = v;
+            if (lp == 1 && m > 0) store_remote(p + 2 * PS, m - 1, v);
+            if (lp == 2 && m < KC - 1) store_remote(p - 2 * PS, m + 1, v);
+        }
+        barrier();
+    }
+    for (int t = threadIdx.x; t < 2 * N * N; t += TC) {
+        const int lp = 1 + t / (N * N), r = t - (lp - 1) * N * N, j = r / N, i = r - j * N, k = 2 * m + lp;
+        if (i < 1 || j < 1 || i > N - 2 || j > N - 2 || k > N - 2) continue;
+        u[k * N * N + r] = su[lp * PS + j * RS + place(i)];
+    }
+    if (events && ev) atomicAdd(events, ev);
+}
+
+cudaLaunchConfig_t config(cudaLaunchAttribute* at, cudaStream_t s)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(KC);
+    cfg.blockDim = dim3(TC);
+    cfg.dynamicSmemBytes = kSmem;
+    cfg.stream = s;
+    at->id = cudaLaunchAttributeClusterDimension;
+    at->val.clusterDim.x = KC;
+    at->val.clusterDim.y = at->val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+// Whether the current device runs such a cluster; the answer and the kernel's
+// limits are set once per device.
+bool ready()
+{
+    static std::atomic<signed char> known[64];   // 0: not asked, 1: yes, -1: no
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+    signed char k = known[dev].load(std::memory_order_acquire);
+    if (k == 0) {
+        cudaLaunchAttribute at{};
+        const cudaLaunchConfig_t cfg = config(&at, nullptr);
+        int clusters = 0;
+        const bool ok =
+            cudaFuncSetAttribute(k_sweeps, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) == cudaSuccess &&
+            cudaFuncSetAttribute(k_sweeps, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+            cudaOccupancyMaxActiveClusters(&clusters, k_sweeps, &cfg) == cudaSuccess && clusters > 0;
+        if (!ok) (void)cudaGetLastError();
+        k = ok ? 1 : -1;
+        known[dev].store(k, std::memory_order_release);
+    }
+    return k > 0;
+}
+
+cudaError_t launch(double* u, const double* rhs, const smoothf2::Params& P, int nsweeps, unsigned long long* events,
+                   cudaStream_t s)
+{
+    cudaLaunchAttribute at{};
+    const cudaLaunchConfig_t cfg = config(&at, s);
+    count_launches(1);
+    return cudaLaunchKernelEx(&cfg, k_sweeps, u, rhs, P, nsweeps, events);
+}
+
+}  // namespace sweep33
 
 // ---------------------------------------------------------------------------
 // Block reduction of (max |x|, sum x^2) in a fixed order (deterministic).
@@ -222,13 +372,13 @@ __global__ void __launch_bounds__(BX * BY) k_coarse_rhs(const double* __restrict
 // r + det(D^2_h u) (SIGN = 1, the coarse right-hand side) or r - det (SIGN = -1,
 // the residual) at a point, with exact integer second differences and a
 // two-float determinant; ld as gather_f2_of takes it.
-template <int SIGN, bool UNORM, bool SMALL, typename Idx, typename Ld>
+template <int SIGN, bool UNORM, int FORM, typename Idx, typename Ld>
 __device__ __forceinline__ double operator_of(Ld ld, Idx sy, Idx sz, double rv, double inv_h6)
 {
     using namespace resid;
     f2::F2 H[6];
     long long b0;
-    if (gather_f2_of<SMALL, Idx>(ld, sy, sz, 0, H, &b0)) {
+    if (gather_f2_of<FORM, Idx>(ld, sy, sz, 0, H, &b0)) {
         const float ih = (float)(SIGN * inv_h6);
         const f2::F2 d = f2::mul(f2::det3<UNORM>(H[0], H[1], H[2], H[3], H[4], H[5]),
                                  f2::F2{ih, (float)(SIGN * inv_h6 - (double)ih)});
@@ -243,7 +393,7 @@ __device__ __forceinline__ double operator_of(Ld ld, Idx sy, Idx sz, double rv, 
 template <int SIGN, bool UNORM>
 __device__ __forceinline__ double operator_point(const double* q, int sy, int sz, double rv, double inv_h6)
 {
-    return operator_of<SIGN, UNORM, true, int>([q](int o) -> long long { return __double_as_longlong(q[o]); }, sy, sz, rv,
+    return operator_of<SIGN, UNORM, resid::kSmall, int>([q](int o) -> long long { return __double_as_longlong(q[o]); }, sy, sz, rv,
                                          inv_h6);
 }
 
@@ -269,7 +419,7 @@ __global__ void __launch_bounds__(BX * BY) k_operator_f2(const double* __restric
         return;
     }
     const long long* q = reinterpret_cast<const long long*>(u) + p;
-    out[p] = operator_of<SIGN, UNORM, !UNORM, long long>([q](long long o) -> long long { return __ldg(q + o); }, n, sz,
+    out[p] = operator_of<SIGN, UNORM, UNORM ? resid::kDirect : resid::kSmall, long long>([q](long long o) -> long long { return __ldg(q + o); }, n, sz,
                                                  __ldg(r + p), inv_h6);
 }
 
@@ -978,6 +1128,7 @@ cudaError_t launch_smooth(double* u, const double* rhs, int n, double h, int nsw
 {
     const smoothf2::Params P = smoothf2::make_params(h);
     if (n >= kF2MinN && P.kexp != smoothf2::kNone) {
+        if (n == sweep33::N && nsweeps > 0 && sweep33::ready()) return sweep33::launch(u, rhs, P, nsweeps, events, s);
         for (int sw = 0; sw < nsweeps; ++sw) {
             cudaError_t e;
             if ((e = launch_smooth_f2<0, 0>(u, rhs, n, P, events, s)) != cudaSuccess) return e;

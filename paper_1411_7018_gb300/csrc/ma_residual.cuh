@@ -310,9 +310,13 @@ struct ResF2 {
 // point, sy and sz are the offsets of a step in j and k.  false (H unset) where
 // the stencil's largest value is zero, huge or tiny.  -20 <= kexp <= 40 keeps
 // every scaled unit inside FP32's range.
-// SMALL: for the smaller grids, where most warps meet a change of binade: the
-// general form at once.
-template <bool SMALL = false, typename Idx, typename Ld>
+// FORM, how a warp that meets a change of binade is served: kDirect, for grids
+// that fill the GPU: stencils of one binade first, the general form for the
+// rest; kSmall, for grids where most warps meet one and a phase is one point's
+// chain: all by a left shift where it serves the warp.
+enum Form { kDirect, kSmall };
+
+template <int FORM = kDirect, typename Idx, typename Ld>
 __device__ __forceinline__ bool gather_f2_of(Ld ld, Idx sy, Idx sz, int kexp, f2::F2* H, long long* centre)
 {
     const long long b0 = ld(0);
@@ -334,7 +338,7 @@ __device__ __forceinline__ bool gather_f2_of(Ld ld, Idx sy, Idx sz, int kexp, f2
     int sign = (int)(h0 & 0x80000000u);   // the ulp of the binade, negated for negative values
     // a quarter of the diagonal entries, and the off-diagonal ones, in ulps
     long long A, B, C, R, S, T;
-    if (!SMALL && (diff >> 20) == 0) {
+    if (FORM == kDirect && (diff >> 20) == 0) {
         if (E < f2::kMinE || E > f2::kMaxE) return false;
         A = (bxp - b0) + (bxm - b0);
         B = (byp - b0) + (bym - b0);
@@ -357,11 +361,6 @@ __device__ __forceinline__ bool gather_f2_of(Ld ld, Idx sy, Idx sz, int kexp, f2
                                  max4(tpp, tmm, tpm, tmp));
         E = (int)(top >> 20);
         if (E < f2::kMinE || E > f2::kMaxE) return false;
-        // (zeros and denormals shift out with the rest: E exceeds 63 by far)
-        auto fix = [E](long long b) -> long long {
-            const long long m = (b & 0x000FFFFFFFFFFFFFll) | 0x0010000000000000ll;
-            return (m << 7) >> min(E - (int)((b >> 52) & 0x7ff), 63);
-        };
         auto sums = [&](auto g) {
             const long long m0 = g(b0);
             A = (g(bxp) - m0) + (g(bxm) - m0);
@@ -371,14 +370,35 @@ __device__ __forceinline__ bool gather_f2_of(Ld ld, Idx sy, Idx sz, int kexp, f2
             S = (g(spp) - g(smp)) - (g(spm) - g(smm));
             T = (g(tpp) - g(tmp)) - (g(tpm) - g(tmm));
         };
-        if (!__any_sync(__activemask(), (int)diff < 0)) {   // one sign each: the unit carries it
+        // (zeros and denormals shift out with the rest: E exceeds 63 by far)
+        auto fix = [E](long long b) -> long long {
+            const long long m = (b & 0x000FFFFFFFFFFFFFll) | 0x0010000000000000ll;
+            return (m << 7) >> min(E - (int)((b >> 52) & 0x7ff), 63);
+        };
+        // all of one sign (the unit carries it) and within seven binades: a left
+        // shift, a third fewer instructions, but 16 registers more (129^3: 48 us
+        // the right-hand side with it, 36 without)
+        const int low = E - 7 + (int)((h0 >> 20) & 0x800);
+        auto left = [low](long long b) { return (int)((unsigned)(b >> 32) >> 20) - low; };
+        bool near = false;
+        if (FORM == kSmall) {
+            const int far = (left(bxp) | left(bxm) | left(byp)) | (left(bym) | left(bzp) | left(bzm)) |
+                            (left(rpp) | left(rmm) | left(rpm)) | (left(rmp) | left(spp) | left(smm)) |
+                            (left(spm) | left(smp) | left(tpp)) | (left(tmm) | left(tpm) | left(tmp)) | left(b0);
+            near = !__any_sync(__activemask(), (unsigned)far > 7u);
+        }
+        if (near) {
+            sums([&](long long b) { return ((b & 0x000FFFFFFFFFFFFFll) | 0x0010000000000000ll) << left(b); });
+        } else if (FORM == kDirect && !__any_sync(__activemask(), (int)diff < 0)) {
             sums(fix);
         } else {
+            // (left shifts about: a stencil of one sign keeps its unit's sign whatever its warp's others hold)
+            const long long mixed = FORM == kSmall ? (int)diff >> 31 : -1;
             sums([&](long long b) {
-                const long long v = fix(b), neg = b >> 63;
+                const long long v = fix(b), neg = (b >> 63) & mixed;
                 return (v ^ neg) - neg;
             });
-            sign = 0;
+            sign &= (int)~mixed;
         }
         E -= 7;
     }
@@ -390,7 +410,7 @@ __device__ __forceinline__ bool gather_f2_of(Ld ld, Idx sy, Idx sz, int kexp, f2
 #define MA_F2_HW(x) big |= (int)((x) >> 32) ^ (int)((x) >> 63)
     MA_F2_HW(A); MA_F2_HW(B); MA_F2_HW(C); MA_F2_HW(R); MA_F2_HW(S); MA_F2_HW(T);
 #undef MA_F2_HW
-    if (!SMALL && big < (1 << 13)) {
+    if (FORM == kDirect && big < (1 << 13)) {
         const float u23 = 8388608.0f * unit, u423 = 8388608.0f * unit4;
         H[0] = f2::from_i45(A, unit4, u423);
         H[1] = f2::from_i45(B, unit4, u423);
@@ -416,7 +436,7 @@ __device__ __forceinline__ bool gather_f2(const double* __restrict__ u, Idx p, I
                                           long long* centre)
 {
     const long long* q = reinterpret_cast<const long long*>(u) + p;
-    return gather_f2_of<false, Idx>([q](Idx o) -> long long { return __ldg(q + o); }, sy, sz, kexp, H, centre);
+    return gather_f2_of<kDirect, Idx>([q](Idx o) -> long long { return __ldg(q + o); }, sy, sz, kexp, H, centre);
 }
 
 template <bool UNORM = false>

@@ -86,14 +86,14 @@ __device__ __forceinline__ resid::f2::F2 shift(resid::f2::F2 a, float z)
 // false: the point needs the FP64 form.  UNORM: det3's sums unnormalised, which
 // saves 15 operations and leaves the root's residual to about 2^-45 of the
 // entries' cube in place of 2^-46; that is below an ulp of u from 33^3 up.
-template <bool UNORM, bool SMALL, typename Idx, typename Ld>
+template <bool UNORM, int FORM, typename Idx, typename Ld>
 __device__ __forceinline__ bool update(Ld ld, Idx sy, Idx sz, double b, const Params& P, double* v)
 {
     using namespace resid;
     f2::F2 H[6];
     long long b0;
     // rhs > 0 by its bits (NaN passes and fails to converge below)
-    if (!gather_f2_of<SMALL, Idx>(ld, sy, sz, P.kexp, H, &b0) || __double_as_longlong(b) <= 0) return false;
+    if (!gather_f2_of<FORM, Idx>(ld, sy, sz, P.kexp, H, &b0) || __double_as_longlong(b) <= 0) return false;
     const f2::F2 r6 = f2::mul(f2::from_f64(b), f2::F2{P.chi, P.clo});
     HessSf F;
     F.A = H[0].hi; F.B = H[1].hi; F.C = H[2].hi;
@@ -128,14 +128,14 @@ __device__ __forceinline__ bool update(Ld ld, Idx sy, Idx sz, double b, const Pa
 }
 
 // A point of a grid in global memory, in place.
-template <bool UNORM, typename Idx>
+template <bool UNORM, int FORM, typename Idx>
 __device__ __forceinline__ void point(double* u, const double* __restrict__ rhs, Idx p, Idx sy, Idx sz,
                                       const Params& P, unsigned long long* events)
 {
     const long long* q = reinterpret_cast<const long long*>(u) + p;
     const double b = __ldg(rhs + p);
     double v;
-    if (update<UNORM, !UNORM, Idx>([q](Idx o) -> long long { return __ldg(q + o); }, sy, sz, b, P, &v)) {
+    if (update<UNORM, FORM, Idx>([q](Idx o) -> long long { return __ldg(q + o); }, sy, sz, b, P, &v)) {
         u[p] = v;   // (one store after both forms: 10 % slower at 257^3)
         return;
     }
@@ -149,7 +149,7 @@ __device__ __forceinline__ double point_sm(const double* q, int sy, int sz, doub
 {
     double v;
     if (P.kexp != kNone &&
-        update<false, true, int>([q](int o) -> long long { return __double_as_longlong(q[o]); }, sy, sz, b, P, &v))
+        update<false, resid::kSmall, int>([q](int o) -> long long { return __double_as_longlong(q[o]); }, sy, sz, b, P, &v))
         return v;
     return point_f64(q, sy, sz, __dmul_rn(P.h6, b), nonconvex);
 }
