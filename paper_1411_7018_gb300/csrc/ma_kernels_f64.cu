@@ -294,22 +294,32 @@ cudaError_t launch(double* u, const double* rhs, const smoothf2::Params& P, int 
 // ---------------------------------------------------------------------------
 // Block reduction of (max |x|, sum x^2) in a fixed order (deterministic).
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void block_reduce_store(double mx, double ss, double* partials, int slot)
+__device__ __forceinline__ void block_reduce_store(unsigned long long mx, double ss, double* partials, int slot)
 {
-    __shared__ double smx[BX * BY / 32], sss[BX * BY / 32];
+    __shared__ unsigned long long smx[BX * BY / 32];
+    __shared__ double sss[BX * BY / 32];
     for (int o = 16; o > 0; o >>= 1) {
-        mx = fmax(mx, __shfl_down_sync(0xffffffffu, mx, o));
+        mx = max(mx, __shfl_down_sync(0xffffffffu, mx, o));
         ss += __shfl_down_sync(0xffffffffu, ss, o);
     }
     const int t = threadIdx.y * BX + threadIdx.x;
     if ((t & 31) == 0) { smx[t >> 5] = mx; sss[t >> 5] = ss; }
     __syncthreads();
     if (t == 0) {
-        double m = smx[0], q = sss[0];
-        for (int w = 1; w < BX * BY / 32; ++w) { m = fmax(m, smx[w]); q += sss[w]; }
-        partials[2 * slot] = m;
+        unsigned long long m = smx[0];
+        double q = sss[0];
+        for (int w = 1; w < BX * BY / 32; ++w) { m = max(m, smx[w]); q += sss[w]; }
+        partials[2 * slot] = __longlong_as_double((long long)m);
         partials[2 * slot + 1] = q;
     }
+}
+
+// x in FP64, by integer operations where it is normal or zero
+__device__ __forceinline__ double widen(double x) { return x; }
+__device__ __forceinline__ double widen(float x)
+{
+    const unsigned b = __float_as_uint(x) & 0x7fffffffu;
+    return b == 0 || b - 0x00800000u < 0x7f000000u ? f2d(x) : (double)x;
 }
 
 constexpr int KZ = 16;   // z-blocks of the reduction grids; each loops over k
@@ -322,11 +332,12 @@ __device__ __forceinline__ void norm_partials_block(const T* __restrict__ v, int
 {
     const int i = bid.x * BX + threadIdx.x;
     const int j = bid.y * BY + threadIdx.y;
-    double mx = 0.0, ss = 0.0;
-    for (int k = bid.z; k < n; k += gdim.z) {
-        if (i > 0 && j > 0 && k > 0 && i < n - 1 && j < n - 1 && k < n - 1) {
-            const double x = (double)v[lin(i, j, k, n)];
-            mx = fmax(mx, fabs(x));
+    unsigned long long mx = 0;
+    double ss = 0.0;
+    if (i > 0 && j > 0 && i < n - 1 && j < n - 1) {
+        for (int k = bid.z == 0 ? (int)gdim.z : (int)bid.z; k < n - 1; k += gdim.z) {
+            const double x = widen(v[lin(i, j, k, n)]);
+            mx = resid::max_bits(mx, x);
             ss = fma(x, x, ss);
         }
     }

@@ -123,6 +123,15 @@ __global__ void __launch_bounds__(RX * RY) k_residual_col(const double* __restri
     residual_col_block<Out>(u, rhs, out, n, inv_h6, partials, kchunk, blockIdx, gridDim);
 }
 
+// The larger of a magnitude m and |x| as their bit patterns, which order like
+// the values; a NaN is passed over, as fmax does.  (An FP64 maximum holds the
+// FP64 pipe as long as an addition.)
+__device__ __forceinline__ unsigned long long max_bits(unsigned long long m, double x)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
+    return b > m && b <= 0x7ff0000000000000ull ? b : m;
+}
+
 // One block of NF = 256 threads folds the (max, sum of squares) partials in
 // a fixed order: out2 = (max, sqrt(h^3 sum)), the max and discrete L2 norms
 // of the stopping rule (Section 4).
@@ -131,10 +140,12 @@ constexpr int NF = 256;
 __device__ __forceinline__ void norm_final_block(const double* __restrict__ partials, int count, double h3,
                                                  double* out2)
 {
-    __shared__ double smx[NF], sss[NF];
-    double mx = 0.0, ss = 0.0;
+    __shared__ unsigned long long smx[NF];
+    __shared__ double sss[NF];
+    unsigned long long mx = 0;
+    double ss = 0.0;
     for (int q = threadIdx.x; q < count; q += NF) {
-        mx = fmax(mx, partials[2 * q]);
+        mx = max_bits(mx, partials[2 * q]);
         ss += partials[2 * q + 1];
     }
     smx[threadIdx.x] = mx;
@@ -142,13 +153,13 @@ __device__ __forceinline__ void norm_final_block(const double* __restrict__ part
     __syncthreads();
     for (int w = NF / 2; w > 0; w >>= 1) {
         if ((int)threadIdx.x < w) {
-            smx[threadIdx.x] = fmax(smx[threadIdx.x], smx[threadIdx.x + w]);
+            smx[threadIdx.x] = max(smx[threadIdx.x], smx[threadIdx.x + w]);
             sss[threadIdx.x] += sss[threadIdx.x + w];
         }
         __syncthreads();
     }
     if (threadIdx.x == 0) {
-        out2[0] = smx[0];
+        out2[0] = __longlong_as_double((long long)smx[0]);
         out2[1] = sqrt(h3 * sss[0]);
     }
 }
