@@ -554,3 +554,29 @@ def test_coarsest_5_converges_to_the_swept_solution(name, length, start):
     u = dev(u0)
     M.ma_coarsest_solve(u, dev(f), n, h, 0)
     assert np.max(np.abs(host(u) - ref)) <= 1e-12 * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("n", [33, 35, 67])   # from 33 up: sums of bit patterns where a point's 27 values share a binade
+@pytest.mark.parametrize("lo,hi", [(1.0, 2.0), (-1.9, -1.1), (0.25, 3.0), (-1.0, 1.0), (0.0, 0.0), (1e-308, 2e-308)])
+def test_solution_restriction_is_the_exact_weighted_mean(n, lo, hi):
+    """The 27-point weighting against the exact mean rounded once (FP64 split into
+    integers): a form of the exact sum is within half an ulp of it, one in FP64
+    additions within 16 roundings of the largest value."""
+    from fractions import Fraction
+    rng = np.random.default_rng(5)
+    u = lo + (hi - lo) * rng.random((n, n, n))
+    nc = (n + 1) // 2
+    out = torch.empty((nc, nc, nc), dtype=torch.float64, device="cuda")
+    M.ma_restrict_solution(dev(u), n, out, M.MA_APPROX_WEIGHTED, M.MA_FULL_WEIGHTING)
+    got = host(out)
+    for K, J, I in [(1, 1, 1), (nc - 2, nc - 2, nc - 2)] + [tuple(rng.integers(1, nc - 1, 3)) for _ in range(60)]:
+        b = u[2 * K - 1:2 * K + 2, 2 * J - 1:2 * J + 2, 2 * I - 1:2 * I + 2]
+        w = np.array([1, 2, 1])
+        w = w[:, None, None] * w[None, :, None] * w[None, None, :]
+        exact = sum(Fraction(float(x)) * int(c) for x, c in zip(b.ravel(), w.ravel())) / 64
+        one = np.all(np.frexp(b)[1] == np.frexp(b)[1].ravel()[0]) and (np.all(b > 0) or np.all(b < 0))
+        big = float(np.max(np.abs(b)))
+        if one and big > 1e-300:
+            assert got[K, J, I] == float(exact)
+        else:
+            assert abs(Fraction(float(got[K, J, I])) - exact) <= Fraction(16 * EPS * big) + Fraction(5e-324) * 64
