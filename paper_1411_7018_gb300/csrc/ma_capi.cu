@@ -240,12 +240,13 @@ cudaError_t refresh_base(ma_hierarchy* H, int apply, int l0)
     cudaError_t e;
     ma::Level& F = H->lev[l0];
     if ((e = ma::launch_update(F.u, F.e, F.n, apply, s)) != cudaSuccess) return e;
+    ma::RefreshSpec lv[ma::kRefreshLevels];
+    int nlev = 0;
     for (int l = l0 + 1; l < H->L; ++l) {
         ma::Level& A = H->lev[l];
-        if ((e = ma::launch_split_inject(F.u, F.n, 1 << (l - l0), A.hi, A.lo, A.n, s)) != cudaSuccess) return e;
-        if ((e = ma::launch_base_colour(A.hi, A.lo, A.bstore, A.n, A.h, s)) != cudaSuccess) return e;
+        lv[nlev++] = ma::RefreshSpec{A.n, 1 << (l - l0), A.h, A.hi, A.lo, A.bstore};
     }
-    return cudaSuccess;
+    return ma::launch_refresh(F.u, F.n, lv, nlev, s);
 }
 
 // First level of the cycles from l0 that the cluster launch takes (33^3 or

@@ -146,7 +146,16 @@ cudaError_t launch_f32_to_f64(const float* e, double* u, int n, cudaStream_t s);
 cudaError_t launch_interpolate_f32(const float* ec, int nc, float* ef, cudaStream_t s);
 cudaError_t launch_zero_interior_f32(float* e, int n, cudaStream_t s);
 cudaError_t launch_norm_partials_f32(const float* v, int n, double* partials, cudaStream_t s);
-cudaError_t launch_split_inject(const double* u0, int n0, int stride, float* hi, float* lo, int nc, cudaStream_t s);
+// The coarse correction levels' hi/lo splits of the iterate u0 (n0^3, every
+// stride-th point) and their base Hessians from them.
+struct RefreshSpec {
+    int n, stride;
+    double h;
+    float *hi, *lo;
+    void* bstore;
+};
+constexpr int kRefreshLevels = 16;
+cudaError_t launch_refresh(const double* u0, int n0, const RefreshSpec* lv, int nlev, cudaStream_t s);
 cudaError_t launch_residual64_to32(const double* u, const double* rhs, float* r_cm, void* bstore, int n, double h,
                                    double* partials, cudaStream_t s);
 
