@@ -384,10 +384,69 @@ __device__ __forceinline__ void base_colour_block(const float* __restrict__ hi, 
     b[5 * c.cnt] = B.yz;
 }
 
+// The same over kc planes of a column a thread: of a point's 19 values nine are
+// loaded for it, the others were loaded for the planes before (151^3: 39 ->
+// 34.5 us; the coarse levels of a 513^3 solve 972 -> 764 us a solve).
+__device__ __forceinline__ void base_colour_col_block(const float* __restrict__ hi, const float* __restrict__ lo,
+                                                      float* __restrict__ bstore, int n, float inv_h2, int kc,
+                                                      uint3 bid)
+{
+    const int i = bid.x * BX + threadIdx.x;
+    const int j = bid.y * BY + threadIdx.y;
+    const int k0 = 1 + (int)bid.z * kc, k1 = min(n - 2, k0 + kc - 1);
+    if (i < 1 || j < 1 || i > n - 2 || j > n - 2) return;
+    const long long sy = n, sz = (long long)n * n;
+    long long p = lin(i, j, k0, n);
+    auto ld = [&](long long o) -> HiLo { return {__ldg(hi + o), __ldg(lo + o)}; };
+    struct Cross {
+        HiLo c, xp, xm, yp, ym;
+    };
+    auto cross = [&](long long o) -> Cross { return {ld(o), ld(o + 1), ld(o - 1), ld(o + sy), ld(o - sy)}; };
+    const int pi = i & 1, pj = j & 1;
+    const int ni = colour_count(n, pi), nj = colour_count(n, pj);
+    // this column's two colour boxes (k even, odd)
+    const long long plane = (long long)ni * nj, row = ((j - (pj ? 1 : 2)) >> 1) * ni + ((i - (pi ? 1 : 2)) >> 1);
+    const long long cnt0 = plane * colour_count(n, 0), cnt1 = plane * colour_count(n, 1);
+    float* b0 = bstore + 6 * cm_offset(n, pi | (pj << 1)) + ((k0 - 1) >> 1) * plane + row;
+    float* b1 = bstore + 6 * cm_offset(n, pi | (pj << 1) | 4) + (k0 >> 1) * plane + row;
+    Cross m = cross(p - sz), c = cross(p);
+    for (int k = k0; k <= k1; ++k, p += sz) {
+        const Cross q = cross(p + sz);
+        const HiLo pp = ld(p + sy + 1), pm = ld(p - sy + 1), mp = ld(p + sy - 1), mm = ld(p - sy - 1);
+        const S3f B = hess_of(
+            [&](int di, int dj, int dk) -> HiLo {
+                if (dk == 0 && di != 0 && dj != 0) return di > 0 ? (dj > 0 ? pp : pm) : (dj > 0 ? mp : mm);
+                const Cross& w = dk == 0 ? c : (dk > 0 ? q : m);
+                return di > 0 ? w.xp : (di < 0 ? w.xm : (dj > 0 ? w.yp : (dj < 0 ? w.ym : w.c)));
+            },
+            inv_h2);
+        const long long cnt = (k & 1) ? cnt1 : cnt0;
+        float* b = (k & 1) ? b1 : b0;
+        if (k & 1) b1 += plane;
+        else b0 += plane;
+        b[0] = B.xx;
+        b[cnt] = B.yy;
+        b[2 * cnt] = B.zz;
+        b[3 * cnt] = B.xy;
+        b[4 * cnt] = B.xz;
+        b[5 * cnt] = B.yz;
+        m = c;
+        c = q;
+    }
+}
+
+// Planes a thread: one where a grid has too few columns to fill the GPU.
+__host__ __device__ inline int base_chunk(int n) { return n >= 65 ? 8 : 1; }
+dim3 base_grid(int n)
+{
+    const int kc = base_chunk(n);
+    return dim3((n + BX - 1) / BX, (n + BY - 1) / BY, (n - 2 + kc - 1) / kc);
+}
+
 __global__ void __launch_bounds__(BX * BY) k_base_colour(const float* __restrict__ hi, const float* __restrict__ lo,
                                                          float* __restrict__ bstore, int n, float inv_h2)
 {
-    base_colour_block(hi, lo, bstore, n, inv_h2, blockIdx);
+    base_colour_col_block(hi, lo, bstore, n, inv_h2, base_chunk(n), blockIdx);
 }
 
 // Natural-layout interior values -> colour-major order.
@@ -1984,7 +2043,7 @@ __device__ __forceinline__ void split_inject_block(const double* __restrict__ u0
 // Most levels are small, and two launches a level took 1.4 - 2.2 us each
 // whatever their size (33^3 solve with both: 857 -> 806 us, 129^3: 2.45 -> 2.38 ms).
 struct RefreshLevel {
-    int first;          // first block
+    int first[2];       // first block of the split and of the base launch
     int n, stride, gx, gy;
     float inv_h2;
     float *hi, *lo, *b;
@@ -2000,11 +2059,11 @@ template <bool SPLIT>
 __global__ void __launch_bounds__(BX * BY) k_refresh(const __grid_constant__ RefreshArgs A)
 {
     int l = 0;
-    while (l + 1 < A.nlev && (int)blockIdx.x >= A.lev[l + 1].first) ++l;
+    while (l + 1 < A.nlev && (int)blockIdx.x >= A.lev[l + 1].first[!SPLIT]) ++l;
     const RefreshLevel& V = A.lev[l];
-    const uint3 bid = batched::split_block((int)blockIdx.x - V.first, V.gx, V.gy);
+    const uint3 bid = batched::split_block((int)blockIdx.x - V.first[!SPLIT], V.gx, V.gy);
     if (SPLIT) split_inject_block(A.u0, A.n0, V.stride, V.hi, V.lo, V.n, bid);
-    else base_colour_block(V.hi, V.lo, V.b, V.n, V.inv_h2, bid);
+    else base_colour_col_block(V.hi, V.lo, V.b, V.n, V.inv_h2, base_chunk(V.n), bid);
 }
 
 }  // namespace
@@ -2019,7 +2078,7 @@ size_t cm_points(int n) { return n >= 3 ? (size_t)(n - 2) * (n - 2) * (n - 2) : 
 cudaError_t launch_base_colour(const float* hi, const float* lo, void* bstore, int n, double h, cudaStream_t s)
 {
     count_launches(1);
-    k_base_colour<<<grid_of(n), dim3(BX, BY), 0, s>>>(hi, lo, (float*)bstore, n, (float)(1.0 / (h * h)));
+    k_base_colour<<<base_grid(n), dim3(BX, BY), 0, s>>>(hi, lo, (float*)bstore, n, (float)(1.0 / (h * h)));
     return cudaGetLastError();
 }
 
@@ -2506,16 +2565,17 @@ cudaError_t launch_refresh(const double* u0, int n0, const RefreshSpec* lv, int 
     A.u0 = u0;
     A.n0 = n0;
     A.nlev = nlev;
-    int blocks = 0;
+    int blocks[2] = {0, 0};
     for (int l = 0; l < nlev; ++l) {
-        const dim3 g = grid_of(lv[l].n);
-        A.lev[l] = RefreshLevel{blocks, lv[l].n, lv[l].stride, (int)g.x, (int)g.y, (float)(1.0 / (lv[l].h * lv[l].h)),
+        const dim3 g = grid_of(lv[l].n), gb = base_grid(lv[l].n);
+        A.lev[l] = RefreshLevel{{blocks[0], blocks[1]}, lv[l].n, lv[l].stride, (int)g.x, (int)g.y, (float)(1.0 / (lv[l].h * lv[l].h)),
                                 lv[l].hi, lv[l].lo, (float*)lv[l].bstore};
-        blocks += (int)(g.x * g.y * g.z);
+        blocks[0] += (int)(g.x * g.y * g.z);
+        blocks[1] += (int)(gb.x * gb.y * gb.z);
     }
     count_launches(2);
-    k_refresh<true><<<blocks, dim3(BX, BY), 0, s>>>(A);
-    k_refresh<false><<<blocks, dim3(BX, BY), 0, s>>>(A);
+    k_refresh<true><<<blocks[0], dim3(BX, BY), 0, s>>>(A);
+    k_refresh<false><<<blocks[1], dim3(BX, BY), 0, s>>>(A);
     return cudaGetLastError();
 }
 
