@@ -1989,18 +1989,36 @@ struct CmF32Out {
     float* r;
     float* b;        // colour-major B store of the level
     float inv_4h2;   // 1 / (4 h^2)
+    // the two colour boxes of a column (k even, odd): points before the box,
+    // points of it, and the column's first place in it
+    struct Column {
+        long long off0, off1, cnt0, cnt1;
+        int row, plane;
+        __device__ __forceinline__ Column(int i, int j, int n)
+        {
+            const int pi = i & 1, pj = j & 1, ni = colour_count(n, pi), nj = colour_count(n, pj);
+            plane = ni * nj;
+            row = ((j - (pj ? 1 : 2)) >> 1) * ni + ((i - (pi ? 1 : 2)) >> 1);
+            off0 = cm_offset(n, pi | (pj << 1));
+            off1 = cm_offset(n, pi | (pj << 1) | 4);
+            cnt0 = (long long)plane * colour_count(n, 0);
+            cnt1 = (long long)plane * colour_count(n, 1);
+        }
+    };
     // the residual without FP64 arithmetic (resid::residual_f2_block)
-    __device__ __forceinline__ void put2(long long, int i, int j, int k, int n, const resid::ResF2& v) const
+    __device__ __forceinline__ void put2(const Column& c, long long, int k, const resid::ResF2& v) const
     {
-        const CmPos c = cm_pos(i, j, k, n);
-        r[c.off + c.idx] = v.val.hi;
-        float* q = b + 6 * c.off + c.idx;
+        const bool pk = k & 1;
+        const long long off = pk ? c.off1 : c.off0, cnt = pk ? c.cnt1 : c.cnt0;
+        const long long idx = (long long)((k - (pk ? 1 : 2)) >> 1) * c.plane + c.row;
+        r[off + idx] = v.val.hi;
+        float* q = b + 6 * off + idx;
         q[0] = v.H[0].hi * inv_4h2;
-        q[c.cnt] = v.H[1].hi * inv_4h2;
-        q[2 * c.cnt] = v.H[2].hi * inv_4h2;
-        q[3 * c.cnt] = v.H[3].hi * inv_4h2;
-        q[4 * c.cnt] = v.H[4].hi * inv_4h2;
-        q[5 * c.cnt] = v.H[5].hi * inv_4h2;
+        q[cnt] = v.H[1].hi * inv_4h2;
+        q[2 * cnt] = v.H[2].hi * inv_4h2;
+        q[3 * cnt] = v.H[3].hi * inv_4h2;
+        q[4 * cnt] = v.H[4].hi * inv_4h2;
+        q[5 * cnt] = v.H[5].hi * inv_4h2;
     }
     __device__ __forceinline__ void zero(long long) const {}
 };

@@ -476,7 +476,7 @@ __device__ __forceinline__ ResF2 residual_point_f2(const double* __restrict__ u,
 
 // Block body: one (i, j) column per thread over a run of k (as
 // residual_col_block), each point evaluated by residual_point_f2; Out::put2
-// receives (p, i, j, k, n, ResF2).  Norm partials from the FP32 rounding of
+// receives (its Column, p, k, ResF2).  Norm partials from the FP32 rounding of
 // the value.
 template <typename Out, int NN = 0>
 __device__ __forceinline__ void residual_f2_block(const double* __restrict__ u, const double* __restrict__ rhs,
@@ -496,6 +496,7 @@ __device__ __forceinline__ void residual_f2_block(const double* __restrict__ u, 
     float mx = 0.0f, ss = 0.0f;
     if (i < n && j < n && k0 < k1) {
         const bool col_interior = i > 0 && j > 0 && i < n - 1 && j < n - 1;
+        const typename Out::Column col(i, j, n);
         for (int k = k0; k < k1; ++k) {
             const long long p = ((long long)k * n + j) * n + i;
             if (!col_interior || k == 0 || k == n - 1) {
@@ -506,7 +507,7 @@ __device__ __forceinline__ void residual_f2_block(const double* __restrict__ u, 
             const float v32 = r.val.hi;
             mx = fmaxf(mx, fabsf(v32));
             ss = fmaf(v32, v32, ss);
-            out.put2(p, i, j, k, n, r);
+            out.put2(col, p, k, r);
         }
     }
     if (partials) {
@@ -559,7 +560,10 @@ template <bool UNORM>
 struct NaturalF2Out {
     static constexpr bool kUnorm = UNORM;
     double* r;
-    __device__ __forceinline__ void put2(long long p, int, int, int, int, const ResF2& v) const
+    struct Column {
+        __device__ __forceinline__ Column(int, int, int) {}
+    };
+    __device__ __forceinline__ void put2(const Column&, long long p, int, const ResF2& v) const
     {
         r[p] = f2d(v.val.hi) + f2d(v.val.lo);
     }
