@@ -466,7 +466,10 @@ ma_status ma_get_corr_tuning(int n, int *smooth_choice, int *residual_choice);
  * default), or 3, 5, 9 or 17; MA_ERR_INVALID_ARG otherwise.  Hierarchies
  * take the setting when they first record their CUDA graphs.
  *
- * ma_set_corr_tail: the FP32 correction cycles of the mixed and FP32 modes. */
+ * ma_set_corr_tail: the FP32 correction cycles of the mixed and FP32 modes.
+ * Their default also runs the levels of 33^3 and 17^3 with the tail in one
+ * 16-block cluster, where the device runs one: the same bits again.  A bound
+ * set by hand leaves the cluster out. */
 ma_status ma_set_corr_tail(int max_n);
 
 /* ma_set_vcycle_tail: the FP64 V-cycles (ma_vcycle and the FP64 solves, FMG

@@ -94,9 +94,9 @@ cudaError_t launch_colour(double* u, const double* rhs, int n, double h6, unsign
 }
 
 // ---------------------------------------------------------------------------
-// The same sweep with the point update of ma_smooth_f2.cuh.  Colours 3 and 4 follow each other in the order and differ in all three
-// parities, a corner offset the stencil lacks, so they are independent and one
-// launch sweeps both: blocks with z below nk0 take colour C, the rest colour
+// The same sweep with the point update of ma_smooth_f2.cuh.  Colours 3 and 4
+// follow each other in the order and differ in all three parities, a corner
+// offset the stencil lacks, so they are independent and one launch sweeps both: blocks with z below nk0 take colour C, the rest colour
 // D.  NN > 0 fixes the grid size at compile time for the sizes that stream
 // from HBM: the 18 neighbour offsets become immediates of the loads.
 // ---------------------------------------------------------------------------
@@ -411,7 +411,7 @@ __device__ __forceinline__ double operator_point(const double* q, int sy, int sz
 // Over a grid, 0 on the shell: one point a thread, the grid size at compile time
 // for the sizes of a hierarchy's larger levels.  The FP64 forms of the two were
 // bound by the FP64 pipe (257^3: 754 us residual, 800 us right-hand side); this
-// one by issue, 252 us at 257^3, 36 against 98 at 129^3, 8.3 against 22 at 65^3,
+// one by issue, 248 us at 257^3, 36 against 98 at 129^3, 8.3 against 22 at 65^3,
 // 3.8 against 7.2 at 33^3 (Example 4, graph replay).  Runs of planes a thread,
 // as the residual with norms walks them, keep more values live (76 registers
 // for 64): 297 us.

@@ -1473,7 +1473,10 @@ __global__ void __launch_bounds__(TT, 1) k_corr_vcycle_tail(TailArgs A) { corr_t
 // Correction V-cycles from a level of 33^3 or 17^3 down to the coarsest grid
 // and back in one cluster of 16 thread blocks.  Level by level those two grids
 // take 16 colour-pair launches and 4 transfers each a cycle, 1.8 us and more
-// apiece whatever their work.
+// apiece whatever their work: a cycle from 33^3 about 138 us, here 64 us (122 K
+// cycles: sweeps of 33^3 16.5 K each pair, of 17^3 9.6 K, the tail 35 K).  At 80
+// registers, which leaves an SM room for other kernels, 24 solves side by side
+// gain 2 % and a 33^3 solve alone loses 4 %.
 //
 // A block owns planes of k: at 33^3 the odd plane 2m + 1 and the even plane
 // 2m + 2 (m its rank), at 17^3 the plane m + 1, in shared memory with one
@@ -2392,8 +2395,8 @@ int tail_smem_bytes(const int* ns, int nlev)
 // Largest level of the single-block tail: at 17^3 one SM's serial colour
 // phases take longer than the launches they replace, at 9^3 and below the
 // launches cost more (measured on whole solves from 33^3 to 257^3).  By
-// default the cluster takes the levels up to 33^3 (measured per cycle beside
-// k_corr_vcycle_cluster); a bound set by hand leaves it out.
+// default the cluster takes the levels up to 33^3 (a cycle from 33^3: 64 us,
+// level by level above the tail about 138); a bound set by hand leaves it out.
 constexpr int kTailDefault = 9, kClusterDefault = 33;
 std::atomic<int> g_tail_max{kClusterDefault};
 

@@ -8,10 +8,10 @@
 // change to the centre value.
 //
 // Measured per sweep under graph replay (Example 4 / random cosine, us), FP64
-// form -> this one: 257^3 1075 / 1076 -> 343 / 406, 129^3 152 / 152 -> 68 / 80,
-// 65^3 34 / 34 -> 25 / 26, 33^3 26 / 26 -> 20 / 20.  Bound at 257^3 by issue
-// (about 450 integer and FP32 instructions a point); at 33^3 by the length of
-// one point's dependent chain, 7 launches a sweep.  The random cosine's values
+// form -> this one: 257^3 1075 / 1076 -> 329 / 380, 129^3 152 / 152 -> 64 / 74,
+// 65^3 34 / 34 -> 24 / 24, 33^3 26 / 26 -> 15 / 15 (two sweeps in one cluster
+// launch).  Bound at 257^3 by issue (about 450 integer and FP32 instructions a
+// point); at 65^3 and below by the length of one point's dependent chain.  The random cosine's values
 // cross more binades, so more warps take gather_f2's fixed-point branch.
 //
 // Scaling: H = 2^k 4 h^2 D^2_h u with 2^k next to 1 / (4 h^2), so that the
@@ -21,8 +21,9 @@
 //
 // The root is found as smallest_root finds it: in FP32 on the rounded entries
 // (by the iteration of corr_root_fast where it is small, else by Newton from 0,
-// or from left of it where the matrix is not positive definite), then one Newton correction whose residual is evaluated to about 2^-45
-// of the entries' cube (in FP64 there), with the FP32 derivative.  The second
+// or from left of it where the matrix is not positive definite), then one Newton
+// correction whose residual is evaluated to about 2^-45 of the entries' cube (in
+// FP64 there), with the FP32 derivative.  The second
 // differences it starts from are exact, where the FP64 gather rounds the
 // neighbour sums to 2^-53 |u|, so from 17^3 up the result lies closer to the
 // exact update.  A point that smallest_root would not solve by that path
@@ -43,7 +44,6 @@ struct Params {
     int kexp;       // k, or kNone: outside gather_f2's range, every point takes the FP64 form
 };
 constexpr int kNone = 1 << 20;
-
 
 inline Params make_params(double h)
 {
