@@ -1384,6 +1384,7 @@ cudaError_t launch_vcycle_tail(const TailSpec64* lv, int nlev, int nu1, int nu2,
 
 cudaError_t prepare_coarsest_f64()
 {
+    (void)sweep33::ready();   // asked and set up here, outside any capture
     cudaError_t e = cudaFuncSetAttribute(k_coarsest, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)(2 * sizeof(double) * 17 * 17 * 17));
     if (e != cudaSuccess) return e;
