@@ -1016,11 +1016,30 @@ __global__ void __launch_bounds__(BX * BY, 8) k_residual_corr_col(const float* _
     residual_corr_col_block<NN>(e, bstore, rhs_cm, res, n, inv_h2, kc, blockIdx);
 }
 
-// Planes per column run, and the grid of the column residual.
-// (8 planes up to 129^3, 16 from 257^3: measured, 21.1 against 24.6 us at 129^3 and
-// 147.3 against 150.4 us at 257^3 under graph replay)
-__host__ __device__ inline int col_chunk(int n) { return n >= 257 ? 16 : 8; }
+// The grid of the column residual, and the planes per column run: a run loads
+// two planes before its first point, and the last wave of blocks (8 an SM) takes
+// as long as a full one, so the run of 8 to 16 planes with the fewest waves
+// times (planes + 2).  At 129^3 that is 9 planes in two waves, 19.0 us, where 8
+// leave a third wave nearly empty, 21.1 us.  Runs of 3 planes would take 65^3
+// from 6.9 to 5.5 us alone, but cost 24 solves side by side 2 % in loads.  (More
+// resident blocks are slower: 10 an SM 151.8 against 143.6 us at 257^3.)
 inline dim3 col_grid(int n, int kc) { return dim3((n - 2 + CW - 1) / CW, (n - 2 + 3) / 4, (n - 2 + kc - 1) / kc); }
+
+int col_chunk(int n)
+{
+    constexpr long long slots = 152 * 8;
+    int best = 16;
+    long long cost = -1;
+    for (int kc = 16; kc >= 8; --kc) {
+        const dim3 g = col_grid(n, kc);
+        const long long c = ((long long)g.x * g.y * g.z + slots - 1) / slots * (kc + 2);
+        if (cost < 0 || c < cost) {
+            cost = c;
+            best = kc;
+        }
+    }
+    return best;
+}
 
 // The shell of res (faces of the cube) is 0.
 __global__ void k_zero_shell(float* v, int n)
