@@ -403,8 +403,9 @@ __device__ __forceinline__ bool gather_f2_of(Ld ld, Idx sy, Idx sz, int kexp, f2
         } else if (FORM == kDirect && !__any_sync(__activemask(), (int)diff < 0)) {
             sums(fix);
         } else {
-            // (left shifts about: a stencil of one sign keeps its unit's sign whatever its warp's others hold)
-            const long long mixed = FORM == kSmall ? (int)diff >> 31 : -1;
+            // a stencil of one sign keeps its unit's sign whatever its warp's others hold: the conversion of a
+            // sum beyond 2^48 rounds a value and its negative differently, so the bits would depend on them
+            const long long mixed = (int)diff >> 31;
             sums([&](long long b) {
                 const long long v = fix(b), neg = (b >> 63) & mixed;
                 return (v ^ neg) - neg;

@@ -580,3 +580,28 @@ def test_solution_restriction_is_the_exact_weighted_mean(n, lo, hi):
             assert got[K, J, I] == float(exact)
         else:
             assert abs(Fraction(float(got[K, J, I])) - exact) <= Fraction(16 * EPS * big) + Fraction(5e-324) * 64
+
+
+@pytest.mark.parametrize("n", [33, 67, 129])
+def test_two_float_points_do_not_depend_on_their_warp(n):
+    """Rough negative values over two binades, so that every stencil takes the fixed-point
+    sums with all their bits; then one value in every 32 of a row, and in every third row
+    and plane, turned positive.  Points whose own stencil is unchanged keep their bits,
+    whichever form the changed points of their warp need."""
+    rng = np.random.default_rng(n)
+    u = -(1.0 + 3.0 * rng.random((n, n, n)))
+    v = u.copy()
+    v[1::3, 1::3, 20::32] *= -1.0
+    f, r0 = rng.random((n, n, n)), rng.random((n, n, n))
+    h = 1.0 / (n - 1)
+    out = []
+    for w in (u, v):
+        res, rhs = (torch.zeros_like(dev(u)) for _ in range(2))
+        M.ma_residual_f2(dev(w), dev(f), res, n, h)
+        M.ma_coarse_rhs(dev(w), dev(r0), rhs, n, h)
+        out.append((host(res), host(rhs)))
+    changed = np.zeros((n, n, n), bool)
+    for k, j, i in np.argwhere(u != v):
+        changed[max(k - 1, 0):k + 2, max(j - 1, 0):j + 2, max(i - 1, 0):i + 2] = True
+    for a, b in zip(*out):
+        assert np.array_equal(a[~changed], b[~changed])
