@@ -75,7 +75,7 @@ struct Params2 {
     double h4;        // h^4
     double kz;        // 2^-k / 2: z to the change of v
     double inv_h2;
-    float chi, clo;   // (2^k h^2)^2 as two floats
+    double c;         // (2^k h^2)^2
     float ihi, ilo;   // its inverse
     int kexp;         // k, or kNone: the FP64 form everywhere
 };
@@ -103,8 +103,7 @@ Params2 make_params2(double h)
     }
     const double q = std::ldexp(h2, P.kexp), c = q * q;
     P.kz = std::ldexp(0.5, -P.kexp);
-    P.chi = (float)c;
-    P.clo = (float)(c - (double)P.chi);
+    P.c = c;
     P.ihi = (float)(1.0 / c);
     P.ilo = (float)(1.0 / c - (double)P.ihi);
     return P;
@@ -173,8 +172,8 @@ __device__ __forceinline__ bool update2(Ld ld, Idx sy, double b, const Params2& 
     namespace f2 = ma::resid::f2;
     F2 H[3];
     long long c;
+    const F2 r4 = f2::from_f64(__dmul_rn(P.c, b));   // ahead of the gather, which its latency hides behind
     if (!gather2_f2<Idx>(ld, sy, P.kexp, H, &c)) return false;
-    const F2 r4 = f2::mul(f2::from_f64(b), F2{P.chi, P.clo});
     const float A = H[0].hi, B = H[1].hi, Rr = H[2].hi, T = A + B, D = A - B;
     const float scale = fabsf(A) + fabsf(B) + fabsf(Rr);
     const float disc = fmaf(D, D, 4.0f * fmaf(Rr, Rr, r4.hi));

@@ -543,7 +543,7 @@ __device__ __forceinline__ bool newton5(double* u, const double* rhs, const smoo
     const int a = on ? lane : 0;
     const int i = 1 + a % 3, j = 1 + (a / 3) % 3, k = 1 + a / 9, p = (k * 5 + j) * 5 + i;
     const double b = rhs[p], start = u[p];
-    const f2::F2 r6 = f2::mul(f2::from_f64(b), f2::F2{P.chi, P.clo});
+    const f2::F2 r6 = f2::from_f64(__dmul_rn(P.c, b));
     float last = 0.0f;
     bool moved = false, laplace = false;
     for (int it = 0; it < 24; ++it) {

@@ -273,18 +273,20 @@ __device__ __forceinline__ F2 from_i64(long long x, float scale)
     return {r.hi * scale, r.lo * scale};
 }
 
-// A normal double as hi + lo (hi: its leading 24 significand bits, lo: the
-// next 23 of the remaining 29), with integer and FP32 operations only.
+// A double as hi + lo, each rounded to nearest (hi: 24 bits, lo: 24 of the 29
+// below, signed), with integer and FP32 operations only: within 2^-49 of x, and
+// without a bias, for 2^-104 <= |x| < 2^127.  (lo cut off instead of rounded
+// is 5e-15 of x too small on average, which a solve carries into u.)  Below 2^-104 hi
+// alone, within 2^-129; below 2^-126 zero.
 __device__ __forceinline__ F2 from_f64(double x)
 {
-    const int hw = __double2hiint(x);
-    const unsigned lw = (unsigned)__double2loint(x);
-    const int ex = (hw >> 20) & 0x7ff;
-    const unsigned low29 = lw & 0x1fffffffu;
-    const float hi = d2f_trunc(x);
-    if (ex < 1075 - 126 + 6 || low29 == 0) return {hi, 0.0f};   // 2^(ex-1069) below FP32's normal range
-    const float unit = __int_as_float(((ex - 1069 + 127) << 23) | (hw & 0x80000000));   // +-2^(ex-1069)
-    return {hi, u23_to_f(low29 >> 6) * unit};   // the lo part to 23 bits: ~2^-47 of x
+    const long long b = __double_as_longlong(x);
+    const int hw = (int)(b >> 32), ex = (hw >> 20) & 0x7ff;
+    const int low = (int)((unsigned)b << 3) >> 3;   // the low 29 bits, signed: x = hi + low ulps, away from 0
+    const float hi = d2f_trunc(__longlong_as_double(b + (1ll << 28)));
+    if ((unsigned)(ex - 919) > 253u) return {hi, 0.0f};
+    const float unit = __int_as_float(((ex - 1045 + 127) << 23) | (hw & 0x80000000));   // +-2^(ex-1045), 2^30 ulps
+    return {hi, __int2float_rn(low) * 9.31322574615478515625e-10f * unit};              // 2^-30
 }
 
 // det(H) for the symmetric 3x3 H = [[A, R, S], [R, B, T], [S, T, C]]: the

@@ -40,7 +40,7 @@ namespace smoothf2 {
 struct Params {
     double h6;      // 64 h^6, the right-hand side's factor of the FP64 form
     double kz;      // 2^-k / 8: z to the change of u
-    float chi, clo; // (2^k 4 h^2)^3 as two floats
+    double c;       // (2^k 4 h^2)^3
     int kexp;       // k, or kNone: outside gather_f2's range, every point takes the FP64 form
 };
 constexpr int kNone = 1 << 20;
@@ -57,10 +57,9 @@ inline Params make_params(double h)
         P.kexp = kNone;
         return P;
     }
-    const double q = ldexp(4.0 * h2, P.kexp), c = q * q * q;
+    const double q = ldexp(4.0 * h2, P.kexp);
+    P.c = q * q * q;
     P.kz = ldexp(0.125, -P.kexp);
-    P.chi = (float)c;
-    P.clo = (float)(c - (double)P.chi);
     return P;
 }
 
@@ -92,9 +91,9 @@ __device__ __forceinline__ bool update(Ld ld, Idx sy, Idx sz, double b, const Pa
     using namespace resid;
     f2::F2 H[6];
     long long b0;
+    const f2::F2 r6 = f2::from_f64(__dmul_rn(P.c, b));   // ahead of the gather, which its latency hides behind
     // rhs > 0 by its bits (NaN passes and fails to converge below)
     if (!gather_f2_of<FORM, Idx>(ld, sy, sz, P.kexp, H, &b0) || __double_as_longlong(b) <= 0) return false;
-    const f2::F2 r6 = f2::mul(f2::from_f64(b), f2::F2{P.chi, P.clo});
     HessSf F;
     F.A = H[0].hi; F.B = H[1].hi; F.C = H[2].hi;
     F.R = H[3].hi; F.S = H[4].hi; F.T = H[5].hi;
