@@ -316,9 +316,10 @@ ma_status ma_smooth(double *u_dev, const double *rhs_dev, int n, double h, int n
 /* The same sweeps as the cycles of a hierarchy run them: from 5^3 up the
  * second differences are exact integer differences of the values' bit
  * patterns and the determinant is taken in two-float (hi + lo FP32)
- * arithmetic, two FP64 operations a point.  Agrees with ma_smooth to the
+ * arithmetic, three FP64 operations a point.  Agrees with ma_smooth to the
  * rounding of its FP64 sums (a few 2^-53 |u|) and lies closer to the exact
- * update; the smallest-root rule and the events are the same. */
+ * update; the smallest-root rule and the events are the same.  Points outside
+ * the two-float range (ma_residual_f2) take the FP64 form. */
 ma_status ma_smooth_f2(double *u_dev, const double *rhs_dev, int n, double h, int nsweeps,
                        unsigned long long *events_dev, ma_stream_t stream);
 
@@ -327,14 +328,16 @@ ma_status ma_smooth_f2(double *u_dev, const double *rhs_dev, int n, double h, in
 ma_status ma_residual(const double *u_dev, const double *rhs_dev, double *r_dev, int n, double h,
                       ma_stream_t stream);
 
-/* The same residual (Algorithm 1 step 3, Eq. MA_discrete) as the fine-grid
- * residual of MA_MIXED solves computes it, without FP64 arithmetic: the second
+/* The same residual (Algorithm 1 step 3, Eq. MA_discrete) as the cycles and
+ * solves of a hierarchy compute it from 5^3 up: the second
  * differences are integer differences, of the 19 stencil values' bit patterns
  * where they share one sign and one binade (exact), of fixed-point values with 7
- * bits to spare otherwise, and the determinant and rhs - det are taken in
- * two-float (hi + lo FP32) arithmetic, about 48 significant bits; a stencil
- * whose largest value is zero, huge or tiny takes the FP64 evaluation of
- * ma_residual.  Same layout and arguments as ma_residual; asynchronous. */
+ * bits to spare otherwise, the determinant is taken in two-float (hi + lo FP32)
+ * arithmetic, about 48 significant bits, and subtracted from rhs in FP64.  A
+ * point takes the FP64 evaluation of ma_residual where h is below 4e-7 or above
+ * 600, the stencil's largest value is zero or outside [2^-40, 2^20), the
+ * determinant overflows FP32, or it and rhs are both below 2^-64.  Same layout
+ * and arguments as ma_residual; asynchronous. */
 ma_status ma_residual_f2(const double *u_dev, const double *rhs_dev, double *r_dev, int n, double h,
                          ma_stream_t stream);
 
@@ -352,7 +355,8 @@ ma_status ma_restrict_solution(const double *uf_dev, int nf, double *uc_dev, int
                                ma_stream_t stream);
 
 /* tau-corrected coarse right-hand side b_H = det(D^2_H w_H) + r_H on the
- * coarse interior, 0 on the shell (Algorithm 1 step 5). */
+ * coarse interior, 0 on the shell (Algorithm 1 step 5), as the cycles
+ * compute it: from 5^3 up with the two-float determinant of ma_residual_f2. */
 ma_status ma_coarse_rhs(const double *wc_dev, const double *rc_dev, double *bc_dev, int nc, double H,
                         ma_stream_t stream);
 
@@ -377,7 +381,10 @@ ma_status ma_interpolate_cubic(const double *uc_dev, int nc, double *uf_dev, voi
 
 /* Approximate solve on a coarsest grid (Algorithm 1 step 1), one thread
  * block: sweeps > 0 runs that many sweeps, 0 sweeps until
- * max|du| <= 1e-14 max|u| (at most 100).  n <= 17. */
+ * max|du| <= 1e-14 max|u| (at most 100).  n <= 17.  As the cycles run it: the
+ * sweeps are those of ma_smooth_f2 from 5^3 up, and on 5^3 with sweeps = 0
+ * Newton's method comes first, and ends the solve where a sweep would
+ * change its iterate by no more than that. */
 ma_status ma_coarsest_solve(double *u_dev, const double *rhs_dev, int n, double h, int sweeps,
                             unsigned long long *events_dev, ma_stream_t stream);
 

@@ -382,30 +382,27 @@ __global__ void __launch_bounds__(BX * BY) k_coarse_rhs(const double* __restrict
 
 // r + det(D^2_h u) (SIGN = 1, the coarse right-hand side) or r - det (SIGN = -1,
 // the residual) at a point, with exact integer second differences and a
-// two-float determinant; ld as gather_f2_of takes it.
+// two-float determinant, added to r in FP64; ld as gather_f2_of takes it, q the
+// centre's place.
 template <int SIGN, bool UNORM, int FORM, typename Idx, typename Ld>
-__device__ __forceinline__ double operator_of(Ld ld, Idx sy, Idx sz, double rv, double inv_h6)
+__device__ __forceinline__ double operator_of(Ld ld, const double* q, Idx sy, Idx sz, double rv, const resid::Scaling& P)
 {
     using namespace resid;
     f2::F2 H[6];
     long long b0;
-    if (gather_f2_of<FORM, Idx>(ld, sy, sz, 0, H, &b0)) {
-        const float ih = (float)(SIGN * inv_h6);
-        const f2::F2 d = f2::mul(f2::det3<UNORM>(H[0], H[1], H[2], H[3], H[4], H[5]),
-                                 f2::F2{ih, (float)(SIGN * inv_h6 - (double)ih)});
-        const f2::F2 v = f2::add(f2::from_f64(rv), d);
-        return f2d(v.hi) + f2d(v.lo);
+    if (P.kexp != kNone && gather_f2_of<FORM, Idx>(ld, sy, sz, P.kexp, H, &b0)) {
+        const f2::F2 d = f2::det3<UNORM>(H[0], H[1], H[2], H[3], H[4], H[5]);
+        if (usable(d, rv)) return fma(SIGN * (f2d(d.hi) + f2d(d.lo)), P.inv_c, rv);
     }
-    const HessS G = gather_hess_of([&](Idx o) { return __longlong_as_double(ld(o)); }, sy, sz, __longlong_as_double(b0));
-    return fma(SIGN * det0(G), inv_h6, rv);
+    return operator_f64(q, sy, sz, rv, P.inv_h6, SIGN);
 }
 
 // At a point of a grid in shared memory (q points at it).
 template <int SIGN, bool UNORM>
-__device__ __forceinline__ double operator_point(const double* q, int sy, int sz, double rv, double inv_h6)
+__device__ __forceinline__ double operator_point(const double* q, int sy, int sz, double rv, const resid::Scaling& P)
 {
-    return operator_of<SIGN, UNORM, resid::kSmall, int>([q](int o) -> long long { return __double_as_longlong(q[o]); }, sy, sz, rv,
-                                         inv_h6);
+    return operator_of<SIGN, UNORM, resid::kSmall, int>(
+        [q](int o) -> long long { return __double_as_longlong(q[o]); }, q, sy, sz, rv, P);
 }
 
 // Over a grid, 0 on the shell: one point a thread, the grid size at compile time
@@ -417,7 +414,7 @@ __device__ __forceinline__ double operator_point(const double* q, int sy, int sz
 // for 64): 297 us.
 template <int NN, int SIGN, bool UNORM>
 __global__ void __launch_bounds__(BX * BY) k_operator_f2(const double* __restrict__ u, const double* __restrict__ r,
-                                                         double* __restrict__ out, int n_rt, double inv_h6)
+                                                         double* __restrict__ out, int n_rt, resid::Scaling P)
 {
     const int n = NN > 0 ? NN : n_rt;
     const int i = blockIdx.x * BX + threadIdx.x;
@@ -430,23 +427,24 @@ __global__ void __launch_bounds__(BX * BY) k_operator_f2(const double* __restric
         return;
     }
     const long long* q = reinterpret_cast<const long long*>(u) + p;
-    out[p] = operator_of<SIGN, UNORM, UNORM ? resid::kDirect : resid::kSmall, long long>([q](long long o) -> long long { return __ldg(q + o); }, n, sz,
-                                                 __ldg(r + p), inv_h6);
+    out[p] = operator_of<SIGN, UNORM, UNORM ? resid::kDirect : resid::kSmall, long long>(
+        [q](long long o) -> long long { return __ldg(q + o); }, u + p, n, sz, __ldg(r + p), P);
 }
 
 template <int SIGN>
-cudaError_t launch_operator_f2(const double* u, const double* r, double* out, int n, double inv_h6, cudaStream_t s)
+cudaError_t launch_operator_f2(const double* u, const double* r, double* out, int n, const resid::Scaling& P,
+                               cudaStream_t s)
 {
     const dim3 g = xfer::grid_of(n), b(BX, BY);
     switch (n) {
-    case 33: k_operator_f2<33, SIGN, true><<<g, b, 0, s>>>(u, r, out, n, inv_h6); break;
-    case 65: k_operator_f2<65, SIGN, true><<<g, b, 0, s>>>(u, r, out, n, inv_h6); break;
-    case 129: k_operator_f2<129, SIGN, true><<<g, b, 0, s>>>(u, r, out, n, inv_h6); break;
-    case 257: k_operator_f2<257, SIGN, true><<<g, b, 0, s>>>(u, r, out, n, inv_h6); break;
-    case 513: k_operator_f2<513, SIGN, true><<<g, b, 0, s>>>(u, r, out, n, inv_h6); break;
+    case 33: k_operator_f2<33, SIGN, true><<<g, b, 0, s>>>(u, r, out, n, P); break;
+    case 65: k_operator_f2<65, SIGN, true><<<g, b, 0, s>>>(u, r, out, n, P); break;
+    case 129: k_operator_f2<129, SIGN, true><<<g, b, 0, s>>>(u, r, out, n, P); break;
+    case 257: k_operator_f2<257, SIGN, true><<<g, b, 0, s>>>(u, r, out, n, P); break;
+    case 513: k_operator_f2<513, SIGN, true><<<g, b, 0, s>>>(u, r, out, n, P); break;
     default:
-        if (n < kUnormMinN) k_operator_f2<0, SIGN, false><<<g, b, 0, s>>>(u, r, out, n, inv_h6);
-        else k_operator_f2<0, SIGN, true><<<g, b, 0, s>>>(u, r, out, n, inv_h6);
+        if (n < kUnormMinN) k_operator_f2<0, SIGN, false><<<g, b, 0, s>>>(u, r, out, n, P);
+        else k_operator_f2<0, SIGN, true><<<g, b, 0, s>>>(u, r, out, n, P);
     }
     return cudaGetLastError();
 }
@@ -732,7 +730,6 @@ constexpr int T64 = 512;
 
 struct Tail64Level {
     int n;
-    double inv_h6;       // 1 / (64 h^6)
     smoothf2::Params P;
     double* u;           // global iterate (read on the top level, written back there)
     const double* rhs;   // global right-hand side (read on the top level)
@@ -823,7 +820,7 @@ __device__ __forceinline__ void vcycle_tail_body(const Tail64Args& A)
         for (int q = threadIdx.x; q < (nf - 2) * (nf - 2) * (nf - 2); q += T64) {        // (3)
             int i, j, k;
             const int p = GF.interior(q, &i, &j, &k);
-            F.r[p] = operator_point<-1, false>(F.u + p, nf, nf * nf, F.rhs[p], A.lev[l].inv_h6);
+            F.r[p] = operator_point<-1, false>(F.u + p, nf, nf * nf, F.rhs[p], A.lev[l].P);
         }
         __syncthreads();
         // (3)-(4): the interior's two restrictions side by side (both are FP64 sums), the shell's injection
@@ -856,10 +853,10 @@ __device__ __forceinline__ void vcycle_tail_body(const Tail64Args& A)
             int i, j, k;
             const int p = GC.interior(q, &i, &j, &k);
             if (nc >= kF2MinN) {
-                C.rhs[p] = operator_point<1, false>(C.w + p, nc, nc * nc, C.r[p], A.lev[l + 1].inv_h6);
+                C.rhs[p] = operator_point<1, false>(C.w + p, nc, nc * nc, C.r[p], A.lev[l + 1].P);
             } else {
                 const HessS H = gather_hess_of([&](int o) { return C.w[p + o]; }, nc, nc * nc, C.w[p]);
-                C.rhs[p] = fma(det0(H), A.lev[l + 1].inv_h6, C.r[p]);
+                C.rhs[p] = fma(det0(H), A.lev[l + 1].P.inv_h6, C.r[p]);
             }
         }
         __syncthreads();
@@ -1184,18 +1181,17 @@ int norm_partial_count(int n) { return residual_partial_count(n); }
 cudaError_t launch_residual(const double* u, const double* rhs, double* r, int n, double h,
                             double* partials, cudaStream_t s)
 {
-    if (n >= kF2MinN) {
+    const resid::Scaling P = resid::make_scaling(h);
+    if (n >= kF2MinN && P.kexp != resid::kNone) {
         const dim3 g = reduce_grid(n);
         const int kchunk = (n + (int)g.z - 1) / (int)g.z;
         count_launches(1);
-        if (!partials) return launch_operator_f2<-1>(u, rhs, r, n, 1.0 / pow6(h), s);
+        if (!partials) return launch_operator_f2<-1>(u, rhs, r, n, P, s);
         const dim3 gk = resid::grid_for(n, g.z);
         if (n < kUnormMinN)
-            resid::launch_k_residual_f2(gk, s, u, rhs, resid::NaturalF2Out<false>{r}, n, 1.0 / pow6(h), partials,
-                                        kchunk);
+            resid::launch_k_residual_f2(gk, s, u, rhs, resid::NaturalF2Out<false>{r}, n, P, partials, kchunk);
         else
-            resid::launch_k_residual_f2(gk, s, u, rhs, resid::NaturalF2Out<true>{r}, n, 1.0 / pow6(h), partials,
-                                        kchunk);
+            resid::launch_k_residual_f2(gk, s, u, rhs, resid::NaturalF2Out<true>{r}, n, P, partials, kchunk);
         return cudaGetLastError();
     }
     return launch_residual_f64(u, rhs, r, n, h, partials, s);
@@ -1263,9 +1259,9 @@ cudaError_t launch_restrict_level(const double* uf, const double* rf, int nf, do
 cudaError_t launch_coarse_rhs(const double* wc, const double* rc, double* bc, int nc, double H, cudaStream_t s)
 {
     count_launches(1);
-    const double inv_H6 = 1.0 / pow6(H);
-    if (nc >= kF2MinN) return launch_operator_f2<1>(wc, rc, bc, nc, inv_H6, s);
-    k_coarse_rhs<<<grid_of(nc), dim3(BX, BY), 0, s>>>(wc, rc, bc, nc, inv_H6);
+    const resid::Scaling P = resid::make_scaling(H);
+    if (nc >= kF2MinN && P.kexp != resid::kNone) return launch_operator_f2<1>(wc, rc, bc, nc, P, s);
+    k_coarse_rhs<<<grid_of(nc), dim3(BX, BY), 0, s>>>(wc, rc, bc, nc, P.inv_h6);
     return cudaGetLastError();
 }
 
@@ -1365,7 +1361,6 @@ cudaError_t launch_vcycle_tail(const TailSpec64* lv, int nlev, int nu1, int nu2,
     for (int l = 0; l < nlev; ++l) {
         if (lv[l].n > 17 || (l > 0 && lv[l].n != (lv[l - 1].n + 1) / 2)) return cudaErrorInvalidValue;
         A.lev[l].n = ns[l] = lv[l].n;
-        A.lev[l].inv_h6 = 1.0 / pow6(lv[l].h);
         A.lev[l].P = smoothf2::make_params(lv[l].h);
         A.lev[l].u = lv[l].u;
         A.lev[l].rhs = lv[l].rhs;

@@ -2006,11 +2006,22 @@ __global__ void k_f32_to_f64(const float* __restrict__ e, double* __restrict__ u
 // problem's right-hand side), and with it the fine base Hessian B = D^2_h u
 // of the correction operator, rounded to FP32 from the FP64 Hessian the
 // residual already formed; the shell is not stored.
+__device__ __noinline__ float cm_point_f64(const double* q, long long sy, long long sz, double rhs, double inv_h6,
+                                           double kh, float kb, float* r, float* b, long long cnt)
+{
+    auto at = [&](long long o) { return q[o]; };
+    const HessS G = gather_hess_of(at, sy, sz, at(0));
+    const double hs[6] = {G.A, G.B, G.C, G.R, G.S, G.T};
+#pragma unroll
+    for (int v = 0; v < 6; ++v) b[v * cnt] = __double2float_rn(hs[v] * kh) * kb;
+    return *r = __double2float_rn(fma(-det0(G), inv_h6, rhs));
+}
+
 struct CmF32Out {
-    static constexpr bool kUnorm = false;
+    static constexpr bool kF64 = false, kUnorm = false;
     float* r;
-    float* b;        // colour-major B store of the level
-    float inv_4h2;   // 1 / (4 h^2)
+    float* b;    // colour-major B store of the level
+    float kb;    // resid::Scaling's
     // the two colour boxes of a column (k even, odd): points before the box,
     // points of it, and the column's first place in it
     struct Column {
@@ -2033,14 +2044,22 @@ struct CmF32Out {
         const bool pk = k & 1;
         const long long off = pk ? c.off1 : c.off0, cnt = pk ? c.cnt1 : c.cnt0;
         const long long idx = (long long)((k - (pk ? 1 : 2)) >> 1) * c.plane + c.row;
-        r[off + idx] = v.val.hi;
+        r[off + idx] = v.v32;
         float* q = b + 6 * off + idx;
-        q[0] = v.H[0].hi * inv_4h2;
-        q[cnt] = v.H[1].hi * inv_4h2;
-        q[2 * cnt] = v.H[2].hi * inv_4h2;
-        q[3 * cnt] = v.H[3].hi * inv_4h2;
-        q[4 * cnt] = v.H[4].hi * inv_4h2;
-        q[5 * cnt] = v.H[5].hi * inv_4h2;
+        q[0] = v.H[0] * kb;
+        q[cnt] = v.H[1] * kb;
+        q[2 * cnt] = v.H[2] * kb;
+        q[3 * cnt] = v.H[3] * kb;
+        q[4 * cnt] = v.H[4] * kb;
+        q[5 * cnt] = v.H[5] * kb;
+    }
+    __device__ __forceinline__ float put64(const Column& c, long long, int k, const double* q, long long sy, long long sz,
+                                           double rhs, const resid::Scaling& P) const
+    {
+        const bool pk = k & 1;
+        const long long off = pk ? c.off1 : c.off0;
+        const long long idx = (long long)((k - (pk ? 1 : 2)) >> 1) * c.plane + c.row;
+        return cm_point_f64(q, sy, sz, rhs, P.inv_h6, P.kh, kb, r + off + idx, b + 6 * off + idx, pk ? c.cnt1 : c.cnt0);
     }
     __device__ __forceinline__ void zero(long long) const {}
 };
@@ -2621,25 +2640,24 @@ cudaError_t launch_refresh(const double* u0, int n0, const RefreshSpec* lv, int 
 
 cudaError_t launch_residual_f2(const double* u, const double* rhs, double* r, int n, double h, cudaStream_t s)
 {
-    const double h2 = h * h;
     count_launches(1);
     const int kz = n < 16 ? n : 16;
     const int kchunk = (n + kz - 1) / kz;
     resid::launch_k_residual_f2(resid::grid_for(n, kz), s, u, rhs, resid::NaturalF2Out<false>{r}, n,
-                                1.0 / (64.0 * h2 * h2 * h2), nullptr, kchunk);
+                                resid::make_scaling(h), nullptr, kchunk);
     return cudaGetLastError();
 }
 
 cudaError_t launch_residual64_to32(const double* u, const double* rhs, float* r_cm, void* bstore, int n, double h,
                                    double* partials, cudaStream_t s)
 {
-    const double h2 = h * h;
+    const resid::Scaling P = resid::make_scaling(h);
     count_launches(1);
     // without norms one plane a block (the partials' count fixes the grid with them)
     const int kz = n < 16 || !partials ? n : 16;
     const int kchunk = (n + kz - 1) / kz;
-    resid::launch_k_residual_f2(resid::grid_for(n, kz), s, u, rhs, CmF32Out{r_cm, (float*)bstore, (float)(0.25 / h2)},
-                                n, 1.0 / (64.0 * h2 * h2 * h2), partials, kchunk);
+    resid::launch_k_residual_f2(resid::grid_for(n, kz), s, u, rhs, CmF32Out{r_cm, (float*)bstore, P.kb}, n, P,
+                                partials, kchunk);
     return cudaGetLastError();
 }
 
@@ -2882,7 +2900,7 @@ struct OpRes64 {
     static constexpr int NT = resid::RX * resid::RY, MINB = 1;
     struct Job {
         int inst, n, kchunk, gx, gy, gz;
-        double inv_h6;
+        resid::Scaling P;
         const double* u;
         const double* rhs;
         double* partials;
@@ -2890,7 +2908,7 @@ struct OpRes64 {
     };
     static __device__ __forceinline__ void run(const Job& J, int q)
     {
-        resid::residual_f2_block<CmF32Out>(J.u, J.rhs, J.out, J.n, J.inv_h6, J.partials, J.kchunk,
+        resid::residual_f2_block<CmF32Out>(J.u, J.rhs, J.out, J.n, J.P, J.partials, J.kchunk,
                                            split_block(q, J.gx, J.gy),
                                            make_uint3((unsigned)J.gx, (unsigned)J.gy, (unsigned)J.gz));
     }
@@ -3242,7 +3260,6 @@ void build_sequence(TableBuilder& T, const BatchInstance* in, int count, const B
             const BatchInstance& I = in[b];
             const BatchLevel& F = I.lev[0];
             const int n = F.n;
-            const double h2 = F.h * F.h;
             const int kz = n < 16 ? n : 16;
             const dim3 g = resid::grid_for(n, kz);
             OpRes64::Job J;
@@ -3253,11 +3270,11 @@ void build_sequence(TableBuilder& T, const BatchInstance* in, int count, const B
             J.gx = (int)g.x;
             J.gy = (int)g.y;
             J.gz = (int)g.z;
-            J.inv_h6 = 1.0 / (64.0 * h2 * h2 * h2);
+            J.P = resid::make_scaling(F.h);
             J.u = F.u;
             J.rhs = F.rhs;
             J.partials = I.partials;
-            J.out = CmF32Out{F.rhs32, (float*)F.bstore, (float)(0.25 / h2)};
+            J.out = CmF32Out{F.rhs32, (float*)F.bstore, J.P.kb};
             rj.push_back(J);
             rb.push_back((int)(g.x * g.y * g.z));
             OpNorm::Job N{in[b].id, I.npartials, F.h * F.h * F.h, I.partials, I.out2,

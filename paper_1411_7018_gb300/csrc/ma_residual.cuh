@@ -184,8 +184,15 @@ inline dim3 grid_for(int n, int kz) { return dim3((n + RX - 1) / RX, (n + RY - 1
 //    exact product: |error| of a few 2^-46 relative to the sum of the
 //    magnitudes of the determinant's terms.
 // A stencil that changes binade or sign is handled the same way, each value
-// as a fixed-point number of the largest one's scale with 7 bits to spare; one
-// whose largest value is zero, huge or tiny takes the FP64 evaluation.
+// as a fixed-point number of the largest one's scale with 7 bits to spare.
+//
+// FP32 has the digits but not FP64's range, so the differences are held as
+// 2^k 4 h^2 D^2_h u with 2^k next to 1 / (4 h^2) (struct Scaling): they have
+// the size of D^2 u whatever the step, and the factor that takes the
+// determinant back lies near 1.  A point takes the FP64 evaluation where k would
+// leave [-20, 40] (h below 4e-7 or above 600), the stencil's largest value is
+// zero or outside [2^-40, 2^20), the determinant overflows FP32, or it and the
+// right-hand side are both below 2^-64 (usable()).
 // ---------------------------------------------------------------------------
 namespace f2 {
 
@@ -304,18 +311,63 @@ __device__ __forceinline__ F2 det3(const F2& A, const F2& B, const F2& C, const 
     return sum(sum(mul_u(A, c1), neg(mul_u(R, c2))), mul_u(S, c3));
 }
 
-// The exact paths accept binades E with 2^(E-1075) and the cube of the
-// scaled second differences inside FP32's normal range: 2^-40 <= |u| < 2^20
-// (every grid function here lies far inside).
+// The exact paths accept binades E with 2^(E-1075), and a scaling 2^k of it
+// for -20 <= k <= 40, inside FP32's normal range: 2^-40 <= |u| < 2^20.
 constexpr int kMinE = 1023 - 40, kMaxE = 1023 + 20;
 
 }  // namespace f2
 
-// Residual rhs - det(D^2_h u) at interior point p and 4 H (H = h^2 D^2_h u)
-// for outputs that store it: value as two-float, v32 its FP32 rounding.
+// A level's scaling and constants, from its step h.
+struct Scaling {
+    double h6, inv_h6;   // 64 h^6, the right-hand side's factor of the FP64 forms, and its inverse
+    double c, inv_c;     // (2^k 4 h^2)^3 and its inverse
+    double kz;           // 2^-k / 8: a root z of the scaled matrix to the change of u
+    double kh;           // 2^k: 4 h^2 D^2_h u to the scaled differences
+    float kb;            // scaled differences to D^2_h u
+    int kexp;            // k, or kNone: every point takes the FP64 form
+};
+constexpr int kNone = 1 << 20;
+
+inline Scaling make_scaling(double h)
+{
+    Scaling P{};
+    const double h2 = h * h;
+    P.h6 = 64.0 * h2 * h2 * h2;
+    P.inv_h6 = 1.0 / P.h6;
+    int e = 0;
+    const double m = frexp(4.0 * h2, &e);   // 4 h^2 = m 2^e, m in [1/2, 1)
+    P.kexp = m < 0.70710678118654752 ? 1 - e : -e;
+    if (P.kexp < -20 || P.kexp > 40) {
+        P.kexp = kNone;
+        P.kh = 1.0 / (4.0 * h2);   // the FP64 form's differences as D^2_h u
+        P.kb = 1.0f;
+        return P;
+    }
+    const double q = ldexp(4.0 * h2, P.kexp);   // in [0.7, 1.42)
+    P.c = q * q * q;
+    P.inv_c = 1.0 / P.c;
+    P.kz = ldexp(0.125, -P.kexp);
+    P.kh = ldexp(1.0, P.kexp);
+    P.kb = (float)(1.0 / q);
+    return P;
+}
+
+// Whether the two-float determinant d of scaled differences serves rhs - det and
+// rhs + det: none of its products overflowed (an infinity or NaN stays one to the
+// end), and what they lost below FP32's range, some 2^-126, lies below the
+// rounding of the larger of d and rhs.
+__device__ __forceinline__ bool usable(f2::F2 d, double rhs)
+{
+    return fabsf(d.hi) < 3.0e38f &&
+           (fabsf(d.hi) >= 5.421010862427522e-20f || (__double2hiint(rhs) & 0x7ff00000) >= (1023 - 64) << 20);   // 2^-64
+}
+
+// Residual rhs - det(D^2_h u) at an interior point and the scaled differences
+// for outputs that store them.
 struct ResF2 {
-    f2::F2 val;
-    f2::F2 H[6];   // 4 h^2 D^2_h u: xx, yy, zz, xy, xz, yz
+    double v;      // FP64 outputs
+    float v32;     // its FP32 rounding
+    float H[6];    // 2^k 4 h^2 D^2_h u: xx, yy, zz, xy, xz, yz
 };
 
 // H = 2^kexp 4 h^2 D^2_h u at a point, formed exactly in int64 and held as
@@ -453,37 +505,47 @@ __device__ __forceinline__ bool gather_f2(const double* __restrict__ u, Idx p, I
     return gather_f2_of<kDirect, Idx>([q](Idx o) -> long long { return __ldg(q + o); }, sy, sz, kexp, H, centre);
 }
 
-template <bool UNORM = false>
-__device__ __forceinline__ ResF2 residual_point_f2(const double* __restrict__ u, long long p, long long sy,
-                                                   long long sz, double rhs, f2::F2 inv_h6, double inv_h6_d)
+// F64: the value in FP64, the right-hand side with all its digits (two FP64
+// operations); otherwise its FP32 rounding, from two floats.  ic: P.inv_c as two
+// floats.  false: the point needs the FP64 form.
+template <bool F64, bool UNORM>
+__device__ __forceinline__ bool residual_point_f2(const double* __restrict__ u, long long p, long long sy,
+                                                  long long sz, double rhs, const Scaling& P, f2::F2 ic, ResF2* out)
 {
-    ResF2 out;
+    f2::F2 H[6];
     long long b0;
-    if (gather_f2<long long>(u, p, sy, sz, 0, out.H, &b0)) {
-        const f2::F2 d = f2::det3<UNORM>(out.H[0], out.H[1], out.H[2], out.H[3], out.H[4], out.H[5]);
-        out.val = f2::add(f2::from_f64(rhs), f2::neg(f2::mul(d, inv_h6)));
-        return out;
+    if (P.kexp == kNone || !gather_f2<long long>(u, p, sy, sz, P.kexp, H, &b0)) return false;
+    const f2::F2 d = f2::det3<UNORM>(H[0], H[1], H[2], H[3], H[4], H[5]);
+    if (!usable(d, rhs)) return false;
+    if constexpr (F64) {
+        out->v = fma(-(f2d(d.hi) + f2d(d.lo)), P.inv_c, rhs);
+        out->v32 = d2f_trunc(out->v);
+    } else {
+        out->v32 = f2::add(f2::from_f64(rhs), f2::neg(f2::mul(d, ic))).hi;
     }
-    // FP64 evaluation
-    HessS H = gather_hess(u, p, sy, sz, __longlong_as_double(b0));
-    const double v = fma(-det0(H), inv_h6_d, rhs);
-    const double hs[6] = {H.A, H.B, H.C, H.R, H.S, H.T};
-    for (int c = 0; c < 6; ++c) {
-        const float hi = __double2float_rn(hs[c]);
-        out.H[c] = {hi, __double2float_rn(hs[c] - (double)hi)};
-    }
-    const float vh = __double2float_rn(v);
-    out.val = {vh, __double2float_rn(v - (double)vh)};
-    return out;
+    for (int c = 0; c < 6; ++c) out->H[c] = H[c].hi;
+    return true;
+}
+
+// r + sign det(D^2_h u) in FP64, for the points the two-float forms leave (out of
+// line: inline it cost those forms 8 registers); q points at the centre.
+static __device__ __noinline__ double operator_f64(const double* q, long long sy, long long sz, double r, double inv_h6,
+                                                   int sign)
+{
+    auto at = [&](long long o) { return q[o]; };
+    const HessS G = gather_hess_of(at, sy, sz, at(0));
+    return fma(sign * det0(G), inv_h6, r);
 }
 
 // Block body: one (i, j) column per thread over a run of k (as
 // residual_col_block), each point evaluated by residual_point_f2; Out::put2
-// receives (its Column, p, k, ResF2).  Norm partials from the FP32 rounding of
-// the value.
+// receives (its Column, p, k, ResF2).  Out::put64 evaluates the points left in
+// FP64, in a second walk of a run that has any (a call within the first took the
+// 513^3 residual of a mixed solve from 2055 to 2260 us; this one takes 2094).
+// Norm partials from the FP32 rounding of the value.
 template <typename Out, int NN = 0>
 __device__ __forceinline__ void residual_f2_block(const double* __restrict__ u, const double* __restrict__ rhs,
-                                                  const Out& out, int n_rt, double inv_h6_d, double* partials,
+                                                  const Out& out, int n_rt, const Scaling& P, double* partials,
                                                   int kchunk, uint3 bid, uint3 gdim)
 {
     // NN > 0: the grid size at compile time, so the stencil offsets are
@@ -494,23 +556,37 @@ __device__ __forceinline__ void residual_f2_block(const double* __restrict__ u, 
     const int k0 = bid.z * kchunk;
     const int k1 = min(n, k0 + kchunk);
     const long long sy = n, sz = (long long)n * n;
-    const float ih = (float)inv_h6_d;   // the two-float 1 / (64 h^6)
-    const f2::F2 inv_h6 = {ih, (float)(inv_h6_d - (double)ih)};
+    const float ih = (float)P.inv_c;
+    const f2::F2 ic = {ih, (float)(P.inv_c - (double)ih)};
     float mx = 0.0f, ss = 0.0f;
     if (i < n && j < n && k0 < k1) {
         const bool col_interior = i > 0 && j > 0 && i < n - 1 && j < n - 1;
         const typename Out::Column col(i, j, n);
+        bool left = false;   // a point for FP64
         for (int k = k0; k < k1; ++k) {
             const long long p = ((long long)k * n + j) * n + i;
             if (!col_interior || k == 0 || k == n - 1) {
                 out.zero(p);
                 continue;
             }
-            const ResF2 r = residual_point_f2<Out::kUnorm>(u, p, sy, sz, rhs[p], inv_h6, inv_h6_d);
-            const float v32 = r.val.hi;
+            ResF2 r;
+            const double b = rhs[p];
+            if (!residual_point_f2<Out::kF64, Out::kUnorm>(u, p, sy, sz, b, P, ic, &r)) {
+                left = true;
+                continue;
+            }
+            out.put2(col, p, k, r);
+            mx = fmaxf(mx, fabsf(r.v32));
+            ss = fmaf(r.v32, r.v32, ss);
+        }
+        for (int k = max(k0, 1); left && k < min(k1, n - 1); ++k) {
+            const long long p = ((long long)k * n + j) * n + i;
+            ResF2 r;
+            const double b = rhs[p];
+            if (residual_point_f2<Out::kF64, Out::kUnorm>(u, p, sy, sz, b, P, ic, &r)) continue;
+            const float v32 = out.put64(col, p, k, u + p, sy, sz, b, P);
             mx = fmaxf(mx, fabsf(v32));
             ss = fmaf(v32, v32, ss);
-            out.put2(col, p, k, r);
         }
     }
     if (partials) {
@@ -533,10 +609,10 @@ __device__ __forceinline__ void residual_f2_block(const double* __restrict__ u, 
 }
 
 template <typename Out, int NN = 0>
-__global__ void __launch_bounds__(RX * RY) k_residual_f2(const double* __restrict__ u, const double* __restrict__ rhs,
-                                                         Out out, int n, double inv_h6, double* partials, int kchunk)
+__global__ void __launch_bounds__(RX * RY, NN > 0 ? 8 : 5) k_residual_f2(const double* __restrict__ u, const double* __restrict__ rhs,
+                                                         Out out, int n, Scaling P, double* partials, int kchunk)
 {
-    residual_f2_block<Out, NN>(u, rhs, out, n, inv_h6, partials, kchunk, blockIdx, gridDim);
+    residual_f2_block<Out, NN>(u, rhs, out, n, P, partials, kchunk, blockIdx, gridDim);
 }
 
 // Launch with the grid size fixed at compile time for the sizes of a
@@ -544,31 +620,38 @@ __global__ void __launch_bounds__(RX * RY) k_residual_f2(const double* __restric
 // its 64-bit offsets).
 template <typename Out>
 void launch_k_residual_f2(dim3 grid, cudaStream_t s, const double* u, const double* rhs, Out out, int n,
-                          double inv_h6, double* partials, int kchunk)
+                          const Scaling& P, double* partials, int kchunk)
 {
     const dim3 blk(RX, RY);
     switch (n) {
-    case 33: k_residual_f2<Out, 33><<<grid, blk, 0, s>>>(u, rhs, out, n, inv_h6, partials, kchunk); break;
-    case 65: k_residual_f2<Out, 65><<<grid, blk, 0, s>>>(u, rhs, out, n, inv_h6, partials, kchunk); break;
-    case 129: k_residual_f2<Out, 129><<<grid, blk, 0, s>>>(u, rhs, out, n, inv_h6, partials, kchunk); break;
-    case 257: k_residual_f2<Out, 257><<<grid, blk, 0, s>>>(u, rhs, out, n, inv_h6, partials, kchunk); break;
-    case 513: k_residual_f2<Out, 513><<<grid, blk, 0, s>>>(u, rhs, out, n, inv_h6, partials, kchunk); break;
-    default: k_residual_f2<Out, 0><<<grid, blk, 0, s>>>(u, rhs, out, n, inv_h6, partials, kchunk); break;
+    case 33: k_residual_f2<Out, 33><<<grid, blk, 0, s>>>(u, rhs, out, n, P, partials, kchunk); break;
+    case 65: k_residual_f2<Out, 65><<<grid, blk, 0, s>>>(u, rhs, out, n, P, partials, kchunk); break;
+    case 129: k_residual_f2<Out, 129><<<grid, blk, 0, s>>>(u, rhs, out, n, P, partials, kchunk); break;
+    case 257: k_residual_f2<Out, 257><<<grid, blk, 0, s>>>(u, rhs, out, n, P, partials, kchunk); break;
+    case 513: k_residual_f2<Out, 513><<<grid, blk, 0, s>>>(u, rhs, out, n, P, partials, kchunk); break;
+    default: k_residual_f2<Out, 0><<<grid, blk, 0, s>>>(u, rhs, out, n, P, partials, kchunk); break;
     }
 }
 
-// FP64 output of the two-float residual (hi + lo rounded once to double).
-// UNORM: the determinant with unnormalised sums (f2::det3).
+// FP64 output of the two-float residual.  UNORM: the determinant with
+// unnormalised sums (f2::det3).
 template <bool UNORM>
 struct NaturalF2Out {
-    static constexpr bool kUnorm = UNORM;
+    static constexpr bool kF64 = true, kUnorm = UNORM;
     double* r;
     struct Column {
         __device__ __forceinline__ Column(int, int, int) {}
     };
     __device__ __forceinline__ void put2(const Column&, long long p, int, const ResF2& v) const
     {
-        r[p] = f2d(v.val.hi) + f2d(v.val.lo);
+        r[p] = v.v;
+    }
+    __device__ __forceinline__ float put64(const Column&, long long p, int, const double* q, long long sy, long long sz,
+                                           double rhs, const Scaling& P) const
+    {
+        const double v = operator_f64(q, sy, sz, rhs, P.inv_h6, -1);
+        r[p] = v;
+        return d2f_trunc(v);
     }
     __device__ __forceinline__ void zero(long long p) const { r[p] = 0.0; }
 };

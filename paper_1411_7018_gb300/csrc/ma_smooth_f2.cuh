@@ -4,8 +4,8 @@
 // at 85 % of its peak: 137 us per colour at 257^3, against 20 us for the
 // bytes.  Here the six second differences are exact integers
 // (resid::gather_f2), the determinant at the shifted Hessian is taken in
-// two-float arithmetic, and two FP64 operations are left, the addition of the
-// change to the centre value.
+// two-float arithmetic, and three FP64 operations are left: the scaling of the
+// right-hand side and the addition of the change to the centre value.
 //
 // Measured per sweep under graph replay (Example 4 / random cosine, us), FP64
 // form -> this one: 257^3 1075 / 1076 -> 329 / 380, 129^3 152 / 152 -> 64 / 74,
@@ -14,10 +14,9 @@
 // point); at 65^3 and below by the length of one point's dependent chain.  The random cosine's values
 // cross more binades, so more warps take gather_f2's fixed-point branch.
 //
-// Scaling: H = 2^k 4 h^2 D^2_h u with 2^k next to 1 / (4 h^2), so that the
-// entries have the size of D^2 u and their products stay inside FP32's range
-// whatever the step; the local equation det(H - z I) = (2^k 4 h^2)^3 rhs has the
-// root of Eq. (realroots) at v = v0 + z / (8 2^k).
+// Scaling (resid::Scaling): H = 2^k 4 h^2 D^2_h u with 2^k next to 1 / (4 h^2);
+// the local equation det(H - z I) = (2^k 4 h^2)^3 rhs has the root of Eq.
+// (realroots) at v = v0 + z / (8 2^k).
 //
 // The root is found as smallest_root finds it: in FP32 on the rounded entries
 // (by the iteration of corr_root_fast where it is small, else by Newton from 0,
@@ -37,31 +36,9 @@
 namespace ma {
 namespace smoothf2 {
 
-struct Params {
-    double h6;      // 64 h^6, the right-hand side's factor of the FP64 form
-    double kz;      // 2^-k / 8: z to the change of u
-    double c;       // (2^k 4 h^2)^3
-    int kexp;       // k, or kNone: outside gather_f2's range, every point takes the FP64 form
-};
-constexpr int kNone = 1 << 20;
-
-inline Params make_params(double h)
-{
-    Params P{};
-    const double h2 = h * h;
-    P.h6 = 64.0 * h2 * h2 * h2;
-    int e = 0;
-    const double m = frexp(4.0 * h2, &e);   // 4 h^2 = m 2^e, m in [1/2, 1)
-    P.kexp = m < 0.70710678118654752 ? 1 - e : -e;
-    if (P.kexp < -20 || P.kexp > 40) {
-        P.kexp = kNone;
-        return P;
-    }
-    const double q = ldexp(4.0 * h2, P.kexp);
-    P.c = q * q * q;
-    P.kz = ldexp(0.125, -P.kexp);
-    return P;
-}
+using Params = resid::Scaling;
+using resid::kNone;
+inline Params make_params(double h) { return resid::make_scaling(h); }
 
 // The new centre value by the FP64 form, for the points the fast path leaves;
 // q points at the centre.
@@ -91,9 +68,13 @@ __device__ __forceinline__ bool update(Ld ld, Idx sy, Idx sz, double b, const Pa
     using namespace resid;
     f2::F2 H[6];
     long long b0;
-    const f2::F2 r6 = f2::from_f64(__dmul_rn(P.c, b));   // ahead of the gather, which its latency hides behind
+    // on a small grid ahead of the gather, which hides its latency (33^3 solve: 2 % of it); on one that fills the
+    // GPU after it, in fewer registers (257^3 solve: 1 %)
+    f2::F2 r6;
+    if (FORM == kSmall) r6 = f2::from_f64(__dmul_rn(P.c, b));
     // rhs > 0 by its bits (NaN passes and fails to converge below)
     if (!gather_f2_of<FORM, Idx>(ld, sy, sz, P.kexp, H, &b0) || __double_as_longlong(b) <= 0) return false;
+    if (FORM == kDirect) r6 = f2::from_f64(__dmul_rn(P.c, b));
     HessSf F;
     F.A = H[0].hi; F.B = H[1].hi; F.C = H[2].hi;
     F.R = H[3].hi; F.S = H[4].hi; F.T = H[5].hi;
