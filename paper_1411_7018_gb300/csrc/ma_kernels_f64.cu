@@ -526,7 +526,8 @@ __device__ __forceinline__ void run_sweeps64(const SmallGrid& G, const Grid64& S
 // right-hand sides; where they are not positive definite (FMG's zero interior)
 // from the solution of the Poisson equation with right-hand side
 // 3 rhs^(1/3), which a convex solution exceeds and mostly lies near.  If the
-// residual does not fall the iterate is put back.  True
+// residual does not fall, or a step leaves a point that is not positive definite
+// or out of range, the iterate is put back.  True
 // when the changes that a sweep would make (each point's residual over its
 // derivative) are at most 1e-14 max |u|, the sweeps' own rule; otherwise the
 // caller's sweeps decide as they would have.  J: 27 x kJ floats.
@@ -548,7 +549,7 @@ __device__ __forceinline__ bool newton5(double* u, const double* rhs, const smoo
         f2::F2 H[6];
         long long b0;
         auto ld = [&](int o) -> long long { return __double_as_longlong(u[p + o]); };
-        bool usable = gather_f2_of<true, int>(ld, 5, 25, P.kexp, H, &b0);
+        bool usable = gather_f2_of<kSmall, int>(ld, 5, 25, P.kexp, H, &b0);
         if (!usable && ((ld(0) | ld(1) | ld(-1) | ld(5) | ld(-5) | ld(25) | ld(-25)) << 1) == 0) {
             usable = true;   // a zero interior's centre: no Hessian there, which is a Laplacian of 0
             H[0] = H[1] = H[2] = H[3] = H[4] = H[5] = f2::F2{0.0f, 0.0f};
@@ -573,8 +574,9 @@ __device__ __forceinline__ bool newton5(double* u, const double* rhs, const smoo
         const bool bad = __any_sync(FULL, on && !ok);
         const bool start_laplace = bad && !moved && !laplace && __all_sync(FULL, !on || usable);
         if (!start_laplace && (bad || (moved && !(worst < last)))) {
-            // not a point Newton can be trusted from, or the residual no longer falls: round-off, or put it back
-            if ((bad && laplace) || (moved && !__all_sync(FULL, !on || worst <= 1e-11f * fabsf(r6.hi)))) {
+            // not a point Newton can be trusted from (its residual is not known), or the residual no longer falls:
+            // put the iterate back, unless that is round-off
+            if (bad || !__all_sync(FULL, !on || worst <= 1e-11f * fabsf(r6.hi))) {
                 __syncwarp();
                 if (on) u[p] = start;
                 __syncwarp();
@@ -582,7 +584,7 @@ __device__ __forceinline__ bool newton5(double* u, const double* rhs, const smoo
             }
             double big = on ? fabs(__longlong_as_double(b0)) : 0.0;
             for (int o = 16; o > 0; o >>= 1) big = fmax(big, __shfl_xor_sync(FULL, big, o));
-            return moved && __all_sync(FULL, !on || fabsf(g) * (float)P.kz <= 1e-14f * (float)big * m);
+            return __all_sync(FULL, !on || fabsf(g) * (float)P.kz <= 1e-14f * (float)big * m);
         }
         if (start_laplace) g = H[0].hi + H[1].hi + H[2].hi - 3.0f * cbrtf(r6.hi);
         if (!moved || worst > 0.25f * last) {
