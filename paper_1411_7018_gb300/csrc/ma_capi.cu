@@ -162,11 +162,11 @@ cudaError_t vcycle_from(ma_hierarchy* H, int l0)
             spec[q] = ma::TailSpec64{A.n, A.h, A.u, A.rhs};
         }
         if ((e = ma::launch_vcycle_tail(spec, nlev, d.nu1, d.nu2, d.restrict_kind, d.approx_restrict,
-                                        d.coarse_sweeps, H->events, s)) != cudaSuccess)
+                                        d.coarse_sweeps, H->L == 1, H->events, s)) != cudaSuccess)
             return e;
     } else {
         ma::Level& B = H->lev[H->L - 1];
-        if ((e = ma::launch_coarsest(B.u, B.rhs, B.n, B.h, d.coarse_sweeps, H->events, s)) != cudaSuccess)
+        if ((e = ma::launch_coarsest(B.u, B.rhs, B.n, B.h, d.coarse_sweeps, H->L == 1, H->events, s)) != cudaSuccess)
             return e;                                                                                      // (1)
     }
     for (int l = lt - 1; l >= l0; --l) {
@@ -213,7 +213,8 @@ cudaError_t fmg(ma_hierarchy* H, bool finest_vcycle = true)
     }
     ma::Level& B = H->lev[H->L - 1];
     if ((e = ma::launch_zero_interior(B.u, B.n, s)) != cudaSuccess) return e;
-    if ((e = ma::launch_coarsest(B.u, B.rhs, B.n, B.h, H->d.coarse_sweeps, H->events, s)) != cudaSuccess) return e;
+    if ((e = ma::launch_coarsest(B.u, B.rhs, B.n, B.h, H->d.coarse_sweeps, H->L == 1, H->events, s)) != cudaSuccess)
+        return e;
     for (int l = H->L - 2; l >= 0; --l) {
         ma::Level& F = H->lev[l];
         ma::Level& C = H->lev[l + 1];
@@ -1467,7 +1468,7 @@ ma_status ma_coarsest_solve(double* u, const double* rhs, int n, double h, int s
     if (!u || !rhs || !valid_step_grid(n) || n > 17 || !(h > 0.0) || sweeps < 0 || sweeps > 1000)
         return fail(MA_ERR_INVALID_ARG, "ma_coarsest_solve: bad arguments (n <= 17)");
     MA_CK(ma::prepare_kernels());
-    MA_CK(ma::launch_coarsest(u, rhs, n, h, sweeps, events, (cudaStream_t)stream));
+    MA_CK(ma::launch_coarsest(u, rhs, n, h, sweeps, true, events, (cudaStream_t)stream));
     return MA_OK;
 }
 

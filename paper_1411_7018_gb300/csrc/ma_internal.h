@@ -53,7 +53,8 @@ size_t interpolate_cubic_scratch(int nc);
 cudaError_t launch_interpolate_cubic(const double* uc, int nc, double* uf, double* scratch, cudaStream_t s);
 cudaError_t launch_inject(const double* vf, int nf, double* vc, cudaStream_t s);
 cudaError_t launch_zero_interior(double* u, int n, cudaStream_t s);
-cudaError_t launch_coarsest(double* u, const double* rhs, int n, double h, int sweeps,
+// finest: the grid is no other's correction (ma_kernels_f64.cu, newton5)
+cudaError_t launch_coarsest(double* u, const double* rhs, int n, double h, int sweeps, bool finest,
                             unsigned long long* events, cudaStream_t s);
 cudaError_t launch_copy_rhs_bc(const double* f, const double* g, double* rhs, double* u, int n,
                                int* bad, cudaStream_t s);
@@ -69,7 +70,7 @@ struct TailSpec64 {
 int vcycle_tail_max_n();          // 0 when the fused tail is switched off
 bool set_vcycle_tail(int max_n);  // 0 off, 1 default, or 3 / 5 / 9 / 17; false otherwise
 cudaError_t launch_vcycle_tail(const TailSpec64* lv, int nlev, int nu1, int nu2, int kind, int approx,
-                               int coarse_sweeps, unsigned long long* events, cudaStream_t s);
+                               int coarse_sweeps, bool finest, unsigned long long* events, cudaStream_t s);
 
 // Mixed-precision kernels (ma_kernels_mixed.cu).  e, res, w are n^3 floats
 // in the natural layout; hi + lo is the FP32 split of the FP64 iterate; the

@@ -530,10 +530,12 @@ __device__ __forceinline__ void run_sweeps64(const SmallGrid& G, const Grid64& S
 // or out of range, the iterate is put back.  True
 // when the changes that a sweep would make (each point's residual over its
 // derivative) are at most 1e-14 max |u|, the sweeps' own rule; otherwise the
-// caller's sweeps decide as they would have.  J: 27 x kJ floats.
+// caller's sweeps decide as they would have.  finest: the grid is no other's
+// correction, and the last step takes its residual in FP64 (3000 cycles), which on
+// 5^3 rounds less than the two-float determinant does.  J: 27 x kJ floats.
 constexpr int kJ = 29;   // an odd stride: a lane's row and a column of it meet no bank conflicts
 
-__device__ __forceinline__ bool newton5(double* u, const double* rhs, const smoothf2::Params& P, float* J)
+__device__ __forceinline__ bool newton5(double* u, const double* rhs, const smoothf2::Params& P, float* J, bool finest)
 {
     using namespace resid;
     constexpr unsigned FULL = 0xffffffffu;
@@ -545,6 +547,16 @@ __device__ __forceinline__ bool newton5(double* u, const double* rhs, const smoo
     const f2::F2 r6 = f2::from_f64(__dmul_rn(P.c, b));
     float last = 0.0f;
     bool moved = false, laplace = false;
+    auto step = [&](float g) {   // u -= J^-1 g
+        float d = 0.0f;
+        for (int c = 0; c < 27; ++c) {
+            const float gc = __shfl_sync(FULL, g, c);
+            if (on) d = fmaf(-J[lane * kJ + c], gc, d);
+        }
+        __syncwarp();   // every lane has read what it needs of u
+        if (on) u[p] = fma(8.0 * P.kz, f2d(d), u[p]);
+        __syncwarp();
+    };
     for (int it = 0; it < 24; ++it) {
         f2::F2 H[6];
         long long b0;
@@ -584,7 +596,12 @@ __device__ __forceinline__ bool newton5(double* u, const double* rhs, const smoo
             }
             double big = on ? fabs(__longlong_as_double(b0)) : 0.0;
             for (int o = 16; o > 0; o >>= 1) big = fmax(big, __shfl_xor_sync(FULL, big, o));
-            return __all_sync(FULL, !on || fabsf(g) * (float)P.kz <= 1e-14f * (float)big * m);
+            const bool done = __all_sync(FULL, !on || fabsf(g) * (float)P.kz <= 1e-14f * (float)big * m);
+            if (done && finest) {
+                const HessS G = gather_hess_of([&](int o) { return u[p + o]; }, 5, 25, u[p]);
+                step((float)fma(det0(G), P.kh * P.kh * P.kh, -__dmul_rn(P.c, b)));
+            }
+            return done;
         }
         if (start_laplace) g = H[0].hi + H[1].hi + H[2].hi - 3.0f * cbrtf(r6.hi);
         if (!moved || worst > 0.25f * last) {
@@ -623,13 +640,7 @@ __device__ __forceinline__ bool newton5(double* u, const double* rhs, const smoo
                 __syncwarp();
             }
         }
-        float d = 0.0f;
-        for (int c = 0; c < 27; ++c) {
-            const float gc = __shfl_sync(FULL, g, c);
-            if (on) d = fmaf(-J[lane * kJ + c], gc, d);
-        }
-        if (on) u[p] = fma(8.0 * P.kz, f2d(d), u[p]);
-        __syncwarp();
+        step(g);
         if (start_laplace) {
             laplace = true;
             continue;
@@ -645,7 +656,8 @@ __device__ __forceinline__ bool newton5(double* u, const double* rhs, const smoo
 // eighth sweep where it did not finish.  On 3^3 the one unknown's root with a
 // Newton step in FP64 (smallest_root_precise).  Every thread of the block
 // enters; ends with a block barrier.  J: 27 kJ floats.
-__device__ __forceinline__ void coarsest64_sm(const Grid64& S, int n, int sweeps, float* J, unsigned long long* ev)
+__device__ __forceinline__ void coarsest64_sm(const Grid64& S, int n, int sweeps, bool finest, float* J,
+                                              unsigned long long* ev)
 {
     const int max_sweeps = sweeps > 0 ? sweeps : 100;
     const int nt = phase_threads(n, (int)blockDim.x);
@@ -667,7 +679,7 @@ __device__ __forceinline__ void coarsest64_sm(const Grid64& S, int n, int sweeps
     } else if ((int)threadIdx.x < nt) {
         const SmallGrid G(n);
         for (int s = 0; s < max_sweeps; ++s) {
-            if (n == 5 && sweeps == 0 && (s & 7) == 0 && S.P.kexp != smoothf2::kNone && newton5(S.u, S.rhs, S.P, J))
+            if (n == 5 && sweeps == 0 && (s & 7) == 0 && S.P.kexp != smoothf2::kNone && newton5(S.u, S.rhs, S.P, J, finest))
                 break;
             double du = 0.0, um = 0.0;
             run_sweeps64(G, S, 1, nt, ev, [&](double v0, double v) {
@@ -693,7 +705,8 @@ __device__ __forceinline__ void coarsest64_sm(const Grid64& S, int n, int sweeps
 }
 
 __device__ __forceinline__ void coarsest64_body(double* u, const double* __restrict__ rhs, int n,
-                                                const smoothf2::Params& P, int sweeps, unsigned long long* events)
+                                                const smoothf2::Params& P, int sweeps, bool finest,
+                                                unsigned long long* events)
 {
     extern __shared__ double sm[];
     __shared__ int tab[kPhaseTab];
@@ -705,16 +718,16 @@ __device__ __forceinline__ void coarsest64_body(double* u, const double* __restr
     fill_phase_tab(tab, n, false);
     __syncthreads();
     unsigned long long ev = 0;
-    coarsest64_sm(Grid64{su, sr, tab, P}, n, sweeps, J, &ev);
+    coarsest64_sm(Grid64{su, sr, tab, P}, n, sweeps, finest, J, &ev);
     for (int q = threadIdx.x; q < m; q += COARSE_THREADS) u[q] = su[q];
     if (events && ev) atomicAdd(events, ev);
 }
 
 __global__ void __launch_bounds__(COARSE_THREADS) k_coarsest(double* u, const double* __restrict__ rhs, int n,
-                                                             smoothf2::Params P, int sweeps,
+                                                             smoothf2::Params P, int sweeps, bool finest,
                                                              unsigned long long* events)
 {
-    coarsest64_body(u, rhs, n, P, sweeps, events);
+    coarsest64_body(u, rhs, n, P, sweeps, finest, events);
 }
 
 // ---------------------------------------------------------------------------
@@ -741,7 +754,7 @@ struct Tail64Level {
 struct Tail64Args {
     int nlev;
     Tail64Level lev[4];
-    int nu1, nu2, kind, approx, coarse_sweeps;
+    int nu1, nu2, kind, approx, coarse_sweeps, finest;
     unsigned long long* events;
 };
 
@@ -863,7 +876,7 @@ __device__ __forceinline__ void vcycle_tail_body(const Tail64Args& A)
         }
         __syncthreads();
     }
-    coarsest64_sm(grid(L - 1), A.lev[L - 1].n, A.coarse_sweeps, J, &ev);                     // (1)
+    coarsest64_sm(grid(L - 1), A.lev[L - 1].n, A.coarse_sweeps, A.finest != 0, J, &ev);                     // (1)
     for (int l = L - 2; l >= 0; --l) {
         const Tail64Smem F = tail64_fields(A, t64sm, l);
         const Tail64Smem C = tail64_fields(A, t64sm, l + 1);
@@ -982,7 +995,7 @@ struct OpZero64 {
 struct OpCoarsest64 {
     static constexpr int NT = COARSE_THREADS, MINB = 1;
     struct Job {
-        int inst, n, sweeps;
+        int inst, n, sweeps, finest;
         smoothf2::Params P;
         double* u;
         const double* rhs;
@@ -990,7 +1003,7 @@ struct OpCoarsest64 {
     };
     static __device__ __forceinline__ void run(const Job& J, int)
     {
-        coarsest64_body(J.u, J.rhs, J.n, J.P, J.sweeps, J.events);
+        coarsest64_body(J.u, J.rhs, J.n, J.P, J.sweeps, J.finest != 0, J.events);
     }
 };
 
@@ -1058,8 +1071,8 @@ void emit_fmg_f64(TableBuilder& T, const BatchInstance* in, int count, const Bat
             const dim3 g = grid2(V.n);
             zj.push_back(OpZero64::Job{in[b].id, V.n, (int)g.x, (int)g.y, V.u});
             zb.push_back((int)(g.x * g.y * g.z));
-            kj.push_back(OpCoarsest64::Job{in[b].id, V.n, p.coarse_sweeps, smoothf2::make_params(V.h), V.u, V.rhs,
-                                           in[b].events});
+            kj.push_back(OpCoarsest64::Job{in[b].id, V.n, p.coarse_sweeps, in[b].L == 1, smoothf2::make_params(V.h), V.u,
+                                           V.rhs, in[b].events});
             kb.push_back(1);
             ksmem = std::max(ksmem, (int)(2 * sizeof(double) * (size_t)V.n * V.n * V.n));
         }
@@ -1327,12 +1340,12 @@ cudaError_t launch_copy_rhs_bc(const double* f, const double* g, double* rhs, do
     return cudaGetLastError();
 }
 
-cudaError_t launch_coarsest(double* u, const double* rhs, int n, double h, int sweeps,
+cudaError_t launch_coarsest(double* u, const double* rhs, int n, double h, int sweeps, bool finest,
                             unsigned long long* events, cudaStream_t s)
 {
     const size_t smem = 2 * sizeof(double) * (size_t)n * n * n;
     count_launches(1);
-    k_coarsest<<<1, COARSE_THREADS, smem, s>>>(u, rhs, n, smoothf2::make_params(h), sweeps, events);
+    k_coarsest<<<1, COARSE_THREADS, smem, s>>>(u, rhs, n, smoothf2::make_params(h), sweeps, finest, events);
     return cudaGetLastError();
 }
 
@@ -1354,7 +1367,7 @@ bool set_vcycle_tail(int max_n)
 }
 
 cudaError_t launch_vcycle_tail(const TailSpec64* lv, int nlev, int nu1, int nu2, int kind, int approx,
-                               int coarse_sweeps, unsigned long long* events, cudaStream_t s)
+                               int coarse_sweeps, bool finest, unsigned long long* events, cudaStream_t s)
 {
     if (nlev < 1 || nlev > 4) return cudaErrorInvalidValue;
     Tail64Args A{};
@@ -1373,6 +1386,7 @@ cudaError_t launch_vcycle_tail(const TailSpec64* lv, int nlev, int nu1, int nu2,
     A.kind = kind;
     A.approx = approx;
     A.coarse_sweeps = coarse_sweeps;
+    A.finest = finest;
     A.events = events;
     count_launches(1);
     k_vcycle_tail<<<1, T64, tail64_smem_bytes(ns, nlev), s>>>(A);

@@ -669,3 +669,41 @@ def test_coarsest_5_is_swept_where_newton_leaves_the_range(rhs):
     u = dev(pr.u)
     M.ma_coarsest_solve(u, dev(f), n, h, 0)
     assert np.max(np.abs(host(u) - ref)) <= 1e-12 * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("single", [True, False])
+@pytest.mark.parametrize("name", ["exp", "sine"])
+def test_5_cubed_alone_is_solved_to_fp64_digits(name, single):
+    """A 5^3 grid that is the finest, as a hierarchy of one level and as a coarsest solve: the solution's
+    residual in extended precision, in units of what rounding its stencil's values to 2^-53 of each can do
+    to the determinant.  u's own rounding is one unit at most, and a Newton step with FP64 arithmetic adds
+    those of its gather and its determinant: three in all."""
+    n = 5
+    pr = P.make(name, n)
+    u = dev(pr.u)
+    if single:
+        H = M.Hierarchy(M.make_desc(n, length=pr.length, coarsest_n=5, precision=M.MA_FP64))
+        H.set_rhs_bc(dev(pr.f), u)
+        H.solve(tol=0.0, max_cycles=20, init=M.MA_INIT_KEEP, raise_on_error=False)
+        H.get_solution(u)
+        H.close()
+    else:
+        M.ma_coarsest_solve(u, dev(pr.f), n, pr.h, 0)
+    v = host(u).astype(np.longdouble)
+
+    def at(o, w=v):
+        return w[1 + o[2]:n - 1 + o[2], 1 + o[1]:n - 1 + o[1], 1 + o[0]:n - 1 + o[0]]
+
+    def pair(o, w=v):
+        return at(o, w) + at([-x for x in o], w)
+    h2, w = np.longdouble(pr.h) ** 2, np.abs(v)
+    axes = ((1, 0, 0), (0, 1, 0), (0, 0, 1))
+    crosses = (((1, 1, 0), (1, -1, 0)), ((1, 0, 1), (1, 0, -1)), ((0, 1, 1), (0, 1, -1)))
+    a, b, d = ((pair(o) - 2 * at((0, 0, 0))) / h2 for o in axes)
+    r, s, t = ((pair(p) - pair(q)) / (4 * h2) for p, q in crosses)
+    A, B, D = ((pair(o, w) + 2 * at((0, 0, 0), w)) / h2 for o in axes)
+    R, S, T = ((pair(p, w) + pair(q, w)) / (4 * h2) for p, q in crosses)
+    det = a * (b * d - t * t) - r * (r * d - s * t) + s * (r * t - b * s)
+    unit = A * np.abs(b * d - t * t) + B * np.abs(a * d - s * s) + D * np.abs(a * b - r * r) + \
+        2 * (R * np.abs(s * t - r * d) + S * np.abs(r * t - s * b) + T * np.abs(r * s - t * a))
+    assert np.max(np.abs(pr.f[1:-1, 1:-1, 1:-1] - det) / unit) <= 3.0 * 2.0 ** -53
