@@ -85,7 +85,11 @@ constexpr int kNone = 1 << 20;
 // pass at 8193^2 it is 5e-11 from the two-float one, a twentieth of the scheme's
 // error (1.059e-9 against 1.114e-9 for u = exp((x^2 + y^2) / 2)), and grids of
 // that size keep the FP64 values.
-constexpr int kF2Min2 = 5, kF2Max2 = 4097;
+// Hierarchies whose finest grid has fewer than 17^2 points keep FP64 on every
+// level: there the two-float determinant rounds more than the FP64 gather does
+// (4 to 6 units of the stencil's rounding on 9^2 against 1); above, the solutions'
+// errors are no larger than FP64's from 17^2 (3e-17 and 3e-17 rms) and smaller from 33^2.
+constexpr int kF2Min2 = 5, kF2Max2 = 4097, kF2Finest2 = 17;
 __host__ __device__ constexpr bool takes_f2(int n) { return n >= kF2Min2 && n <= kF2Max2; }
 
 Params2 make_params2(double h)
@@ -777,10 +781,9 @@ cudaError_t norm_final2(const double* partials, int count, double h, double* out
 }
 
 // Norms of the residual rhs - S(u) into out2, or (u null) of rhs.
-cudaError_t norms2(const double* u, const double* rhs, int n, double h, double* partials, double* out2, cudaStream_t s)
+cudaError_t norms2(const double* u, const double* rhs, int n, double h, const Params2& P, double* partials, double* out2,
+                   cudaStream_t s)
 {
-    Params2 P = make_params2(h);
-    if (!takes_f2(n)) P.kexp = kNone;
     ma::count_launches(1);
     if (u) k_partials2<true><<<partial_grid2(n), dim3(TX, TY), 0, s>>>(u, rhs, n, P, partials);
     else k_partials2<false><<<partial_grid2(n), dim3(TX, TY), 0, s>>>(nullptr, rhs, n, P, partials);
@@ -898,11 +901,19 @@ size_t layout2(ma2d_hierarchy* H, const ma2d_desc* d, char* base)
     return off;
 }
 
+// Level l's parameters; the FP64 form where the sizes ask for it.
+Params2 level_params2(const ma2d_hierarchy* H, int l)
+{
+    Params2 P = make_params2(H->lev[l].h);
+    if (!takes_f2(H->lev[l].n) || H->lev[0].n < kF2Finest2) P.kexp = kNone;
+    return P;
+}
+
 cudaError_t coarsest_solve2(ma2d_hierarchy* H, int l)
 {
     auto& B = H->lev[l];
     ma::count_launches(1);
-    k_coarsest2<<<1, CT2, 0, H->s>>>(B.u, B.rhs, B.n, make_params2(B.h), H->d.coarse_sweeps, H->d.ordering);
+    k_coarsest2<<<1, CT2, 0, H->s>>>(B.u, B.rhs, B.n, level_params2(H, l), H->d.coarse_sweeps, H->d.ordering);
     return cudaGetLastError();
 }
 
@@ -914,8 +925,7 @@ cudaError_t tail2(ma2d_hierarchy* H, int l)
     A.nlev = H->L - l;
     for (int q = 0; q < A.nlev; ++q) {
         auto& V = H->lev[l + q];
-        A.lev[q] = Tail2Level{V.n, make_params2(V.h), V.u, V.rhs};
-        if (!takes_f2(V.n)) A.lev[q].P.kexp = kNone;
+        A.lev[q] = Tail2Level{V.n, level_params2(H, l + q), V.u, V.rhs};
     }
     A.nu1 = d.nu1;
     A.nu2 = d.nu2;
@@ -1132,16 +1142,17 @@ ma_status ma2d_solve(ma2d_hierarchy* H, const ma_solve_opts* o, ma_solve_result*
     // the norms of the reference, the initial iterate and its residual norms as one graph
     CK2(run_graph2(H, H->g_init[3 * o->init + o->relative], [&]() -> cudaError_t {
         auto& F = H->lev[0];
+        const Params2 P = level_params2(H, 0);
         cudaError_t e = cudaSuccess;
         if (o->relative == MA_REL_INITIAL) {
             if (o->init != MA_INIT_KEEP) e = zero_interior2(F.u, F.n, H->s);
-            if (e == cudaSuccess) e = norms2(F.u, F.rhs, F.n, F.h, H->partials, H->out + 2, H->s);
+            if (e == cudaSuccess) e = norms2(F.u, F.rhs, F.n, F.h, P, H->partials, H->out + 2, H->s);
         } else if (o->relative == MA_REL_RHS) {
-            e = norms2(nullptr, F.rhs, F.n, F.h, H->partials, H->out + 2, H->s);
+            e = norms2(nullptr, F.rhs, F.n, F.h, P, H->partials, H->out + 2, H->s);
         }
         if (e == cudaSuccess && o->init == MA_INIT_FMG) e = fmg2(H);
         if (e == cudaSuccess && o->init == MA_INIT_ZERO) e = zero_interior2(F.u, F.n, H->s);
-        return e != cudaSuccess ? e : norms2(F.u, F.rhs, F.n, F.h, H->partials, H->out, H->s);
+        return e != cudaSuccess ? e : norms2(F.u, F.rhs, F.n, F.h, P, H->partials, H->out, H->s);
     }));
     double mx = 0.0, l2 = 0.0, scale = 1.0;
     ma_status st = read_norms2(H, &mx, &l2);
@@ -1157,8 +1168,9 @@ ma_status ma2d_solve(ma2d_hierarchy* H, const ma_solve_opts* o, ma_solve_result*
            stagnant < ma::kFloorStagnantCycles) {
         CK2(run_graph2(H, H->g_cycle, [&]() -> cudaError_t {
             auto& F = H->lev[0];
+            const Params2 P = level_params2(H, 0);
             const cudaError_t e = vcycle2_from(H, 0);
-            return e != cudaSuccess ? e : norms2(F.u, F.rhs, F.n, F.h, H->partials, H->out, H->s);
+            return e != cudaSuccess ? e : norms2(F.u, F.rhs, F.n, F.h, P, H->partials, H->out, H->s);
         }));
         res->cycles += 1;
         if ((st = read_norms2(H, &mx, &l2)) != MA_OK) return st;

@@ -172,3 +172,36 @@ def test_cycles_from_a_zero_interior_match_oracle(n, opts, scale, shift):
     ref = g.copy()
     O2.solve(ref, f, pr.h, tol=0.0, max_cycles=2, init_fmg=False, params=O2.Params2D(**opts))
     assert np.max(np.abs(got - ref)) <= 1e-11 * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("ordering", [M.MA2D_REDBLACK, M.MA2D_COLOUR4])
+@pytest.mark.parametrize("coarsest", [3, 5])
+@pytest.mark.parametrize("n", [5, 9])
+def test_smallest_grids_are_solved_to_fp64_digits(n, coarsest, ordering):
+    """The residual of a solution on 5^2 and 9^2, in extended precision and in units of what rounding its
+    stencil's values to 2^-53 of each can do to u_xx u_yy - u_xy^2.  u's own rounding is one unit
+    at most, and an update in FP64 arithmetic adds those of its sums and its root: three in all."""
+    h = 1.0 / (n - 1)
+    y, x = np.meshgrid(np.arange(n) * h - 0.05, np.arange(n) * h - 0.03, indexing="ij")
+    u0 = 0.5 * (x * x + y * y) + 0.1 * np.sin(2 * x) * np.cos(y) - 0.3
+    f = (1 - 0.4 * np.sin(2 * x) * np.cos(y)) * (1 - 0.1 * np.sin(2 * x) * np.cos(y)) - (0.2 * np.cos(2 * x) * np.sin(y)) ** 2
+    H = M.Hierarchy2D(M.make_desc2d(n, coarsest_n=coarsest, ordering=ordering))
+    H.set_rhs_bc(dev(f), dev(u0))
+    H.solve(tol=0.0, max_cycles=40, raise_on_error=False)
+    out = torch.empty((n, n), dtype=torch.float64, device="cuda")
+    H.get_solution(out)
+    H.close()
+    v = host(out).astype(np.longdouble)
+
+    def at(i, j, w):
+        return w[1 + j:n - 1 + j, 1 + i:n - 1 + i]
+
+    def pair(i, j, w):
+        return at(i, j, w) + at(-i, -j, w)
+    h2, w = np.longdouble(h) ** 2, np.abs(v)
+    a, b = ((pair(*o, v) - 2 * at(0, 0, v)) / h2 for o in ((1, 0), (0, 1)))
+    r = (pair(1, 1, v) - pair(1, -1, v)) / (4 * h2)
+    A, B = ((pair(*o, w) + 2 * at(0, 0, w)) / h2 for o in ((1, 0), (0, 1)))
+    R = (pair(1, 1, w) + pair(1, -1, w)) / (4 * h2)
+    unit = A * np.abs(b) + B * np.abs(a) + 2 * R * np.abs(r)
+    assert np.max(np.abs(f[1:-1, 1:-1] - (a * b - r * r)) / unit) <= 3.0 * 2.0 ** -53
