@@ -76,7 +76,7 @@ struct Params2 {
     double kz;        // 2^-k / 2: z to the change of v
     double inv_h2;
     double c;         // (2^k h^2)^2
-    float ihi, ilo;   // its inverse
+    double inv_c;     // its inverse
     int kexp;         // k, or kNone: the FP64 form everywhere
 };
 constexpr int kNone = 1 << 20;
@@ -108,8 +108,7 @@ Params2 make_params2(double h)
     const double q = std::ldexp(h2, P.kexp), c = q * q;
     P.kz = std::ldexp(0.5, -P.kexp);
     P.c = c;
-    P.ihi = (float)(1.0 / c);
-    P.ilo = (float)(1.0 / c - (double)P.ihi);
+    P.inv_c = 1.0 / c;
     return P;
 }
 
@@ -196,7 +195,7 @@ __device__ __forceinline__ bool update2(Ld ld, Idx sy, double b, const Params2& 
     return true;
 }
 
-// rv + S_h(u) (SIGN = 1) or rv - S_h(u) (SIGN = -1).
+// rv + S_h(u) (SIGN = 1) or rv - S_h(u) (SIGN = -1), the sum in FP64: rv may be of any size.
 template <int SIGN, typename Idx, typename Ld>
 __device__ __forceinline__ double operator2(Ld ld, Idx sy, double rv, const Params2& P)
 {
@@ -206,10 +205,8 @@ __device__ __forceinline__ double operator2(Ld ld, Idx sy, double rv, const Para
     if (P.kexp != kNone && gather2_f2<Idx>(ld, sy, P.kexp, H, &c)) {
         const float scale = fabsf(H[0].hi) + fabsf(H[1].hi) + fabsf(H[2].hi);
         if ((scale > 1.0e-11f && scale < 1.0e15f) || scale == 0.0f) {   // the products' low parts in FP32's range
-            F2 d = f2::mul(f2::add(f2::mul_u(H[0], H[1]), f2::neg(f2::mul_u(H[2], H[2]))), F2{P.ihi, P.ilo});
-            if (SIGN < 0) d = f2::neg(d);
-            const F2 v = f2::add(f2::from_f64(rv), d);
-            return ma::f2d(v.hi) + ma::f2d(v.lo);
+            const F2 d = f2::add(f2::mul_u(H[0], H[1]), f2::neg(f2::mul_u(H[2], H[2])));
+            return fma(SIGN * (ma::f2d(d.hi) + ma::f2d(d.lo)), P.inv_c, rv);
         }
     }
     auto at = [&](Idx o) { return __longlong_as_double(ld(o)); };

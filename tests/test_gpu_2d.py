@@ -205,3 +205,24 @@ def test_smallest_grids_are_solved_to_fp64_digits(n, coarsest, ordering):
     R = (pair(1, 1, w) + pair(1, -1, w)) / (4 * h2)
     unit = A * np.abs(b) + B * np.abs(a) + 2 * R * np.abs(r)
     assert np.max(np.abs(f[1:-1, 1:-1] - (a * b - r * r)) / unit) <= 3.0 * 2.0 ** -53
+
+
+# cube edge and data scale: with u = s L^2 u0(x / L), f is s^2 times that of u0
+@pytest.mark.parametrize("length,s", [(1e-6, 1.0), (1e-3, 1.0), (1e3, 1.0), (1.0, 1e-4), (1.0, 3e-11), (1.0, 1e-12), (1.0, 1e7)])
+@pytest.mark.parametrize("n", [33, 129, 513])
+def test_solves_over_scales(n, length, s):
+    """Solves converge at every scale, and to the unscaled solution: with residuals of tol max f both are
+    within tol |u| of the discrete one.  s = 3e-11 has f about 1e-21."""
+    tol = 1e-10 if n < 513 else 1e-9
+    out = []
+    for L, c in ((1.0, 1.0), (length, s)):
+        pr = P2.make2d("ex1", n)
+        H = M.Hierarchy2D(M.make_desc2d(n, length=L))
+        H.set_rhs_bc(dev(c * c * pr.f), dev(c * L * L * pr.initial()))
+        r = H.solve(tol=tol, max_cycles=25)
+        u = torch.empty((n, n), dtype=torch.float64, device="cuda")
+        H.get_solution(u)
+        H.close()
+        assert r.res <= tol
+        out.append(host(u) / (c * L * L))
+    assert np.max(np.abs(out[0] - out[1])) <= 10 * tol * np.max(np.abs(out[0]))
