@@ -1596,12 +1596,13 @@ struct PhaseSync {
     {
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(now()), "r"(bytes) : "memory");
     }
+    // (acquire at cluster scope: what has come was written by other blocks)
     __device__ __forceinline__ void wait()
     {
         const unsigned b = now(), parity = (t >> 1) & 1;
         unsigned done = 0;
         for (int spin = 0; spin < (1 << 20) && !done && !lost; ++spin)
-            asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+            asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
                          "selp.u32 %0, 1, 0, p;\n}"
                          : "=r"(done)
                          : "r"(b), "r"(parity)
