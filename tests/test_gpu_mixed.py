@@ -511,3 +511,24 @@ def test_fused_tail_cycle_is_bitwise_the_level_by_level_cycle(name, n, coarsest,
     for u, cycles, res in outs[:-1]:
         assert cycles == outs[-1][1] and res == outs[-1][2]
         assert np.array_equal(u, outs[-1][0])
+
+
+@pytest.mark.parametrize("s", [1.0, 1.75, 0.875])
+def test_correction_roots_are_rounded_as_a_newton_step_rounds_them(s):
+    """One colour from e = 0 about u = s |x|^2 / 2, whose Hessian s I, with T = 3 s and M = 3 s^2, is
+    exact in FP32: e / (h^2 / 2) is the root z of (s - z)^3 = s^3 + rhs.  A root between
+    1e-4 and 3e-3 of the entries, where the short iteration gives way to Newton's: rounding M - z (T - z)
+    and z are 2^-24 of z each, and stopping leaves at most 1e-8."""
+    n, h = 33, 1.0 / 32
+    x, y, z = P.grid_coords(n)
+    hi, lo = split(0.5 * s * (x * x + y * y + z * z))
+    assert not lo.any()
+    rng = np.random.default_rng(9)
+    rhs = (3 * s ** 3 * 10.0 ** rng.uniform(-4, -2.5, (n, n, n)) * rng.choice([-1, 1], (n, n, n))).astype(np.float32)
+    e = torch.zeros((n, n, n), dtype=torch.float32, device="cuda")
+    _keep, scr, nb = M.correction_scratch(n)
+    M.ma_smooth_correction_colour(e, dev(hi), dev(lo), dev(rhs), n, h, 0, scr, nb)
+    at = (slice(2, n - 1, 2),) * 3
+    root = s - np.cbrt(s ** 3 + rhs[at].astype(np.longdouble))
+    got = host(e)[at].astype(np.longdouble) / (0.5 * h * h)
+    assert np.max(np.abs(got - root) / np.abs(root)) <= 2 * 2.0 ** -24 + 1e-8
