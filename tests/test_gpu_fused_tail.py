@@ -165,3 +165,33 @@ def test_cluster_cycle_is_bitwise_the_level_by_level_cycle(n, precision, kw, pai
         assert np.array_equal(u, v, equal_nan=True)
         assert (r.cycles, r.status, r.nonconvex_root_events) == (q.cycles, q.status, q.nonconvex_root_events)
         assert r.res == q.res or (np.isnan(r.res) and np.isnan(q.res))
+
+
+@pytest.mark.parametrize("precision", [M.MA_MIXED, M.MA_FP32])
+@pytest.mark.parametrize("n,kw", [(17, {}), (33, {}), (65, {}), (33, dict(coarsest_n=9))])
+def test_the_cluster_runs_where_it_is_the_default(n, kw, precision):
+    """A default cycle's launches against those with a tail bound of 9 set by hand, which leaves the cluster
+    out and nothing else: one cluster launch stands for the levels of 17^3 and 33^3, tens of launches a cycle."""
+    pr = P.make("exp", n)
+    counts = []
+    try:
+        for tail in (True, 9):
+            M.ma_set_corr_tail(tail)
+            H = M.Hierarchy(M.make_desc(n, precision=precision, **kw))
+            H.set_rhs_bc(dev(pr.f), dev(pr.initial()))
+            before = M.ma_kernel_launch_count()
+            H.solve(tol=0.0, max_cycles=2, init=M.MA_INIT_ZERO, raise_on_error=False)
+            counts.append(M.ma_kernel_launch_count() - before)
+            H.close()
+    finally:
+        M.ma_set_corr_tail(True)
+    assert counts[1] - counts[0] >= 20
+
+
+def test_fp64_33_sweeps_are_one_launch():
+    pr = P.make("exp", 33)
+    u = dev(pr.initial())
+    M.ma_smooth_f2(u, dev(pr.f), 33, pr.h, 2)
+    before = M.ma_kernel_launch_count()
+    M.ma_smooth_f2(u, dev(pr.f), 33, pr.h, 2)
+    assert M.ma_kernel_launch_count() - before == 1
