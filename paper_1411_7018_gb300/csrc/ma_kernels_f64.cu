@@ -483,9 +483,17 @@ struct Grid64 {
     smoothf2::Params P;
 };
 
+// A point's new value in FP64 throughout, with a second Newton step: the root to a few ulps.
+__device__ __noinline__ double point_precise(const double* q, int sy, int sz, double rhs6, bool* nonconvex)
+{
+    const double v0 = q[0];
+    const HessS H = gather_hess_of([&](int o) { return q[o]; }, sy, sz, v0);
+    return fma(0.125, smallest_root_precise(H, rhs6, nonconvex), v0);
+}
+
 // nsw sweeps in ascending order; each(p, old, new) sees every update.  The
-// grid's phase threads enter.
-template <typename Each>
+// grid's phase threads enter.  PRECISE: the points by point_precise.
+template <bool PRECISE, typename Each>
 __device__ __forceinline__ void run_sweeps64(const SmallGrid& G, const Grid64& S, int nsw, int nt,
                                              unsigned long long* ev, Each each)
 {
@@ -493,7 +501,8 @@ __device__ __forceinline__ void run_sweeps64(const SmallGrid& G, const Grid64& S
     auto update = [&](int p) {
         const double v0 = S.u[p];
         bool nonconvex = false;
-        const double v = smoothf2::point_sm(S.u + p, n, n * n, S.rhs[p], S.P, &nonconvex);
+        const double v = PRECISE ? point_precise(S.u + p, n, n * n, __dmul_rn(S.P.h6, S.rhs[p]), &nonconvex)
+                                 : smoothf2::point_sm(S.u + p, n, n * n, S.rhs[p], S.P, &nonconvex);
         S.u[p] = v;
         *ev += nonconvex ? 1ull : 0ull;
         each(v0, v);
@@ -653,8 +662,10 @@ __device__ __forceinline__ bool newton5(double* u, const double* rhs, const smoo
 
 // The coarsest grid in shared memory: sweeps until max |du| <= 1e-14 max |u| (at
 // most 100), or a fixed count; on 5^3 Newton's method first, again after every
-// eighth sweep where it did not finish.  On 3^3 the one unknown's root with a
-// Newton step in FP64 (smallest_root_precise).  Every thread of the block
+// eighth sweep where it did not finish.  A fixed count's sweeps, and the one unknown
+// of 3^3, have a second Newton step in FP64 (smallest_root_precise): one leaves
+// 1e-15 of u behind on 5^3 while the points still move, which sweeps to
+// convergence do not see.  Every thread of the block
 // enters; ends with a block barrier.  J: 27 kJ floats.
 __device__ __forceinline__ void coarsest64_sm(const Grid64& S, int n, int sweeps, bool finest, float* J,
                                               unsigned long long* ev)
@@ -678,15 +689,15 @@ __device__ __forceinline__ void coarsest64_sm(const Grid64& S, int n, int sweeps
         }
     } else if ((int)threadIdx.x < nt) {
         const SmallGrid G(n);
-        for (int s = 0; s < max_sweeps; ++s) {
-            if (n == 5 && sweeps == 0 && (s & 7) == 0 && S.P.kexp != smoothf2::kNone && newton5(S.u, S.rhs, S.P, J, finest))
+        if (sweeps > 0) run_sweeps64<true>(G, S, sweeps, nt, ev, [](double, double) {});
+        for (int s = 0; s < max_sweeps && sweeps == 0; ++s) {
+            if (n == 5 && (s & 7) == 0 && S.P.kexp != smoothf2::kNone && newton5(S.u, S.rhs, S.P, J, finest))
                 break;
             double du = 0.0, um = 0.0;
-            run_sweeps64(G, S, 1, nt, ev, [&](double v0, double v) {
+            run_sweeps64<false>(G, S, 1, nt, ev, [&](double v0, double v) {
                 du = fmax(du, fabs(v - v0));
                 um = fmax(um, fabs(v));
             });
-            if (sweeps > 0) continue;
             for (int o = 16; o > 0; o >>= 1) {
                 du = fmax(du, __shfl_xor_sync(0xffffffffu, du, o));
                 um = fmax(um, __shfl_xor_sync(0xffffffffu, um, o));
@@ -790,7 +801,7 @@ __device__ __forceinline__ Tail64Smem tail64_fields(const Tail64Args& A, double*
 __device__ __forceinline__ void tail64_smooth(const Grid64& S, int n, int nsw, unsigned long long* ev)
 {
     const int nt = phase_threads(n, T64);
-    if ((int)threadIdx.x < nt && nsw > 0) run_sweeps64(SmallGrid(n), S, nsw, nt, ev, [](double, double) {});
+    if ((int)threadIdx.x < nt && nsw > 0) run_sweeps64<false>(SmallGrid(n), S, nsw, nt, ev, [](double, double) {});
     __syncthreads();
 }
 

@@ -707,3 +707,42 @@ def test_5_cubed_alone_is_solved_to_fp64_digits(name, single):
     unit = A * np.abs(b * d - t * t) + B * np.abs(a * d - s * s) + D * np.abs(a * b - r * r) + \
         2 * (R * np.abs(s * t - r * d) + S * np.abs(r * t - s * b) + T * np.abs(r * s - t * a))
     assert np.max(np.abs(pr.f[1:-1, 1:-1, 1:-1] - det) / unit) <= 3.0 * 2.0 ** -53
+
+
+def _extended_sweep(u, f, h):
+    """One eight-colour Gauss-Seidel sweep in place, in extended precision (Newton from the centre)."""
+    n = u.shape[0]
+    h2 = np.longdouble(h) ** 2
+    for c in range(8):
+        par = (c & 1, (c >> 1) & 1, (c >> 2) & 1)   # of i, j, k
+
+        def at(i, j, k):
+            return u[tuple(slice((1 if p else 2) + o, n - 1 + o, 2) for p, o in zip(par[::-1], (k, j, i)))]
+        if at(0, 0, 0).size == 0:
+            continue
+        v = at(0, 0, 0)
+        a, b, d = (((at(*o) - v) + (at(*(-x for x in o)) - v)) / h2 for o in ((1, 0, 0), (0, 1, 0), (0, 0, 1)))
+        r, s, t = ((at(*p) + at(*(-x for x in p)) - at(*q) - at(*(-x for x in q))) / (4 * h2)
+                   for p, q in (((1, 1, 0), (1, -1, 0)), ((1, 0, 1), (1, 0, -1)), ((0, 1, 1), (0, 1, -1))))
+        rhs = f[tuple(slice(1 if p else 2, n - 1, 2) for p in par[::-1])]
+        z = np.zeros_like(v)
+        for _ in range(12):
+            x, y, w = a - z, b - z, d - z
+            g = x * (y * w - t * t) - r * (r * w - s * t) + s * (r * t - y * s) - rhs
+            z = z + g / (x * y - r * r + x * w - s * s + y * w - t * t)
+        v += h2 * z / 2
+
+
+@pytest.mark.parametrize("name,n,sweeps", [("exp", 5, 1), ("exp", 5, 4), ("sine", 5, 2), ("exp", 7, 2), ("exp", 9, 2),
+                                           ("sine", 17, 1)])
+def test_fixed_coarsest_sweeps_are_rounded_as_fp64(name, n, sweeps):
+    """A fixed number of coarsest sweeps from a rough start against the same in extended precision.  A point's
+    update averages its neighbours: their sums, the centre's and the result are rounded at 2^-53 |u| each, and
+    a point takes over its neighbours' errors at most once in the average, sweep by sweep: 4 (sweeps + 1)."""
+    pr, u0 = perturbed(name, n, 1e-2 / (n - 1) ** 2)
+    ref = u0.astype(np.longdouble)
+    for _ in range(sweeps):
+        _extended_sweep(ref, pr.f, pr.h)
+    u = dev(u0)
+    M.ma_coarsest_solve(u, dev(pr.f), n, pr.h, sweeps)
+    assert np.max(np.abs(host(u) - ref)) <= 4 * (sweeps + 1) * 2.0 ** -53 * np.max(np.abs(u0))
