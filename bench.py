@@ -740,7 +740,9 @@ def main():
                          "launch_ms_stream_launched": corr_launch_ms_stream,
                          "bytes_per_point": CORR_SMOOTH_BYTES_PER_POINT,
                          "peak_source": peak_src},
-            "roofline_fp64_smoother": {"bound": "alu", "kernel": "k_smooth_colour (FP64 smoother, one colour phase)",
+            "roofline_fp64_smoother": {"bound": "alu",
+                                       "kernel": "k_smooth_colour (ma_smooth, the FP64 single step, one colour "
+                                                 "phase; FP64 cycles run k_smooth_f2, off the FP64 pipe)",
                                        "achieved": f64_gops, "peak": fp64_peak_gops, "unit": "GFP64op/s",
                                        "frac": f64_gops / fp64_peak_gops, "launch_ms": f64_launch_ms,
                                        "ops_per_point": SMOOTH_FP64_OPS_PER_POINT,

@@ -49,7 +49,10 @@ typedef struct {
 ma_status ma2d_hierarchy_footprint(const ma2d_desc *desc, size_t *bytes);
 
 /* Build a hierarchy in the caller's workspace (>= footprint bytes, 256-byte
- * aligned; the caller keeps it alive until ma2d_destroy_hierarchy). */
+ * aligned; the caller keeps it alive until ma2d_destroy_hierarchy).  It also
+ * holds 32 bytes of pinned host memory, a stream for graph capture, and one CUDA
+ * graph for the cycle and for each kind of start that ma2d_solve has run (recorded
+ * on first use). */
 ma_status ma2d_create_hierarchy(const ma2d_desc *desc, void *dev_workspace, size_t bytes, ma_stream_t stream,
                                 ma2d_hierarchy **out);
 

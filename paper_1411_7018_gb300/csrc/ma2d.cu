@@ -80,11 +80,11 @@ struct Params2 {
     int kexp;         // k, or kNone: the FP64 form everywhere
 };
 constexpr int kNone = 1 << 20;
-// Grids that take the two-float forms.  Above 4097^2 the rounding of the FP64
-// forms (eps |u| / h^2, 1e-8 of D^2 u) shows in the solution itself: after the FMG
-// pass at 8193^2 it is 5e-11 from the two-float one, a twentieth of the scheme's
-// error (1.059e-9 against 1.114e-9 for u = exp((x^2 + y^2) / 2)), and grids of
-// that size keep the FP64 values.
+// Grids that take the two-float forms.  The upper bound is there for the paper's
+// Table 1: at 8193^2 the rounding of the FP64 forms (eps |u| / h^2, 1e-8 of D^2 u)
+// moves the solution after one FMG pass by 5e-11, which happens to bring its error
+// nearer to the printed 1.0e-9 (1.059e-9, against 1.114e-9 in two floats, a quarter of
+// 4097^2's as the scheme has it).  Values of that size are kept as they were.
 // Hierarchies whose finest grid has fewer than 17^2 points keep FP64 on every
 // level: there the two-float determinant rounds more than the FP64 gather does
 // (4 to 6 units of the stencil's rounding on 9^2 against 1); above, the solutions'

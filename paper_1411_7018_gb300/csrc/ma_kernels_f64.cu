@@ -9,9 +9,11 @@
 //   prolongation    Section 3 trilinear, Algorithm 1 steps 7-8
 //   coarsest solve  Algorithm 1 step 1, one thread block
 //
-// FP64 throughput is the bound of these kernels on GB300 (FP64 issues at
-// about 1/70 of the FP32 rate), so the point solve keeps its FP64 work to the
-// stencil, one determinant and one Newton correction (ma_point.cuh).
+// GB300 issues FP64 at about 1/70 of its FP32 rate.  The cycles' sweeps,
+// residuals and coarse right-hand sides therefore take integer differences and
+// two floats (ma_smooth_f2.cuh, ma_residual.cuh), two or three FP64 operations a
+// point.  The single steps ma_smooth and ma_residual are FP64 throughout
+// (ma_point.cuh), and bound by that pipe, as are the transfers.
 #include <algorithm>
 #include <atomic>
 #include <cstring>
@@ -408,8 +410,8 @@ __device__ __forceinline__ double operator_point(const double* q, int sy, int sz
 // Over a grid, 0 on the shell: one point a thread, the grid size at compile time
 // for the sizes of a hierarchy's larger levels.  The FP64 forms of the two were
 // bound by the FP64 pipe (257^3: 754 us residual, 800 us right-hand side); this
-// one by issue, 248 us at 257^3, 36 against 98 at 129^3, 8.3 against 22 at 65^3,
-// 3.8 against 7.2 at 33^3 (Example 4, graph replay).  Runs of planes a thread,
+// one by issue, 250 us at 257^3, 36 against 98 at 129^3, 8.7 against 22 at 65^3,
+// 4.0 against 7.2 at 33^3 (Example 4, graph replay).  Runs of planes a thread,
 // as the residual with norms walks them, keep more values live (76 registers
 // for 64): 297 us.
 template <int NN, int SIGN, bool UNORM>
@@ -1360,10 +1362,11 @@ cudaError_t launch_coarsest(double* u, const double* rhs, int n, double h, int s
     return cudaGetLastError();
 }
 
-// Largest level of the fused FP64 tail.  One block runs the tail on one SM,
-// whose FP64 pipe then does all the point solves: at 17^3 (3375 points a
-// sweep) that costs more than 8 colour launches spread over the GPU, at 9^3
-// and below the launches cost more.
+// Largest level of the fused FP64 tail.  At 17^3 one SM's phases (512 points,
+// a warp's chain on every scheduler four deep) take longer than 7 launches a
+// sweep spread over the GPU, at 9^3 and below (91 points) the launches do.  FP64
+// solves to 1e-10 with a bound of 5 / 9 / 17, ms: 33^3 2.95 / 2.54 / 2.90, 65^3 4.75 /
+// 4.25 / 4.69, 129^3 8.95 / 8.47 / 8.94, 257^3 30.5 / 30.0 / 30.6.
 constexpr int kVTailDefault = 9;
 static std::atomic<int> g_vtail_max{kVTailDefault};
 

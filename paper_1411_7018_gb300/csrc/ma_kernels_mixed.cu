@@ -1024,7 +1024,8 @@ __global__ void __launch_bounds__(BX * BY, 8) k_residual_corr_col(const float* _
 // times (planes + 2).  At 129^3 that is 9 planes in two waves, 19.0 us, where 8
 // leave a third wave nearly empty, 21.1 us.  Runs of 3 planes would take 65^3
 // from 6.9 to 5.5 us alone, but cost 24 solves side by side 2 % in loads.  (More
-// resident blocks are slower: 10 an SM 151.8 against 143.6 us at 257^3.)
+// resident blocks are slower: 10 an SM 151.8 against 143.6 us at 257^3.)  152 SMs are a
+// whole GB300; on a part of one the waves are counted wrong, which costs time only.
 inline dim3 col_grid(int n, int kc) { return dim3((n - 2 + CW - 1) / CW, (n - 2 + 3) / 4, (n - 2 + kc - 1) / kc); }
 
 int col_chunk(int n)

@@ -178,11 +178,12 @@ inline dim3 grid_for(int n, int kz) { return dim3((n + RX - 1) / RX, (n + RY - 1
 //    differences of 4 h^2 D^2_h u (the sums of Eq. MA_discrete's stencil,
 //    Section 2) are formed exactly in int64 -- more accurately than the FP64
 //    gather, which rounds the sums u(x+h) + u(x-h).
-//  * The determinant and rhs - det / (64 h^6) are then evaluated in
-//    two-float arithmetic (value = hi + lo, two FP32 numbers, about 48
-//    significant bits), with Knuth's two-sum and the FMA form of Dekker's
-//    exact product: |error| of a few 2^-46 relative to the sum of the
-//    magnitudes of the determinant's terms.
+//  * The determinant is then evaluated in two-float arithmetic (value = hi +
+//    lo, two FP32 numbers, about 48 significant bits), with Knuth's two-sum and
+//    the FMA form of Dekker's exact product: |error| of a few 2^-46 relative to
+//    the sum of the magnitudes of the determinant's terms, 3e-15 rms and without
+//    a bias.  rhs - det is taken in FP64 where the output is FP64, in two floats
+//    where it is FP32.
 // A stencil that changes binade or sign is handled the same way, each value
 // as a fixed-point number of the largest one's scale with 7 bits to spare.
 //
@@ -608,6 +609,8 @@ __device__ __forceinline__ void residual_f2_block(const double* __restrict__ u, 
     }
 }
 
+// (8 and 5 resident blocks: the registers, 64 and 96, that the code took before it had FP64 calls, which
+// alone would take 72; none spill)
 template <typename Out, int NN = 0>
 __global__ void __launch_bounds__(RX * RY, NN > 0 ? 8 : 5) k_residual_f2(const double* __restrict__ u, const double* __restrict__ rhs,
                                                          Out out, int n, Scaling P, double* partials, int kchunk)
