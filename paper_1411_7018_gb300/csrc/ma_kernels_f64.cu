@@ -410,13 +410,15 @@ __device__ __forceinline__ double operator_point(const double* q, int sy, int sz
 // Over a grid, 0 on the shell: one point a thread, the grid size at compile time
 // for the sizes of a hierarchy's larger levels.  The FP64 forms of the two were
 // bound by the FP64 pipe (257^3: 754 us residual, 800 us right-hand side); this
-// one by issue, 250 us at 257^3, 36 against 98 at 129^3, 8.7 against 22 at 65^3,
-// 4.0 against 7.2 at 33^3 (Example 4, graph replay).  Runs of planes a thread,
-// as the residual with norms walks them, keep more values live (76 registers
-// for 64): 297 us.
+// one by issue, 240 us at 257^3, 35 against 98 at 129^3, 8.7 against 22 at 65^3,
+// 3.9 against 7.2 at 33^3 (Example 4, graph replay; nine resident blocks, 56
+// registers and 8 bytes of spills, against eight: 253 us at 257^3).  Runs of
+// planes a thread, as the residual with norms walks them, keep more values live
+// (76 registers for 64): 297 us.
 template <int NN, int SIGN, bool UNORM>
-__global__ void __launch_bounds__(BX * BY) k_operator_f2(const double* __restrict__ u, const double* __restrict__ r,
-                                                         double* __restrict__ out, int n_rt, resid::Scaling P)
+__global__ void __launch_bounds__(BX * BY, NN > 0 ? 9 : (UNORM ? 8 : 6))
+    k_operator_f2(const double* __restrict__ u, const double* __restrict__ r, double* __restrict__ out, int n_rt,
+                  resid::Scaling P)
 {
     const int n = NN > 0 ? NN : n_rt;
     const int i = blockIdx.x * BX + threadIdx.x;
