@@ -609,11 +609,12 @@ __device__ __forceinline__ void residual_f2_block(const double* __restrict__ u, 
     }
 }
 
-// (8 and 5 resident blocks: the registers, 64 and 96, that the code took before it had FP64 calls, which
-// alone would take 72; none spill)
+// 8 resident blocks at 64 registers (5 at 96 with the size at run time): left to
+// itself the compiler takes 72 for the calls of the second walk.  None spill.
 template <typename Out, int NN = 0>
-__global__ void __launch_bounds__(RX * RY, NN > 0 ? 8 : 5) k_residual_f2(const double* __restrict__ u, const double* __restrict__ rhs,
-                                                         Out out, int n, Scaling P, double* partials, int kchunk)
+__global__ void __launch_bounds__(RX * RY, NN > 0 ? 8 : 5)
+    k_residual_f2(const double* __restrict__ u, const double* __restrict__ rhs, Out out, int n, Scaling P,
+                  double* partials, int kchunk)
 {
     residual_f2_block<Out, NN>(u, rhs, out, n, P, partials, kchunk, blockIdx, gridDim);
 }
